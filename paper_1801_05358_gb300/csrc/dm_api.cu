@@ -46,15 +46,16 @@ void free_all(dm_plan *p) {
   void *ptrs[] = {p->rings, p->pairs, p->phase, p->bhat, p->twid, p->rec, p->seed, p->seed_exp, p->cl,
                   p->filt, p->w, p->mask, p->sigma, p->rc, p->a, p->apart, p->wd, p->norms, p->state,
                   p->lev, p->tmpmap, p->tmpmap2, p->tmpalm, p->seeds_dev, p->coef_tmp,
-                  p->ptab, p->rc32, p->apart32, p->s32, p->w32, p->wd32, p->phase32, p->bhat32, p->twid32,
+                  p->rc32, p->apart32, p->s32, p->w32, p->wd32, p->phase32, p->bhat32, p->twid32,
                   p->a_hi, p->g_hi, p->shi32, p->s64, p->rhi, p->tc_err, p->ring_order, p->pair_order,
                   p->tc_synA[0], p->tc_synA[1], p->tc_anaA[0], p->tc_anaA[1], p->tc_soff, p->tc_aoff,
-                  p->tc_synB[0], p->tc_synB[1], p->ptab_lo, p->e32, p->c32, p->clev, p->filt32,
+                  p->tc_synB[0], p->tc_synB[1], p->e32, p->c32, p->clev, p->filt32,
                   p->twr, p->twr32, p->chirp, p->chirp32, p->wcov, p->diag_tab, p->diag_alm, p->diag_part,
                   p->diag_ao, p->covdraw, p->jsrc, p->jacc, p->bhatT[0], p->bhatT[1], p->bhatT32[0],
-                  p->bhatT32[1], p->ck0, p->ck2, p->cko, p->rq0, p->rq2, p->rq2d, p->ffs, p->ffs_lo};
+                  p->bhatT32[1], p->ck0, p->ck2, p->cko, p->rq0, p->rq2, p->rq2d};
   for (void *q : ptrs)
     if (q) cudaFree(q);
+  split_release(p);
   if (p->ev_begin) cudaEventDestroy(p->ev_begin);
   if (p->ev_end) cudaEventDestroy(p->ev_end);
 }
@@ -466,6 +467,9 @@ dm_status plan_workspace(dm_plan *p, dm_plan **out) {
   if ((e = dalloc(p, &p->coef_tmp, 4 * (size_t)L))) return bad(e, "alloc coef");
   if ((e = dalloc(p, &p->s64, (size_t)B * n3))) return bad(e, "alloc s");
   if ((e = dalloc(p, &p->rhi, (size_t)B * n3))) return bad(e, "alloc rhi");
+  if ((e = dalloc(p, &p->tc_err, 1))) return bad(e, "alloc");
+  cudaMemset(p->tc_err, 0, sizeof(int));
+  if (!p->flat) split_new(p);
   if ((e = cudaEventCreate(&p->ev_begin)) || (e = cudaEventCreate(&p->ev_end))) return bad(e, "events");
   cudaMemset(p->rc, 0, sizeof(double2) * (size_t)B * 3 * (p->mmax + 1) * p->npairs * 2);
   cudaMemset(p->mask, 1, (size_t)B * p->npix);
@@ -526,7 +530,7 @@ dm_status dm_plan_info(const dm_plan *p, int64_t *npix, int64_t *nalm, int *nrin
   if (npix) *npix = p->npix;
   if (nalm) *nalm = p->nalm;
   if (nrings) *nrings = p->nrings;
-  if (ws) *ws = p->bytes;
+  if (ws) *ws = p->bytes + split_bytes(p);
   return DM_OK;
 }
 
@@ -924,10 +928,7 @@ dm_status dm_set_ff_slab_bytes(dm_plan *p, int64_t bytes) {
   if (p->session) return DM_EBUSY;
   p->ffs_cap = bytes;
   p->ffs_cap_set = true;
-  if (p->ffs) cudaFree(p->ffs);
-  if (p->ffs_lo) cudaFree(p->ffs_lo);
-  p->ffs = p->ffs_lo = nullptr;
-  p->ffs_m.clear();
+  split_forget(p);
   return DM_OK;
 }
 

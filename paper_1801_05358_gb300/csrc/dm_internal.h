@@ -67,6 +67,8 @@ struct RingClass {
   int poff, pcount;  // pair_order[poff .. poff + pcount): the northern (or equatorial) rings of the class
 };
 
+struct SplitTables;  // dm_split.cu
+
 struct LevelDev {
   int n_levels;
   int max_iter;
@@ -140,7 +142,6 @@ struct dm_plan {
   double2 *apart = nullptr;     // [B][nchunk][3][nalm] analysis partial sums
   int nchunk = 0;               // pair chunks of the analysis
   int nslot = 0;                // chunk slots of apart per RHS (nslot < nchunk: the analysis runs in waves)
-  int nchunk32 = 0;             // chunks of apart32 per RHS: nchunk, or 1 (tensor-core analysis only) when that is over 24 GiB
   double *wd = nullptr;         // [B][3][npix] w * d
   double *norms = nullptr;      // [B][3][nrings][2] Cauchy partial sums
   dmwf::SolveState *state = nullptr;   // [B]
@@ -155,21 +156,16 @@ struct dm_plan {
   int64_t bytes = 0;
   // DM_MIXED_FP32 resources (allocated by dm_set_precision)
   bool fp32_ready = false;      // the buffers of the FP32 modes exist (setup_fp32 succeeded)
-  // Full FP32 tables: built on first use by the kernels that read them (the
-  // CUDA-core FP32 Legendre stages and the stored-table tensor-core tiles).
-  // The float-float stages read them when present and otherwise generate
-  // them per slab of orders m into ffs / ffs_lo.
-  float *ptab = nullptr;        // [3][nalm][npairs] lambda, lam+, lam- in FP32 (FP64 recurrence)
-  float *ptab_lo = nullptr;     // [3][nalm][npairs] FP64 value - ptab: float-float tables
-  float *ffs = nullptr, *ffs_lo = nullptr;  // slab tables of the float-float stages
-  std::vector<int> ffs_m;       // slab boundaries in m (first orders, then mmax + 1)
-  int64_t ffs_cap = (int64_t)1 << 30;  // bytes of the largest slab (hi and lo)
-  bool ffs_cap_set = false;     // dm_set_ff_slab_bytes was called: slabs of that size, no full tables
+  // digit tables of the split products (dm_split.cu): shared with the views of the plan
+  dmwf::SplitTables *split = nullptr;
+  int64_t split_cap = (int64_t)24 << 30;  // largest whole table kept
+  int64_t ffs_cap = (int64_t)1 << 30;  // bytes of the largest slab when the table is not kept whole
+  bool ffs_cap_set = false;     // dm_set_ff_slab_bytes was called: slabs of that size, no whole table
   bool ff_legendre = false;     // DM_FLOAT_FLOAT: Legendre stages in float-float
   bool anchor_ff = true;        // mixed-mode anchors in float-float (else FP64)
   bool ff_now = false;          // inside a float-float anchor
   float2 *rc32 = nullptr;       // [B][3][mmax+1][npairs][2]
-  float2 *apart32 = nullptr;    // [B][nchunk][3][nalm]
+  float2 *apart32 = nullptr;    // [B][3][nalm] analysis sums
   float *s32 = nullptr;         // [B][3][npix] iteration map
   float *w32 = nullptr;         // [B][3][npix]
   float *wd32 = nullptr;        // [B][3][npix]
@@ -191,7 +187,7 @@ struct dm_plan {
   bool use_tc = true;           // tcgen05 Legendre stages when the batch allows
   int *tc_err = nullptr;        // device flag: a bounded tensor-core wait gave up
   int tc_withhold = 0;          // test hook: one withheld arrival in the spin-0 analysis (dm_test_tc_withhold)
-  // tiled BF16 hi/lo copies of ptab for the tensor-core stages ([0] = lambda, [1] = lam+/lam-)
+  // tiled BF16 hi/lo Legendre tables of the tensor-core stages ([0] = lambda, [1] = lam+/lam-)
   unsigned char *tc_synA[2] = {nullptr, nullptr}, *tc_anaA[2] = {nullptr, nullptr};
   int64_t *tc_soff = nullptr, *tc_aoff = nullptr;  // block offsets per m / per (m, parity)
   unsigned char *tc_synB[2] = {nullptr, nullptr};   // per-iteration synthesis B operand tiles
@@ -305,7 +301,7 @@ cudaError_t cov_ring_stage(dm_plan *p, cudaStream_t st);
 cudaError_t cov_ring_stage32(dm_plan *p, cudaStream_t st);      // the mixed mode's (FP32 state)
 cudaError_t anchor_residual_wd_cov(dm_plan *p, const double *s_hi, cudaStream_t st);
 cudaError_t setup_fp32(dm_plan *p);
-cudaError_t ensure_ptab(dm_plan *p);  // the full FP32 tables, built on first use
+cudaError_t gen_tables32(dm_plan *p, float *tab, cudaStream_t st);  // FP32 Legendre tables (dm_legendre.cu)
 // Raise a kernel's dynamic shared-memory limit on the current device to at
 // least `bytes`, never lowering it.  The limit is a process-wide attribute of
 // the function: set per launch, a smaller value set by a plan on another host
@@ -318,7 +314,18 @@ inline cudaError_t dyn_smem_allow(F *func, size_t bytes) {
 }
 // first alm index of order m (m = mmax + 1 = lmax + 1 gives nalm): idx(l, m) = start(m) + l - m
 inline int64_t alm_start_h(int lmax, int m) { return (int64_t)m * (2 * lmax + 3 - m) / 2; }
-cudaError_t gen_tables32_slab(dm_plan *p, float *hi, float *lo, int m0, int m1, cudaStream_t st);                          // tables and buffers of DM_MIXED_FP32
+// split products of the Legendre stages (dm_split.cu)
+void split_new(dm_plan *p);
+void split_release(dm_plan *p);
+void split_forget(dm_plan *p);
+int64_t split_bytes(const dm_plan *p);
+size_t split_table_bytes(int lmax, int mmax, int npairs);
+size_t split_scratch_bytes(int lmax, int npairs, int batch);  // upper bound of the column digits
+void split_disable(dm_plan *p);                                // the direct kernels only
+cudaError_t split_synthesis64(dm_plan *p, const double2 *alm, cudaStream_t st, bool *ran);
+cudaError_t split_analysis64(dm_plan *p, cudaStream_t st, bool *ran);
+cudaError_t split_synthesis32(dm_plan *p, const double2 *alm, const float2 *e32, cudaStream_t st);
+cudaError_t split_analysis32(dm_plan *p, cudaStream_t st);
 cudaError_t copy_s32_to_user(dm_plan *p, double *s_out, cudaStream_t st);
 // anchor residual: r = w (d - s_hi) (or d on observed pixels when s_hi == nullptr),
 // written to p->wd; shi32 = s_hi in FP32
@@ -337,10 +344,8 @@ bool tc_generate(dm_plan *p);                               // the plan's resolv
 size_t gen_bytes(int lmax, int mmax, int npairs);
 cudaError_t syn_gen_launch(dm_plan *p, bool run0, bool run1, cudaStream_t st);
 cudaError_t ana_gen_launch(dm_plan *p, cudaStream_t st);
-cudaError_t legendre_synthesis_ff(dm_plan *p, const double2 *alm, cudaStream_t st);
 cudaError_t anchor_c32(dm_plan *p, cudaStream_t st);     // c = F (a_hi + g_hi) - a_hi, e = 0
 cudaError_t materialize_a(dm_plan *p, cudaStream_t st);  // a = a_hi + e
-cudaError_t legendre_analysis_ff_parts(dm_plan *p, cudaStream_t st, int *used);
 cudaError_t fold_slots(dm_plan *p, int nused, int m0, int m1, cudaStream_t st);
 // Partial sums of the FP64-class analysis over every pair chunk into apart,
 // in waves of at most nslot chunks when the plan holds fewer slots than

@@ -107,7 +107,9 @@ cudaError_t legendre_analysis32(dm_plan *p, int epilogue, double2 *out, cudaStre
 cudaError_t legendre_synthesis(dm_plan *p, const double2 *alm, cudaStream_t st) {
   if (p->flat) return flat_synthesis(p, alm, st);  // flat sky: column transforms (dm_flat.cu)
   if (p->prec != DM_FP64) return legendre_synthesis32(p, alm, st);
-  if (p->ff_legendre || p->ff_now) return legendre_synthesis_ff(p, alm, st);
+  bool ran = false;
+  cudaError_t e = split_synthesis64(p, alm, st, &ran);
+  if (e || ran) return e;
   dim3 grid((p->npairs + SYN_THREADS - 1) / SYN_THREADS, p->mmax + 1, p->batch);
   k_leg_syn64<<<grid, SYN_THREADS, 0, st>>>(p->pairs, p->rec, p->seed, p->seed_exp, alm, p->rc, p->lmax, p->mmax,
                                            p->npairs, p->nalm, p->state_active ? p->state : nullptr);
@@ -289,9 +291,11 @@ cudaError_t legendre_analysis(dm_plan *p, int epilogue, double2 *out, cudaStream
   if (p->prec != DM_FP64) return legendre_analysis32(p, epilogue, out, st, mid);
   const SolveState *stp = p->state_active ? p->state : nullptr;
   int used = p->nchunk;
-  cudaError_t e = (p->ff_legendre || p->ff_now) ? legendre_analysis_ff_parts(p, st, &used)
-                                                : analysis64_parts(p, st, &used);
+  bool ran = false;
+  cudaError_t e = split_analysis64(p, st, &ran);
+  if (!e && !ran) e = analysis64_parts(p, st, &used);
   if (e) return e;
+  if (ran) used = 1;
   if (mid) cudaEventRecord(mid, st);
   double omega = 4.0 * M_PI / (double)p->npix;
   dim3 g2((unsigned)((p->lmax + 1 + 127) / 128), p->batch, p->mmax + 1);
@@ -325,19 +329,16 @@ cudaError_t apply_filter_level(dm_plan *p, const double *coef, const double2 *in
 }
 
 // ======================================================================
-// DM_MIXED_FP32: Legendre values from the FP64 recurrence, stored once in
-// FP32 tables ptab[f][idx(l, m)][pair] (f = lambda, lam+, lam-); FP32
-// contraction; FP32 ring coefficients; FP64 harmonic state and filter.
+// DM_MIXED_FP32: FP32 ring coefficients and harmonic state between anchors.
 // ======================================================================
 
-// Tables of the orders m0 + blockIdx.y: entry (idx(l, m) - base0) * npairs +
-// pair of each function plane (plane entries apart), base0 = idx(m0, m0).
+// FP32 tables [3][nalm][npairs] of lambda, lam+, lam- from the FP64
+// recurrence, from which the stored BF16 tiles are cut.
 __global__ void __launch_bounds__(128) k_gen_tables(const PairDev *__restrict__ pairs, const RecCoef *__restrict__ rec,
                                                     const double *__restrict__ seed, const int *__restrict__ seed_exp,
-                                                    float *__restrict__ ptab, float *__restrict__ ptab_lo, int lmax,
-                                                    int npairs, int m0, int64_t base0, int64_t plane) {
+                                                    float *__restrict__ ptab, int lmax, int npairs, int64_t plane) {
   __shared__ RecCoef sc[SYN_CH];
-  const int m = m0 + blockIdx.y;
+  const int m = blockIdx.y;
   const int p = blockIdx.x * 128 + threadIdx.x;
   const bool act = p < npairs;
   const int pp = act ? p : npairs - 1;
@@ -353,244 +354,37 @@ __global__ void __launch_bounds__(128) k_gen_tables(const PairDev *__restrict__ 
     for (int j = 0; j < cnt; ++j) {
       const int l = lc + j;
       if (act) {
-        const int64_t o = (base + l - base0) * (int64_t)npairs + p;
+        const int64_t o = (base + l) * (int64_t)npairs + p;
         const bool live = (s.S == 0);
-        const double v0 = live ? s.l0 : 0.0, v1 = live ? 0.5 * (s.p0 + s.q0) : 0.0,
-                     v2 = live ? 0.5 * (s.p0 - s.q0) : 0.0;
-        const float h0 = (float)v0, h1 = (float)v1, h2 = (float)v2;
-        ptab[o] = h0;
-        ptab[plane + o] = h1;
-        ptab[2 * plane + o] = h2;
-        ptab_lo[o] = (float)(v0 - (double)h0);
-        ptab_lo[plane + o] = (float)(v1 - (double)h1);
-        ptab_lo[2 * plane + o] = (float)(v2 - (double)h2);
+        ptab[o] = live ? (float)s.l0 : 0.f;
+        ptab[plane + o] = live ? (float)(0.5 * (s.p0 + s.q0)) : 0.f;
+        ptab[2 * plane + o] = live ? (float)(0.5 * (s.p0 - s.q0)) : 0.f;
       }
       if (l < lmax) rec_advance(s, sc[j], x, m, l, seed, pp, npairs);
     }
   }
 }
 
-// Tables of the orders [m0, m1) into hi / lo, laid out as the full tables
-// restricted to those orders (planes of (idx(m1, m1) - idx(m0, m0)) x npairs).
-cudaError_t gen_tables32_slab(dm_plan *p, float *hi, float *lo, int m0, int m1, cudaStream_t st) {
-  if (m1 <= m0) return cudaSuccess;
-  const int64_t b0 = alm_start_h(p->lmax, m0), b1 = alm_start_h(p->lmax, m1);
-  dim3 g((p->npairs + 127) / 128, m1 - m0);
-  k_gen_tables<<<g, 128, 0, st>>>(p->pairs, p->rec, p->seed, p->seed_exp, hi, lo, p->lmax, p->npairs, m0, b0,
-                                  (b1 - b0) * (int64_t)p->npairs);
+cudaError_t gen_tables32(dm_plan *p, float *tab, cudaStream_t st) {
+  dim3 g((p->npairs + 127) / 128, p->mmax + 1);
+  k_gen_tables<<<g, 128, 0, st>>>(p->pairs, p->rec, p->seed, p->seed_exp, tab, p->lmax, p->npairs,
+                                  p->nalm * (int64_t)p->npairs);
   return cudaGetLastError();
 }
 
-// Synthesis, FP32 contraction over l; NB right-hand sides per thread.
-// grid: (batch / NB, pair blocks, m); consecutive blocks share the table tile in L2.
-template <int NB>
-__global__ void __launch_bounds__(SYN_THREADS) k_leg_syn32(const float *__restrict__ ptab,
-                                                           const double2 *__restrict__ alm,
-                                                           const double2 *__restrict__ a_sub,
-                                                           const float2 *__restrict__ e32,
-                                                           float2 *__restrict__ rc, int lmax, int mmax, int npairs,
-                                                           int64_t nalm, const SolveState *__restrict__ state) {
-  __shared__ float2 sT[NB][SYN_CH], sE[NB][SYN_CH], sB[NB][SYN_CH];
-  const int b0 = blockIdx.x * NB, m = blockIdx.z;
-  bool any = false;
-  for (int k = 0; k < NB; ++k) any = any || state == nullptr || !state[b0 + k].done;
-  if (!any) return;
-  const int p = blockIdx.y * SYN_THREADS + threadIdx.x;
-  const bool act = p < npairs;
-  const int pp = act ? p : npairs - 1;
-  float2 T0[NB], T1[NB], Q0[NB], Q1[NB], U0[NB], U1[NB];
-#pragma unroll
-  for (int k = 0; k < NB; ++k) {
-    T0[k] = T1[k] = Q0[k] = Q1[k] = U0[k] = U1[k] = make_float2(0.f, 0.f);
-  }
-  const int64_t base = alm_base(lmax, m);
-  const int64_t plane = nalm * (int64_t)npairs;
-  const float *P0 = ptab + base * npairs + pp, *Pp = P0 + plane, *Pq = P0 + 2 * plane;
-  for (int lc = m; lc <= lmax; lc += SYN_CH) {
-    const int cnt = min(SYN_CH, lmax + 1 - lc);
-    __syncthreads();
-    for (int i = threadIdx.x; i < cnt * NB; i += SYN_THREADS) {
-      const int k = i / cnt, j = i % cnt;
-      const int64_t ob = (int64_t)(b0 + k) * 3 * nalm + base + lc + j;
-      if (e32 != nullptr) {  // FP32 iteration state e = a - a_hi
-        const float2 t = e32[ob], e = e32[ob + nalm], bb = e32[ob + 2 * nalm];
-        sT[k][j] = t;
-        sE[k][j] = make_float2(-e.x, -e.y);
-        sB[k][j] = make_float2(-bb.x, -bb.y);
-        continue;
-      }
-      double2 t = alm[ob], e = alm[ob + nalm], bb = alm[ob + 2 * nalm];
-      if (a_sub != nullptr) {  // correction e = a - a_hi (FP64 difference, then FP32)
-        t = csub(t, a_sub[ob]);
-        e = csub(e, a_sub[ob + nalm]);
-        bb = csub(bb, a_sub[ob + 2 * nalm]);
-      }
-      sT[k][j] = make_float2((float)t.x, (float)t.y);
-      sE[k][j] = make_float2((float)-e.x, (float)-e.y);
-      sB[k][j] = make_float2((float)-bb.x, (float)-bb.y);
-    }
-    __syncthreads();
-    for (int j = 0; j < cnt; ++j) {
-      const int l = lc + j;
-      const int64_t o = (int64_t)l * npairs;  // table entry idx(l, m) = base + l
-      const float lam = P0[o], lp = Pp[o], lq = Pq[o];
-      if (((l - m) & 1) == 0) {
-#pragma unroll
-        for (int k = 0; k < NB; ++k) {
-          const float2 t = sT[k][j], ne = sE[k][j], nb = sB[k][j];
-          T0[k].x = fmaf(t.x, lam, T0[k].x); T0[k].y = fmaf(t.y, lam, T0[k].y);
-          Q0[k].x = fmaf(ne.x, lp, Q0[k].x); Q0[k].y = fmaf(ne.y, lp, Q0[k].y);
-          U0[k].x = fmaf(nb.x, lp, U0[k].x); U0[k].y = fmaf(nb.y, lp, U0[k].y);
-          Q1[k].x = fmaf(-nb.y, lq, Q1[k].x); Q1[k].y = fmaf(nb.x, lq, Q1[k].y);
-          U1[k].x = fmaf(ne.y, lq, U1[k].x); U1[k].y = fmaf(-ne.x, lq, U1[k].y);
-        }
-      } else {
-#pragma unroll
-        for (int k = 0; k < NB; ++k) {
-          const float2 t = sT[k][j], ne = sE[k][j], nb = sB[k][j];
-          T1[k].x = fmaf(t.x, lam, T1[k].x); T1[k].y = fmaf(t.y, lam, T1[k].y);
-          Q1[k].x = fmaf(ne.x, lp, Q1[k].x); Q1[k].y = fmaf(ne.y, lp, Q1[k].y);
-          U1[k].x = fmaf(nb.x, lp, U1[k].x); U1[k].y = fmaf(nb.y, lp, U1[k].y);
-          Q0[k].x = fmaf(-nb.y, lq, Q0[k].x); Q0[k].y = fmaf(nb.x, lq, Q0[k].y);
-          U0[k].x = fmaf(ne.y, lq, U0[k].x); U0[k].y = fmaf(-ne.x, lq, U0[k].y);
-        }
-      }
-    }
-  }
-  if (!act) return;
-  const bool equator = (p == npairs - 1);
-#pragma unroll
-  for (int k = 0; k < NB; ++k) {
-    const int b = b0 + k;
-    if (state != nullptr && state[b].done) continue;
-    float2 *o0 = rc + rc_index2(b, 0, m, mmax, p, npairs);
-    float2 *o1 = rc + rc_index2(b, 1, m, mmax, p, npairs);
-    float2 *o2 = rc + rc_index2(b, 2, m, mmax, p, npairs);
-    o0[0] = cadd(T0[k], T1[k]);
-    o1[0] = cadd(Q0[k], Q1[k]);
-    o2[0] = cadd(U0[k], U1[k]);
-    if (!equator) {
-      o0[1] = csub(T0[k], T1[k]);
-      o1[1] = csub(Q0[k], Q1[k]);
-      o2[1] = csub(U0[k], U1[k]);
-    }
-  }
-}
-
-// Analysis, FP32: P tile from the table into smem, then the per-l contraction
-// over the pairs of the chunk (same structure as k_leg_ana64), NB RHS per block.
-template <int NB>
-__global__ void __launch_bounds__(ANA_P) k_leg_ana32(const float *__restrict__ ptab, const float2 *__restrict__ rc,
-                                                     float2 *__restrict__ apart, int lmax, int mmax, int npairs,
-                                                     int64_t nalm, int nchunk, const SolveState *__restrict__ state) {
-  __shared__ float P0[ANA_P][ANA_L + 1], Pp[ANA_P][ANA_L + 1], Pq[ANA_P][ANA_L + 1];
-  __shared__ float4 G[ANA_P][NB][3];  // (GT_e, GT_o), (GQ_e, GQ_o), (GU_e, GU_o)
-  __shared__ float red[ANA_PARTS][ANA_L][NB][6];
-  const int b0 = blockIdx.x * NB, chunk = blockIdx.y, m = blockIdx.z;
-  bool any = false;
-  for (int k = 0; k < NB; ++k) any = any || state == nullptr || !state[b0 + k].done;
-  if (!any) return;
-  const int t = threadIdx.x;
-  const int p = chunk * ANA_P + t;
-  const bool act = p < npairs;
-  const int pp = act ? p : npairs - 1;
-#pragma unroll
-  for (int k = 0; k < NB; ++k) {
-    float2 gn[3], gs[3];
-    for (int f = 0; f < 3; ++f) {
-      const float2 *g = rc + rc_index2(b0 + k, f, m, mmax, pp, npairs);
-      gn[f] = act ? g[0] : make_float2(0.f, 0.f);
-      gs[f] = (act && p != npairs - 1) ? g[1] : make_float2(0.f, 0.f);
-    }
-    for (int f = 0; f < 3; ++f) {
-      float2 e = cadd(gn[f], gs[f]), o = csub(gn[f], gs[f]);
-      G[t][k][f] = make_float4(e.x, e.y, o.x, o.y);
-    }
-  }
-  const int64_t base = alm_base(lmax, m);
-  const int64_t plane = nalm * (int64_t)npairs;
-  const int lj = t % ANA_L, part = t / ANA_L;
-  for (int lc = m; lc <= lmax; lc += ANA_L) {
-    const int cnt = min(ANA_L, lmax + 1 - lc);
-    __syncthreads();
-    // phase A: tile of the tables, coalesced over pairs
-    for (int j = 0; j < cnt; ++j) {
-      const int64_t o = (base + lc + j) * (int64_t)npairs + pp;
-      P0[t][j] = act ? ptab[o] : 0.f;
-      Pp[t][j] = act ? ptab[plane + o] : 0.f;
-      Pq[t][j] = act ? ptab[2 * plane + o] : 0.f;
-    }
-    __syncthreads();
-    float acc[NB][6];
-#pragma unroll
-    for (int k = 0; k < NB; ++k)
-#pragma unroll
-      for (int i = 0; i < 6; ++i) acc[k][i] = 0.f;
-    if (lj < cnt) {
-      const int l = lc + lj;
-      const bool odd = ((l - m) & 1) != 0;
-      for (int q = part * ANA_L; q < (part + 1) * ANA_L; ++q) {
-        const float lam = P0[q][lj], lp = Pp[q][lj], lq = Pq[q][lj];
-#pragma unroll
-        for (int k = 0; k < NB; ++k) {
-          const float4 gt4 = G[q][k][0], gq4 = G[q][k][1], gu4 = G[q][k][2];
-          const float2 gt = odd ? make_float2(gt4.z, gt4.w) : make_float2(gt4.x, gt4.y);
-          const float2 gqp = odd ? make_float2(gq4.z, gq4.w) : make_float2(gq4.x, gq4.y);
-          const float2 gup = odd ? make_float2(gu4.z, gu4.w) : make_float2(gu4.x, gu4.y);
-          const float2 gqo = odd ? make_float2(gq4.x, gq4.y) : make_float2(gq4.z, gq4.w);
-          const float2 guo = odd ? make_float2(gu4.x, gu4.y) : make_float2(gu4.z, gu4.w);
-          acc[k][0] = fmaf(lam, gt.x, acc[k][0]);
-          acc[k][1] = fmaf(lam, gt.y, acc[k][1]);
-          acc[k][2] = fmaf(-lp, gqp.x, fmaf(lq, guo.y, acc[k][2]));
-          acc[k][3] = fmaf(-lp, gqp.y, fmaf(-lq, guo.x, acc[k][3]));
-          acc[k][4] = fmaf(-lp, gup.x, fmaf(-lq, gqo.y, acc[k][4]));
-          acc[k][5] = fmaf(-lp, gup.y, fmaf(lq, gqo.x, acc[k][5]));
-        }
-      }
-    }
-#pragma unroll
-    for (int k = 0; k < NB; ++k)
-#pragma unroll
-      for (int i = 0; i < 6; ++i) red[part][lj][k][i] = acc[k][i];
-    __syncthreads();
-    if (part == 0 && lj < cnt) {
-      const int l = lc + lj;
-#pragma unroll
-      for (int k = 0; k < NB; ++k) {
-        float v[6];
-        for (int i = 0; i < 6; ++i) {
-          float a = red[0][lj][k][i];
-          for (int q = 1; q < ANA_PARTS; ++q) a += red[q][lj][k][i];
-          v[i] = a;
-        }
-        float2 *o = apart + ((int64_t)(b0 + k) * nchunk + chunk) * 3 * nalm + base + l;
-        o[0] = make_float2(v[0], v[1]);
-        o[nalm] = make_float2(v[2], v[3]);
-        o[2 * nalm] = make_float2(v[4], v[5]);
-      }
-    }
-  }
-}
-
-__global__ void k_ana_reduce32(const float2 *__restrict__ apart, double2 *out, int lmax, int64_t nalm, int nchunk,
-                               double omega, int epilogue, const double *__restrict__ filt, int nlev,
+__global__ void k_ana_reduce32(const float2 *__restrict__ apart, double2 *out, int lmax, int64_t nalm, double omega, int epilogue, const double *__restrict__ filt, int nlev,
                                const SolveState *__restrict__ state, const double2 *__restrict__ g_add) {
   const int b = blockIdx.y, m = blockIdx.z;
   if (state != nullptr && state[b].done) return;
   const int l = m + blockIdx.x * blockDim.x + threadIdx.x;
   if (l > lmax) return;
   const int64_t i = alm_base(lmax, m) + l;
-  // chunk sum in FP32 (it carries the analysis of the FP32 correction only),
-  // harmonic step and filter in FP64
+  // the FP32 sums carry the analysis of the FP32 correction only; harmonic
+  // step and filter in FP64
   double2 acc[3];
   for (int f = 0; f < 3; ++f) {
-    float ax = 0.f, ay = 0.f;
-    for (int c = 0; c < nchunk; ++c) {
-      const float2 v = apart[(((int64_t)b * nchunk + c) * 3 + f) * nalm + i];
-      ax += v.x;
-      ay += v.y;
-    }
-    acc[f] = make_double2(omega * (double)ax, omega * (double)ay);
+    const float2 v = apart[((int64_t)b * 3 + f) * nalm + i];
+    acc[f] = make_double2(omega * (double)v.x, omega * (double)v.y);
   }
   double2 *o = out + (int64_t)b * 3 * nalm + i;
   if (epilogue == ANA_PLAIN) {
@@ -614,21 +408,7 @@ __global__ void k_ana_reduce32(const float2 *__restrict__ apart, double2 *out, i
 
 cudaError_t legendre_synthesis32(dm_plan *p, const double2 *alm, cudaStream_t st) {
   if (p->use_tc && tc_batch_ok(p->batch)) return legendre_synthesis_tc(p, alm, st);
-  if (cudaError_t e = ensure_ptab(p)) return e;
-  const SolveState *stp = p->state_active ? p->state : nullptr;
-  const int pb = (p->npairs + SYN_THREADS - 1) / SYN_THREADS;
-  if (p->batch % 4 == 0) {
-    dim3 g(p->batch / 4, pb, p->mmax + 1);
-    k_leg_syn32<4><<<g, SYN_THREADS, 0, st>>>(p->ptab, alm, p->anchor_active ? p->a_hi : nullptr,
-                                              p->anchor_active ? p->e32 : nullptr, p->rc32, p->lmax, p->mmax,
-                                              p->npairs, p->nalm, stp);
-  } else {
-    dim3 g(p->batch, pb, p->mmax + 1);
-    k_leg_syn32<1><<<g, SYN_THREADS, 0, st>>>(p->ptab, alm, p->anchor_active ? p->a_hi : nullptr,
-                                              p->anchor_active ? p->e32 : nullptr, p->rc32, p->lmax, p->mmax,
-                                              p->npairs, p->nalm, stp);
-  }
-  return cudaGetLastError();
+  return split_synthesis32(p, alm, p->anchor_active ? p->e32 : nullptr, st);
 }
 
 // Filtered harmonic step of an anchored mixed iteration, on the FP32 state
@@ -638,7 +418,7 @@ cudaError_t legendre_synthesis32(dm_plan *p, const double2 *alm, cudaStream_t st
 // c depends on the level's filter F; it is formed in FP64 (and e_new with it)
 // whenever the level differs from the one c was formed at (clev, advanced by
 // the level control after this kernel), otherwise the step is all FP32.
-__global__ void k_ana_step_e32(const float2 *__restrict__ apart, int nchunk, float omega, int lmax, int64_t nalm,
+__global__ void k_ana_step_e32(const float2 *__restrict__ apart, float omega, int lmax, int64_t nalm,
                                const double *__restrict__ filt, const float *__restrict__ filt32, int nlev,
                                const SolveState *__restrict__ state, const int *__restrict__ clev,
                                const double2 *__restrict__ a_hi, const double2 *__restrict__ g_hi,
@@ -650,13 +430,8 @@ __global__ void k_ana_step_e32(const float2 *__restrict__ apart, int nchunk, flo
   const int64_t i = alm_base(lmax, m) + l, ib = (int64_t)b * 3 * nalm + i;
   float2 acc[3];
   for (int f = 0; f < 3; ++f) {
-    float ax = 0.f, ay = 0.f;
-    for (int c = 0; c < nchunk; ++c) {
-      const float2 v = apart[(((int64_t)b * nchunk + c) * 3 + f) * nalm + i];
-      ax += v.x;
-      ay += v.y;
-    }
-    acc[f] = make_float2(omega * ax, omega * ay);
+    const float2 v = apart[((int64_t)b * 3 + f) * nalm + i];
+    acc[f] = make_float2(omega * v.x, omega * v.y);
   }
   const int lev = state[b].level;
   const int64_t co = (((int64_t)b * nlev + lev) * (lmax + 1) + l) * 4;
@@ -745,33 +520,17 @@ cudaError_t materialize_a(dm_plan *p, cudaStream_t st) {
 
 cudaError_t legendre_analysis32(dm_plan *p, int epilogue, double2 *out, cudaStream_t st, cudaEvent_t mid) {
   const SolveState *stp = p->state_active ? p->state : nullptr;
-  int nchunk = p->nchunk;
-  if (p->use_tc && tc_batch_ok(p->batch)) {
-    cudaError_t e = legendre_analysis_tc(p, st);
-    if (e) return e;
-    nchunk = 1;
-  } else if (p->nchunk32 < p->nchunk) {
-    return cudaErrorInvalidValue;  // the CUDA-core FP32 analysis needs every chunk (see setup_fp32)
-  } else if (cudaError_t e = ensure_ptab(p)) {
+  if (cudaError_t e = (p->use_tc && tc_batch_ok(p->batch)) ? legendre_analysis_tc(p, st) : split_analysis32(p, st))
     return e;
-  } else if (p->batch % 4 == 0) {
-    dim3 g(p->batch / 4, p->nchunk, p->mmax + 1);
-    k_leg_ana32<4><<<g, ANA_P, 0, st>>>(p->ptab, p->rc32, p->apart32, p->lmax, p->mmax, p->npairs, p->nalm,
-                                        p->nchunk, stp);
-  } else {
-    dim3 g(p->batch, p->nchunk, p->mmax + 1);
-    k_leg_ana32<1><<<g, ANA_P, 0, st>>>(p->ptab, p->rc32, p->apart32, p->lmax, p->mmax, p->npairs, p->nalm,
-                                        p->nchunk, stp);
-  }
   if (mid) cudaEventRecord(mid, st);
   double omega = 4.0 * M_PI / (double)p->npix;
   dim3 g2((unsigned)((p->lmax + 1 + 127) / 128), p->batch, p->mmax + 1);
   if (epilogue == ANA_DM_STEP && p->anchor_active) {  // FP32 state e between anchors
-    k_ana_step_e32<<<g2, 128, 0, st>>>(p->apart32, nchunk, (float)omega, p->lmax, p->nalm, p->filt, p->filt32,
+    k_ana_step_e32<<<g2, 128, 0, st>>>(p->apart32, (float)omega, p->lmax, p->nalm, p->filt, p->filt32,
                                        p->filt_levels, p->state, p->clev, p->a_hi, p->g_hi, p->e32, p->c32);
     return cudaGetLastError();
   }
-  k_ana_reduce32<<<g2, 128, 0, st>>>(p->apart32, out, p->lmax, p->nalm, nchunk, omega, epilogue, p->filt,
+  k_ana_reduce32<<<g2, 128, 0, st>>>(p->apart32, out, p->lmax, p->nalm, omega, epilogue, p->filt,
                                      p->filt_levels,
                                      epilogue == ANA_DM_STEP ? p->state : stp,
                                      (p->anchor_active && epilogue == ANA_DM_STEP) ? p->g_hi : nullptr);

@@ -529,7 +529,6 @@ static cudaError_t tc_scratch(dm_plan *p) {
 static cudaError_t tc_tables(dm_plan *p) {
   if (p->tc_synA[1] && p->tc_anaA[1]) return cudaSuccess;
   cudaError_t e = tc_scratch(p);
-  if (!e) e = ensure_ptab(p);  // the tiles are cut from the FP32 tables
   if (e) return e;
   const int npt = (p->npairs + 127) / 128, nps = (p->npairs + 15) / 16;
   int64_t ssteps = 0, atiles = 0;
@@ -543,26 +542,38 @@ static cudaError_t tc_tables(dm_plan *p) {
   }
   const size_t sbytes[2] = {(size_t)ssteps * npt * 2 * 2 * TILE_A, (size_t)ssteps * npt * 4 * 2 * TILE_A};
   const size_t abytes[2] = {(size_t)atiles * nps * 1 * 2 * TILE_A, (size_t)atiles * nps * 2 * 2 * TILE_A};
+  // the tiles are cut from FP32 tables that live as long as that takes; on an
+  // error none of them stays
+  float *ptab = nullptr;
+  auto undo = [&](cudaError_t err) {
+    cudaFree(ptab);
+    for (int part = 0; part < 2; ++part) {
+      cudaFree(p->tc_synA[part]);
+      cudaFree(p->tc_anaA[part]);
+      p->tc_synA[part] = p->tc_anaA[part] = nullptr;
+    }
+    return err;
+  };
   for (int part = 0; part < 2; ++part) {
-    if (!p->tc_synA[part]) {
-      if ((e = cudaMalloc(&p->tc_synA[part], sbytes[part]))) return e;
-      p->bytes += (int64_t)sbytes[part];
-    }
-    if (!p->tc_anaA[part]) {
-      if ((e = cudaMalloc(&p->tc_anaA[part], abytes[part]))) return e;
-      p->bytes += (int64_t)abytes[part];
-    }
+    if ((e = cudaMalloc(&p->tc_synA[part], sbytes[part]))) return undo(e);
+    if ((e = cudaMalloc(&p->tc_anaA[part], abytes[part]))) return undo(e);
   }
+  if ((e = cudaMalloc(&ptab, sizeof(float) * 3 * (size_t)p->nalm * p->npairs))) return undo(e);
+  if ((e = gen_tables32(p, ptab, 0))) return undo(e);
   dim3 gs(syn_steps(p->lmax, 0), npt, p->mmax + 1);
-  k_tab_syn<0><<<gs, 256>>>(p->ptab, p->tc_synA[0], p->tc_soff, p->lmax, p->npairs, p->nalm, npt);
-  k_tab_syn<1><<<gs, 256>>>(p->ptab, p->tc_synA[1], p->tc_soff, p->lmax, p->npairs, p->nalm, npt);
+  k_tab_syn<0><<<gs, 256>>>(ptab, p->tc_synA[0], p->tc_soff, p->lmax, p->npairs, p->nalm, npt);
+  k_tab_syn<1><<<gs, 256>>>(ptab, p->tc_synA[1], p->tc_soff, p->lmax, p->npairs, p->nalm, npt);
   if (max_lt > 0) {
     dim3 ga(nps, max_lt, 2 * (p->mmax + 1));
-    k_tab_ana<0><<<ga, 256>>>(p->ptab, p->tc_anaA[0], p->tc_aoff, p->lmax, p->npairs, p->nalm, nps);
-    k_tab_ana<1><<<ga, 256>>>(p->ptab, p->tc_anaA[1], p->tc_aoff, p->lmax, p->npairs, p->nalm, nps);
+    k_tab_ana<0><<<ga, 256>>>(ptab, p->tc_anaA[0], p->tc_aoff, p->lmax, p->npairs, p->nalm, nps);
+    k_tab_ana<1><<<ga, 256>>>(ptab, p->tc_anaA[1], p->tc_aoff, p->lmax, p->npairs, p->nalm, nps);
   }
-  if ((e = cudaGetLastError())) return e;
-  return cudaDeviceSynchronize();
+  e = cudaGetLastError();
+  if (!e) e = cudaDeviceSynchronize();
+  if (e) return undo(e);
+  cudaFree(ptab);
+  for (int part = 0; part < 2; ++part) p->bytes += (int64_t)(sbytes[part] + abytes[part]);
+  return cudaSuccess;
 }
 
 // stages per CTA: as many as fit in the shared memory of one CTA, or of two

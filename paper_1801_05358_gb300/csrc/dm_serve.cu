@@ -70,6 +70,7 @@ struct Pool {
   uint64_t cl_hash = 0;
   dm_precision prec = DM_FP64;  // mode the plan was set to (DM_FLOAT_FLOAT kept as such)
   dm_plan *plan = nullptr;
+  size_t reserved = 0;          // bytes of the memory budget it holds
   cudaStream_t stream = nullptr;
   std::vector<Slot> slots;
   // a round in flight: its iterations and the copy of the solver states into
@@ -121,7 +122,7 @@ dm_plan make_view(const dm_plan *p, int b) {
   v.filt += (size_t)b * p->filt_levels * 4 * (p->lmax + 1);
   if (p->fp32_ready) {
     v.rc32 += b * nrc;
-    v.apart32 += (size_t)b * p->nchunk32 * na;
+    v.apart32 += (size_t)b * na;
     v.s32 += b * n3;
     v.w32 += b * n3;
     v.wd32 += b * n3;
@@ -149,8 +150,10 @@ __global__ void k_sub_maps(const double *__restrict__ x, double *__restrict__ y,
     y[i] = x[i] - y[i];
 }
 
-// rough device footprint of a pool, from the plan's own allocation list
-size_t estimate_bytes(int nside, int lmax, int S, dm_precision prec) {
+// rough device footprint of a pool, from the plan's own allocation list;
+// *tables: the part of it that Legendre tables beyond the FP32 ones may take
+size_t estimate_bytes(int nside, int lmax, int S, dm_precision prec, double *tables) {
+  *tables = 0;
   const double npix = 12.0 * nside * nside, nalm = (lmax + 1.0) * (lmax + 2.0) / 2.0, npairs = 2.0 * nside;
   const double nchunk = ceil(npairs / 64.0);
   double b = 0;
@@ -163,11 +166,14 @@ size_t estimate_bytes(int nside, int lmax, int S, dm_precision prec) {
   const bool stored = tc && dmwf::tc_tables_fit(lmax, lmax, (int)npairs, S);
   if (prec != DM_FP64) {                         // DM_MIXED_FP32 and DM_FLOAT_FLOAT
     const double full = 3 * nalm * npairs * 4 * 2;  // FP32 tables, hi and lo
-    if (stored || (prec == DM_MIXED_FP32 && !tc) || (prec == DM_FLOAT_FLOAT && full <= 32.0 * (1u << 30)) ||
-        full <= (double)(1u << 30))
+    const bool fp32_tab = stored || (prec == DM_MIXED_FP32 && !tc);
+    if (fp32_tab || (prec == DM_FLOAT_FLOAT && full <= 32.0 * (1u << 30)) || full <= (double)(1u << 30)) {
       b += full;
-    else
-      b += (double)(1u << 30);                   // per-slab tables of the float-float stages
+      *tables = fp32_tab ? full / 2 : full;
+    } else {
+      b += (double)(1u << 30);
+      *tables = (double)(1u << 30);
+    }
     b += S * 3 * (lmax + 1.0) * npairs * 2 * 8;  // rc32
     b += S * nchunk * 3 * nalm * 8;              // apart32
     b += S * 3 * npix * 4 * 4;                   // s32, w32, wd32, shi32
@@ -232,14 +238,15 @@ Pool *make_pool(dm_server *S, const Request &r, dm_status *why) {
   *why = DM_ENOMEM;
   const int slots = S->cfg.slots_per_plan;
   const dm_precision prec = request_prec(S, r);
-  size_t need = estimate_bytes(r.nside, r.lmax, slots, prec);
+  double tables = 0;
+  size_t need = estimate_bytes(r.nside, r.lmax, slots, prec, &tables);
   if (S->used + need > S->cfg.hbm_budget_bytes) {
     // free idle pools (no busy slot) to make room
     std::lock_guard<std::mutex> lk(S->mu);
     for (size_t i = 0; i < S->pools.size();) {
       Pool *q = S->pools[i].get();
       if (q->busy() == 0) {
-        S->used -= estimate_bytes(q->nside, q->lmax, slots, q->prec);
+        S->used -= q->reserved;
         release_pool(q);
         S->pools.erase(S->pools.begin() + i);
       } else {
@@ -259,6 +266,30 @@ Pool *make_pool(dm_server *S, const Request &r, dm_status *why) {
     return nullptr;
   }
   dm_plan *p = pool->plan;
+  {
+    // The digit tables of the FP64-class stages take what the estimate left
+    // for tables and what the budget has beyond it: the whole table, else
+    // slabs, else none (the direct FP64 kernels), so that no request the
+    // budget held without them is turned away for them.
+    const double room = tables + (double)(S->cfg.hbm_budget_bytes - S->used - need);
+    const double scratch = (double)split_scratch_bytes(r.lmax, p->npairs, slots);
+    const double whole = (double)split_table_bytes(r.lmax, p->mmax, p->npairs);
+    double take = 0;
+    if (whole <= (double)p->split_cap && whole + scratch <= room) {
+      take = whole + scratch;
+    } else if (std::min(whole, (double)p->ffs_cap) + scratch <= room) {
+      p->split_cap = 0;
+      take = std::min(whole, (double)p->ffs_cap) + scratch;
+    } else if (prec == DM_FP64) {
+      split_disable(p);
+    } else {  // the other modes have no kernels without tables: slabs within what the estimate left
+      p->split_cap = 0;
+      p->ffs_cap = (int64_t)std::max((double)(1 << 20), std::min(whole, tables));
+      take = tables;
+    }
+    if (take > tables) need += (size_t)(take - tables);
+  }
+  pool->reserved = need;
   dm_schedule sc = S->cfg.sched;
   sc.iters_per_level = 0;
   if ((rs = dm_set_schedule(p, &sc)) != DM_OK || (rs = dm_set_spectra(p, r.cl.data())) != DM_OK ||

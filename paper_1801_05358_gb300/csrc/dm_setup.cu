@@ -598,11 +598,9 @@ __global__ void k_d2f2(const double2 *in, float2 *out, int64_t n) {
     out[i] = make_float2((float)in[i].x, (float)in[i].y);
 }
 
-cudaError_t gen_tables32(dm_plan *p);  // dm_legendre.cu
-
 // Buffers of DM_MIXED_FP32 and DM_FLOAT_FLOAT: FP32 copies of the FFT tables,
-// FP32 ring coefficients and maps.  The FP32 Legendre tables are not made
-// here: the kernels that read them build them on first use (ensure_ptab).
+// FP32 ring coefficients and maps.  The Legendre tables are made on first use
+// (dm_split.cu, dm_legendre_tc.cu, dm_legendre_otf.cu).
 cudaError_t setup_fp32(dm_plan *p) {
   if (p->fp32_ready) return cudaSuccess;  // set only after everything below succeeded
   cudaError_t e;
@@ -613,7 +611,7 @@ cudaError_t setup_fp32(dm_plan *p) {
                     (void **)&p->twr32,   (void **)&p->rc32,
                     (void **)&p->apart32, (void **)&p->s32,    (void **)&p->w32,     (void **)&p->wd32,
                     (void **)&p->a_hi,    (void **)&p->g_hi,   (void **)&p->shi32,   (void **)&p->e32,
-                    (void **)&p->c32,     (void **)&p->clev,   (void **)&p->tc_err};
+                    (void **)&p->c32,     (void **)&p->clev};
   // the workspace figure goes back to what it was on entry, so a failed
   // set-up (and its retries) does not inflate dm_plan_info's byte count
   const int64_t bytes_on_entry = p->bytes;
@@ -640,11 +638,7 @@ cudaError_t setup_fp32(dm_plan *p) {
   if ((e = al(&p->twid32, p->fft_M_max - 1))) return undo(e);
   if ((e = al(&p->twr32, p->twr_words))) return undo(e);
   if ((e = al(&p->rc32, (size_t)B * 3 * (p->mmax + 1) * p->npairs * 2))) return undo(e);
-  {
-    const double full = (double)B * p->nchunk * 3 * p->nalm * sizeof(float2);
-    p->nchunk32 = full <= 24.0 * (1u << 30) ? p->nchunk : 1;
-  }
-  if ((e = al(&p->apart32, (size_t)B * p->nchunk32 * 3 * p->nalm))) return undo(e);
+  if ((e = al(&p->apart32, (size_t)B * 3 * p->nalm))) return undo(e);
   if ((e = al(&p->s32, (size_t)B * n3))) return undo(e);
   if ((e = al(&p->w32, (size_t)B * n3))) return undo(e);
   if ((e = al(&p->wd32, (size_t)B * n3))) return undo(e);
@@ -654,8 +648,6 @@ cudaError_t setup_fp32(dm_plan *p) {
   if ((e = al(&p->e32, (size_t)B * 3 * p->nalm))) return undo(e);
   if ((e = al(&p->c32, (size_t)B * 3 * p->nalm))) return undo(e);
   if ((e = al(&p->clev, (size_t)B))) return undo(e);
-  if ((e = al(&p->tc_err, 1))) return undo(e);
-  cudaMemset(p->tc_err, 0, sizeof(int));
   cudaMemset(p->rc32, 0, sizeof(float2) * (size_t)B * 3 * (p->mmax + 1) * p->npairs * 2);
   k_d2f2<<<512, 256>>>(p->phase, p->phase32, p->ph_total);
   if (p->bh_total > 0) k_d2f2<<<512, 256>>>(p->bhat, p->bhat32, p->bh_total);
@@ -666,26 +658,6 @@ cudaError_t setup_fp32(dm_plan *p) {
   if (p->twr_words > 0) k_d2f2<<<64, 256>>>(p->twr, p->twr32, p->twr_words);
   if ((e = cudaDeviceSynchronize())) return undo(e);
   p->fp32_ready = true;
-  return cudaSuccess;
-}
-
-// The full FP32 Legendre tables (3 x nalm x npairs, hi and lo), made once.
-cudaError_t ensure_ptab(dm_plan *p) {
-  if (p->ptab) return cudaSuccess;
-  const size_t n = (size_t)3 * p->nalm * p->npairs;
-  float *hi = nullptr, *lo = nullptr;
-  cudaError_t e = cudaMalloc(&hi, sizeof(float) * n);
-  if (!e) e = cudaMalloc(&lo, sizeof(float) * n);
-  if (!e) e = gen_tables32_slab(p, hi, lo, 0, p->mmax + 1, 0);
-  if (!e) e = cudaDeviceSynchronize();
-  if (e) {
-    cudaFree(hi);
-    cudaFree(lo);
-    return e;
-  }
-  p->ptab = hi;
-  p->ptab_lo = lo;
-  p->bytes += (int64_t)(2 * sizeof(float) * n);
   return cudaSuccess;
 }
 

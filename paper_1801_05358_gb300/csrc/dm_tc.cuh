@@ -54,10 +54,21 @@ __device__ __forceinline__ void mma_bf16(uint32_t d_tmem, uint64_t adesc, uint64
       "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate));
 }
 
-__device__ __forceinline__ void commit(uint64_t *mbar) {
-  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-                   smem_u32(mbar))
-               : "memory");
+__device__ __forceinline__ void commit_at(uint32_t mbar) {
+  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(mbar) : "memory");
+}
+__device__ __forceinline__ void commit(uint64_t *mbar) { commit_at(smem_u32(mbar)); }
+// the MMA with the accumulation known when compiled
+template <bool ACC>
+__device__ __forceinline__ void mma_bf16_c(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc) {
+  if (ACC)
+    asm volatile("{\n\t.reg .pred p;\n\tsetp.eq.u32 p, 0, 0;\n\t"
+                 "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}\n" ::"r"(d_tmem),
+                 "l"(adesc), "l"(bdesc), "r"(idesc));
+  else
+    asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.u32 p, 0, 0;\n\t"
+                 "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}\n" ::"r"(d_tmem),
+                 "l"(adesc), "l"(bdesc), "r"(idesc));
 }
 
 __device__ __forceinline__ void mbar_init(uint64_t *mbar, uint32_t count) {
@@ -82,8 +93,7 @@ constexpr uint64_t MBAR_TIMEOUT_NS = 1000000000ull;
 // advance (at least tens of milliseconds, at most about 17 s).  Returns false
 // (and sets *err, when given) when it gives up.
 constexpr uint32_t MBAR_SUSPEND_NS = 4000;
-__device__ __forceinline__ bool mbar_wait(uint64_t *mbar, uint32_t phase, int *err) {
-  const uint32_t a = smem_u32(mbar);
+__device__ __forceinline__ bool mbar_wait_at(uint32_t a, uint32_t phase, int *err) {  // a: shared address
   uint64_t t0 = 0;
   for (uint32_t it = 0; it < (1u << 22); ++it) {
     uint32_t ok;
@@ -106,6 +116,9 @@ __device__ __forceinline__ bool mbar_wait(uint64_t *mbar, uint32_t phase, int *e
   if (err) atomicExch(err, 1);
   return false;
 }
+__device__ __forceinline__ bool mbar_wait(uint64_t *mbar, uint32_t phase, int *err) {
+  return mbar_wait_at(smem_u32(mbar), phase, err);
+}
 
 // Plain arrival of this thread on an mbarrier.
 __device__ __forceinline__ void mbar_arrive(uint64_t *mbar) {
@@ -113,18 +126,22 @@ __device__ __forceinline__ void mbar_arrive(uint64_t *mbar) {
 }
 
 // Arrive on an mbarrier (count 1) and add bytes to the transaction count of its current phase.
+__device__ __forceinline__ void mbar_expect_tx_at(uint32_t mbar, uint32_t bytes) {
+  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(mbar), "r"(bytes) : "memory");
+}
 __device__ __forceinline__ void mbar_expect_tx(uint64_t *mbar, uint32_t bytes) {
-  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(mbar)), "r"(bytes)
-               : "memory");
+  mbar_expect_tx_at(smem_u32(mbar), bytes);
 }
 
 // Bulk copy global -> shared (16-byte aligned addresses, size a multiple of 16),
 // completion reported to the mbarrier as transaction bytes.
-__device__ __forceinline__ void bulk_g2s(void *dst, const void *src, uint32_t bytes, uint64_t *mbar) {
-  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
-                   smem_u32(dst)),
-               "l"(src), "r"(bytes), "r"(smem_u32(mbar))
+__device__ __forceinline__ void bulk_g2s_at(uint32_t dst, const void *src, uint32_t bytes, uint32_t mbar) {
+  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst),
+               "l"(src), "r"(bytes), "r"(mbar)
                : "memory");
+}
+__device__ __forceinline__ void bulk_g2s(void *dst, const void *src, uint32_t bytes, uint64_t *mbar) {
+  bulk_g2s_at(smem_u32(dst), src, bytes, smem_u32(mbar));
 }
 
 __device__ __forceinline__ void fence_proxy_async() {
