@@ -56,6 +56,7 @@ void free_all(dm_plan *p) {
   for (void *q : ptrs)
     if (q) cudaFree(q);
   split_release(p);
+  dft_release(p);
   if (p->ev_begin) cudaEventDestroy(p->ev_begin);
   if (p->ev_end) cudaEventDestroy(p->ev_end);
 }
@@ -469,7 +470,10 @@ dm_status plan_workspace(dm_plan *p, dm_plan **out) {
   if ((e = dalloc(p, &p->rhi, (size_t)B * n3))) return bad(e, "alloc rhi");
   if ((e = dalloc(p, &p->tc_err, 1))) return bad(e, "alloc");
   cudaMemset(p->tc_err, 0, sizeof(int));
-  if (!p->flat) split_new(p);
+  if (!p->flat) {
+    split_new(p);
+    dft_new(p);
+  }
   if ((e = cudaEventCreate(&p->ev_begin)) || (e = cudaEventCreate(&p->ev_end))) return bad(e, "events");
   cudaMemset(p->rc, 0, sizeof(double2) * (size_t)B * 3 * (p->mmax + 1) * p->npairs * 2);
   cudaMemset(p->mask, 1, (size_t)B * p->npix);
@@ -530,7 +534,7 @@ dm_status dm_plan_info(const dm_plan *p, int64_t *npix, int64_t *nalm, int *nrin
   if (npix) *npix = p->npix;
   if (nalm) *nalm = p->nalm;
   if (nrings) *nrings = p->nrings;
-  if (ws) *ws = p->bytes + split_bytes(p);
+  if (ws) *ws = p->bytes + split_bytes(p) + dft_bytes(p);
   return DM_OK;
 }
 
@@ -1001,6 +1005,7 @@ dm_status dm_set_tc_tiles(dm_plan *p, int generate) {
 dm_status dm_set_ring_radix(dm_plan *p, int lr) {
   if (!p || (lr != 0 && lr != 3 && lr != 4)) return DM_EINVAL;
   p->ring_lr = lr;
+  p->ring_fft = true;
   for (int i = 0; i < DM_TUNE_MAX_CLASSES; ++i) p->tune_ring_lr[i] = -1;  // an explicit radix overrides a tuned one
   return DM_OK;
 }

@@ -1,0 +1,961 @@
+// dm_dft.cu -- the FP64-class ring transforms (inverse and forward ring DFTs of
+// the dual messenger step, Algorithm 1, with the update of Eq. 9 between them)
+// as exact integer products on the tensor cores (split products, dm_split.cu).
+//
+// Why: an FFT in FP64 is bound by the FP64 pipe (2 FMA a clock and SM), and the
+// polar rings of 4i pixels need Bluestein's convolution, four transforms of
+// twice the size.  A ring's DFT is a product with a matrix that every
+// right-hand side, field and ring of the same length shares, and the tensor
+// cores do 26 digit products faster than the FP64 pipe does the FFT.
+//
+// Folding.  The pixels of a ring sit at phi_j = 2 pi (j + s) / n, s = 1/2 or 0,
+// and n is a multiple of 4, so the ring maps onto itself under phi -> -phi and
+// phi -> pi - phi.  With cos m(pi - phi) = (-1)^m cos m phi and
+// sin m(pi - phi) = -(-1)^m sin m phi, the four pixels of an orbit combine to
+// one value for each of four matrices: cosines and sines of even and of odd m
+// (CE, CO, SE, SO), each of about n/4 x n/4: a quarter of the plain product
+// each way.  Orders beyond n/2 alias: F_{kn+q} = (-1)^{2sk} F_q and
+// F_{kn-q} = (-1)^{2sk} conj F_q, so only q <= n/2 meet the matrix.
+//
+// Passes of an iteration: k_dft_xinv (alias fold of F_m, digits), k_dft<false>
+// (orbit sums, FP64), k_dft_pix (unfold, s, Cauchy partials, t - s = w (d - s),
+// fold, digits), k_dft<true> (F_q, q <= n/2), k_dft_alias (the orders beyond).
+// One matrix set per ring length and shift (each polar radius; two for the
+// belt), kept as digit planes of 8 x 8 core matrices (4 matrices x n^2/16 x 12
+// bytes: 268 MB in all at nside 256, 2.1 GB at nside 512) that serve both
+// directions, K-major forward and MN-major inverse.
+#include <algorithm>
+#include <vector>
+
+#include "dm_internal.h"
+#include "dm_split.cuh"
+
+namespace dmwf {
+
+constexpr int DFT_CHUNK = 8;       // K steps of 16 per drain
+constexpr int DFT_DRAIN_WARPS = 8;
+constexpr int DFT_THREADS = 32 * (DFT_DRAIN_WARPS + 2);
+constexpr int DFT_MAX_STAGES = 8;
+constexpr size_t DFT_SCRATCH = (size_t)1 << 30;  // column digits of one direction and group of right-hand sides
+
+// A matrix set: the rings of one length and shift.
+struct DftSet {
+  int n, nj;            // pixels; orbits (n/4, or n/4 + 1 without the half-pixel shift)
+  int shift;            // 1: s = 1/2
+  int mx;               // largest order kept (min(mmax, n/2))
+  int rq;               // row octets of each matrix (even)
+  int nyo;              // column octets (orbits)
+  int pair0, npr;       // pairs of this length in the pair list
+};
+// The same in a cut of nl lanes (right-hand sides x fields of a group).
+struct DftCol {
+  int nct, w, n0;       // column tiles, columns per tile, padded columns
+  int ksi, ksf;         // K steps of the inverse and forward products
+  int col0;             // first column of the set
+  int64_t xi, xf;       // bytes into the inverse and forward column digits
+  int64_t v;            // values into the orbit sums
+  int njp;              // padded orbits
+};
+struct DftTile {
+  int set, fun;         // matrix: CE 0, CO 1, SE 2, SO 3 (forward: the parity; cosine and sine in one tile)
+  int row, ct, ks;
+  int z, zfun;          // table row octet of the tile; distance to the sine matrix
+  int n0;
+  int64_t x, xfun;      // column digits of K step 0; distance to the sine columns
+};
+struct DftCut {
+  int nl = 0;
+  DftCol *cols = nullptr;              // device
+  DftTile *tiles[2][5] = {};           // device, by direction and NQ
+  int ntiles[2][5] = {};
+  int ncol = 0;
+  size_t xbytes = 0, vcount = 0;
+};
+struct DftTables {
+  std::vector<DftSet> sets;
+  std::vector<int64_t> off;            // digit table offset of each set
+  unsigned char *dig = nullptr;
+  DftSet *sets_dev = nullptr;
+  CUtensorMap *maps = nullptr;         // device: [set][inverse, forward]
+  int *pair_of = nullptr, *set_of = nullptr;  // pair list and its sets
+  int nlist = 0;
+  std::vector<DftCut> cuts;
+  unsigned char *x = nullptr;
+  size_t xbytes = 0;
+  double *v = nullptr;
+  size_t vcount = 0;
+  int *xexp = nullptr;                 // [2][columns]
+  int xexp_n = 0;
+  int64_t bytes = 0;
+  bool failed = false;
+};
+
+namespace {
+
+// cos(pi t / n), n a multiple of 4: the argument is brought into [0, pi/4] in
+// integers, so that the rounding of t / n costs less than the result's own
+__device__ double cos_frac(long long t, long long n) {
+  t %= 2 * n;
+  if (t < 0) t += 2 * n;
+  if (t > n) t = 2 * n - t;
+  double sgn = 1.0;
+  if (2 * t > n) {
+    t = n - t;
+    sgn = -1.0;
+  }
+  if (4 * t > n) return sgn * sinpi((double)(n / 2 - t) / (double)n);
+  return sgn * cospi((double)t / (double)n);
+}
+
+// Digits of one set: one thread per (matrix, row, octet of orbits).
+__global__ void k_dft_gen(const DftSet s, unsigned char *__restrict__ dig) {
+  const int64_t total = (int64_t)4 * s.rq * 8 * s.nyo;
+  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x) {
+    const int jo = (int)(i % s.nyo), rr = (int)(i / s.nyo), fun = rr / (8 * s.rq), r = rr % (8 * s.rq);
+    const int q = 2 * r + (fun & 1);
+    long long v[8];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+      const int j = 8 * jo + k;
+      v[k] = 0;
+      if (q <= s.mx && j < s.nj) {
+        const long long t = (long long)q * (2 * j + s.shift);  // q phi_j = pi t / n
+        const double c = cos_frac(fun < 2 ? t : t - s.n / 2, s.n);
+        v[k] = c == 1.0 ? 1ll << 53 : (c == -1.0 ? -(1ll << 53) : fixed53(c, 0));
+      }
+    }
+    int d[8][SPLIT_S];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) Fixed<SPLIT_S>::digits(v[k], d[k]);
+#pragma unroll
+    for (int j = 0; j < SPLIT_S; ++j) {
+      uint4 w;
+      w.x = bf16_pair(d[0][j], d[1][j]);
+      w.y = bf16_pair(d[2][j], d[3][j]);
+      w.z = bf16_pair(d[4][j], d[5][j]);
+      w.w = bf16_pair(d[6][j], d[7][j]);
+      *reinterpret_cast<uint4 *>(
+          dig + ((((int64_t)j * 4 * s.rq + fun * s.rq + (r >> 3)) * s.nyo + jo) * 128 + (r & 7) * 16)) = w;
+    }
+  }
+}
+
+// column of (pair of the set, lane, side): its tile and place there
+__device__ __forceinline__ void col_place(const DftCol &c, int col, int &ct, int &cit) {
+  ct = col / c.w;
+  cit = col - ct * c.w;
+}
+
+// Inverse columns of one pair and lane (both sides): C_q = sum of the orders
+// that alias to q, times 2 beyond m = 0; cosines meet Re C, sines Im C.
+__global__ void __launch_bounds__(128) k_dft_xinv(const double2 *__restrict__ rc, unsigned char *__restrict__ x,
+                                                  int *__restrict__ xexp, const DftSet *__restrict__ sets,
+                                                  const DftCol *__restrict__ cols, const int *__restrict__ pair_of,
+                                                  const int *__restrict__ set_of, int nl, int lane0, int mmax,
+                                                  int npairs, const SolveState *__restrict__ state) {
+  extern __shared__ __align__(16) double2 sc[];  // [groups][2 sides][mx + 1], 256 entries at least
+  __shared__ int red[4];
+  const int g = blockIdx.x, lane = blockIdx.y, pair = pair_of[g];
+  if (state != nullptr && state[(lane0 + lane) / 3].done) return;
+  const DftSet S = sets[set_of[g]];
+  const DftCol C = cols[set_of[g]];
+  const int n = S.n, h = n / 2, nq = S.mx + 1;
+  const bool equator = pair == npairs - 1;
+  const double2 *src = rc + ((int64_t)(lane0 + lane) * (mmax + 1) * npairs + pair) * 2;
+  const int64_t ms = (int64_t)npairs * 2;
+  int ex[2] = {-100000, -100000};
+  // short rings: groups of threads share the aliases of an order
+  const int ng = nq < 128 ? 128 / nq : 1, grp = ng > 1 ? threadIdx.x / nq : 0;
+  for (int q = ng > 1 ? threadIdx.x % nq : threadIdx.x; q < nq && grp < ng; q += 128) {
+    double2 a = make_double2(0, 0), b = make_double2(0, 0);
+    auto add = [&](int m, double re, double im) {  // re, im: signs of the real and imaginary parts
+      const double2 u = src[m * ms], w = equator ? make_double2(0, 0) : src[m * ms + 1];
+      a.x = fma(re, u.x, a.x);
+      a.y = fma(im, u.y, a.y);
+      b.x = fma(re, w.x, b.x);
+      b.y = fma(im, w.y, b.y);
+    };
+    if (grp == 0) add(q, q ? 2.0 : 1.0, q ? 2.0 : 1.0);
+    for (int k = 1 + grp; k * n - q <= mmax; k += ng) {
+      const double sg = (S.shift & k & 1) ? -2.0 : 2.0;
+      if (q > 0 && q < h) add(k * n - q, sg, -sg);
+      if (k * n + q <= mmax) add(k * n + q, sg, sg);
+    }
+    sc[(2 * grp) * nq + q] = a;
+    sc[(2 * grp + 1) * nq + q] = b;
+    if (ng > 1) break;
+    ex[0] = max(ex[0], max(exp_of(a.x), exp_of(a.y)));
+    ex[1] = max(ex[1], max(exp_of(b.x), exp_of(b.y)));
+  }
+  __syncthreads();
+  if (ng > 1) {  // the groups' sums, in order
+    const int q = threadIdx.x;
+    if (q < nq)
+      for (int side = 0; side < 2; ++side) {
+        double2 a = sc[side * nq + q];
+        for (int g2 = 1; g2 < ng; ++g2) {
+          const double2 u = sc[(2 * g2 + side) * nq + q];
+          a.x += u.x;
+          a.y += u.y;
+        }
+        sc[side * nq + q] = a;  // (its own group's slot)
+        ex[side] = max(exp_of(a.x), exp_of(a.y));
+      }
+    __syncthreads();
+  }
+  for (int side = 0; side < (equator ? 1 : 2); ++side) {
+    int e = max(-1000, block_max(ex[side], red));
+    if (e >= SPLIT_NAN) e = SPLIT_NAN;
+    const int pl = g - S.pair0, col = (pl * nl + lane) * 2 + side;
+    if (threadIdx.x == 0) xexp[C.col0 + col] = e;
+    int ct, cit;
+    col_place(C, col, ct, cit);
+    const int64_t blk = (int64_t)SPLIT_S * C.n0 * 32;
+    const double2 *c = sc + side * nq;
+    for (int it = threadIdx.x; it < 8 * S.rq; it += 128) {
+      const int fun = it / (2 * S.rq), hq = it - fun * 2 * S.rq, o = hq >> 1;
+      long long v[4];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const int q = 2 * (4 * hq + i) + (fun & 1);
+        v[i] = (e >= SPLIT_NAN || q >= nq) ? 0 : fixed53(fun < 2 ? c[q].x : c[q].y, e);
+      }
+      put_digits<6, 4>(x + C.xi + (((int64_t)fun * C.nct + ct) * C.ksi + (o >> 1)) * blk, C.n0, cit, o & 1, hq & 1, v,
+                       false, 0);
+    }
+  }
+}
+
+// One ring and lane: pixels from the orbit sums (inverse), their update or
+// output, and the orbit combinations of the forward product as digits.
+template <int MODE>
+__global__ void __launch_bounds__(128, 8) k_dft_pix(const RingDev *__restrict__ rings, const double *__restrict__ v,
+                                                 unsigned char *__restrict__ x, const int *__restrict__ xexp_in,
+                                                 int *__restrict__ xexp_out, const DftSet *__restrict__ sets,
+                                                 const DftCol *__restrict__ cols, const int *__restrict__ pair_of,
+                                                 const int *__restrict__ set_of, int nl, int lane0, int npairs,
+                                                 int nrings, int64_t npix, const double *__restrict__ in_map,
+                                                 double *__restrict__ out_map, const double *__restrict__ w,
+                                                 const double *__restrict__ wd, double *__restrict__ norms,
+                                                 const SolveState *__restrict__ state) {
+  extern __shared__ __align__(16) double so[];  // [4][nj] orbit combinations
+  __shared__ int red[4];
+  __shared__ double rsum[4][2];
+  const int g = blockIdx.x >> 1, side = blockIdx.x & 1, lane = blockIdx.y, pair = pair_of[g];
+  if (side && pair == npairs - 1) return;
+  const int al = lane0 + lane;
+  if ((MODE == RING_ITER || MODE == RING_INIT) && state != nullptr && state[al / 3].done) return;
+  const DftSet S = sets[set_of[g]];
+  const DftCol C = cols[set_of[g]];
+  const int ring = side ? nrings - 1 - pair : pair;
+  const int64_t mo = (int64_t)al * npix + rings[ring].start;
+  const int pl = g - S.pair0, col = (pl * nl + lane) * 2 + side;
+  const int n = S.n, nj = S.nj;
+  const double *vc = v + C.v + (int64_t)col * 4 * C.njp;
+  bool bad = false;
+  if (MODE == RING_ITER || MODE == RING_INV_MAP) bad = xexp_in[C.col0 + col] >= SPLIT_NAN;
+  double dd = 0.0, ss = 0.0;
+  int ex = -100000;
+  auto pixel = [&](int j, double s) -> double {  // value of pixel j after the inverse -> its residual
+    const int64_t i = mo + j;
+    if (MODE == RING_INV_MAP) {
+      out_map[i] = s;
+      return 0.0;
+    }
+    if (MODE == RING_ITER) {
+      const double d = s - out_map[i];
+      dd = fma(d, d, dd);
+      ss = fma(s, s, ss);
+      out_map[i] = s;
+      return fma(-w[i], s, wd[i]);
+    }
+    if (MODE == RING_INIT) return w[i] > 0.0 ? in_map[i] : 0.0;
+    return in_map[i];
+  };
+  for (int j = threadIdx.x; j < nj; j += 128) {
+    double a1 = 0, a2 = 0, b1 = 0, b2 = 0;
+    if (MODE == RING_ITER || MODE == RING_INV_MAP) {
+      const double ce = vc[j], co = vc[C.njp + j], se = vc[2 * C.njp + j], sn = vc[3 * C.njp + j];
+      a1 = ce + co;
+      a2 = ce - co;
+      b1 = sn + se;
+      b2 = sn - se;
+      if (bad) a1 = a2 = NAN;
+    }
+    double ce, co, se, sn;
+    if (S.shift || (j > 0 && 4 * j < n)) {
+      // the orbit of phi_j: j and its mirrors under phi -> pi - phi, -phi, pi + phi
+      const int jm = (S.shift ? n / 2 - 1 : n / 2) - j, jn = (S.shift ? n - 1 : n) - j, jp = n / 2 + j;
+      const double r0 = pixel(j, a1 - b1), r1 = pixel(jm, a2 - b2), r2 = pixel(jn, a1 + b1), r3 = pixel(jp, a2 + b2);
+      const double c0 = r0 + r2, c1 = r1 + r3, d0 = r0 - r2, d1 = r1 - r3;
+      ce = c0 + c1;
+      co = c0 - c1;
+      se = d0 - d1;
+      sn = d0 + d1;
+    } else if (j == 0) {  // phi = 0 and pi
+      const double r0 = pixel(0, a1), r1 = pixel(n / 2, a2);
+      ce = r0 + r1;
+      co = r0 - r1;
+      se = sn = 0.0;
+    } else {  // phi = pi/2 and 3 pi/2
+      const double r0 = pixel(j, a1 - b1), r2 = pixel(n - j, a1 + b1);
+      ce = r0 + r2;
+      co = se = 0.0;
+      sn = r0 - r2;
+    }
+    if (MODE != RING_INV_MAP) {
+      so[j] = ce;
+      so[nj + j] = co;
+      so[2 * nj + j] = se;
+      so[3 * nj + j] = sn;
+      ex = max(max(ex, max(exp_of(ce), exp_of(co))), max(exp_of(se), exp_of(sn)));
+    }
+  }
+  if (MODE == RING_INV_MAP) return;
+  if (MODE == RING_ITER) {
+    for (int o = 16; o > 0; o >>= 1) {
+      dd += __shfl_down_sync(0xffffffffu, dd, o);
+      ss += __shfl_down_sync(0xffffffffu, ss, o);
+    }
+    if ((threadIdx.x & 31) == 0) {
+      rsum[threadIdx.x >> 5][0] = dd;
+      rsum[threadIdx.x >> 5][1] = ss;
+    }
+  }
+  int e = max(-1000, block_max(ex, red));  // (its barriers cover the sums and the combinations too)
+  if (e >= SPLIT_NAN) e = SPLIT_NAN;
+  if (threadIdx.x == 0) {
+    xexp_out[C.col0 + col] = e;
+    if (MODE == RING_ITER) {
+      const int64_t no = ((int64_t)al * nrings + ring) * 2;
+      norms[no] = (rsum[0][0] + rsum[1][0]) + (rsum[2][0] + rsum[3][0]);
+      norms[no + 1] = (rsum[0][1] + rsum[1][1]) + (rsum[2][1] + rsum[3][1]);
+    }
+  }
+  int ct, cit;
+  col_place(C, col, ct, cit);
+  const int64_t blk = (int64_t)SPLIT_S * C.n0 * 32;
+  for (int it = threadIdx.x; it < 4 * 4 * C.ksf; it += 128) {
+    const int fun = it / (4 * C.ksf), hq = it - fun * 4 * C.ksf, o = hq >> 1;
+    long long d[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const int j = 4 * hq + i;
+      d[i] = (e >= SPLIT_NAN || j >= nj) ? 0 : fixed53(so[fun * nj + j], e);
+    }
+    put_digits<6, 4>(x + C.xf + (((int64_t)fun * C.nct + ct) * C.ksf + (o >> 1)) * blk, C.n0, cit, o & 1, hq & 1, d,
+                     false, 0);
+  }
+}
+
+// Orders beyond n/2 from the ones they alias with: thread = pair, so that the
+// stores of one order run along the pairs; blockIdx.y the order, blockIdx.z
+// the lane.  (In the products' epilogue one thread wrote all aliases of its
+// order: the shortest rings then took longest.)
+__global__ void __launch_bounds__(128) k_dft_alias(double2 *__restrict__ rc, int lane0, int mmax, int npairs,
+                                                   int nside, int nrun, const SolveState *__restrict__ state) {
+  const int m = blockIdx.y + 3, p = blockIdx.x * 128 + threadIdx.x, al = lane0 + blockIdx.z;
+  const int n = 4 * min(p + 1, nside);  // the orders up to n / 2 are the products' own
+  if (p >= nrun || 2 * m <= n) return;
+  if (state != nullptr && state[al / 3].done) return;
+  const bool shift = p < nside || !((p - nside + 1) & 1);
+  const int k0 = m / n, r = m - k0 * n;
+  const bool fold = 2 * r > n;
+  const int q = fold ? n - r : r, k = fold ? k0 + 1 : k0;
+  const double re = (shift && (k & 1)) ? -1.0 : 1.0, im = fold ? -re : re;
+  double2 *o = rc + ((int64_t)al * (mmax + 1) * npairs + p) * 2;
+  const double2 a = o[(int64_t)q * npairs * 2];
+  o[(int64_t)m * npairs * 2] = make_double2(re * a.x, im * a.y);
+  if (p == npairs - 1) return;  // the equator has no mirror ring
+  const double2 b = o[(int64_t)q * npairs * 2 + 1];
+  o[(int64_t)m * npairs * 2 + 1] = make_double2(re * b.x, im * b.y);
+}
+
+struct DftArgs {
+  const DftTile *tiles;
+  int ntiles;
+  const CUtensorMap *maps;
+  const DftSet *sets;
+  const DftCol *cols;
+  const int *pair_of;
+  const unsigned char *x;
+  const int *xexp;
+  int nl, lane0, mmax, npairs;
+  double *v;            // inverse: orbit sums
+  double2 *rc;          // forward: ring coefficients
+  const SolveState *state;
+  int nstages;
+  int *err;
+};
+
+__device__ __forceinline__ void map_acquire(const CUtensorMap *map) {
+  asm volatile("fence.proxy.tensormap::generic.acquire.gpu [%0], 128;" ::"l"(map) : "memory");
+}
+
+// FWD: rows are orders of one parity (cosine and sine sums in one tile), K the
+// orbits; else rows are orbits of one matrix, K the orders.  The structure of
+// the Legendre products (k_split): warps 0-7 drain, warp 8 streams, warp 9
+// issues.
+template <bool FWD, int NQ>
+__global__ void __launch_bounds__(DFT_THREADS, 1) k_dft(const DftArgs A) {
+  constexpr int S = SPLIT_S, G = Weights<S>::G, N0 = 8 * NQ;
+  constexpr int SET = (G * N0 + ((N0 & 15) ? 8 : 0) + 15) / 16 * 16;
+  constexpr int COLS = 2 * SET <= 128 ? 128 : (2 * SET <= 256 ? 256 : 512);
+  constexpr int ABYTES = S * 4096, BBYTES = S * N0 * 32, ZBYTES = (N0 + 8) * 32, STAGE = ABYTES + BBYTES + ZBYTES;
+  constexpr int NF = FWD ? 2 : 1;
+  extern __shared__ __align__(1024) unsigned char sm[];
+  __shared__ uint64_t bars[2 * DFT_MAX_STAGES + 5];
+  __shared__ uint32_t tslot;
+  __shared__ int cta_bad;
+  uint64_t *full = bars, *empty = bars + DFT_MAX_STAGES, *tfull = bars + 2 * DFT_MAX_STAGES, *tempty = tfull + 2,
+           *fin = tempty + 2;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int NS = A.nstages;
+  if (tid == 0) {
+    for (int i = 0; i < NS; ++i) {
+      mbar_init(&full[i], 1);
+      mbar_init(&empty[i], 1);
+    }
+    for (int i = 0; i < 2; ++i) {
+      mbar_init(&tfull[i], 1);
+      mbar_init(&tempty[i], DFT_DRAIN_WARPS);
+    }
+    mbar_init(fin, 1);
+    cta_bad = 0;
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  for (int i = tid; i < NS * (ZBYTES / 16); i += DFT_THREADS)
+    *reinterpret_cast<uint4 *>(sm + (size_t)(i / (ZBYTES / 16)) * STAGE + ABYTES + BBYTES + (i % (ZBYTES / 16)) * 16) =
+        make_uint4(0, 0, 0, 0);
+  fence_proxy_async();
+  if (warp == 0) tmem_alloc(&tslot, COLS);
+  fence_before_sync();
+  __syncthreads();
+  fence_after_sync();
+  const uint32_t tbase = tslot;
+  int issued = 0;
+  const uint32_t sm_a = smem_u32(sm), full_a = smem_u32(full), empty_a = smem_u32(empty);
+
+  if (warp == DFT_DRAIN_WARPS) {
+    if (lane == 0) {
+      bool ok = true;
+      StageAt at;
+      for (int t = blockIdx.x; ok && t < A.ntiles; t += gridDim.x) {
+        const DftTile T = A.tiles[t];
+        const CUtensorMap *map = A.maps + 2 * T.set + (FWD ? 1 : 0);
+        map_acquire(map);
+        for (int k0 = 0; ok && k0 < T.ks; k0 += DFT_CHUNK)
+          for (int f = 0; ok && f < NF; ++f)
+            for (int k = k0; k < min(k0 + DFT_CHUNK, T.ks); ++k) {
+              if (issued >= NS && !mbar_wait_at(empty_a + 8 * at.s, at.phase ^ 1, A.err)) {
+                ok = false;
+                break;
+              }
+              const uint32_t dst = sm_a + at.s * STAGE, bar = full_a + 8 * at.s;
+              mbar_expect_tx_at(bar, ABYTES + BBYTES);
+              const int z = T.z + f * T.zfun;
+              if (FWD)
+                tma_box_at(dst, map, 2 * k, z, bar);
+              else
+                tma_box_at(dst, map, 16 * T.row, z + 2 * k, bar);
+              bulk_g2s_at(dst + ABYTES, A.x + T.x + f * T.xfun + (int64_t)k * BBYTES, BBYTES, bar);
+              ++issued;
+              at.next(NS);
+            }
+      }
+      if (!ok) cta_bad = 1;
+    }
+  } else if (warp == DFT_DRAIN_WARPS + 1) {
+    if (lane == 0) {
+      bool ok = true;
+      int cc = 0;
+      StageAt at;
+      const uint64_t ad0 = FWD ? split_desc(sm_a, 128, 256) : split_desc(sm_a, 2048, 128);
+      const uint64_t bd0 = split_desc(sm_a + ABYTES, 128, 256);
+      for (int t = blockIdx.x; ok && t < A.ntiles; t += gridDim.x) {
+        const int ks = A.tiles[t].ks, nch = NF * ((ks + DFT_CHUNK - 1) / DFT_CHUNK);
+        for (int c = 0; ok && c < nch; ++c, ++cc) {
+          const int set = cc & 1;
+          if (cc >= 2 && !mbar_wait(&tempty[set], ((cc >> 1) - 1) & 1, A.err)) {
+            ok = false;
+            break;
+          }
+          fence_after_sync();
+          const int nstep = min(DFT_CHUNK, ks - (c / NF) * DFT_CHUNK);
+          const uint32_t d = tbase + set * SET;
+          for (int k = 0; k < nstep; ++k) {
+            if (!mbar_wait_at(full_a + 8 * at.s, at.phase, A.err)) {
+              ok = false;
+              break;
+            }
+            fence_after_sync();
+            const uint64_t off = (uint64_t)(at.s * (STAGE >> 4));
+            if (k == 0)
+              split_step<S, N0, 4096, !FWD, true>(d, ad0 + off, bd0 + off);
+            else
+              split_step<S, N0, 4096, !FWD, false>(d, ad0 + off, bd0 + off);
+            commit_at(empty_a + 8 * at.s);
+            at.next(NS);
+          }
+          if (ok) commit(&tfull[set]);
+        }
+      }
+      if (!ok) cta_bad = 1;
+      commit(fin);
+      mbar_wait(fin, 0, A.err);
+    }
+  } else {
+    const int half = warp >> 2, wq = warp & 3;
+    bool ok = true;
+    int cc = 0;
+    for (int t = blockIdx.x; ok && t < A.ntiles; t += gridDim.x) {
+      const DftTile T = A.tiles[t];
+      const DftSet D = A.sets[T.set];
+      const DftCol C = A.cols[T.set];
+      const int ncol = D.npr * A.nl * 2, c0 = T.ct * C.w + half * NQ * 4;
+      const int cend = min(ncol, (T.ct + 1) * C.w);  // columns of the tile end here
+      const int nch = NF * ((T.ks + DFT_CHUNK - 1) / DFT_CHUNK);
+      Acc<S> acc[NF][NQ][4];
+      for (int c = 0; c < nch; ++c, ++cc) {
+        const int set = cc & 1;
+        if (!mbar_wait(&tfull[set], (cc >> 1) & 1, A.err)) {
+          ok = false;
+          break;
+        }
+        __syncwarp();
+        fence_after_sync();
+        const uint32_t tcol = tbase + ((uint32_t)(wq * 32) << 16) + set * SET + half * NQ * 4;
+#pragma unroll
+        for (int q = 0; q < NQ; ++q) {
+          if (c0 + 4 * q >= cend) break;
+          uint32_t g[G][4];
+#pragma unroll
+          for (int k = 0; k < G; ++k) tmem_ld4(tcol + k * N0 + q * 4, g[k]);
+          tmem_wait_ld();
+#pragma unroll
+          for (int e = 0; e < 4; ++e) {
+            int w[G];
+#pragma unroll
+            for (int k = 0; k < G; ++k) w[k] = __float2int_rn(__uint_as_float(g[k][e]));
+            if (NF == 2 && (c & 1))
+              acc[NF - 1][q][e].add(w);
+            else
+              acc[0][q][e].add(w);
+          }
+        }
+        fence_before_sync();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&tempty[set]);
+      }
+      if (!ok) break;
+      const int row = T.row * 128 + wq * 32 + lane;
+      if (!FWD) {
+        if (row < D.nj) {
+#pragma unroll
+          for (int q = 0; q < NQ; ++q)
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+              const int col = c0 + 4 * q + e;
+              if (col >= cend) break;
+              A.v[C.v + ((int64_t)col * 4 + T.fun) * C.njp + row] = value_of(acc[0][q][e], A.xexp[C.col0 + col]);
+            }
+        }
+      } else {
+        const int qo = 2 * row + T.fun;  // the order
+        if (qo <= D.mx) {
+#pragma unroll
+          for (int q = 0; q < NQ; ++q)
+#pragma unroll
+            for (int e = 0; e < 4; e += 2) {  // the two sides of one pair and lane
+              const int col = c0 + 4 * q + e;
+              if (col >= cend) break;
+              const int pc = col >> 1, pl = pc / A.nl, ln = pc - pl * A.nl, al = A.lane0 + ln;
+              if (A.state != nullptr && A.state[al / 3].done) continue;
+              const int pair = A.pair_of[D.pair0 + pl];
+              const bool equator = pair == A.npairs - 1;
+              const int en = A.xexp[C.col0 + col], es = equator ? 0 : A.xexp[C.col0 + col + 1];
+              double2 f = make_double2(value_of(acc[0][q][e], en), -value_of(acc[NF - 1][q][e], en));
+              double2 s = make_double2(value_of(acc[0][q][e + 1], es), -value_of(acc[NF - 1][q][e + 1], es));
+              if (en >= SPLIT_NAN) f.x = f.y = NAN;
+              if (es >= SPLIT_NAN) s.x = s.y = NAN;
+              double2 *o = A.rc + (((int64_t)al * (A.mmax + 1) + qo) * A.npairs + pair) * 2;
+              o[0] = f;
+              if (!equator) o[1] = s;
+            }
+        }
+      }
+    }
+    if (!ok && lane == 0) cta_bad = 1;
+  }
+  __syncthreads();
+  if (cta_bad && warp == DFT_DRAIN_WARPS && lane == 0)
+    for (int c = max(0, issued - NS); c < issued; ++c) mbar_wait(&full[c % NS], (c / NS) & 1, A.err);
+  fence_before_sync();
+  __syncthreads();
+  if (warp == 0) tmem_dealloc(tbase, COLS);
+}
+
+void drop_cut(DftCut &c) {
+  if (c.cols) cudaFree(c.cols);
+  for (auto &d : c.tiles)
+    for (DftTile *t : d)
+      if (t) cudaFree(t);
+}
+
+}  // namespace
+
+// Matrix sets of a plan: polar radii, then the belt with and without the shift.
+static std::vector<DftSet> dft_sets(const dm_plan *p, std::vector<int> *pairs, std::vector<int> *set_of) {
+  std::vector<DftSet> sets;
+  auto make = [&](int n, int shift) {
+    DftSet s{};
+    s.n = n;
+    s.shift = shift;
+    s.nj = n / 4 + (shift ? 0 : 1);
+    s.mx = std::min(p->mmax, n / 2);
+    s.rq = 2 * ((s.mx / 2 + 16) / 16);
+    s.nyo = (s.nj + 7) / 8;
+    s.pair0 = (int)pairs->size();
+    return s;
+  };
+  for (int i = 1; i < p->nside; ++i) {
+    DftSet s = make(4 * i, 1);
+    s.npr = 1;
+    pairs->push_back(i - 1);
+    sets.push_back(s);
+  }
+  for (int shift = 1; shift >= 0; --shift) {
+    DftSet s = make(4 * p->nside, shift);
+    for (int q = p->nside - 1; q < p->npairs; ++q)
+      if (p->rings_h[q].shift == shift) pairs->push_back(q);
+    s.npr = (int)pairs->size() - s.pair0;
+    if (s.npr > 0) sets.push_back(s);
+  }
+  for (size_t k = 0; k < sets.size(); ++k)
+    for (int q = 0; q < sets[k].npr; ++q) set_of->push_back((int)k);
+  return sets;
+}
+
+static size_t set_bytes(const DftSet &s) { return (size_t)SPLIT_S * 4 * s.rq * s.nyo * 128; }
+
+// Bytes of the matrix sets of a sphere plan.
+size_t dft_table_bytes(int nside, int mmax) {
+  double b = 0;
+  for (int i = 1; i <= nside; ++i)
+    b += (double)SPLIT_S * 4 * 2 * ((std::min(mmax, 2 * i) / 2 + 16) / 16) * ((i + 8) / 8) * 128 * (i == nside ? 2 : 1);
+  return (size_t)b;
+}
+
+void dft_release(dm_plan *p) {
+  DftTables *T = p->dft;
+  if (!T) return;
+  for (DftCut &c : T->cuts) drop_cut(c);
+  for (void *q : {(void *)T->dig, (void *)T->sets_dev, (void *)T->maps, (void *)T->pair_of, (void *)T->set_of,
+                  (void *)T->x, (void *)T->v, (void *)T->xexp})
+    if (q) cudaFree(q);
+  delete T;
+  p->dft = nullptr;
+}
+void dft_new(dm_plan *p) { p->dft = new DftTables(); }
+void dft_disable(dm_plan *p) { p->dft->failed = true; }
+int64_t dft_bytes(const dm_plan *p) { return p->dft ? p->dft->bytes : 0; }
+
+static cudaError_t dft_setup(dm_plan *p, cudaStream_t st) {
+  DftTables *T = p->dft;
+  if (T->dig) return cudaSuccess;
+  if (!encode_fn()) return cudaErrorNotSupported;
+  std::vector<int> pairs, set_of;
+  T->sets = dft_sets(p, &pairs, &set_of);
+  T->nlist = (int)pairs.size();
+  const int ns = (int)T->sets.size();
+  int64_t total = 0;
+  T->off.clear();
+  for (const DftSet &s : T->sets) {
+    T->off.push_back(total);
+    total += (int64_t)set_bytes(s);
+  }
+  cudaError_t e;
+  unsigned char *dig = nullptr;
+  auto up = [&](auto **dst, const auto *src, size_t count) {
+    if (*dst == nullptr)
+      if (cudaError_t r = cudaMalloc((void **)dst, sizeof(*src) * count)) return r;
+    return cudaMemcpyAsync((void *)*dst, src, sizeof(*src) * count, cudaMemcpyHostToDevice, st);
+  };
+  if ((e = cudaMalloc(&dig, (size_t)total))) return e;
+  std::vector<CUtensorMap> maps(2 * ns);
+  for (int k = 0; k < ns && !e; ++k) {
+    const DftSet &s = T->sets[k];
+    for (int dir = 0; dir < 2; ++dir) {
+      const cuuint64_t dims[4] = {64, (cuuint64_t)s.nyo, (cuuint64_t)(4 * s.rq), SPLIT_S};
+      const cuuint64_t strides[3] = {128, (cuuint64_t)s.nyo * 128, (cuuint64_t)(4 * s.rq) * s.nyo * 128};
+      const cuuint32_t box[4] = {64, dir == 0 ? 16u : 2u, dir == 0 ? 2u : 16u, SPLIT_S};
+      const cuuint32_t one[4] = {1, 1, 1, 1};
+      if (encode_fn()(&maps[2 * k + dir], CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, dig + T->off[k], dims, strides, box,
+                      one, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
+                      CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
+        e = cudaErrorInvalidValue;
+    }
+    const int64_t items = (int64_t)4 * s.rq * 8 * s.nyo;
+    k_dft_gen<<<(unsigned)std::min<int64_t>((items + 127) / 128, 4096), 128, 0, st>>>(s, dig + T->off[k]);
+  }
+  if (!e) e = cudaGetLastError();
+  if (!e) e = up(&T->maps, maps.data(), maps.size());
+  if (!e) e = up(&T->sets_dev, T->sets.data(), T->sets.size());
+  if (!e) e = up(&T->pair_of, pairs.data(), pairs.size());
+  if (!e) e = up(&T->set_of, set_of.data(), set_of.size());
+  if (!e) e = cudaStreamSynchronize(st);
+  if (e) {
+    cudaFree(dig);
+    return e;
+  }
+  T->dig = dig;
+  T->bytes += total + (int64_t)(sizeof(CUtensorMap) * maps.size() + sizeof(DftSet) * ns + 2 * sizeof(int) * pairs.size());
+  return cudaSuccess;
+}
+
+// Column digits of nl lanes: bytes of the larger direction.
+static size_t cut_layout(const DftTables *T, int nl, std::vector<DftCol> *cols, int *ncol, size_t *vcount) {
+  size_t xi = 0, xf = 0, v = 0;
+  int c0 = 0;
+  cols->clear();
+  for (const DftSet &s : T->sets) {
+    DftCol c{};
+    const int n = s.npr * nl * 2;
+    c.nct = (n + 31) / 32;
+    c.w = ((n + c.nct - 1) / c.nct + 3) / 4 * 4;
+    c.nct = (n + c.w - 1) / c.w;
+    c.n0 = (c.w + 7) / 8 * 8;
+    c.ksi = s.rq / 2;
+    c.ksf = (s.nj + 15) / 16;
+    c.col0 = c0;
+    c.njp = (s.nj + 3) / 4 * 4;
+    c.xi = (int64_t)xi;
+    c.xf = (int64_t)xf;
+    c.v = (int64_t)v;
+    const size_t blk = (size_t)SPLIT_S * c.n0 * 32;
+    xi += 4 * (size_t)c.nct * c.ksi * blk;
+    xf += 4 * (size_t)c.nct * c.ksf * blk;
+    v += (size_t)n * 4 * c.njp;
+    c0 += n;
+    cols->push_back(c);
+  }
+  *ncol = c0;
+  *vcount = v;
+  return std::max(xi, xf);
+}
+
+static cudaError_t dft_cut(dm_plan *p, int nl, cudaStream_t st) {
+  DftTables *T = p->dft;
+  DftCut K;
+  K.nl = nl;
+  std::vector<DftCol> cols;
+  K.xbytes = cut_layout(T, nl, &cols, &K.ncol, &K.vcount);
+  cudaError_t e = cudaMalloc(&K.cols, sizeof(DftCol) * cols.size());
+  if (!e) e = cudaMemcpyAsync(K.cols, cols.data(), sizeof(DftCol) * cols.size(), cudaMemcpyHostToDevice, st);
+  for (int dir = 0; dir < 2 && !e; ++dir) {
+    std::vector<DftTile> tiles[5];
+    for (int k = 0; k < (int)T->sets.size(); ++k) {
+      const DftSet &s = T->sets[k];
+      const DftCol &c = cols[k];
+      const int64_t blk = (int64_t)SPLIT_S * c.n0 * 32;
+      const int ks = dir == 0 ? c.ksi : c.ksf;
+      for (int fun = 0; fun < (dir == 0 ? 4 : 2); ++fun) {
+        const int rows = dir == 0 ? s.nj : (s.mx - fun) / 2 + (s.mx >= fun ? 1 : 0);
+        for (int r = 0; r < (rows + 127) / 128; ++r)
+          for (int ct = 0; ct < c.nct; ++ct) {
+            DftTile t{};
+            t.set = k;
+            t.fun = fun;
+            t.row = r;
+            t.ct = ct;
+            t.ks = ks;
+            t.z = fun * s.rq + (dir == 0 ? 0 : 16 * r);
+            t.zfun = 2 * s.rq;
+            t.n0 = c.n0;
+            t.x = (dir == 0 ? c.xi : c.xf) + ((int64_t)fun * c.nct + ct) * ks * blk;
+            t.xfun = (int64_t)2 * c.nct * ks * blk;
+            tiles[c.n0 / 8].push_back(t);
+          }
+      }
+    }
+    for (int q = 1; q < 5 && !e; ++q) {
+      if (tiles[q].empty()) continue;
+      std::stable_sort(tiles[q].begin(), tiles[q].end(), [](const DftTile &a, const DftTile &b) { return a.ks > b.ks; });
+      e = cudaMalloc(&K.tiles[dir][q], sizeof(DftTile) * tiles[q].size());
+      if (!e)
+        e = cudaMemcpyAsync(K.tiles[dir][q], tiles[q].data(), sizeof(DftTile) * tiles[q].size(),
+                            cudaMemcpyHostToDevice, st);
+      if (!e) e = cudaStreamSynchronize(st);
+      K.ntiles[dir][q] = (int)tiles[q].size();
+    }
+  }
+  if (!e) e = cudaStreamSynchronize(st);
+  if (!e && T->xbytes < K.xbytes) {
+    if (T->x) cudaFree(T->x);
+    T->bytes += (int64_t)K.xbytes - (int64_t)T->xbytes;
+    T->x = nullptr;
+    T->xbytes = 0;
+    if (!(e = cudaMalloc(&T->x, K.xbytes))) T->xbytes = K.xbytes;
+  }
+  if (!e && T->vcount < K.vcount) {
+    if (T->v) cudaFree(T->v);
+    T->bytes += (int64_t)(8 * (K.vcount - T->vcount));
+    T->v = nullptr;
+    T->vcount = 0;
+    if (!(e = cudaMalloc(&T->v, sizeof(double) * K.vcount))) T->vcount = K.vcount;
+  }
+  if (!e && T->xexp_n < K.ncol) {
+    if (T->xexp) cudaFree(T->xexp);
+    T->xexp = nullptr;
+    T->xexp_n = 0;
+    if (!(e = cudaMalloc(&T->xexp, sizeof(int) * 2 * K.ncol))) T->xexp_n = K.ncol;
+  }
+  if (e) {
+    drop_cut(K);
+    return e;
+  }
+  if (T->cuts.size() >= 6) {
+    for (DftCut &c : T->cuts) drop_cut(c);
+    T->cuts.clear();
+  }
+  T->cuts.push_back(K);
+  return cudaSuccess;
+}
+
+// Right-hand sides per group: as many as the column digits of DFT_SCRATCH bytes hold.
+static int dft_group(const dm_plan *p) {
+  std::vector<DftCol> cols;
+  int nc;
+  size_t v;
+  int g = p->batch;
+  while (g > 1 && cut_layout(p->dft, 3 * g, &cols, &nc, &v) > DFT_SCRATCH) g = (g + 1) / 2;
+  return g;
+}
+
+size_t dft_scratch_bytes(int nside, int batch) {  // bound of the column digits and orbit sums
+  const double px = 12.0 * nside * nside * 3 * batch;
+  return (size_t)(std::min(1.5 * px * 12.0, 2.0 * (double)DFT_SCRATCH) + std::min(1.3 * px * 8.0, 1.5 * (double)DFT_SCRATCH)) +
+         ((size_t)32 << 20);
+}
+
+static const DftCut *dft_ready(dm_plan *p, int nl, cudaStream_t st) {
+  DftTables *T = p->dft;
+  if (!T || T->failed) return nullptr;
+  for (const DftCut &c : T->cuts)
+    if (c.nl == nl) return &c;
+  cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(st, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone) {
+    cudaGetLastError();
+    return nullptr;
+  }
+  cudaError_t e = (int64_t)dft_table_bytes(p->nside, p->mmax) > p->dft_cap ? cudaErrorMemoryAllocation
+                                                                            : dft_setup(p, st);
+  if (!e) e = dft_cut(p, nl, st);
+  if (e) {
+    cudaGetLastError();
+    T->failed = true;
+    return nullptr;
+  }
+  return &T->cuts.back();
+}
+
+template <bool FWD>
+static cudaError_t dft_products(dm_plan *p, const DftCut &K, int lane0, const SolveState *state, cudaStream_t st) {
+  DftTables *T = p->dft;
+  int dev = 0, sms = 0;
+  cudaGetDevice(&dev);
+  if (cudaError_t r = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) return r;
+  for (int q = 4; q >= 1; --q) {
+    const int nt = K.ntiles[FWD][q];
+    if (nt == 0) continue;
+    DftArgs A;
+    A.tiles = K.tiles[FWD][q];
+    A.ntiles = nt;
+    A.maps = T->maps;
+    A.sets = T->sets_dev;
+    A.cols = K.cols;
+    A.pair_of = T->pair_of;
+    A.x = T->x;
+    A.xexp = T->xexp + (FWD ? T->xexp_n : 0);
+    A.nl = K.nl;
+    A.lane0 = lane0;
+    A.mmax = p->mmax;
+    A.npairs = p->npairs;
+    A.v = T->v;
+    A.rc = p->rc;
+    A.state = state;
+    A.err = p->tc_err;
+    const int n0 = 8 * q, stage = SPLIT_S * 4096 + SPLIT_S * n0 * 32 + (n0 + 8) * 32;
+    A.nstages = std::min(DFT_MAX_STAGES, (int)((224u << 10) / stage));
+    const size_t smem = (size_t)A.nstages * stage;
+    auto go = [&](auto kern) {
+      if (cudaError_t r = dyn_smem_allow(kern, smem)) return r;
+      kern<<<std::min(sms, nt), DFT_THREADS, smem, st>>>(A);
+      return cudaGetLastError();
+    };
+    cudaError_t e;
+    switch (q) {
+      case 1: e = go(k_dft<FWD, 1>); break;
+      case 2: e = go(k_dft<FWD, 2>); break;
+      case 3: e = go(k_dft<FWD, 3>); break;
+      default: e = go(k_dft<FWD, 4>); break;
+    }
+    if (e) return e;
+  }
+  return cudaSuccess;
+}
+
+// The FP64 ring stage (modes of ring_stage) as split products; *ran = false
+// when the FFT kernels have to do it.
+cudaError_t dft_ring_stage(dm_plan *p, int mode, const double *in_map, double *out_map, cudaStream_t st, bool *ran) {
+  *ran = false;
+  if (p->flat || !p->dft || p->dft->failed || p->ring_fft || p->tune_only_class >= 0) return cudaSuccess;
+  if (!p->dft->dig && !dft_ready(p, 3, st)) return cudaSuccess;  // the tables, before the group is known
+  const int gb = dft_group(p);
+  for (int b0 = 0; b0 < p->batch; b0 += gb)
+    if (!dft_ready(p, 3 * std::min(gb, p->batch - b0), st)) return cudaSuccess;
+  *ran = true;
+  DftTables *T = p->dft;
+  const SolveState *state = (mode == RING_ITER || mode == RING_INIT) ? p->state : nullptr;
+  for (int b0 = 0; b0 < p->batch; b0 += gb) {
+    const int nl = 3 * std::min(gb, p->batch - b0), lane0 = 3 * b0;
+    const DftCut *K = dft_ready(p, nl, st);
+    if (!K) return cudaErrorMemoryAllocation;
+    cudaError_t e;
+    int *ei = T->xexp, *ef = T->xexp + T->xexp_n;
+    if (mode == RING_ITER || mode == RING_INV_MAP) {
+      const size_t sm = sizeof(double2) * std::max(256, 2 * (p->mmax + 1));
+      if ((e = dyn_smem_allow(k_dft_xinv, sm))) return e;
+      k_dft_xinv<<<dim3(T->nlist, nl), 128, sm, st>>>(p->rc, T->x, ei, T->sets_dev, K->cols, T->pair_of, T->set_of, nl,
+                                                      lane0, p->mmax, p->npairs, state);
+      if ((e = dft_products<false>(p, *K, lane0, state, st))) return e;
+    }
+    const size_t sp = sizeof(double) * 4 * (p->nside + 1);
+    auto pix = [&](auto kern) {
+      if (cudaError_t r = dyn_smem_allow(kern, sp)) return r;
+      kern<<<dim3(2 * T->nlist, nl), 128, sp, st>>>(p->rings, T->v, T->x, ei, ef, T->sets_dev, K->cols, T->pair_of,
+                                                    T->set_of, nl, lane0, p->npairs, p->nrings, p->npix, in_map,
+                                                    out_map, p->w, p->wd, p->norms, state);
+      return cudaGetLastError();
+    };
+    switch (mode) {
+      case RING_ITER: e = pix(k_dft_pix<RING_ITER>); break;
+      case RING_INV_MAP: e = pix(k_dft_pix<RING_INV_MAP>); break;
+      case RING_INIT: e = pix(k_dft_pix<RING_INIT>); break;
+      default: e = pix(k_dft_pix<RING_FWD_MAP>); break;
+    }
+    if (e) return e;
+    if (mode == RING_INV_MAP) continue;
+    if ((e = dft_products<true>(p, *K, lane0, state, st))) return e;
+    // pairs with orders beyond n / 2: the shorter polar rings, and the belt where mmax exceeds 2 nside
+    const int nrun = p->mmax > 2 * p->nside ? p->npairs : std::min(p->nside - 1, (p->mmax + 1) / 2);
+    if (nrun > 0 && p->mmax >= 3) {
+      k_dft_alias<<<dim3((nrun + 127) / 128, p->mmax - 2, nl), 128, 0, st>>>(p->rc, lane0, p->mmax, p->npairs,
+                                                                             p->nside, nrun, state);
+      if ((e = cudaGetLastError())) return e;
+    }
+  }
+  return cudaSuccess;
+}
+
+}  // namespace dmwf

@@ -68,6 +68,7 @@ struct RingClass {
 };
 
 struct SplitTables;  // dm_split.cu
+struct DftTables;    // dm_dft.cu
 
 struct LevelDev {
   int n_levels;
@@ -121,6 +122,7 @@ struct dm_plan {
   int twr_off[2][16] = {{-1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1}, {-1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1}};  // [LR - 3][LOGM]: offset in twr (-1: not built)
   int twr_words = 0;
   int ring_lr = 3;              // radix 2^ring_lr of the fixed-size ring transforms (0: generic kernels)
+  bool ring_fft = false;        // dm_set_ring_radix was called: the FFT kernels in the FP64-class modes too
   int *ring_order = nullptr;    // [nrings] ring ids grouped by FFT size class
   int *pair_order = nullptr;    // [npairs] the side-0 ring of each pair, grouped by class
   std::vector<int> pair_order_h;
@@ -158,6 +160,9 @@ struct dm_plan {
   bool fp32_ready = false;      // the buffers of the FP32 modes exist (setup_fp32 succeeded)
   // digit tables of the split products (dm_split.cu): shared with the views of the plan
   dmwf::SplitTables *split = nullptr;
+  // ring DFT matrices of the FP64-class modes (dm_dft.cu), shared likewise
+  dmwf::DftTables *dft = nullptr;
+  int64_t dft_cap = (int64_t)8 << 30;  // largest matrix table kept (else the FFT kernels)
   int64_t split_cap = (int64_t)24 << 30;  // largest whole table kept
   int64_t ffs_cap = (int64_t)1 << 30;  // bytes of the largest slab when the table is not kept whole
   bool ffs_cap_set = false;     // dm_set_ff_slab_bytes was called: slabs of that size, no whole table
@@ -314,6 +319,14 @@ inline cudaError_t dyn_smem_allow(F *func, size_t bytes) {
 }
 // first alm index of order m (m = mmax + 1 = lmax + 1 gives nalm): idx(l, m) = start(m) + l - m
 inline int64_t alm_start_h(int lmax, int m) { return (int64_t)m * (2 * lmax + 3 - m) / 2; }
+// FP64-class ring transforms as split products (dm_dft.cu)
+void dft_new(dm_plan *p);
+void dft_release(dm_plan *p);
+void dft_disable(dm_plan *p);
+int64_t dft_bytes(const dm_plan *p);
+size_t dft_table_bytes(int nside, int mmax);
+size_t dft_scratch_bytes(int nside, int batch);
+cudaError_t dft_ring_stage(dm_plan *p, int mode, const double *in_map, double *out_map, cudaStream_t st, bool *ran);
 // split products of the Legendre stages (dm_split.cu)
 void split_new(dm_plan *p);
 void split_release(dm_plan *p);

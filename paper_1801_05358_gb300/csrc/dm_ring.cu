@@ -728,6 +728,9 @@ int ring_lanes_per_block(size_t word_bytes, int tw_words, int ph_words, int lane
 // the caller's s buffer; FP32: the plan's s32).
 cudaError_t ring_stage(dm_plan *p, int mode, const double *in_map, double *out_map, cudaStream_t st) {
   if (p->prec == DM_FP64) {
+    bool ran = false;
+    cudaError_t e = dft_ring_stage(p, mode, in_map, out_map, st, &ran);
+    if (e || ran) return e;
     switch (mode) {
       case RING_FWD_MAP:
         return launch_ring<double, double2, RING_FWD_MAP>(p, p->phase, p->bhat, p->chirp, p->twid, p->rc, in_map, nullptr,

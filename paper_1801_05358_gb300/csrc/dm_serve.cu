@@ -287,6 +287,12 @@ Pool *make_pool(dm_server *S, const Request &r, dm_status *why) {
       p->ffs_cap = (int64_t)std::max((double)(1 << 20), std::min(whole, tables));
       take = tables;
     }
+    // the ring DFT matrices with what is left, else the FFT kernels
+    const double rings = (double)dft_table_bytes(r.nside, p->mmax) + (double)dft_scratch_bytes(r.nside, slots);
+    if (take + rings <= room)
+      take += rings;
+    else
+      dft_disable(p);
     if (take > tables) need += (size_t)(take - tables);
   }
   pool->reserved = need;
