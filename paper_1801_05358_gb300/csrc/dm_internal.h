@@ -194,6 +194,7 @@ struct dm_plan {
   int tc_withhold = 0;          // test hook: one withheld arrival in the spin-0 analysis (dm_test_tc_withhold)
   // tiled BF16 hi/lo Legendre tables of the tensor-core stages ([0] = lambda, [1] = lam+/lam-)
   unsigned char *tc_synA[2] = {nullptr, nullptr}, *tc_anaA[2] = {nullptr, nullptr};
+  int *tc_ks = nullptr;         // first K step of every tile (visible_steps)
   int64_t *tc_soff = nullptr, *tc_aoff = nullptr;  // block offsets per m / per (m, parity)
   unsigned char *tc_synB[2] = {nullptr, nullptr};   // per-iteration synthesis B operand tiles
   // tensor-core Legendre tiles generated in the kernels (dm_legendre_otf.cu):
@@ -329,6 +330,7 @@ size_t dft_scratch_bytes(int nside, int batch);
 cudaError_t dft_ring_stage(dm_plan *p, int mode, const double *in_map, double *out_map, cudaStream_t st, bool *ran);
 // split products of the Legendre stages (dm_split.cu)
 void split_new(dm_plan *p);
+cudaError_t visible_steps(dm_plan *p, int floor_exp, int **out);
 void split_release(dm_plan *p);
 void split_forget(dm_plan *p);
 int64_t split_bytes(const dm_plan *p);

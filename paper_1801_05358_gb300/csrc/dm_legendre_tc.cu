@@ -36,6 +36,12 @@ namespace {
 
 constexpr int TC_THREADS = 256;
 
+// K steps before the first Legendre value of a tile that reaches 2^-60 are
+// left out: the evanescent region (m well above l sin theta), where a value
+// this small changes no bit of an FP32 sum with those of the other rings.  It
+// holds 10 % of the K steps at nside 256 / lmax 512, 20 % at nside 512 / 1024.
+constexpr int TC_FLOOR_EXP = -60;
+
 __device__ __forceinline__ float2 e_of(const double2 *a, const double2 *ahi, int64_t i) {
   double2 v = a[i];
   if (ahi != nullptr) {
@@ -192,9 +198,10 @@ constexpr int TC_MAX_STAGES = 8;
 template <int PART>
 __global__ void __launch_bounds__(128, 1) k_syn_tc(const unsigned char *__restrict__ tab,
                                                    const unsigned char *__restrict__ bt,
-                                                   const int64_t *__restrict__ soff, float2 *__restrict__ rc,
-                                                   int lmax, int mmax, int npairs, int B, int NS, uint32_t ncols,
-                                                   int *err) {
+                                                   const int64_t *__restrict__ soff,
+                                                   const int *__restrict__ ks, int ks_stride,
+                                                   float2 *__restrict__ rc, int lmax, int mmax, int npairs, int B,
+                                                   int NS, uint32_t ncols, int *err) {
   extern __shared__ __align__(1024) unsigned char sm[];
   __shared__ uint64_t mbar[2 * TC_MAX_STAGES];  // done[NS] (MMAs of the stage finished), full[NS] (operands landed)
   __shared__ uint32_t tslot;
@@ -218,11 +225,14 @@ __global__ void __launch_bounds__(128, 1) k_syn_tc(const unsigned char *__restri
   __syncthreads();
   fence_after_sync();
   const uint32_t tbase = tslot;
-  const int nsteps = syn_steps(lmax, m);
+  const int all_steps = syn_steps(lmax, m);
+  // first K step (32 multipoles) with a visible value; one step at least, so that the accumulators are written
+  const int first = min(all_steps - 1, ks[((int64_t)PART * (mmax + 1) + m) * ks_stride + pt] >> 1);
+  const int nsteps = all_steps - first;
   const int nunits = nsteps * UPS;
   if (tid == 0) {
-    const unsigned char *tabm = tab + (soff[m] * npt + (int64_t)pt * nsteps) * (int64_t)abytes;
-    const unsigned char *btm = bt + soff[m] * (int64_t)bbytes;
+    const unsigned char *tabm = tab + (soff[m] * npt + (int64_t)pt * all_steps + first) * (int64_t)abytes;
+    const unsigned char *btm = bt + (soff[m] + first) * (int64_t)bbytes;
     const uint32_t idesc = idesc_bf16(128, NC);
     // tile j of unit u: spin 0 tiles {0, 1}; spin 2 parity e tiles {0, 3}, parity o tiles {1, 2}
     auto tile = [&](int u, int j) { return PART == 0 ? j : ((u & 1) == 0 ? 3 * j : 1 + j); };
@@ -336,6 +346,7 @@ constexpr int ANA_MAX_STAGES = 4;
 template <int PART>
 __global__ void __launch_bounds__(ANA_THREADS, 1) k_ana_tc(const unsigned char *__restrict__ tab,
                                                           const int64_t *__restrict__ aoff,
+                                                          const int *__restrict__ ks, int npt, int nlt,
                                                           const float2 *__restrict__ rc, float2 *__restrict__ out,
                                                           int lmax, int mmax, int npairs, int64_t nalm, int B,
                                                           int LT, uint32_t ncols, int S, int *err, int withhold) {
@@ -377,13 +388,17 @@ __global__ void __launch_bounds__(ANA_THREADS, 1) k_ana_tc(const unsigned char *
   fence_after_sync();
   const uint32_t tbase = tslot;
   const int64_t base = abase(lmax, m);
-  const int nsteps = (npairs + 15) / 16;
+  const int all_steps = (npairs + 15) / 16;
+  // first K step (16 ring pairs) visible at the last multipole of the CTA's tiles; one step at least
+  const int llast = par + 2 * (128 * (lt0 + nt) - 1);
+  const int first = min(all_steps - 1, ks[((int64_t)PART * (mmax + 1) + m) * (npt + nlt) + npt + min(nlt - 1, llast / 128)]);
+  const int nsteps = all_steps - first;
   int issued = 0;  // K steps whose A copies the producer issued
   if (warp < nconv * ngroups) {
     const int grp = warp / nconv, task = tid - grp * 32 * nconv;
     const bool has = task < ntask;
     float2 v[16];
-    if (has && grp < nsteps) load_ana_b<PART>(task, rc, m, grp, mmax, npairs, v);
+    if (has && grp < nsteps) load_ana_b<PART>(task, rc, m, first + grp, mmax, npairs, v);
     for (int c = grp; c < nsteps; c += ngroups) {
       const int s = c % S, k = c / S;
       if (c >= S && !mbar_wait(&done[s], (k - 1) & 1, err)) {
@@ -392,7 +407,7 @@ __global__ void __launch_bounds__(ANA_THREADS, 1) k_ana_tc(const unsigned char *
       }
       if (has) {
         convert_ana_b<PART>(task, sm + s * stage + LT * abytes, tileB, par, v);
-        if (c + ngroups < nsteps) load_ana_b<PART>(task, rc, m, c + ngroups, mmax, npairs, v);
+        if (c + ngroups < nsteps) load_ana_b<PART>(task, rc, m, first + c + ngroups, mmax, npairs, v);
       }
       fence_proxy_async();  // generic-proxy writes -> tensor-core reads
       // test hook (dm_test_tc_withhold): the first converter thread of the
@@ -403,8 +418,8 @@ __global__ void __launch_bounds__(ANA_THREADS, 1) k_ana_tc(const unsigned char *
         mbar_arrive(&full_b[s]);
     }
   } else if (warp == 8 && lane == 0) {
-    const unsigned char *tabm = tab + (aoff[2 * m + par] + lt0) * nsteps * (int64_t)abytes;
-    const int64_t tstride = (int64_t)nsteps * abytes;  // next l tile
+    const unsigned char *tabm = tab + ((aoff[2 * m + par] + lt0) * all_steps + first) * (int64_t)abytes;
+    const int64_t tstride = (int64_t)all_steps * abytes;  // next l tile
     for (int c = 0; c < nsteps; ++c) {
       const int s = c % S, k = c / S;
       if (c >= S && !mbar_wait(&done[s], (k - 1) & 1, err)) {
@@ -570,6 +585,7 @@ static cudaError_t tc_tables(dm_plan *p) {
   }
   e = cudaGetLastError();
   if (!e) e = cudaDeviceSynchronize();
+  if (!e && !p->tc_ks) e = visible_steps(p, TC_FLOOR_EXP, &p->tc_ks);
   if (e) return undo(e);
   cudaFree(ptab);
   for (int part = 0; part < 2; ++part) p->bytes += (int64_t)(sbytes[part] + abytes[part]);
@@ -596,7 +612,7 @@ cudaError_t legendre_synthesis_tc(dm_plan *p, const double2 *alm, cudaStream_t s
   if (e) return e;
   const int B = p->batch;
   const double2 *ahi = p->anchor_active ? p->a_hi : nullptr;
-  const int npt = (p->npairs + 127) / 128;
+  const int npt = (p->npairs + 127) / 128, nlt = (p->lmax + 128) / 128;
   dim3 gb(syn_steps(p->lmax, 0), p->mmax + 1);
   const float2 *e32 = p->anchor_active ? p->e32 : nullptr;  // iteration: the FP32 state e
   const bool run0 = p->tune_only_part != 1, run1 = p->tune_only_part != 0;
@@ -611,7 +627,7 @@ cudaError_t legendre_synthesis_tc(dm_plan *p, const double2 *alm, cudaStream_t s
     p->syn_ns_used[0] = ns;
     const size_t sm = tc_smem_n(stage, ns, nc);
     dyn_smem_allow(k_syn_tc<0>, sm);
-    k_syn_tc<0><<<g, 128, sm, st>>>(p->tc_synA[0], p->tc_synB[0], p->tc_soff, p->rc32, p->lmax, p->mmax,
+    k_syn_tc<0><<<g, 128, sm, st>>>(p->tc_synA[0], p->tc_synB[0], p->tc_soff, p->tc_ks, npt + nlt, p->rc32, p->lmax, p->mmax,
                                     p->npairs, B, ns, nc, p->tc_err);
   }
   if (run1) {
@@ -621,7 +637,7 @@ cudaError_t legendre_synthesis_tc(dm_plan *p, const double2 *alm, cudaStream_t s
     p->syn_ns_used[1] = ns;
     const size_t sm = tc_smem_n(stage, ns, nc);
     dyn_smem_allow(k_syn_tc<1>, sm);
-    k_syn_tc<1><<<g, 128, sm, st>>>(p->tc_synA[1], p->tc_synB[1], p->tc_soff, p->rc32, p->lmax, p->mmax,
+    k_syn_tc<1><<<g, 128, sm, st>>>(p->tc_synA[1], p->tc_synB[1], p->tc_soff, p->tc_ks, npt + nlt, p->rc32, p->lmax, p->mmax,
                                     p->npairs, B, ns, nc, p->tc_err);
   }
   return cudaGetLastError();
@@ -659,6 +675,7 @@ cudaError_t legendre_analysis_tc(dm_plan *p, cudaStream_t st) {
   if (e) return e;
   const int B = p->batch;
   const int ltiles = ana_tiles(p->lmax, 0, 0);
+  const int npt = (p->npairs + 127) / 128, nlt = (p->lmax + 128) / 128;
   if (p->tune_only_part != 1) {
     const int NC = 2 * B, LT = ana_lt_pick(p->tune_ana_lt[0], NC);
     const uint32_t nc = pow2_cols(LT * NC);
@@ -669,7 +686,7 @@ cudaError_t legendre_analysis_tc(dm_plan *p, cudaStream_t st) {
     const size_t sm = tc_smem_n(stage, S, nc);
     dim3 g((ltiles + LT - 1) / LT, 2, p->mmax + 1);
     dyn_smem_allow(k_ana_tc<0>, sm);
-    k_ana_tc<0><<<g, ANA_THREADS, sm, st>>>(p->tc_anaA[0], p->tc_aoff, p->rc32, p->apart32, p->lmax, p->mmax,
+    k_ana_tc<0><<<g, ANA_THREADS, sm, st>>>(p->tc_anaA[0], p->tc_aoff, p->tc_ks, npt, nlt, p->rc32, p->apart32, p->lmax, p->mmax,
                                             p->npairs, p->nalm, B, LT, nc, S, p->tc_err, p->tc_withhold);
   }
   if (p->tune_only_part != 0) {
@@ -682,7 +699,7 @@ cudaError_t legendre_analysis_tc(dm_plan *p, cudaStream_t st) {
     const size_t sm = tc_smem_n(stage, S, nc);
     dim3 g((ltiles + LT - 1) / LT, 2, p->mmax + 1);
     dyn_smem_allow(k_ana_tc<1>, sm);
-    k_ana_tc<1><<<g, ANA_THREADS, sm, st>>>(p->tc_anaA[1], p->tc_aoff, p->rc32, p->apart32, p->lmax, p->mmax,
+    k_ana_tc<1><<<g, ANA_THREADS, sm, st>>>(p->tc_anaA[1], p->tc_aoff, p->tc_ks, npt, nlt, p->rc32, p->apart32, p->lmax, p->mmax,
                                             p->npairs, p->nalm, B, LT, nc, S, p->tc_err, 0);
   }
   return cudaGetLastError();

@@ -119,13 +119,14 @@ __device__ __forceinline__ int64_t sp_alm_base(int lmax, int m) { return (int64_
 // thread per ring pair and order.  The running maximum of a row grows through
 // buckets of 16 exponents; the multipole at which it entered each is kept, so
 // that one pass of the recurrence finds the first value within 2^-55 of the
-// final maximum (to a bucket, never late).
+// final maximum and above 2^floor_exp (to a bucket, never late).
 constexpr int SC_BUCKETS = 40;  // exponents -600 .. 39
 __global__ void __launch_bounds__(64) k_split_scale(const PairDev *__restrict__ pairs,
                                                     const RecCoef *__restrict__ rec,
                                                     const double *__restrict__ seed,
                                                     const int *__restrict__ seed_exp, int16_t *__restrict__ esc,
-                                                    uint16_t *__restrict__ lfirst, int lmax, int mmax, int npairs) {
+                                                    uint16_t *__restrict__ lfirst, int lmax, int mmax, int npairs,
+                                                    int floor_exp) {
   __shared__ uint16_t enter[2][SC_BUCKETS][64];
   __shared__ RecCoef sc[64];
   const int m = blockIdx.y, t = threadIdx.x, p = min((int)blockIdx.x * 64 + t, npairs - 1);
@@ -157,8 +158,8 @@ __global__ void __launch_bounds__(64) k_split_scale(const PairDev *__restrict__ 
   for (int f = 0; f < 2; ++f) {
     const int64_t o = ((int64_t)f * (mmax + 1) + m) * npairs + p;
     esc[o] = (int16_t)max(e[f], SPLIT_MIN_EXP);
-    const int bk = max(0, (e[f] - 55 - SPLIT_MIN_EXP) >> 4);
-    lfirst[o] = (uint16_t)(top[f] < 0 ? lmax - m + 1 : enter[f][min(bk, top[f])][t]);
+    const int thr = max(e[f] - 55, floor_exp), bk = max(0, (thr - SPLIT_MIN_EXP) >> 4);
+    lfirst[o] = (uint16_t)(top[f] < 0 || e[f] < thr ? lmax - m + 1 : enter[f][min(bk, top[f])][t]);
   }
 }
 
@@ -751,6 +752,33 @@ void split_forget(dm_plan *p) {
   drop_cuts(T);
 }
 
+// First K steps (units of 16 multipoles or ring pairs) of every tile of 128
+// ring pairs and of 128 multipoles whose values reach 2^floor_exp, as k_split_ks
+// lays them out, in a new device array.
+cudaError_t visible_steps(dm_plan *p, int floor_exp, int **out) {
+  const int nm = p->mmax + 1, npt = (p->npairs + 127) / 128, nlt = (p->lmax + 128) / 128;
+  const size_t n = 2 * (size_t)nm * p->npairs;
+  int16_t *esc = nullptr;
+  int *ks = nullptr;
+  cudaError_t e = cudaMalloc(&esc, sizeof(int16_t) * 2 * n);
+  if (!e) e = cudaMalloc(&ks, sizeof(int) * 2 * nm * (size_t)(npt + nlt));
+  if (!e) {
+    uint16_t *lf = reinterpret_cast<uint16_t *>(esc + n);
+    k_split_scale<<<dim3((p->npairs + 63) / 64, nm), 64>>>(p->pairs, p->rec, p->seed, p->seed_exp, esc, lf, p->lmax,
+                                                           p->mmax, p->npairs, floor_exp);
+    k_split_ks<<<dim3(nm, 2), 32>>>(lf, ks, p->mmax, p->npairs, npt, nlt);
+    e = cudaGetLastError();
+  }
+  if (!e) e = cudaDeviceSynchronize();
+  cudaFree(esc);
+  if (e) {
+    cudaFree(ks);
+    return e;
+  }
+  *out = ks;
+  return cudaSuccess;
+}
+
 // Row exponents, first visible multipoles, slabs and tensor maps: once per
 // plan.  The whole table is kept when it takes at most p->split_cap bytes,
 // else slabs of p->ffs_cap bytes are generated before their products.
@@ -781,7 +809,7 @@ static cudaError_t split_setup(dm_plan *p, cudaStream_t st) {
     if (!e) {
       k_split_scale<<<dim3((npairs + 63) / 64, nm), 64, 0, st>>>(p->pairs, p->rec, p->seed, p->seed_exp,
                                                                  reinterpret_cast<int16_t *>(esc), lf, lmax, p->mmax,
-                                                                 npairs);
+                                                                 npairs, -100000);
       k_split_ks<<<dim3(nm, 2), 32, 0, st>>>(lf, ks, p->mmax, npairs, npt, nlt);
       e = cudaGetLastError();
     }
