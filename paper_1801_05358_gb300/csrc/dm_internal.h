@@ -158,6 +158,10 @@ struct dm_plan {
   int64_t bytes = 0;
   // DM_MIXED_FP32 resources (allocated by dm_set_precision)
   bool fp32_ready = false;      // the buffers of the FP32 modes exist (setup_fp32 succeeded)
+  // FP32 Legendre tables of the mixed mode's small plans and batches (dm_legendre32.cu)
+  float *tab32 = nullptr;       // [3][nalm][npairs up to a multiple of 4] lambda, lam+, lam-
+  bool tab32_failed = false;    // they did not fit: the split products run
+  bool is_view = false;         // a one-RHS view of a serving pool (makes no tables of its own)
   // digit tables of the split products (dm_split.cu): shared with the views of the plan
   dmwf::SplitTables *split = nullptr;
   // ring DFT matrices of the FP64-class modes (dm_dft.cu), shared likewise
@@ -307,7 +311,11 @@ cudaError_t cov_ring_stage(dm_plan *p, cudaStream_t st);
 cudaError_t cov_ring_stage32(dm_plan *p, cudaStream_t st);      // the mixed mode's (FP32 state)
 cudaError_t anchor_residual_wd_cov(dm_plan *p, const double *s_hi, cudaStream_t st);
 cudaError_t setup_fp32(dm_plan *p);
-cudaError_t gen_tables32(dm_plan *p, float *tab, cudaStream_t st);  // FP32 Legendre tables (dm_legendre.cu)
+bool syn32_ready(dm_plan *p, cudaStream_t st);
+bool ana32_ready(dm_plan *p, cudaStream_t st);
+cudaError_t syn32(dm_plan *p, const double2 *alm, const float2 *e32, cudaStream_t st);
+cudaError_t ana32(dm_plan *p, cudaStream_t st);
+cudaError_t gen_tables32(dm_plan *p, float *tab, int ld, cudaStream_t st);  // FP32 Legendre tables (dm_legendre.cu)
 // Raise a kernel's dynamic shared-memory limit on the current device to at
 // least `bytes`, never lowering it.  The limit is a process-wide attribute of
 // the function: set per launch, a smaller value set by a plan on another host
@@ -327,10 +335,12 @@ void dft_disable(dm_plan *p);
 int64_t dft_bytes(const dm_plan *p);
 size_t dft_table_bytes(int nside, int mmax);
 size_t dft_scratch_bytes(int nside, int batch);
+cudaError_t dft_flat_columns(dm_plan *p, const double2 *alm, const SolveState *state, cudaStream_t st, bool *ran);
 cudaError_t dft_ring_stage(dm_plan *p, int mode, const double *in_map, double *out_map, cudaStream_t st, bool *ran);
 // split products of the Legendre stages (dm_split.cu)
 void split_new(dm_plan *p);
 cudaError_t visible_steps(dm_plan *p, int floor_exp, int **out);
+cudaError_t first_steps(const uint16_t *lfirst, int *ks, int mmax, int npairs, int npt, int nlt);
 void split_release(dm_plan *p);
 void split_forget(dm_plan *p);
 int64_t split_bytes(const dm_plan *p);

@@ -332,11 +332,13 @@ cudaError_t apply_filter_level(dm_plan *p, const double *coef, const double2 *in
 // DM_MIXED_FP32: FP32 ring coefficients and harmonic state between anchors.
 // ======================================================================
 
-// FP32 tables [3][nalm][npairs] of lambda, lam+, lam- from the FP64
-// recurrence, from which the stored BF16 tiles are cut.
+// FP32 tables [3][nalm][ld] (ld >= npairs) of lambda, lam+, lam- from the FP64
+// recurrence: k_syn32 and k_ana32 read them, the stored BF16 tiles are cut
+// from them.
 __global__ void __launch_bounds__(128) k_gen_tables(const PairDev *__restrict__ pairs, const RecCoef *__restrict__ rec,
                                                     const double *__restrict__ seed, const int *__restrict__ seed_exp,
-                                                    float *__restrict__ ptab, int lmax, int npairs, int64_t plane) {
+                                                    float *__restrict__ ptab, int lmax, int npairs, int ld,
+                                                    int64_t plane) {
   __shared__ RecCoef sc[SYN_CH];
   const int m = blockIdx.y;
   const int p = blockIdx.x * 128 + threadIdx.x;
@@ -354,7 +356,7 @@ __global__ void __launch_bounds__(128) k_gen_tables(const PairDev *__restrict__ 
     for (int j = 0; j < cnt; ++j) {
       const int l = lc + j;
       if (act) {
-        const int64_t o = (base + l) * (int64_t)npairs + p;
+        const int64_t o = (base + l) * (int64_t)ld + p;
         const bool live = (s.S == 0);
         ptab[o] = live ? (float)s.l0 : 0.f;
         ptab[plane + o] = live ? (float)(0.5 * (s.p0 + s.q0)) : 0.f;
@@ -365,14 +367,15 @@ __global__ void __launch_bounds__(128) k_gen_tables(const PairDev *__restrict__ 
   }
 }
 
-cudaError_t gen_tables32(dm_plan *p, float *tab, cudaStream_t st) {
+cudaError_t gen_tables32(dm_plan *p, float *tab, int ld, cudaStream_t st) {
   dim3 g((p->npairs + 127) / 128, p->mmax + 1);
-  k_gen_tables<<<g, 128, 0, st>>>(p->pairs, p->rec, p->seed, p->seed_exp, tab, p->lmax, p->npairs,
-                                  p->nalm * (int64_t)p->npairs);
+  k_gen_tables<<<g, 128, 0, st>>>(p->pairs, p->rec, p->seed, p->seed_exp, tab, p->lmax, p->npairs, ld,
+                                  p->nalm * (int64_t)ld);
   return cudaGetLastError();
 }
 
-__global__ void k_ana_reduce32(const float2 *__restrict__ apart, double2 *out, int lmax, int64_t nalm, double omega, int epilogue, const double *__restrict__ filt, int nlev,
+__global__ void k_ana_reduce32(const float2 *__restrict__ apart, double2 *out, int lmax, int64_t nalm,
+                               double omega, int epilogue, const double *__restrict__ filt, int nlev,
                                const SolveState *__restrict__ state, const double2 *__restrict__ g_add) {
   const int b = blockIdx.y, m = blockIdx.z;
   if (state != nullptr && state[b].done) return;
@@ -408,6 +411,7 @@ __global__ void k_ana_reduce32(const float2 *__restrict__ apart, double2 *out, i
 
 cudaError_t legendre_synthesis32(dm_plan *p, const double2 *alm, cudaStream_t st) {
   if (p->use_tc && tc_batch_ok(p->batch)) return legendre_synthesis_tc(p, alm, st);
+  if (syn32_ready(p, st)) return syn32(p, alm, p->anchor_active ? p->e32 : nullptr, st);
   return split_synthesis32(p, alm, p->anchor_active ? p->e32 : nullptr, st);
 }
 
@@ -520,7 +524,9 @@ cudaError_t materialize_a(dm_plan *p, cudaStream_t st) {
 
 cudaError_t legendre_analysis32(dm_plan *p, int epilogue, double2 *out, cudaStream_t st, cudaEvent_t mid) {
   const SolveState *stp = p->state_active ? p->state : nullptr;
-  if (cudaError_t e = (p->use_tc && tc_batch_ok(p->batch)) ? legendre_analysis_tc(p, st) : split_analysis32(p, st))
+  if (cudaError_t e = (p->use_tc && tc_batch_ok(p->batch)) ? legendre_analysis_tc(p, st)
+                      : ana32_ready(p, st)                     ? ana32(p, st)
+                                                               : split_analysis32(p, st))
     return e;
   if (mid) cudaEventRecord(mid, st);
   double omega = 4.0 * M_PI / (double)p->npix;

@@ -36,12 +36,6 @@ namespace {
 
 constexpr int TC_THREADS = 256;
 
-// K steps before the first Legendre value of a tile that reaches 2^-60 are
-// left out: the evanescent region (m well above l sin theta), where a value
-// this small changes no bit of an FP32 sum with those of the other rings.  It
-// holds 10 % of the K steps at nside 256 / lmax 512, 20 % at nside 512 / 1024.
-constexpr int TC_FLOOR_EXP = -60;
-
 __device__ __forceinline__ float2 e_of(const double2 *a, const double2 *ahi, int64_t i) {
   double2 v = a[i];
   if (ahi != nullptr) {
@@ -574,7 +568,7 @@ static cudaError_t tc_tables(dm_plan *p) {
     if ((e = cudaMalloc(&p->tc_anaA[part], abytes[part]))) return undo(e);
   }
   if ((e = cudaMalloc(&ptab, sizeof(float) * 3 * (size_t)p->nalm * p->npairs))) return undo(e);
-  if ((e = gen_tables32(p, ptab, 0))) return undo(e);
+  if ((e = gen_tables32(p, ptab, p->npairs, 0))) return undo(e);
   dim3 gs(syn_steps(p->lmax, 0), npt, p->mmax + 1);
   k_tab_syn<0><<<gs, 256>>>(ptab, p->tc_synA[0], p->tc_soff, p->lmax, p->npairs, p->nalm, npt);
   k_tab_syn<1><<<gs, 256>>>(ptab, p->tc_synA[1], p->tc_soff, p->lmax, p->npairs, p->nalm, npt);

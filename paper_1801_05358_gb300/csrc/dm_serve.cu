@@ -99,6 +99,7 @@ uint64_t hash_bytes(const void *p, size_t n) {  // FNV-1a
 dm_plan make_view(const dm_plan *p, int b) {
   dm_plan v = *p;
   v.batch = 1;
+  v.is_view = true;
   v.prof_on = false;
   v.ev.clear();
   const size_t n3 = 3 * (size_t)p->npix, na = 3 * (size_t)p->nalm;

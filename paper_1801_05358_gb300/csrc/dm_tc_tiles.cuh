@@ -14,6 +14,12 @@ using namespace tc;
 
 constexpr int TILE_A = 4096;  // 128 x 16 BF16
 
+// K steps before the first Legendre value of a tile that reaches 2^-60 are
+// left out: the evanescent region (m well above l sin theta), where a value
+// this small changes no bit of an FP32 sum with those of the other rings.  It
+// holds 10 % of the K steps at nside 256 / lmax 512, 20 % at nside 512 / 1024.
+constexpr int TC_FLOOR_EXP = -60;
+
 __device__ __forceinline__ int64_t abase(int lmax, int m) { return (int64_t)m * (2 * lmax + 1 - m) / 2; }
 
 // byte offset of the 16-byte core-matrix row (row, k-octet ko) of a [rows x 16] K-major tile
