@@ -108,7 +108,8 @@ __device__ __forceinline__ Xs xs_of(const PairDev *pairs, int p) {
 __global__ void __launch_bounds__(128) k_ckpt(const PairDev *__restrict__ pairs, const RecCoef *__restrict__ rec,
                                               const double *__restrict__ seed, const int *__restrict__ seed_exp,
                                               const int64_t *__restrict__ cko, float4 *__restrict__ ck0,
-                                              float4 *__restrict__ ck2, int lmax, int npairs) {
+                                              float4 *__restrict__ ck2, uint16_t *__restrict__ lfirst, int lmax,
+                                              int npairs) {
   const int m = blockIdx.y, p = blockIdx.x * blockDim.x + threadIdx.x;
   if (p >= npairs) return;
   const double x = pairs[p].x;
@@ -116,7 +117,14 @@ __global__ void __launch_bounds__(128) k_ckpt(const PairDev *__restrict__ pairs,
   Rec s;
   rec_init(s, seed, seed_exp, m, p, npairs);
   const int64_t base = abase(lmax, m);
+  // first l - m with a value of 2^TC_FLOOR_EXP or more (spin 0; spin 2)
+  int f0 = lmax - m + 1, f2 = f0;
+  const double vis = ldexp(1.0, TC_FLOOR_EXP);
   for (int l = m; l <= lmax; ++l) {
+    if (s.S == 0 && (f0 > lmax - m || f2 > lmax - m)) {
+      if (f0 > lmax - m && fabs(s.l0) >= vis) f0 = l - m;
+      if (f2 > lmax - m && (fabs(s.p0) >= vis || fabs(s.q0) >= vis)) f2 = l - m;
+    }
     const int j = (l - m) / CKL;
     const int64_t o = (cko[m] + j) * (int64_t)npairs + p;
     if (l == m + CKL * j) {
@@ -137,6 +145,8 @@ __global__ void __launch_bounds__(128) k_ckpt(const PairDev *__restrict__ pairs,
     }
     if (l < lmax) rec_advance(s, rec[base + l + 1], x, m, l, seed, p, npairs);
   }
+  lfirst[(int64_t)m * npairs + p] = (uint16_t)f0;
+  lfirst[((int64_t)gridDim.y + m) * npairs + p] = (uint16_t)f2;
 }
 
 // FP32 coefficients of target l: (al, bl, al - 1 - bl), (a, ac, b) and
@@ -410,8 +420,8 @@ __global__ void __launch_bounds__(AGEN_THREADS, 1) k_ana_gen(
     const float4 *__restrict__ ck0, const float4 *__restrict__ ck2, const int64_t *__restrict__ cko,
     const float4 *__restrict__ rq0, const float4 *__restrict__ rq2, const float2 *__restrict__ rq2d,
     const PairDev *__restrict__ pairs,
-    const float2 *__restrict__ rc, float2 *__restrict__ out, int lmax, int mmax, int npairs, int64_t nalm, int B,
-    int LT, uint32_t ncols, int S, int *err, int withhold) {
+    const int *__restrict__ ks, int npt, int nlt, const float2 *__restrict__ rc, float2 *__restrict__ out, int lmax,
+    int mmax, int npairs, int64_t nalm, int B, int LT, uint32_t ncols, int S, int *err, int withhold) {
   extern __shared__ __align__(1024) unsigned char sm[];
   __shared__ uint64_t bars[2 * AGEN_MAX_S + 1];
   __shared__ uint32_t tslot;
@@ -462,7 +472,11 @@ __global__ void __launch_bounds__(AGEN_THREADS, 1) k_ana_gen(
   fence_after_sync();
   const uint32_t tbase = tslot;
   const int64_t base = abase(lmax, m);
-  const int nsteps = (npairs + 15) / 16;
+  // K steps (16 ring pairs) from the first one visible at the last multipole of the CTA's tiles; one at least
+  const int all_steps = (npairs + 15) / 16, llast = par + 2 * (128 * (lt0 + nt) - 1);
+  const int first =
+      min(all_steps - 1, ks[((int64_t)PART * (mmax + 1) + m) * (npt + nlt) + npt + min(nlt - 1, llast / 128)]);
+  const int nsteps = all_steps - first;
   const int nblk = (lmax - m + 1 + CKL - 1) / CKL;
   if (warp < S) {
     // This CTA's checkpoint blocks: J = 4 lt0 + bi for bi < nvalid.  A lane
@@ -488,7 +502,7 @@ __global__ void __launch_bounds__(AGEN_THREADS, 1) k_ana_gen(
       if (PART == 0) {
         for (int task = lane; task < 2 * B; task += 32) {
           float2 v[16];
-          load_ana_b<0>(task, rc, m, c, mmax, npairs, v);
+          load_ana_b<0>(task, rc, m, first + c, mmax, npairs, v);
           convert_ana_b<0>(task, Bst, tileB, par, v);
         }
       } else {
@@ -497,17 +511,17 @@ __global__ void __launch_bounds__(AGEN_THREADS, 1) k_ana_gen(
           float2 vq[16], vu[16];
           const int64_t fq = (((int64_t)b * 3 + 1) * (mmax + 1) + m) * npairs * 2;
           const int64_t fu = (((int64_t)b * 3 + 2) * (mmax + 1) + m) * npairs * 2;
-          load_pairs8(rc + fq, 16 * c + 8 * ko, npairs, vq);
-          load_pairs8(rc + fu, 16 * c + 8 * ko, npairs, vu);
+          load_pairs8(rc + fq, 16 * (first + c) + 8 * ko, npairs, vq);
+          load_pairs8(rc + fu, 16 * (first + c) + 8 * ko, npairs, vu);
           convert_b_pq(b, ko, Bst, Bst + 2 * tileB, tileB, par, vq, vu);
         }
       }
       // A tile rows of block J, pairs 16 c + 8 g + PPL sl ..
       if (gen) {
         unsigned char *At = Ast + (j * nA + f) * ATS;
-        const int p0 = 16 * c + 8 * g + PPL * sl;
+        const int p0 = 16 * (first + c) + 8 * g + PPL * sl;
         const int64_t orow = (cko[m] + J) * (int64_t)npairs;
-        const bool df = pair_dform(pairs, min(16 * c + 8 * g, npairs - 1));
+        const bool df = pair_dform(pairs, min(16 * (first + c) + 8 * g, npairs - 1));
         const int l0 = m + CKL * J;
         if (df) {
           if (par == 0)
@@ -666,8 +680,8 @@ __global__ void __launch_bounds__(160, 1) k_syn_gen(
     const float4 *__restrict__ ck0, const float4 *__restrict__ ck2, const int64_t *__restrict__ cko,
     const float4 *__restrict__ rq0, const float4 *__restrict__ rq2, const float2 *__restrict__ rq2d,
     const PairDev *__restrict__ pairs,
-    const unsigned char *__restrict__ bt, const int64_t *__restrict__ soff, float2 *__restrict__ rc, int lmax,
-    int mmax, int npairs, int B, int NS, uint32_t ncols, int *err) {
+    const unsigned char *__restrict__ bt, const int64_t *__restrict__ soff, const int *__restrict__ ks, int ks_stride,
+    float2 *__restrict__ rc, int lmax, int mmax, int npairs, int B, int NS, uint32_t ncols, int *err) {
   extern __shared__ __align__(1024) unsigned char sm[];
   __shared__ uint64_t mbar[3 * SGEN_MAX_NS];
   __shared__ uint32_t tslot;
@@ -695,7 +709,10 @@ __global__ void __launch_bounds__(160, 1) k_syn_gen(
   __syncthreads();
   fence_after_sync();
   const uint32_t tbase = tslot;
-  const int nsteps = syn_steps(lmax, m);
+  // K steps (32 multipoles) from the checkpoint block of the first visible value; one block at least
+  const int all_steps = syn_steps(lmax, m);
+  const int first = min((all_steps - 1) & ~1, (ks[((int64_t)PART * (mmax + 1) + m) * ks_stride + pt] >> 1) & ~1);
+  const int nsteps = all_steps - first;
   const int nunits = nsteps * UPS;
   if (warp < 4) {
     const int r = tid, pair = p0 + r;
@@ -704,7 +721,7 @@ __global__ void __launch_bounds__(160, 1) k_syn_gen(
     const Xs xs = xs_of(pairs, pp);
     const bool df = pair_dform(pairs, pp);
     const int64_t base = abase(lmax, m);
-    const int64_t ckb = cko[m] * (int64_t)npairs + pp;
+    const int64_t ckb = (cko[m] + (first >> 1)) * (int64_t)npairs + pp;
     const int ls = (PART == 1 && m < 2) ? 2 : 0;  // spin 2 starts at l = 2
     float a0 = 0.f, a1 = 0.f, b0 = 0.f, b1 = 0.f, sc = 1.f;
     int S = 0;
@@ -712,7 +729,7 @@ __global__ void __launch_bounds__(160, 1) k_syn_gen(
     // current K step c (cA, cD) and the next one (nA, nD), loaded a step ahead;
     // the checkpoint of the next block is loaded a block ahead (k0, k2)
     auto coef = [&](int c, float4 &ca, float2 &cd) {
-      const int l1 = m + 32 * c + lane + 1;
+      const int l1 = m + 32 * (first + c) + lane + 1;
       ca = make_float4(0.f, 0.f, 0.f, 0.f);
       cd = make_float2(0.f, 0.f);
       if (l1 <= lmax) {
@@ -752,14 +769,14 @@ __global__ void __launch_bounds__(160, 1) k_syn_gen(
       }
       unsigned char *Ae = sm + ((c * UPS) % NS) * stage;
       unsigned char *Ao = PART == 0 ? Ae : sm + ((c * UPS + 1) % NS) * stage;
-      syn_step<PART>(Ae, Ao, r, m + 32 * c, lmax, ls, act, a0, a1, b0, b1, S, sc, xs, df, cA, cD);
+      syn_step<PART>(Ae, Ao, r, m + 32 * (first + c), lmax, ls, act, a0, a1, b0, b1, S, sc, xs, df, cA, cD);
       cA = nA;
       cD = nD;
       fence_proxy_async();
       for (int h = 0; h < UPS; ++h) mbar_arrive(&full_a[(c * UPS + h) % NS]);
     }
   } else if (warp == 4 && lane == 0) {
-    const unsigned char *btm = bt + soff[m] * (int64_t)bbytes;
+    const unsigned char *btm = bt + (soff[m] + first) * (int64_t)bbytes;
     const uint32_t idesc = idesc_bf16(128, NC);
     auto tile = [&](int u, int j) { return PART == 0 ? j : ((u & 1) == 0 ? 3 * j : 1 + j); };
     auto issue = [&](int u) {
@@ -859,6 +876,9 @@ cudaError_t gen_setup(dm_plan *p) {
   std::vector<int64_t> cko(p->mmax + 2, 0);
   for (int m = 0; m <= p->mmax; ++m) cko[m + 1] = cko[m] + (p->lmax - m + 1 + CKL - 1) / CKL;
   const size_t nrec = (size_t)cko[p->mmax + 1] * p->npairs;
+  const int nm = p->mmax + 1, npt = (p->npairs + 127) / 128, nlt = (p->lmax + 128) / 128;
+  uint16_t *lf = nullptr;
+  int *ks = nullptr;
   float4 *ck0 = nullptr, *ck2 = nullptr, *rq0 = nullptr, *rq2 = nullptr;
   float2 *rq2d = nullptr;
   int64_t *ckod = nullptr;
@@ -869,6 +889,8 @@ cudaError_t gen_setup(dm_plan *p) {
     cudaFree(rq2);
     cudaFree(rq2d);
     cudaFree(ckod);
+    cudaFree(lf);
+    cudaFree(ks);
     return e;
   };
   cudaError_t e;
@@ -878,13 +900,18 @@ cudaError_t gen_setup(dm_plan *p) {
   if ((e = cudaMalloc(&rq2, sizeof(float4) * (size_t)p->nalm))) return fail(e);
   if ((e = cudaMalloc(&rq2d, sizeof(float2) * (size_t)p->nalm))) return fail(e);
   if ((e = cudaMalloc(&ckod, sizeof(int64_t) * cko.size()))) return fail(e);
+  if ((e = cudaMalloc(&lf, sizeof(uint16_t) * 2 * nm * (size_t)p->npairs))) return fail(e);
+  if ((e = cudaMalloc(&ks, sizeof(int) * 2 * nm * (size_t)(npt + nlt)))) return fail(e);
   cudaMemset(ck0, 0, sizeof(float4) * nrec);
   cudaMemset(ck2, 0, sizeof(float4) * nrec);
   cudaMemcpy(ckod, cko.data(), sizeof(int64_t) * cko.size(), cudaMemcpyHostToDevice);
   k_rec32<<<512, 256>>>(p->rec, rq0, rq2, rq2d, p->nalm);
   k_ckpt<<<dim3((p->npairs + 127) / 128, p->mmax + 1), 128>>>(p->pairs, p->rec, p->seed, p->seed_exp, ckod, ck0,
-                                                              ck2, p->lmax, p->npairs);
-  if ((e = cudaGetLastError()) || (e = cudaDeviceSynchronize())) return fail(e);
+                                                              ck2, lf, p->lmax, p->npairs);
+  if ((e = first_steps(lf, ks, p->mmax, p->npairs, npt, nlt)) || (e = cudaDeviceSynchronize())) return fail(e);
+  cudaFree(lf);
+  cudaFree(p->tc_ks);
+  p->tc_ks = ks;
   p->ck0 = ck0;
   p->ck2 = ck2;
   p->rq0 = rq0;
@@ -931,7 +958,7 @@ static int sgen_stages(int want, int stage_bytes, uint32_t ncols) {
 cudaError_t syn_gen_launch(dm_plan *p, bool run0, bool run1, cudaStream_t st) {
   cudaError_t e = gen_setup(p);
   if (e) return e;
-  const int B = p->batch, npt = (p->npairs + 127) / 128;
+  const int B = p->batch, npt = (p->npairs + 127) / 128, ks_stride = npt + (p->lmax + 128) / 128;
   dim3 g(npt, p->mmax + 1);
   if (run0) {
     const int stage = 2 * 2 * TILE_A + 2 * 2 * (2 * B * 32);
@@ -941,7 +968,7 @@ cudaError_t syn_gen_launch(dm_plan *p, bool run0, bool run1, cudaStream_t st) {
     const size_t sm = tc_smem_n(stage, ns, nc);
     dyn_smem_allow(k_syn_gen<0>, sm);
     k_syn_gen<0><<<g, 160, sm, st>>>(p->ck0, p->ck2, p->cko, p->rq0, p->rq2, p->rq2d, p->pairs, p->tc_synB[0], p->tc_soff,
-                                     p->rc32, p->lmax, p->mmax, p->npairs, B, ns, nc, p->tc_err);
+                                     p->tc_ks, ks_stride, p->rc32, p->lmax, p->mmax, p->npairs, B, ns, nc, p->tc_err);
   }
   if (run1) {
     const int stage = 2 * 2 * TILE_A + 2 * 2 * (4 * B * 32);
@@ -951,7 +978,7 @@ cudaError_t syn_gen_launch(dm_plan *p, bool run0, bool run1, cudaStream_t st) {
     const size_t sm = tc_smem_n(stage, ns, nc);
     dyn_smem_allow(k_syn_gen<1>, sm);
     k_syn_gen<1><<<g, 160, sm, st>>>(p->ck0, p->ck2, p->cko, p->rq0, p->rq2, p->rq2d, p->pairs, p->tc_synB[1], p->tc_soff,
-                                     p->rc32, p->lmax, p->mmax, p->npairs, B, ns, nc, p->tc_err);
+                                     p->tc_ks, ks_stride, p->rc32, p->lmax, p->mmax, p->npairs, B, ns, nc, p->tc_err);
   }
   return cudaGetLastError();
 }
@@ -969,11 +996,14 @@ cudaError_t ana_gen_launch(dm_plan *p, cudaStream_t st) {
   if (e) return e;
   const int B = p->batch;
   const int ltiles = ana_tiles(p->lmax, 0, 0);
+  const int npt = (p->npairs + 127) / 128, nlt = (p->lmax + 128) / 128;
   for (int part = 0; part < 2; ++part) {
     if (p->tune_only_part == 1 - part) continue;
     const int NC = part == 0 ? 2 * B : 4 * B;
     const int ltmax = std::max(1, std::min(part == 0 ? 4 : 2, 512 / (int)pow2_cols(NC)));
-    const int LT = p->tune_ana_lt[part] > 0 ? std::min(p->tune_ana_lt[part], ltmax) : ltmax;
+    // two l tiles unless tuned: a wider block sees more of the ring pairs at its last multipole and leaves out
+    // fewer (nside 1024, 8 right-hand sides: 51.4 ms with four and two, 46.6 with two, 53 with one)
+    const int LT = p->tune_ana_lt[part] > 0 ? std::min(p->tune_ana_lt[part], ltmax) : std::min(2, ltmax);
     const int stage = agen_stage_bytes(part, LT, B);
     const int coef_bytes = ((coef_slots(LT) * (part == 0 ? 16 : 24)) + 1023) & ~1023;
     const int fit = (int)(((227u << 10) - 1024u - (unsigned)coef_bytes) / (unsigned)stage);
@@ -987,13 +1017,13 @@ cudaError_t ana_gen_launch(dm_plan *p, cudaStream_t st) {
     dim3 g((ltiles + LT - 1) / LT, 2, p->mmax + 1);
     if (part == 0) {
       dyn_smem_allow(k_ana_gen<0>, sm);
-      k_ana_gen<0><<<g, AGEN_THREADS, sm, st>>>(p->ck0, p->ck2, p->cko, p->rq0, p->rq2, p->rq2d, p->pairs, p->rc32,
-                                                p->apart32, p->lmax, p->mmax, p->npairs, p->nalm, B, LT, nc, S,
+      k_ana_gen<0><<<g, AGEN_THREADS, sm, st>>>(p->ck0, p->ck2, p->cko, p->rq0, p->rq2, p->rq2d, p->pairs, p->tc_ks,
+                                                npt, nlt, p->rc32, p->apart32, p->lmax, p->mmax, p->npairs, p->nalm, B, LT, nc, S,
                                                 p->tc_err, p->tc_withhold);
     } else {
       dyn_smem_allow(k_ana_gen<1>, sm);
-      k_ana_gen<1><<<g, AGEN_THREADS, sm, st>>>(p->ck0, p->ck2, p->cko, p->rq0, p->rq2, p->rq2d, p->pairs, p->rc32,
-                                                p->apart32, p->lmax, p->mmax, p->npairs, p->nalm, B, LT, nc, S,
+      k_ana_gen<1><<<g, AGEN_THREADS, sm, st>>>(p->ck0, p->ck2, p->cko, p->rq0, p->rq2, p->rq2d, p->pairs, p->tc_ks,
+                                                npt, nlt, p->rc32, p->apart32, p->lmax, p->mmax, p->npairs, p->nalm, B, LT, nc, S,
                                                 p->tc_err, 0);
     }
   }

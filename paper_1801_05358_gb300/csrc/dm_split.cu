@@ -752,6 +752,11 @@ void split_forget(dm_plan *p) {
   drop_cuts(T);
 }
 
+cudaError_t first_steps(const uint16_t *lfirst, int *ks, int mmax, int npairs, int npt, int nlt) {
+  k_split_ks<<<dim3(mmax + 1, 2), 32>>>(lfirst, ks, mmax, npairs, npt, nlt);
+  return cudaGetLastError();
+}
+
 // First K steps (units of 16 multipoles or ring pairs) of every tile of 128
 // ring pairs and of 128 multipoles whose values reach 2^floor_exp, as k_split_ks
 // lays them out, in a new device array.
