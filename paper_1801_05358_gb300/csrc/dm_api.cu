@@ -470,10 +470,8 @@ dm_status plan_workspace(dm_plan *p, dm_plan **out) {
   if ((e = dalloc(p, &p->rhi, (size_t)B * n3))) return bad(e, "alloc rhi");
   if ((e = dalloc(p, &p->tc_err, 1))) return bad(e, "alloc");
   cudaMemset(p->tc_err, 0, sizeof(int));
-  if (!p->flat) {
-    split_new(p);
-    dft_new(p);
-  }
+  if (!p->flat) split_new(p);
+  dft_new(p);
   if ((e = cudaEventCreate(&p->ev_begin)) || (e = cudaEventCreate(&p->ev_end))) return bad(e, "events");
   cudaMemset(p->rc, 0, sizeof(double2) * (size_t)B * 3 * (p->mmax + 1) * p->npairs * 2);
   cudaMemset(p->mask, 1, (size_t)B * p->npix);

@@ -27,6 +27,7 @@
 #include <algorithm>
 #include <vector>
 
+#include "dm_fft.cuh"
 #include "dm_internal.h"
 #include "dm_split.cuh"
 
@@ -36,6 +37,14 @@ constexpr int DFT_CHUNK = 8;       // K steps of 16 per drain
 constexpr int DFT_DRAIN_WARPS = 8;
 constexpr int DFT_THREADS = 32 * (DFT_DRAIN_WARPS + 2);
 constexpr int DFT_MAX_STAGES = 8;
+constexpr size_t DFT_SMEM = 224u << 10;  // dynamic shared memory that a block may have here
+// Below this many pixels of a plan (all right-hand sides) the FFT kernels are
+// faster: a stage here is five dependent launches of few tiles, there one to
+// three.  64 iterations of a solve, products against FFTs: nside 16, B 1 22.1
+// and 11.5 ms; nside 64, B 1 23.8 and 19.7; nside 64, B 2 (the line) 26.7 and
+// 30.0; nside 32, B 8 (the line) 28.9 and 29.8; nside 128, B 2 58 and 101;
+// flat N = 256, B 1 15.6 and 13.3, B 2 20.9 and 24.1; N = 1024, B 4 387 and 510.
+constexpr int64_t DFT_MIN_PIXELS = 12 * 64 * 64 * 2;
 constexpr size_t DFT_SCRATCH = (size_t)1 << 30;  // column digits of one direction and group of right-hand sides
 
 // A matrix set: the rings of one length and shift.
@@ -146,24 +155,58 @@ __device__ __forceinline__ void col_place(const DftCol &c, int col, int &ct, int
   cit = col - ct * c.w;
 }
 
+// Slot of the i-th value of a row of staged values: one slot of padding every
+// 4, so that threads on neighbouring groups of 4 read different banks.
+__device__ __forceinline__ int slot4(int i) { return i + (i >> 2); }
+__host__ __device__ constexpr int slots4(int n) { return n + n / 4 + 1; }
+
+// Digits of four staged values per item, the items ordered so that the 16-byte
+// rows of the two sides (neighbouring columns) leave as one 32-byte sector.
+// row(side, fun) -> staged values; col/place of side 0 in ct, cit.
+template <typename Row>
+__device__ __forceinline__ void digit_items(unsigned char *x, const DftCol &C, int ks, int ct, int cit, int count,
+                                            const int e[2], int nsides, Row row) {
+  const int64_t blk = (int64_t)SPLIT_S * C.n0 * 32;
+  for (int it = threadIdx.x; it < 4 * 4 * ks * 2; it += blockDim.x) {
+    const int hf = it & 1, side = (it >> 1) & 1, r = it >> 2, fun = r / (2 * ks), o = r - fun * 2 * ks;
+    if (side >= nsides) continue;
+    const double *v = row(side, fun);
+    long long d[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const int j = 8 * o + 4 * hf + i;
+      d[i] = (e[side] >= SPLIT_NAN || j >= count) ? 0 : fixed53(v[slot4(j)], e[side]);
+    }
+    put_digits<6, 4>(x + (((int64_t)fun * C.nct + ct) * ks + (o >> 1)) * blk, C.n0, cit + side, o & 1, hf, d, false,
+                     0);
+  }
+}
+
 // Inverse columns of one pair and lane (both sides): C_q = sum of the orders
 // that alias to q, times 2 beyond m = 0; cosines meet Re C, sines Im C.
 __global__ void __launch_bounds__(128) k_dft_xinv(const double2 *__restrict__ rc, unsigned char *__restrict__ x,
                                                   int *__restrict__ xexp, const DftSet *__restrict__ sets,
                                                   const DftCol *__restrict__ cols, const int *__restrict__ pair_of,
                                                   const int *__restrict__ set_of, int nl, int lane0, int mmax,
-                                                  int npairs, const SolveState *__restrict__ state) {
-  extern __shared__ __align__(16) double2 sc[];  // [groups][2 sides][mx + 1], 256 entries at least
+                                                  int npairs, int eq, const SolveState *__restrict__ state) {
+  extern __shared__ __align__(16) double vals[];  // [side][CE, CO, SE, SO][slots of an order's half]
+  __shared__ double2 part[256];                   // partial alias sums of the short rings
   __shared__ int red[4];
   const int g = blockIdx.x, lane = blockIdx.y, pair = pair_of[g];
   if (state != nullptr && state[(lane0 + lane) / 3].done) return;
   const DftSet S = sets[set_of[g]];
   const DftCol C = cols[set_of[g]];
-  const int n = S.n, h = n / 2, nq = S.mx + 1;
-  const bool equator = pair == npairs - 1;
+  const int n = S.n, h = n / 2, nq = S.mx + 1, ld = slots4(S.mx / 2 + 1);
+  const bool equator = pair == eq;
   const double2 *src = rc + ((int64_t)(lane0 + lane) * (mmax + 1) * npairs + pair) * 2;
   const int64_t ms = (int64_t)npairs * 2;
   int ex[2] = {-100000, -100000};
+  auto keep = [&](int q, int side, double2 v) {
+    double *o = vals + (side * 4 + (q & 1)) * ld + slot4(q >> 1);
+    o[0] = v.x;
+    o[2 * ld] = v.y;
+    ex[side] = max(ex[side], max(exp_of(v.x), exp_of(v.y)));
+  };
   // short rings: groups of threads share the aliases of an order
   const int ng = nq < 128 ? 128 / nq : 1, grp = ng > 1 ? threadIdx.x / nq : 0;
   for (int q = ng > 1 ? threadIdx.x % nq : threadIdx.x; q < nq && grp < ng; q += 128) {
@@ -181,134 +224,152 @@ __global__ void __launch_bounds__(128) k_dft_xinv(const double2 *__restrict__ rc
       if (q > 0 && q < h) add(k * n - q, sg, -sg);
       if (k * n + q <= mmax) add(k * n + q, sg, sg);
     }
-    sc[(2 * grp) * nq + q] = a;
-    sc[(2 * grp + 1) * nq + q] = b;
-    if (ng > 1) break;
-    ex[0] = max(ex[0], max(exp_of(a.x), exp_of(a.y)));
-    ex[1] = max(ex[1], max(exp_of(b.x), exp_of(b.y)));
+    if (ng > 1) {
+      part[(2 * grp) * nq + q] = a;
+      part[(2 * grp + 1) * nq + q] = b;
+      break;
+    }
+    keep(q, 0, a);
+    keep(q, 1, b);
   }
   __syncthreads();
   if (ng > 1) {  // the groups' sums, in order
     const int q = threadIdx.x;
     if (q < nq)
       for (int side = 0; side < 2; ++side) {
-        double2 a = sc[side * nq + q];
+        double2 a = part[side * nq + q];
         for (int g2 = 1; g2 < ng; ++g2) {
-          const double2 u = sc[(2 * g2 + side) * nq + q];
+          const double2 u = part[(2 * g2 + side) * nq + q];
           a.x += u.x;
           a.y += u.y;
         }
-        sc[side * nq + q] = a;  // (its own group's slot)
-        ex[side] = max(exp_of(a.x), exp_of(a.y));
+        keep(q, side, a);
       }
-    __syncthreads();
   }
-  for (int side = 0; side < (equator ? 1 : 2); ++side) {
-    int e = max(-1000, block_max(ex[side], red));
-    if (e >= SPLIT_NAN) e = SPLIT_NAN;
-    const int pl = g - S.pair0, col = (pl * nl + lane) * 2 + side;
-    if (threadIdx.x == 0) xexp[C.col0 + col] = e;
-    int ct, cit;
-    col_place(C, col, ct, cit);
-    const int64_t blk = (int64_t)SPLIT_S * C.n0 * 32;
-    const double2 *c = sc + side * nq;
-    for (int it = threadIdx.x; it < 8 * S.rq; it += 128) {
-      const int fun = it / (2 * S.rq), hq = it - fun * 2 * S.rq, o = hq >> 1;
-      long long v[4];
-#pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        const int q = 2 * (4 * hq + i) + (fun & 1);
-        v[i] = (e >= SPLIT_NAN || q >= nq) ? 0 : fixed53(fun < 2 ? c[q].x : c[q].y, e);
-      }
-      put_digits<6, 4>(x + C.xi + (((int64_t)fun * C.nct + ct) * C.ksi + (o >> 1)) * blk, C.n0, cit, o & 1, hq & 1, v,
-                       false, 0);
-    }
+  int e[2];
+  const int col = ((g - S.pair0) * nl + lane) * 2, nsides = equator ? 1 : 2;
+  for (int side = 0; side < 2; ++side) {
+    e[side] = max(-1000, block_max(ex[side], red));  // (its barriers cover the staged values too)
+    if (e[side] >= SPLIT_NAN) e[side] = SPLIT_NAN;
+    if (threadIdx.x == 0 && side < nsides) xexp[C.col0 + col + side] = e[side];
   }
+  int ct, cit;
+  col_place(C, col, ct, cit);
+  // rows of the odd matrices end half an order earlier when mx is even
+  const int ne = S.mx / 2 + 1, no = (S.mx + 1) / 2;
+  if (no < ne && threadIdx.x < 4) vals[(2 * threadIdx.x + 1) * ld + slot4(no)] = 0.0;
+  __syncthreads();
+  digit_items(x + C.xi, C, C.ksi, ct, cit, ne, e, nsides,
+              [&](int side, int fun) { return vals + (side * 4 + fun) * ld; });
 }
 
-// One ring and lane: pixels from the orbit sums (inverse), their update or
-// output, and the orbit combinations of the forward product as digits.
+// One pair of rings and lane (threads 0-127 the northern ring, 128-255 the
+// southern): pixels from the orbit sums (inverse), their update or output, and
+// the orbit combinations of the forward product as digits.  The loads of an
+// orbit's four pixels go out together: the pass is bound by their latency and
+// the FP64 pipe, not by its bytes.
 template <int MODE>
-__global__ void __launch_bounds__(128, 8) k_dft_pix(const RingDev *__restrict__ rings, const double *__restrict__ v,
+__global__ void __launch_bounds__(256) k_dft_pix(const RingDev *__restrict__ rings, const double *__restrict__ v,
                                                  unsigned char *__restrict__ x, const int *__restrict__ xexp_in,
                                                  int *__restrict__ xexp_out, const DftSet *__restrict__ sets,
                                                  const DftCol *__restrict__ cols, const int *__restrict__ pair_of,
-                                                 const int *__restrict__ set_of, int nl, int lane0, int npairs,
+                                                 const int *__restrict__ set_of, int nl, int lane0, int eq,
                                                  int nrings, int64_t npix, const double *__restrict__ in_map,
                                                  double *__restrict__ out_map, const double *__restrict__ w,
                                                  const double *__restrict__ wd, double *__restrict__ norms,
                                                  const SolveState *__restrict__ state) {
-  extern __shared__ __align__(16) double so[];  // [4][nj] orbit combinations
-  __shared__ int red[4];
-  __shared__ double rsum[4][2];
-  const int g = blockIdx.x >> 1, side = blockIdx.x & 1, lane = blockIdx.y, pair = pair_of[g];
-  if (side && pair == npairs - 1) return;
+  extern __shared__ __align__(16) double so[];  // [side][CE, CO, SE, SO][slots of nj]
+  __shared__ int red[8];
+  __shared__ double rsum[8][2];
+  const int g = blockIdx.x, lane = blockIdx.y, pair = pair_of[g], side = threadIdx.x >> 7, tx = threadIdx.x & 127;
   const int al = lane0 + lane;
   if ((MODE == RING_ITER || MODE == RING_INIT) && state != nullptr && state[al / 3].done) return;
   const DftSet S = sets[set_of[g]];
   const DftCol C = cols[set_of[g]];
+  const int nsides = pair == eq ? 1 : 2;
+  const bool on = side < nsides;
   const int ring = side ? nrings - 1 - pair : pair;
-  const int64_t mo = (int64_t)al * npix + rings[ring].start;
-  const int pl = g - S.pair0, col = (pl * nl + lane) * 2 + side;
-  const int n = S.n, nj = S.nj;
-  const double *vc = v + C.v + (int64_t)col * 4 * C.njp;
-  bool bad = false;
-  if (MODE == RING_ITER || MODE == RING_INV_MAP) bad = xexp_in[C.col0 + col] >= SPLIT_NAN;
+  const int col = ((g - S.pair0) * nl + lane) * 2;
+  const int n = S.n, nj = S.nj, ld = slots4(nj);
   double dd = 0.0, ss = 0.0;
   int ex = -100000;
-  auto pixel = [&](int j, double s) -> double {  // value of pixel j after the inverse -> its residual
-    const int64_t i = mo + j;
-    if (MODE == RING_INV_MAP) {
-      out_map[i] = s;
-      return 0.0;
-    }
-    if (MODE == RING_ITER) {
-      const double d = s - out_map[i];
-      dd = fma(d, d, dd);
-      ss = fma(s, s, ss);
-      out_map[i] = s;
-      return fma(-w[i], s, wd[i]);
-    }
-    if (MODE == RING_INIT) return w[i] > 0.0 ? in_map[i] : 0.0;
-    return in_map[i];
-  };
-  for (int j = threadIdx.x; j < nj; j += 128) {
-    double a1 = 0, a2 = 0, b1 = 0, b2 = 0;
-    if (MODE == RING_ITER || MODE == RING_INV_MAP) {
-      const double ce = vc[j], co = vc[C.njp + j], se = vc[2 * C.njp + j], sn = vc[3 * C.njp + j];
-      a1 = ce + co;
-      a2 = ce - co;
-      b1 = sn + se;
-      b2 = sn - se;
-      if (bad) a1 = a2 = NAN;
-    }
-    double ce, co, se, sn;
-    if (S.shift || (j > 0 && 4 * j < n)) {
-      // the orbit of phi_j: j and its mirrors under phi -> pi - phi, -phi, pi + phi
-      const int jm = (S.shift ? n / 2 - 1 : n / 2) - j, jn = (S.shift ? n - 1 : n) - j, jp = n / 2 + j;
-      const double r0 = pixel(j, a1 - b1), r1 = pixel(jm, a2 - b2), r2 = pixel(jn, a1 + b1), r3 = pixel(jp, a2 + b2);
-      const double c0 = r0 + r2, c1 = r1 + r3, d0 = r0 - r2, d1 = r1 - r3;
-      ce = c0 + c1;
-      co = c0 - c1;
-      se = d0 - d1;
-      sn = d0 + d1;
-    } else if (j == 0) {  // phi = 0 and pi
-      const double r0 = pixel(0, a1), r1 = pixel(n / 2, a2);
-      ce = r0 + r1;
-      co = r0 - r1;
-      se = sn = 0.0;
-    } else {  // phi = pi/2 and 3 pi/2
-      const double r0 = pixel(j, a1 - b1), r2 = pixel(n - j, a1 + b1);
-      ce = r0 + r2;
-      co = se = 0.0;
-      sn = r0 - r2;
-    }
-    if (MODE != RING_INV_MAP) {
-      so[j] = ce;
-      so[nj + j] = co;
-      so[2 * nj + j] = se;
-      so[3 * nj + j] = sn;
-      ex = max(max(ex, max(exp_of(ce), exp_of(co))), max(exp_of(se), exp_of(sn)));
+  if (on) {
+    const int64_t mo = (int64_t)al * npix + rings[ring].start;
+    const double *vc = v + C.v + (int64_t)(col + side) * 4 * C.njp;
+    double *sv = so + side * 4 * ld;
+    bool bad = false;
+    if (MODE == RING_ITER || MODE == RING_INV_MAP) bad = xexp_in[C.col0 + col + side] >= SPLIT_NAN;
+    // orbit j: its mirrors under phi -> pi - phi, -phi and pi + phi; without
+    // the shift orbit 0 stands for the two half orbits phi = 0, pi and
+    // phi = pi/2, 3 pi/2
+    for (int j = tx; j < n / 4; j += 128) {
+      const bool two = !S.shift && j == 0;
+      int at[4] = {j, (S.shift ? n / 2 - 1 : n / 2) - j, (S.shift ? n - 1 : n) - j, n / 2 + j};
+      if (two) {
+        at[1] = n / 2;
+        at[2] = n / 4;
+        at[3] = 3 * (n / 4);
+      }
+      double p[4], pw[4], pd[4], o[4], r[4];
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        if (MODE == RING_ITER) {
+          p[k] = out_map[mo + at[k]];
+          pw[k] = w[mo + at[k]];
+          pd[k] = wd[mo + at[k]];
+        } else if (MODE == RING_INIT) {
+          pw[k] = w[mo + at[k]];
+          p[k] = in_map[mo + at[k]];
+        } else if (MODE == RING_FWD_MAP) {
+          p[k] = in_map[mo + at[k]];
+        }
+      }
+      if (MODE == RING_ITER || MODE == RING_INV_MAP) {
+        const double ce = vc[j], co = vc[C.njp + j], se = vc[2 * C.njp + j], sn = vc[3 * C.njp + j];
+        const double a1 = ce + co, a2 = ce - co, b1 = sn + se, b2 = sn - se;
+        o[0] = a1 - b1;
+        o[1] = a2 - b2;
+        o[2] = a1 + b1;
+        o[3] = a2 + b2;
+        if (two) {
+          const double c4 = vc[n / 4] + vc[C.njp + n / 4], s4 = vc[2 * C.njp + n / 4] + vc[3 * C.njp + n / 4];
+          o[0] = a1;
+          o[1] = a2;
+          o[2] = c4 - s4;
+          o[3] = c4 + s4;
+        }
+        if (bad) o[0] = o[1] = o[2] = o[3] = NAN;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) out_map[mo + at[k]] = o[k];
+      }
+      if (MODE == RING_INV_MAP) continue;
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        if (MODE == RING_ITER) {
+          const double d = o[k] - p[k];
+          dd = fma(d, d, dd);
+          ss = fma(o[k], o[k], ss);
+          r[k] = fma(-pw[k], o[k], pd[k]);
+        } else if (MODE == RING_INIT) {
+          r[k] = pw[k] > 0.0 ? p[k] : 0.0;
+        } else {
+          r[k] = p[k];
+        }
+      }
+      auto keep = [&](int i, double ce, double co, double se, double sn) {
+        sv[slot4(i)] = ce;
+        sv[ld + slot4(i)] = co;
+        sv[2 * ld + slot4(i)] = se;
+        sv[3 * ld + slot4(i)] = sn;
+        ex = max(max(ex, max(exp_of(ce), exp_of(co))), max(exp_of(se), exp_of(sn)));
+      };
+      if (two) {
+        keep(0, r[0] + r[1], r[0] - r[1], 0.0, 0.0);
+        keep(n / 4, r[2] + r[3], 0.0, 0.0, r[2] - r[3]);
+      } else {
+        const double c0 = r[0] + r[2], c1 = r[1] + r[3], d0 = r[0] - r[2], d1 = r[1] - r[3];
+        keep(j, c0 + c1, c0 - c1, d0 - d1, d0 + d1);
+      }
     }
   }
   if (MODE == RING_INV_MAP) return;
@@ -322,30 +383,28 @@ __global__ void __launch_bounds__(128, 8) k_dft_pix(const RingDev *__restrict__ 
       rsum[threadIdx.x >> 5][1] = ss;
     }
   }
-  int e = max(-1000, block_max(ex, red));  // (its barriers cover the sums and the combinations too)
-  if (e >= SPLIT_NAN) e = SPLIT_NAN;
-  if (threadIdx.x == 0) {
-    xexp_out[C.col0 + col] = e;
+  for (int o = 16; o > 0; o >>= 1) ex = max(ex, __shfl_xor_sync(0xffffffffu, ex, o));
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = ex;
+  __syncthreads();
+  int e[2];
+#pragma unroll
+  for (int k = 0; k < 2; ++k) {
+    e[k] = max(-1000, max(max(red[4 * k], red[4 * k + 1]), max(red[4 * k + 2], red[4 * k + 3])));
+    if (e[k] >= SPLIT_NAN) e[k] = SPLIT_NAN;
+  }
+  if (tx == 0 && on) {
+    xexp_out[C.col0 + col + side] = e[side];
     if (MODE == RING_ITER) {
       const int64_t no = ((int64_t)al * nrings + ring) * 2;
-      norms[no] = (rsum[0][0] + rsum[1][0]) + (rsum[2][0] + rsum[3][0]);
-      norms[no + 1] = (rsum[0][1] + rsum[1][1]) + (rsum[2][1] + rsum[3][1]);
+      const int q = 4 * side;
+      norms[no] = (rsum[q][0] + rsum[q + 1][0]) + (rsum[q + 2][0] + rsum[q + 3][0]);
+      norms[no + 1] = (rsum[q][1] + rsum[q + 1][1]) + (rsum[q + 2][1] + rsum[q + 3][1]);
     }
   }
   int ct, cit;
   col_place(C, col, ct, cit);
-  const int64_t blk = (int64_t)SPLIT_S * C.n0 * 32;
-  for (int it = threadIdx.x; it < 4 * 4 * C.ksf; it += 128) {
-    const int fun = it / (4 * C.ksf), hq = it - fun * 4 * C.ksf, o = hq >> 1;
-    long long d[4];
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      const int j = 4 * hq + i;
-      d[i] = (e >= SPLIT_NAN || j >= nj) ? 0 : fixed53(so[fun * nj + j], e);
-    }
-    put_digits<6, 4>(x + C.xf + (((int64_t)fun * C.nct + ct) * C.ksf + (o >> 1)) * blk, C.n0, cit, o & 1, hq & 1, d,
-                     false, 0);
-  }
+  digit_items(x + C.xf, C, C.ksf, ct, cit, nj, e, nsides,
+              [&](int sd, int fun) { return so + (sd * 4 + fun) * ld; });
 }
 
 // Orders beyond n/2 from the ones they alias with: thread = pair, so that the
@@ -371,6 +430,176 @@ __global__ void __launch_bounds__(128) k_dft_alias(double2 *__restrict__ rc, int
   o[(int64_t)m * npairs * 2 + 1] = make_double2(re * b.x, im * b.y);
 }
 
+// ---- the columns of a flat patch: complex transforms of the same length over
+// the N rows.  Column kx takes the place of a row pair, its real and imaginary
+// parts those of the two rows, so tables, cuts and products are the rows' own.
+constexpr int FLAT_NB = 8;  // right-hand sides per block (the E/B rotation of a column is formed once)
+
+// Column digits of field f: C_q = h_q + h_-q to the cosines, i (h_q - h_-q) to
+// the sines, h the rotated modes.  grid (columns, 3 x groups of FLAT_NB).
+__global__ void __launch_bounds__(256) k_flat_xsyn(const double2 *__restrict__ alm, unsigned char *__restrict__ x,
+                                                   int *__restrict__ xexp, const DftSet *__restrict__ sets,
+                                                   const DftCol *__restrict__ cols, int nl, int b0, double inv_area,
+                                                   int64_t nmodes, const SolveState *__restrict__ state) {
+  extern __shared__ __align__(16) double vals[];  // [re, im][CE, CO, SE, SO][slots], then cos, sin 2 phi
+  __shared__ int red[8];
+  const DftSet S = sets[0];
+  const DftCol C = cols[0];
+  const int N = S.n, ne = N / 4, ld = slots4(ne), kx = blockIdx.x, f = blockIdx.y % 3;
+  double *rot = vals + 8 * ld;
+  if (f > 0)
+    for (int q = threadIdx.x; q < N / 2; q += 256) {
+      double c, s;
+      rot2(kx, q, c, s);
+      rot[2 * q] = inv_area * c;
+      rot[2 * q + 1] = inv_area * s;
+    }
+  for (int b = (blockIdx.y / 3) * FLAT_NB; b < min(nl / 3, (int)(blockIdx.y / 3 + 1) * FLAT_NB); ++b) {
+    if (state != nullptr && state[b0 + b].done) continue;
+    __syncthreads();
+    const double2 *a = alm + (int64_t)(b0 + b) * 3 * nmodes + (int64_t)kx * N;
+    int ex[2] = {-100000, -100000};
+    for (int q = threadIdx.x; q < N / 2; q += 256) {
+      auto mode = [&](int ky, double sgn) {
+        if (f == 0) return make_double2(inv_area * a[ky].x, inv_area * a[ky].y);
+        const double2 e = a[nmodes + ky], bb = a[2 * nmodes + ky];
+        const double c = rot[2 * q], s = sgn * rot[2 * q + 1];
+        return f == 1 ? make_double2(e.x * c - bb.x * s, e.y * c - bb.y * s)
+                      : make_double2(e.x * s + bb.x * c, e.y * s + bb.y * c);
+      };
+      const double2 hp = mode(q, 1.0);
+      double2 cs = hp, sn = make_double2(0, 0);
+      if (q > 0) {
+        const double2 hm = mode(N - q, -1.0);
+        cs = make_double2(hp.x + hm.x, hp.y + hm.y);
+        sn = make_double2(hp.x - hm.x, hp.y - hm.y);
+      }
+      auto keep = [&](int ri, double c, double t) {
+        double *o = vals + (ri * 4 + (q & 1)) * ld + slot4(q >> 1);
+        o[0] = c;
+        o[2 * ld] = t;
+        ex[ri] = max(ex[ri], max(exp_of(c), exp_of(t)));
+      };
+      keep(0, cs.x, sn.y);
+      keep(1, cs.y, -sn.x);
+    }
+    int e[2];
+    const int col = (kx * nl + 3 * b + f) * 2;
+    for (int ri = 0; ri < 2; ++ri) {
+      e[ri] = max(-1000, block_max(ex[ri], red));  // (its barriers cover the staged values too)
+      if (e[ri] >= SPLIT_NAN) e[ri] = SPLIT_NAN;
+      if (threadIdx.x == 0) xexp[C.col0 + col + ri] = e[ri];
+    }
+    int ct, cit;
+    col_place(C, col, ct, cit);
+    digit_items(x + C.xi, C, C.ksi, ct, cit, ne, e, 2, [&](int ri, int fun) { return vals + (ri * 4 + fun) * ld; });
+  }
+}
+
+// Place of row y in a column of the ring coefficients (pairs (y, N - 1 - y)).
+__device__ __forceinline__ int flat_place(int y, int N) { return y < N / 2 ? 2 * y : 2 * (N - 1 - y) + 1; }
+
+// The rows of orbit j under y -> N - y and N/2 - y; orbit 0 stands for the half
+// orbits y = 0, N/2 and y = N/4, 3N/4.
+__device__ __forceinline__ void flat_orbit(int j, int N, int at[4]) {
+  at[0] = j;
+  at[1] = N / 2 - j;
+  at[2] = j ? N - j : N / 4;
+  at[3] = j ? N / 2 + j : 3 * (N / 4);
+}
+
+// Orbit sums of a column into its rows.  grid (columns, lanes)
+__global__ void __launch_bounds__(256) k_flat_unfold(const double *__restrict__ v, const int *__restrict__ xexp,
+                                                     double2 *__restrict__ rc, const DftSet *__restrict__ sets,
+                                                     const DftCol *__restrict__ cols, int nl, int lane0, int mmax,
+                                                     const SolveState *__restrict__ state) {
+  const int kx = blockIdx.x, lane = blockIdx.y, al = lane0 + lane;
+  if (state != nullptr && state[al / 3].done) return;
+  const DftCol C = cols[0];
+  const int N = sets[0].n, col = (kx * nl + lane) * 2;
+  const double *vc = v + C.v + (int64_t)col * 4 * C.njp;
+  double2 *o = rc + ((int64_t)al * (mmax + 1) + kx) * N;
+  for (int j = threadIdx.x; j < N / 4; j += 256) {
+    double s[2][4];
+#pragma unroll
+    for (int ri = 0; ri < 2; ++ri) {
+      const double *u = vc + ri * 4 * C.njp;
+      const double ce = u[j], co = u[C.njp + j], se = u[2 * C.njp + j], so = u[3 * C.njp + j];
+      const double a1 = ce + co, a2 = ce - co, b1 = so + se, b2 = so - se;
+      s[ri][0] = a1 - b1;
+      s[ri][1] = a2 - b2;
+      s[ri][2] = a1 + b1;
+      s[ri][3] = a2 + b2;
+      if (j == 0) {
+        const int h = N / 4;
+        const double c4 = u[h] + u[C.njp + h], s4 = u[2 * C.njp + h] + u[3 * C.njp + h];
+        s[ri][0] = a1;
+        s[ri][1] = a2;
+        s[ri][2] = c4 - s4;
+        s[ri][3] = c4 + s4;
+      }
+      if (xexp[C.col0 + col + ri] >= SPLIT_NAN) s[ri][0] = s[ri][1] = s[ri][2] = s[ri][3] = NAN;
+    }
+    int at[4];
+    flat_orbit(j, N, at);
+#pragma unroll
+    for (int k = 0; k < 4; ++k) o[flat_place(at[k], N)] = make_double2(s[0][k], s[1][k]);
+  }
+}
+
+// The rows of a column folded over their orbits, as digits.  grid (columns, lanes)
+__global__ void __launch_bounds__(256) k_flat_xana(const double2 *__restrict__ rc, unsigned char *__restrict__ x,
+                                                   int *__restrict__ xexp, const DftSet *__restrict__ sets,
+                                                   const DftCol *__restrict__ cols, int nl, int lane0, int mmax,
+                                                   const SolveState *__restrict__ state) {
+  extern __shared__ __align__(16) double vals[];  // [re, im][CE, CO, SE, SO][slots of nj]
+  __shared__ int red[8];
+  const int kx = blockIdx.x, lane = blockIdx.y, al = lane0 + lane;
+  if (state != nullptr && state[al / 3].done) return;
+  const DftSet S = sets[0];
+  const DftCol C = cols[0];
+  const int N = S.n, ld = slots4(S.nj), col = (kx * nl + lane) * 2;
+  const double2 *src = rc + ((int64_t)al * (mmax + 1) + kx) * N;
+  int ex[2] = {-100000, -100000};
+  for (int j = threadIdx.x; j < N / 4; j += 256) {
+    int at[4];
+    flat_orbit(j, N, at);
+    double2 r[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) r[k] = src[flat_place(at[k], N)];
+#pragma unroll
+    for (int ri = 0; ri < 2; ++ri) {
+      double y[4];
+#pragma unroll
+      for (int k = 0; k < 4; ++k) y[k] = ri ? r[k].y : r[k].x;
+      auto keep = [&](int i, double ce, double co, double se, double so) {
+        double *o = vals + ri * 4 * ld + slot4(i);
+        o[0] = ce;
+        o[ld] = co;
+        o[2 * ld] = se;
+        o[3 * ld] = so;
+        ex[ri] = max(max(ex[ri], max(exp_of(ce), exp_of(co))), max(exp_of(se), exp_of(so)));
+      };
+      if (j == 0) {
+        keep(0, y[0] + y[1], y[0] - y[1], 0.0, 0.0);
+        keep(N / 4, y[2] + y[3], 0.0, 0.0, y[2] - y[3]);
+      } else {
+        const double c0 = y[0] + y[2], c1 = y[1] + y[3], d0 = y[0] - y[2], d1 = y[1] - y[3];
+        keep(j, c0 + c1, c0 - c1, d0 - d1, d0 + d1);
+      }
+    }
+  }
+  int e[2];
+  for (int ri = 0; ri < 2; ++ri) {
+    e[ri] = max(-1000, block_max(ex[ri], red));
+    if (e[ri] >= SPLIT_NAN) e[ri] = SPLIT_NAN;
+    if (threadIdx.x == 0) xexp[C.col0 + col + ri] = e[ri];
+  }
+  int ct, cit;
+  col_place(C, col, ct, cit);
+  digit_items(x + C.xf, C, C.ksf, ct, cit, S.nj, e, 2, [&](int ri, int fun) { return vals + (ri * 4 + fun) * ld; });
+}
+
 struct DftArgs {
   const DftTile *tiles;
   int ntiles;
@@ -381,6 +610,8 @@ struct DftArgs {
   const unsigned char *x;
   const int *xexp;
   int nl, lane0, mmax, npairs;
+  int eq;               // the pair without a mirror ring (-1: none)
+  bool columns;         // forward: columns of a flat patch, modes +-q of complex sums
   double *v;            // inverse: orbit sums
   double2 *rc;          // forward: ring coefficients
   const SolveState *state;
@@ -572,12 +803,18 @@ __global__ void __launch_bounds__(DFT_THREADS, 1) k_dft(const DftArgs A) {
               const int pc = col >> 1, pl = pc / A.nl, ln = pc - pl * A.nl, al = A.lane0 + ln;
               if (A.state != nullptr && A.state[al / 3].done) continue;
               const int pair = A.pair_of[D.pair0 + pl];
-              const bool equator = pair == A.npairs - 1;
+              const bool equator = pair == A.eq;
               const int en = A.xexp[C.col0 + col], es = equator ? 0 : A.xexp[C.col0 + col + 1];
               double2 f = make_double2(value_of(acc[0][q][e], en), -value_of(acc[NF - 1][q][e], en));
               double2 s = make_double2(value_of(acc[0][q][e + 1], es), -value_of(acc[NF - 1][q][e + 1], es));
               if (en >= SPLIT_NAN) f.x = f.y = NAN;
               if (es >= SPLIT_NAN) s.x = s.y = NAN;
+              if (A.columns) {  // f, s: the sums of the real and imaginary parts
+                double2 *o = A.rc + ((int64_t)al * (A.mmax + 1) + pair) * D.n;
+                o[qo] = make_double2(f.x - s.y, f.y + s.x);
+                if (qo > 0) o[D.n - qo] = make_double2(f.x + s.y, s.x - f.y);
+                continue;
+              }
               double2 *o = A.rc + (((int64_t)al * (A.mmax + 1) + qo) * A.npairs + pair) * 2;
               o[0] = f;
               if (!equator) o[1] = s;
@@ -604,7 +841,7 @@ void drop_cut(DftCut &c) {
 
 }  // namespace
 
-// Matrix sets of a plan: polar radii, then the belt with and without the shift.
+// Matrix sets of a plan: polar radii, then the belt with and without the shift; a flat patch has one.
 static std::vector<DftSet> dft_sets(const dm_plan *p, std::vector<int> *pairs, std::vector<int> *set_of) {
   std::vector<DftSet> sets;
   auto make = [&](int n, int shift) {
@@ -618,6 +855,14 @@ static std::vector<DftSet> dft_sets(const dm_plan *p, std::vector<int> *pairs, s
     s.pair0 = (int)pairs->size();
     return s;
   };
+  if (p->flat) {  // every row of the grid
+    DftSet s = make(p->flatN, 0);
+    for (int q = 0; q < p->npairs; ++q) pairs->push_back(q);
+    s.npr = p->npairs;
+    sets.push_back(s);
+    set_of->assign(p->npairs, 0);
+    return sets;
+  }
   for (int i = 1; i < p->nside; ++i) {
     DftSet s = make(4 * i, 1);
     s.npr = 1;
@@ -848,7 +1093,7 @@ static const DftCut *dft_ready(dm_plan *p, int nl, cudaStream_t st) {
     cudaGetLastError();
     return nullptr;
   }
-  cudaError_t e = (int64_t)dft_table_bytes(p->nside, p->mmax) > p->dft_cap ? cudaErrorMemoryAllocation
+  cudaError_t e = !p->flat && (int64_t)dft_table_bytes(p->nside, p->mmax) > p->dft_cap ? cudaErrorMemoryAllocation
                                                                             : dft_setup(p, st);
   if (!e) e = dft_cut(p, nl, st);
   if (e) {
@@ -860,7 +1105,8 @@ static const DftCut *dft_ready(dm_plan *p, int nl, cudaStream_t st) {
 }
 
 template <bool FWD>
-static cudaError_t dft_products(dm_plan *p, const DftCut &K, int lane0, const SolveState *state, cudaStream_t st) {
+static cudaError_t dft_products(dm_plan *p, const DftCut &K, int lane0, const SolveState *state, cudaStream_t st,
+                                bool columns = false) {
   DftTables *T = p->dft;
   int dev = 0, sms = 0;
   cudaGetDevice(&dev);
@@ -881,6 +1127,8 @@ static cudaError_t dft_products(dm_plan *p, const DftCut &K, int lane0, const So
     A.lane0 = lane0;
     A.mmax = p->mmax;
     A.npairs = p->npairs;
+    A.eq = p->flat ? -1 : p->npairs - 1;
+    A.columns = columns;
     A.v = T->v;
     A.rc = p->rc;
     A.state = state;
@@ -905,17 +1153,29 @@ static cudaError_t dft_products(dm_plan *p, const DftCut &K, int lane0, const So
   return cudaSuccess;
 }
 
+static size_t xinv_smem(const dm_plan *p) { return sizeof(double) * 8 * slots4(p->mmax / 2 + 1); }
+static size_t pix_smem(const dm_plan *p) { return sizeof(double) * 8 * slots4((p->flat ? p->flatN / 4 : p->nside) + 1); }
+
+// Whether the products run, their tables and the cuts of all groups made.
+static bool dft_use(dm_plan *p, cudaStream_t st) {
+  if (!p->dft || p->dft->failed || p->ring_fft || p->tune_only_class >= 0) return false;
+  if (p->npix * p->batch < DFT_MIN_PIXELS || std::max(xinv_smem(p), pix_smem(p)) > DFT_SMEM) return false;
+  if (!p->dft->dig && !dft_ready(p, 3, st)) return false;  // the tables, before the group is known
+  const int gb = dft_group(p);
+  for (int b0 = 0; b0 < p->batch; b0 += gb)
+    if (!dft_ready(p, 3 * std::min(gb, p->batch - b0), st)) return false;
+  return true;
+}
+
 // The FP64 ring stage (modes of ring_stage) as split products; *ran = false
 // when the FFT kernels have to do it.
 cudaError_t dft_ring_stage(dm_plan *p, int mode, const double *in_map, double *out_map, cudaStream_t st, bool *ran) {
   *ran = false;
-  if (p->flat || !p->dft || p->dft->failed || p->ring_fft || p->tune_only_class >= 0) return cudaSuccess;
-  if (!p->dft->dig && !dft_ready(p, 3, st)) return cudaSuccess;  // the tables, before the group is known
+  if (!dft_use(p, st)) return cudaSuccess;
   const int gb = dft_group(p);
-  for (int b0 = 0; b0 < p->batch; b0 += gb)
-    if (!dft_ready(p, 3 * std::min(gb, p->batch - b0), st)) return cudaSuccess;
   *ran = true;
   DftTables *T = p->dft;
+  const int eq = p->flat ? -1 : p->npairs - 1;
   const SolveState *state = (mode == RING_ITER || mode == RING_INIT) ? p->state : nullptr;
   for (int b0 = 0; b0 < p->batch; b0 += gb) {
     const int nl = 3 * std::min(gb, p->batch - b0), lane0 = 3 * b0;
@@ -924,18 +1184,18 @@ cudaError_t dft_ring_stage(dm_plan *p, int mode, const double *in_map, double *o
     cudaError_t e;
     int *ei = T->xexp, *ef = T->xexp + T->xexp_n;
     if (mode == RING_ITER || mode == RING_INV_MAP) {
-      const size_t sm = sizeof(double2) * std::max(256, 2 * (p->mmax + 1));
+      const size_t sm = xinv_smem(p);
       if ((e = dyn_smem_allow(k_dft_xinv, sm))) return e;
       k_dft_xinv<<<dim3(T->nlist, nl), 128, sm, st>>>(p->rc, T->x, ei, T->sets_dev, K->cols, T->pair_of, T->set_of, nl,
-                                                      lane0, p->mmax, p->npairs, state);
+                                                      lane0, p->mmax, p->npairs, eq, state);
       if ((e = dft_products<false>(p, *K, lane0, state, st))) return e;
     }
-    const size_t sp = sizeof(double) * 4 * (p->nside + 1);
+    const size_t sp = pix_smem(p);
     auto pix = [&](auto kern) {
       if (cudaError_t r = dyn_smem_allow(kern, sp)) return r;
-      kern<<<dim3(2 * T->nlist, nl), 128, sp, st>>>(p->rings, T->v, T->x, ei, ef, T->sets_dev, K->cols, T->pair_of,
-                                                    T->set_of, nl, lane0, p->npairs, p->nrings, p->npix, in_map,
-                                                    out_map, p->w, p->wd, p->norms, state);
+      kern<<<dim3(T->nlist, nl), 256, sp, st>>>(p->rings, T->v, T->x, ei, ef, T->sets_dev, K->cols, T->pair_of,
+                                                T->set_of, nl, lane0, eq, p->nrings, p->npix, in_map, out_map, p->w,
+                                                p->wd, p->norms, state);
       return cudaGetLastError();
     };
     switch (mode) {
@@ -948,11 +1208,45 @@ cudaError_t dft_ring_stage(dm_plan *p, int mode, const double *in_map, double *o
     if (mode == RING_INV_MAP) continue;
     if ((e = dft_products<true>(p, *K, lane0, state, st))) return e;
     // pairs with orders beyond n / 2: the shorter polar rings, and the belt where mmax exceeds 2 nside
-    const int nrun = p->mmax > 2 * p->nside ? p->npairs : std::min(p->nside - 1, (p->mmax + 1) / 2);
+    const int nrun = p->flat ? 0 : p->mmax > 2 * p->nside ? p->npairs : std::min(p->nside - 1, (p->mmax + 1) / 2);
     if (nrun > 0 && p->mmax >= 3) {
       k_dft_alias<<<dim3((nrun + 127) / 128, p->mmax - 2, nl), 128, 0, st>>>(p->rc, lane0, p->mmax, p->npairs,
                                                                              p->nside, nrun, state);
       if ((e = cudaGetLastError())) return e;
+    }
+  }
+  return cudaSuccess;
+}
+
+// Column transforms of a flat patch as the same products; *ran = false when
+// the FFT kernels have to do them.  Synthesis: modes to the ring coefficients;
+// analysis: in place, to F[lane][kx][ky] (without the Nyquist modes).
+cudaError_t dft_flat_columns(dm_plan *p, const double2 *alm, const SolveState *state, cudaStream_t st, bool *ran) {
+  *ran = false;
+  if (!dft_use(p, st)) return cudaSuccess;
+  *ran = true;
+  DftTables *T = p->dft;
+  const int N = p->flatN, gb = dft_group(p);
+  const size_t sx = sizeof(double) * (8 * slots4(N / 4) + N), sf = sizeof(double) * 8 * slots4(N / 4 + 1);
+  for (int b0 = 0; b0 < p->batch; b0 += gb) {
+    const int nb = std::min(gb, p->batch - b0), nl = 3 * nb, lane0 = 3 * b0;
+    const DftCut *K = dft_ready(p, nl, st);
+    if (!K) return cudaErrorMemoryAllocation;
+    cudaError_t e;
+    int *ei = T->xexp, *ef = T->xexp + T->xexp_n;
+    if (alm) {
+      if ((e = dyn_smem_allow(k_flat_xsyn, sx))) return e;
+      k_flat_xsyn<<<dim3(N / 2, 3 * ((nb + FLAT_NB - 1) / FLAT_NB)), 256, sx, st>>>(
+          alm, T->x, ei, T->sets_dev, K->cols, nl, b0, 1.0 / (p->flatL * p->flatL), p->nmodes, state);
+      if ((e = dft_products<false>(p, *K, lane0, state, st))) return e;
+      k_flat_unfold<<<dim3(N / 2, nl), 256, 0, st>>>(T->v, ei, p->rc, T->sets_dev, K->cols, nl, lane0, p->mmax,
+                                                     state);
+      if ((e = cudaGetLastError())) return e;
+    } else {
+      if ((e = dyn_smem_allow(k_flat_xana, sf))) return e;
+      k_flat_xana<<<dim3(N / 2, nl), 256, sf, st>>>(p->rc, T->x, ef, T->sets_dev, K->cols, nl, lane0, p->mmax,
+                                                    state);
+      if ((e = dft_products<true>(p, *K, lane0, state, st, true))) return e;
     }
   }
   return cudaSuccess;

@@ -686,4 +686,16 @@ __device__ __forceinline__ void fused_dit_dif(T2 *x, const T2 *tw, int t, F f) {
   for (int q = 0; q < R; ++q) x[sslot(t + brev_bits(q, LR) * L)] = b[q];
 }
 
+// cos 2phi, sin 2phi of a flat patch's mode (kx, ky signed), exactly from the integers
+__device__ __forceinline__ void rot2(int kx, int ky, double &c, double &s) {
+  const double x = (double)kx, y = (double)ky, r = x * x + y * y;
+  if (r == 0.0) {
+    c = 1.0;
+    s = 0.0;
+  } else {
+    c = (x * x - y * y) / r;
+    s = 2.0 * x * y / r;
+  }
+}
+
 }  // namespace dmwf

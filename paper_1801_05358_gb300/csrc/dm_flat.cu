@@ -44,16 +44,55 @@ __device__ __forceinline__ int64_t flat_rc(int b, int f, int kx, int mmax, int y
   return ((((int64_t)b * 3 + f) * (mmax + 1) + kx) * (N / 2) + pair) * 2 + side;
 }
 
-// cos 2phi, sin 2phi of the mode (kx, ky signed), exactly from the integers
-__device__ __forceinline__ void rot2(int kx, int ky, double &c, double &s) {
-  const double x = (double)kx, y = (double)ky, r = x * x + y * y;
-  if (r == 0.0) {
-    c = 1.0;
-    s = 0.0;
-  } else {
-    c = (x * x - y * y) / r;
-    s = 2.0 * x * y / r;
+// One mode's epilogue: from the column sums g0, g1, g2 of its fields to a_l, the
+// DM step or the signal draw (w: the sums' scale; cw, sw: the rotation times it;
+// all 0 on the Nyquist row).
+__device__ __forceinline__ void flat_mode(double2 g0, double2 g1, double2 g2, double cw, double sw, double w,
+                                          int epilogue, const double *__restrict__ filt, int level, int64_t mode,
+                                          int64_t nmodes, double2 *o, const double2 *g) {
+  if (epilogue == ANA_FLAT_DRAW) {
+    // the signal draw of a constrained realisation: the 2-D FFT of white
+    // noise maps, unrotated and scaled by L/N (passed as omega), times the
+    // per-mode Cholesky factor of the TE block and sqrt(BB) (filt holds the
+    // spectra, [4][nmodes]: TT, EE, BB, TE), so that <a a^H> = L^2 S
+    const double tt = filt[mode], ee = filt[nmodes + mode], bb = filt[2 * nmodes + mode],
+                 te = filt[3 * nmodes + mode];
+    const double l11 = sqrt(fmax(tt, 0.0));
+    const double l21 = (l11 > 0.0) ? te / l11 : 0.0;
+    const double l22 = sqrt(fmax(ee - l21 * l21, 0.0));
+    const double lbb = sqrt(fmax(bb, 0.0));
+    const double2 h0 = make_double2(w * g0.x, w * g0.y), h1 = make_double2(w * g1.x, w * g1.y),
+                  h2 = make_double2(w * g2.x, w * g2.y);
+    o[0] = make_double2(l11 * h0.x, l11 * h0.y);
+    o[nmodes] = make_double2(l21 * h0.x + l22 * h1.x, l21 * h0.y + l22 * h1.y);
+    o[2 * nmodes] = make_double2(lbb * h2.x, lbb * h2.y);
+    return;
   }
+  double2 t = make_double2(0, 0), e = t, bb = t;
+  if (epilogue == ANA_DM_STEP) {
+    t = o[0];
+    e = o[nmodes];
+    bb = o[2 * nmodes];
+    if (g != nullptr) {  // the harmonic source of a Jacobi refinement's W~ run, before the filter
+      t = cadd(t, g[0]);
+      e = cadd(e, g[nmodes]);
+      bb = cadd(bb, g[2 * nmodes]);
+    }
+  }
+  double2 aT = make_double2(fma(w, g0.x, t.x), fma(w, g0.y, t.y));
+  double2 aE = make_double2(fma(g1.x, cw, fma(g2.x, sw, e.x)), fma(g1.y, cw, fma(g2.y, sw, e.y)));
+  double2 aB = make_double2(fma(-g1.x, sw, fma(g2.x, cw, bb.x)), fma(-g1.y, sw, fma(g2.y, cw, bb.y)));
+  if (epilogue == ANA_DM_STEP) {
+    const double *cf = filt + ((int64_t)level * nmodes + mode) * 4;
+    t = aT;
+    e = aE;
+    aT = make_double2(cf[0] * t.x + cf[1] * e.x, cf[0] * t.y + cf[1] * e.y);
+    aE = make_double2(cf[1] * t.x + cf[2] * e.x, cf[1] * t.y + cf[2] * e.y);
+    aB = make_double2(cf[3] * aB.x, cf[3] * aB.y);
+  }
+  o[0] = aT;
+  o[nmodes] = aE;
+  o[2 * nmodes] = aB;
 }
 
 // One column kx of one RHS per block, the three fields as lanes y = 0, 1, 2
@@ -85,46 +124,35 @@ __global__ void __launch_bounds__(768) k_flat_ana(const double2 *__restrict__ rc
     const bool keep = ky != N / 2;
     double c, s;
     rot2(kx, kys, c, s);
+    const int64_t mode = (int64_t)kx * N + ky, ob = (int64_t)b * 3 * nmodes + mode;
     const double w = keep ? omega : 0.0;
-    double2 aT = make_double2(w * g0.x, w * g0.y);
-    double2 aE = make_double2(w * (g1.x * c + g2.x * s), w * (g1.y * c + g2.y * s));
-    double2 aB = make_double2(w * (-g1.x * s + g2.x * c), w * (-g1.y * s + g2.y * c));
-    const int64_t mode = (int64_t)kx * N + ky;
-    double2 *o = out + (int64_t)b * 3 * nmodes + mode;
-    if (epilogue == ANA_FLAT_DRAW) {
-      // the signal draw of a constrained realisation: the 2-D FFT of white
-      // noise maps, unrotated and scaled by L/N (passed as omega), times the
-      // per-mode Cholesky factor of the TE block and sqrt(BB) (filt holds the
-      // spectra, [4][nmodes]: TT, EE, BB, TE), so that <a a^H> = L^2 S
-      const double tt = filt[mode], ee = filt[nmodes + mode], bb = filt[2 * nmodes + mode],
-                   te = filt[3 * nmodes + mode];
-      const double l11 = sqrt(fmax(tt, 0.0));
-      const double l21 = (l11 > 0.0) ? te / l11 : 0.0;
-      const double l22 = sqrt(fmax(ee - l21 * l21, 0.0));
-      const double lbb = sqrt(fmax(bb, 0.0));
-      const double2 h0 = make_double2(w * g0.x, w * g0.y), h1 = make_double2(w * g1.x, w * g1.y),
-                    h2 = make_double2(w * g2.x, w * g2.y);
-      o[0] = make_double2(l11 * h0.x, l11 * h0.y);
-      o[nmodes] = make_double2(l21 * h0.x + l22 * h1.x, l21 * h0.y + l22 * h1.y);
-      o[2 * nmodes] = make_double2(lbb * h2.x, lbb * h2.y);
-      continue;
-    }
-    if (epilogue == ANA_DM_STEP) {
-      const double *cf = filt + ((int64_t)state[b].level * nmodes + mode) * 4;
-      double2 t = cadd(o[0], aT), e = cadd(o[nmodes], aE), bb = cadd(o[2 * nmodes], aB);
-      if (src != nullptr) {  // the harmonic source of a Jacobi refinement's W~ run, before the filter
-        const double2 *g = src + (int64_t)b * 3 * nmodes + mode;
-        t = cadd(t, g[0]);
-        e = cadd(e, g[nmodes]);
-        bb = cadd(bb, g[2 * nmodes]);
-      }
-      aT = make_double2(cf[0] * t.x + cf[1] * e.x, cf[0] * t.y + cf[1] * e.y);
-      aE = make_double2(cf[1] * t.x + cf[2] * e.x, cf[1] * t.y + cf[2] * e.y);
-      aB = make_double2(cf[3] * bb.x, cf[3] * bb.y);
-    }
-    o[0] = aT;
-    o[nmodes] = aE;
-    o[2 * nmodes] = aB;
+    flat_mode(g0, g1, g2, w * c, w * s, w, epilogue, filt, epilogue == ANA_DM_STEP ? state[b].level : 0, mode,
+              nmodes, out + ob, src ? src + ob : nullptr);
+  }
+}
+
+// The epilogue alone, after the column products (dft_flat_columns): rc holds
+// F[b][f][mode].  Bound by its loads; each thread takes FLAT_EPI_NB right-hand
+// sides of one mode, whose rotation it forms once.
+constexpr int FLAT_EPI_NB = 8;
+__global__ void __launch_bounds__(256) k_flat_modes(const double2 *__restrict__ rc, double2 *out, int N, int batch,
+                                                    double omega, int epilogue, const double *__restrict__ filt,
+                                                    int64_t nmodes, const SolveState *__restrict__ state,
+                                                    const double2 *__restrict__ src) {
+  const int64_t mode = (int64_t)blockIdx.x * 256 + threadIdx.x;
+  if (mode >= nmodes) return;
+  const int kx = (int)(mode / N), ky = (int)(mode - (int64_t)kx * N);
+  const bool keep = ky != N / 2;
+  double c, s;
+  rot2(kx, ky < N / 2 ? ky : ky - N, c, s);
+  const double w = keep ? omega : 0.0, cw = w * c, sw = w * s;
+  for (int b = blockIdx.y * FLAT_EPI_NB; b < min(batch, (int)(blockIdx.y + 1) * FLAT_EPI_NB); ++b) {
+    if (state != nullptr && state[b].done) continue;
+    const int64_t ob = (int64_t)b * 3 * nmodes + mode;
+    const double2 z = make_double2(0, 0);
+    flat_mode(keep ? rc[ob] : z, keep ? rc[ob + nmodes] : z, keep ? rc[ob + 2 * nmodes] : z, cw, sw, w, epilogue,
+              filt, epilogue == ANA_DM_STEP ? state[b].level : 0, mode, nmodes, out + ob,
+              src ? src + ob : nullptr);
   }
 }
 
@@ -172,9 +200,11 @@ size_t flat_smem(int N) { return sizeof(double2) * ((size_t)(N - 1) + 3 * (size_
 
 cudaError_t flat_synthesis(dm_plan *p, const double2 *alm, cudaStream_t st) {
   const int N = p->flatN;
+  bool ran = false;
+  cudaError_t e = dft_flat_columns(p, alm, p->state_active ? p->state : nullptr, st, &ran);
+  if (e || ran) return e;
   const size_t sm = flat_smem(N);
-  cudaError_t e = dyn_smem_allow(k_flat_syn, sm);
-  if (e) return e;
+  if ((e = dyn_smem_allow(k_flat_syn, sm))) return e;
   const int T = std::min(256, std::max(32, N / 4));
   k_flat_syn<<<dim3(N / 2, p->batch), dim3(T, 3), sm, st>>>(alm, p->rc, p->twid, N, p->mmax,
                                                             1.0 / (p->flatL * p->flatL), p->nmodes,
@@ -184,16 +214,24 @@ cudaError_t flat_synthesis(dm_plan *p, const double2 *alm, cudaStream_t st) {
 
 cudaError_t flat_analysis(dm_plan *p, int epilogue, double2 *out, cudaStream_t st, cudaEvent_t mid) {
   const int N = p->flatN;
-  const size_t sm = flat_smem(N);
-  cudaError_t e = dyn_smem_allow(k_flat_ana, sm);
-  if (e) return e;
-  const int T = std::min(256, std::max(32, N / 4));
   const double h = p->flatL / N;
   const bool draw = epilogue == ANA_FLAT_DRAW;
   const SolveState *stp = (epilogue == ANA_DM_STEP || (p->state_active && !draw)) ? p->state : nullptr;
   const double2 *src = (epilogue == ANA_DM_STEP && p->src_active) ? p->jsrc : nullptr;
-  k_flat_ana<<<dim3(N / 2, p->batch), dim3(T, 3), sm, st>>>(p->rc, out, p->twid, N, p->mmax, draw ? h : h * h,
-                                                            epilogue, draw ? p->cl : p->filt, p->nmodes, stp, src);
+  const double omega = draw ? h : h * h, *filt = draw ? p->cl : p->filt;
+  bool ran = false;
+  cudaError_t e = dft_flat_columns(p, nullptr, stp, st, &ran);
+  if (e) return e;
+  if (ran) {
+    k_flat_modes<<<dim3((unsigned)((p->nmodes + 255) / 256), (p->batch + FLAT_EPI_NB - 1) / FLAT_EPI_NB), 256, 0, st>>>(
+        p->rc, out, N, p->batch, omega, epilogue, filt, p->nmodes, stp, src);
+  } else {
+    const size_t sm = flat_smem(N);
+    if ((e = dyn_smem_allow(k_flat_ana, sm))) return e;
+    const int T = std::min(256, std::max(32, N / 4));
+    k_flat_ana<<<dim3(N / 2, p->batch), dim3(T, 3), sm, st>>>(p->rc, out, p->twid, N, p->mmax, omega, epilogue, filt,
+                                                              p->nmodes, stp, src);
+  }
   if (mid) cudaEventRecord(mid, st);
   return cudaGetLastError();
 }

@@ -297,8 +297,9 @@ __global__ void __launch_bounds__(128) k_split_xsyn(const C *__restrict__ alm, u
   const int64_t k0 = (int64_t)(roff[m] - roff[m0]) / 2 * nct + (int64_t)ct * nk;
   unsigned char *xo = x + part * xpart + k0 * blk;
   const int nconv = part == 0 ? 2 : 4;
+  const int lc = part == 0 ? 1 : 2;  // neighbouring items write neighbouring 16-byte rows
   for (int it = threadIdx.x; it < 4 * nk * nconv; it += 128) {
-    const int c = it / (4 * nk), hq = it - c * 4 * nk, oc = hq >> 1, hf = hq & 1;
+    const int hf = it & 1, c = (it >> 1) & (nconv - 1), oc = it >> (1 + lc);
     typename Fixed<S>::type v[4];
 #pragma unroll
     for (int i = 0; i < 4; ++i) v[i] = ex >= SPLIT_NAN ? 0 : Fixed<S>::of(comp(c, 8 * oc + 4 * hf + i), ex);
@@ -385,13 +386,15 @@ __global__ void __launch_bounds__(256) k_split_xana(const C *__restrict__ rc, un
     }
     const int nh = min(pchunk, 16 * nk - p0) / 4;  // groups of four pairs
     for (int it = threadIdx.x; it < nh * nconv; it += 256) {
-      const int c = it / nh, hq = it - c * nh, pl = 4 * hq, p = p0 + pl, oc = p >> 3;
+      // neighbouring items write neighbouring 16-byte rows
+      const int r8 = it >> 3, no = nh / 2, reg = r8 / no, ol = r8 - reg * no;
+      const int c = 4 * reg + ((it >> 1) & 3), pl = 8 * ol + 4 * (it & 1), p = p0 + pl, oc = p >> 3;
       typename Fixed<S>::type v[4];
 #pragma unroll
       for (int i = 0; i < 4; ++i)
         v[i] = (ex >= SPLIT_NAN || p + i >= npairs) ? 0 : Fixed<S>::of(col[c * ld + slot(pl + i)], ex - es[p + i]);
       unsigned char *xo = x + (int64_t)(part == 0 ? 0 : 1 + (c >> 2)) * xpart + k0 * blk;
-      put_digits<S, 4>(xo + (int64_t)(oc >> 1) * blk, n0, 4 * r + (c & 3), oc & 1, hq & 1, v, false, 0);
+      put_digits<S, 4>(xo + (int64_t)(oc >> 1) * blk, n0, 4 * r + (c & 3), oc & 1, it & 1, v, false, 0);
     }
   }
 }
