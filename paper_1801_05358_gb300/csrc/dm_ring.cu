@@ -605,6 +605,14 @@ static void pick_fixed(int logm, void (*&kern)(const RingDev *, const int *, con
   }
 }
 
+// FP32 iterations of 512 to 2048 points take the register-capped radix-16
+// kernels from this many right-hand sides on: fewer passes over shared memory
+// per point, but half the threads per ring.  Whole mixed solves, radix 8
+// against radix 16, per size class: nside 128, B 1 8 % slower, B 4 2.5 %
+// slower, B 8 (the line) 1.2 % faster; nside 256, B 64 4.0 % faster; nside
+// 512, B 16 2.5 % faster.
+constexpr int RING_WIDE_BATCH = 8;
+
 template <typename R, typename C, int MODE>
 static cudaError_t launch_ring(dm_plan *p, const C *phase, const C *bhat, const C *chirps, const C *twid, C *rc,
                                const double *in_map, double *out_user, R *s_state, const R *w, const R *wd,
@@ -619,7 +627,11 @@ static cudaError_t launch_ring(dm_plan *p, const C *phase, const C *bhat, const 
     const RingClass &rc_cls = p->ring_classes[ci];
     if (p->tune_only_class >= 0 && ci != p->tune_only_class) continue;
     const bool tcls = ci < DM_TUNE_MAX_CLASSES;
-    const int lr = (tcls && p->tune_ring_lr[ci] >= 0) ? p->tune_ring_lr[ci] : p->ring_lr;
+    const int logm = 31 - __builtin_clz((unsigned)rc_cls.M);
+    const bool tuned = tcls && p->tune_ring_lr[ci] >= 0;
+    const bool wide = sizeof(R) == 4 && MODE == RING_ITER && !tuned && !p->ring_fft &&
+                      p->batch >= RING_WIDE_BATCH && logm >= 9 && logm <= 11;
+    const int lr = tuned ? p->tune_ring_lr[ci] : wide ? 4 : p->ring_lr;
     int tw_words = std::max(1, rc_cls.M - 1);
     int ph_words = rc_cls.n / 2 + 1;
     int buf_words = rc_cls.M + rc_cls.M / 32 + 1;  // slots spad(0..M)
@@ -631,7 +643,6 @@ static cudaError_t launch_ring(dm_plan *p, const C *phase, const C *bhat, const 
       if (sizeof(C) * (size_t)lane_words > (227u << 10)) return cudaErrorInvalidValue;
     }
     const bool compact = (tw_words == 0);
-    const int logm = 31 - __builtin_clz((unsigned)rc_cls.M);
     const bool fixed = MODE == RING_ITER && !compact && twr != nullptr && (lr == 3 || lr == 4) &&
                        rc_cls.M == (1 << logm) && logm >= 9 && logm <= 12 && p->twr_off[lr - 3][logm] >= 0 &&
                        (bhatT == nullptr || bhatT[lr - 3] != nullptr || p->bh_total == 0);
@@ -646,7 +657,7 @@ static cudaError_t launch_ring(dm_plan *p, const C *phase, const C *bhat, const 
         // variant 2: the FP32 radix-16 kernels of up to 2048 points compiled
         // for three blocks of 256 threads per SM (80 registers a thread)
         // instead of 128 registers and two blocks
-        const bool cap = sizeof(R) == 4 && tcls && p->tune_ring_fuse[ci] == 2 && lr == 4 && logm <= 11;
+        const bool cap = sizeof(R) == 4 && lr == 4 && logm <= 11 && (wide || (tcls && p->tune_ring_fuse[ci] == 2));
         if (lr == 3) {
           fuse ? pick_fixed<R, C, MODE, 3, true>(logm, kern) : pick_fixed<R, C, MODE, 3, false>(logm, kern);
         } else if (cap) {
