@@ -34,8 +34,13 @@
 namespace dmwf {
 
 constexpr int DFT_CHUNK = 8;       // K steps of 16 per drain
-constexpr int DFT_DRAIN_WARPS = 8;
-constexpr int DFT_THREADS = 32 * (DFT_DRAIN_WARPS + 2);
+// Warps that drain the accumulators (FP32 to integer, 64-bit sums: latency
+// bound; with 8 the tensor pipe was 48 % busy): 16 where the column quads
+// divide.  Forward products of 32 columns, 8 and 16 warps: flat N = 1024, 16
+// right-hand sides 987 and 905 us; nside 100, 5 right-hand sides 49 and 42.
+// The inverse ones, half the sums, stay as they were (855 and 866).
+__host__ __device__ constexpr int dft_drain_warps(int nq) { return nq % 2 == 0 ? 16 : 8; }
+__host__ __device__ constexpr int dft_threads(int nq) { return 32 * (dft_drain_warps(nq) + 2); }
 constexpr int DFT_MAX_STAGES = 8;
 constexpr size_t DFT_SMEM = 224u << 10;  // dynamic shared memory that a block may have here
 // Below this many pixels of a plan (all right-hand sides) the FFT kernels are
@@ -433,6 +438,9 @@ __global__ void __launch_bounds__(128) k_dft_alias(double2 *__restrict__ rc, int
 // ---- the columns of a flat patch: complex transforms of the same length over
 // the N rows.  Column kx takes the place of a row pair, its real and imaginary
 // parts those of the two rows, so tables, cuts and products are the rows' own.
+// At N = 1024 with 16 right-hand sides, against one FP64 FFT kernel each:
+// synthesis 2.53 -> 1.66 ms (digits 0.53, products 0.86, unfolding 0.27),
+// analysis 2.79 -> 1.64 (digits 0.32, products 0.91, epilogue 0.41).
 constexpr int FLAT_NB = 8;  // right-hand sides per block (the E/B rotation of a column is formed once)
 
 // Column digits of field f: C_q = h_q + h_-q to the cosines, i (h_q - h_-q) to
@@ -625,10 +633,11 @@ __device__ __forceinline__ void map_acquire(const CUtensorMap *map) {
 
 // FWD: rows are orders of one parity (cosine and sine sums in one tile), K the
 // orbits; else rows are orbits of one matrix, K the orders.  The structure of
-// the Legendre products (k_split): warps 0-7 drain, warp 8 streams, warp 9
-// issues.
+// the Legendre products (k_split): the first warps drain, then one streams
+// and one issues.
 template <bool FWD, int NQ>
-__global__ void __launch_bounds__(DFT_THREADS, 1) k_dft(const DftArgs A) {
+__global__ void __launch_bounds__(dft_threads(NQ), 1) k_dft(const DftArgs A) {
+  constexpr int DRAIN = dft_drain_warps(NQ), THREADS = dft_threads(NQ), QW = 8 * NQ / DRAIN;  // QW: column quads per warp
   constexpr int S = SPLIT_S, G = Weights<S>::G, N0 = 8 * NQ;
   constexpr int SET = (G * N0 + ((N0 & 15) ? 8 : 0) + 15) / 16 * 16;
   constexpr int COLS = 2 * SET <= 128 ? 128 : (2 * SET <= 256 ? 256 : 512);
@@ -649,13 +658,13 @@ __global__ void __launch_bounds__(DFT_THREADS, 1) k_dft(const DftArgs A) {
     }
     for (int i = 0; i < 2; ++i) {
       mbar_init(&tfull[i], 1);
-      mbar_init(&tempty[i], DFT_DRAIN_WARPS);
+      mbar_init(&tempty[i], DRAIN);
     }
     mbar_init(fin, 1);
     cta_bad = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
-  for (int i = tid; i < NS * (ZBYTES / 16); i += DFT_THREADS)
+  for (int i = tid; i < NS * (ZBYTES / 16); i += THREADS)
     *reinterpret_cast<uint4 *>(sm + (size_t)(i / (ZBYTES / 16)) * STAGE + ABYTES + BBYTES + (i % (ZBYTES / 16)) * 16) =
         make_uint4(0, 0, 0, 0);
   fence_proxy_async();
@@ -667,7 +676,7 @@ __global__ void __launch_bounds__(DFT_THREADS, 1) k_dft(const DftArgs A) {
   int issued = 0;
   const uint32_t sm_a = smem_u32(sm), full_a = smem_u32(full), empty_a = smem_u32(empty);
 
-  if (warp == DFT_DRAIN_WARPS) {
+  if (warp == DRAIN) {
     if (lane == 0) {
       bool ok = true;
       StageAt at;
@@ -696,7 +705,7 @@ __global__ void __launch_bounds__(DFT_THREADS, 1) k_dft(const DftArgs A) {
       }
       if (!ok) cta_bad = 1;
     }
-  } else if (warp == DFT_DRAIN_WARPS + 1) {
+  } else if (warp == DRAIN + 1) {
     if (lane == 0) {
       bool ok = true;
       int cc = 0;
@@ -736,17 +745,17 @@ __global__ void __launch_bounds__(DFT_THREADS, 1) k_dft(const DftArgs A) {
       mbar_wait(fin, 0, A.err);
     }
   } else {
-    const int half = warp >> 2, wq = warp & 3;
+    const int part = warp >> 2, wq = warp & 3;
     bool ok = true;
     int cc = 0;
     for (int t = blockIdx.x; ok && t < A.ntiles; t += gridDim.x) {
       const DftTile T = A.tiles[t];
       const DftSet D = A.sets[T.set];
       const DftCol C = A.cols[T.set];
-      const int ncol = D.npr * A.nl * 2, c0 = T.ct * C.w + half * NQ * 4;
+      const int ncol = D.npr * A.nl * 2, c0 = T.ct * C.w + part * QW * 4;
       const int cend = min(ncol, (T.ct + 1) * C.w);  // columns of the tile end here
       const int nch = NF * ((T.ks + DFT_CHUNK - 1) / DFT_CHUNK);
-      Acc<S> acc[NF][NQ][4];
+      Acc<S> acc[NF][QW][4];
       for (int c = 0; c < nch; ++c, ++cc) {
         const int set = cc & 1;
         if (!mbar_wait(&tfull[set], (cc >> 1) & 1, A.err)) {
@@ -755,9 +764,9 @@ __global__ void __launch_bounds__(DFT_THREADS, 1) k_dft(const DftArgs A) {
         }
         __syncwarp();
         fence_after_sync();
-        const uint32_t tcol = tbase + ((uint32_t)(wq * 32) << 16) + set * SET + half * NQ * 4;
+        const uint32_t tcol = tbase + ((uint32_t)(wq * 32) << 16) + set * SET + part * QW * 4;
 #pragma unroll
-        for (int q = 0; q < NQ; ++q) {
+        for (int q = 0; q < QW; ++q) {
           if (c0 + 4 * q >= cend) break;
           uint32_t g[G][4];
 #pragma unroll
@@ -783,7 +792,7 @@ __global__ void __launch_bounds__(DFT_THREADS, 1) k_dft(const DftArgs A) {
       if (!FWD) {
         if (row < D.nj) {
 #pragma unroll
-          for (int q = 0; q < NQ; ++q)
+          for (int q = 0; q < QW; ++q)
 #pragma unroll
             for (int e = 0; e < 4; ++e) {
               const int col = c0 + 4 * q + e;
@@ -795,7 +804,7 @@ __global__ void __launch_bounds__(DFT_THREADS, 1) k_dft(const DftArgs A) {
         const int qo = 2 * row + T.fun;  // the order
         if (qo <= D.mx) {
 #pragma unroll
-          for (int q = 0; q < NQ; ++q)
+          for (int q = 0; q < QW; ++q)
 #pragma unroll
             for (int e = 0; e < 4; e += 2) {  // the two sides of one pair and lane
               const int col = c0 + 4 * q + e;
@@ -825,7 +834,7 @@ __global__ void __launch_bounds__(DFT_THREADS, 1) k_dft(const DftArgs A) {
     if (!ok && lane == 0) cta_bad = 1;
   }
   __syncthreads();
-  if (cta_bad && warp == DFT_DRAIN_WARPS && lane == 0)
+  if (cta_bad && warp == DRAIN && lane == 0)
     for (int c = max(0, issued - NS); c < issued; ++c) mbar_wait(&full[c % NS], (c / NS) & 1, A.err);
   fence_before_sync();
   __syncthreads();
@@ -1138,7 +1147,7 @@ static cudaError_t dft_products(dm_plan *p, const DftCut &K, int lane0, const So
     const size_t smem = (size_t)A.nstages * stage;
     auto go = [&](auto kern) {
       if (cudaError_t r = dyn_smem_allow(kern, smem)) return r;
-      kern<<<std::min(sms, nt), DFT_THREADS, smem, st>>>(A);
+      kern<<<std::min(sms, nt), dft_threads(q), smem, st>>>(A);
       return cudaGetLastError();
     };
     cudaError_t e;

@@ -65,8 +65,11 @@ using namespace tc;
 constexpr int SPLIT_ROWS = 128;        // rows of a tile (ring pairs or multipoles)
 constexpr int SPLIT_CHUNK = 8;         // K steps of 16 per drain
 constexpr int SPLIT_MIN_EXP = -600;    // smallest row scale
-constexpr int SPLIT_DRAIN_WARPS = 8;
-constexpr int SPLIT_THREADS = 32 * (SPLIT_DRAIN_WARPS + 2);
+// Drain warps: 16 where the columns divide (the drain is latency bound).  Both
+// stages and the rings' products alike, a solve at nside 128 with 8 right-hand
+// sides 24.6 -> 23.2 ms, alm2map at nside 256 with 64 8.73 -> 7.98 ms.
+__host__ __device__ constexpr int split_drain_warps(int nq) { return nq % 2 == 0 ? 16 : 8; }
+__host__ __device__ constexpr int split_threads(int nq) { return 32 * (split_drain_warps(nq) + 2); }
 constexpr int SPLIT_MAX_STAGES = 12;
 constexpr size_t SPLIT_SCRATCH = (size_t)1 << 30;  // column digits of one launch
 
@@ -424,11 +427,12 @@ struct SplitArgs {
 };
 
 // SYN: rows are ring pairs, K the multipoles; else rows are multipoles, K the
-// ring pairs.  NQ: right-hand sides per drain warp group (N0 = 8 NQ columns).
+// ring pairs.  N0 = 8 NQ columns, four per right-hand side.
 template <bool SYN, int S, int NQ>
-__global__ void __launch_bounds__(SPLIT_THREADS, 1) k_split(const __grid_constant__ CUtensorMap map,
+__global__ void __launch_bounds__(split_threads(NQ), 1) k_split(const __grid_constant__ CUtensorMap map,
                                                             const SplitArgs A) {
-  constexpr int N0 = 8 * NQ;
+  constexpr int N0 = 8 * NQ, DRAIN = split_drain_warps(NQ), THREADS = split_threads(NQ);
+  constexpr int QW = 8 * NQ / DRAIN;  // right-hand sides per drain warp
   constexpr int G = Weights<S>::G;
   constexpr int SET = (G * N0 + ((N0 & 15) ? 8 : 0) + 15) / 16 * 16;  // accumulator columns of one set
   constexpr int COLS = 2 * SET <= 64 ? 64 : (2 * SET <= 128 ? 128 : (2 * SET <= 256 ? 256 : 512));
@@ -454,21 +458,21 @@ __global__ void __launch_bounds__(SPLIT_THREADS, 1) k_split(const __grid_constan
     }
     for (int i = 0; i < 2; ++i) {
       mbar_init(&tfull[i], 1);
-      mbar_init(&tempty[i], SPLIT_DRAIN_WARPS);
+      mbar_init(&tempty[i], DRAIN);
     }
     mbar_init(fin, 1);
     cta_bad = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (tid < 16) live_mask[tid] = 0;
-  for (int i = tid; i < NS * (ZBYTES / 16); i += SPLIT_THREADS)
+  for (int i = tid; i < NS * (ZBYTES / 16); i += THREADS)
     *reinterpret_cast<uint4 *>(sm + (size_t)(i / (ZBYTES / 16)) * STAGE + ABYTES + KS * BBYTES +
                               (i % (ZBYTES / 16)) * 16) =
         make_uint4(0, 0, 0, 0);
   fence_proxy_async();
   if (warp == 0) tmem_alloc(&tslot, COLS);
   __syncthreads();
-  for (int b = tid; b < A.batch; b += SPLIT_THREADS)
+  for (int b = tid; b < A.batch; b += THREADS)
     if (A.state == nullptr || !A.state[b].done) atomicOr(&live_mask[(b / A.nb) >> 5], 1u << ((b / A.nb) & 31));
   fence_before_sync();
   __syncthreads();
@@ -478,7 +482,7 @@ __global__ void __launch_bounds__(SPLIT_THREADS, 1) k_split(const __grid_constan
   int issued = 0;  // stages filled (producer)
   const uint32_t sm_a = smem_u32(sm), full_a = smem_u32(full), empty_a = smem_u32(empty);
 
-  if (warp == SPLIT_DRAIN_WARPS) {
+  if (warp == DRAIN) {
     if (lane == 0) {
       bool ok = true;
       StageAt at;
@@ -513,7 +517,7 @@ __global__ void __launch_bounds__(SPLIT_THREADS, 1) k_split(const __grid_constan
       }
       if (!ok) cta_bad = 1;
     }
-  } else if (warp == SPLIT_DRAIN_WARPS + 1) {
+  } else if (warp == DRAIN + 1) {
     if (lane == 0) {
       bool ok = true;
       int cc = 0;
@@ -564,7 +568,7 @@ __global__ void __launch_bounds__(SPLIT_THREADS, 1) k_split(const __grid_constan
       mbar_wait(fin, 0, A.err);  // every MMA has finished before the tensor memory goes
     }
   } else {
-    const int half = warp >> 2, wq = warp & 3;
+    const int part = warp >> 2, wq = warp & 3;
     bool ok = true;
     int cc = 0;
     for (int t = blockIdx.x; ok && t < total; t += gridDim.x) {
@@ -573,9 +577,9 @@ __global__ void __launch_bounds__(SPLIT_THREADS, 1) k_split(const __grid_constan
       const SplitTile T = A.tiles[t / A.nct];
       const int nfun = T.part == 0 ? 1 : 2;
       const int nch = nfun * ((T.nk + SPLIT_CHUNK - 1) / SPLIT_CHUNK);
-      const int nrhs = min(NQ, min(A.nb, A.batch - ct * A.nb) - half * NQ);  // of this warp group (may be <= 0)
+      const int nrhs = min(QW, min(A.nb, A.batch - ct * A.nb) - part * QW);  // of this warp group (may be <= 0)
       constexpr int NF = SYN ? 2 : 1;
-      Acc<S> acc[NF][NQ][4];
+      Acc<S> acc[NF][QW][4];
       for (int c = 0; c < nch; ++c, ++cc) {
         const int set = cc & 1;
         if (!mbar_wait(&tfull[set], (cc >> 1) & 1, A.err)) {
@@ -584,10 +588,10 @@ __global__ void __launch_bounds__(SPLIT_THREADS, 1) k_split(const __grid_constan
         }
         __syncwarp();
         fence_after_sync();
-        const uint32_t tcol = tbase + ((uint32_t)(wq * 32) << 16) + set * SET + half * NQ * 4;
+        const uint32_t tcol = tbase + ((uint32_t)(wq * 32) << 16) + set * SET + part * QW * 4;
         const int fa = SYN && nfun == 2 ? (c & 1) : 0;
 #pragma unroll
-        for (int q = 0; q < NQ; ++q) {
+        for (int q = 0; q < QW; ++q) {
           if (q >= nrhs) break;
           uint32_t g[G][4];
 #pragma unroll
@@ -617,9 +621,9 @@ __global__ void __launch_bounds__(SPLIT_THREADS, 1) k_split(const __grid_constan
           cplx *rc = reinterpret_cast<cplx *>(A.out);
           const bool equator = row == A.npairs - 1;
 #pragma unroll
-          for (int q = 0; q < NQ; ++q) {
+          for (int q = 0; q < QW; ++q) {
             if (q >= nrhs) break;
-            const int b = ct * A.nb + half * NQ + q;
+            const int b = ct * A.nb + part * QW + q;
             if (A.state != nullptr && A.state[b].done) continue;
             const int ex = A.xexp[((int64_t)T.m * A.batch + b) * 2 + T.part];
             const int e = ex + er;
@@ -654,9 +658,9 @@ __global__ void __launch_bounds__(SPLIT_THREADS, 1) k_split(const __grid_constan
           const int64_t i = sp_alm_base(A.lmax, T.m) + l;
           const int sg = ((l + T.m) & 1) ? -1 : 1;
 #pragma unroll
-          for (int q = 0; q < NQ; ++q) {
+          for (int q = 0; q < QW; ++q) {
             if (q >= nrhs) break;
-            const int b = ct * A.nb + half * NQ + q;
+            const int b = ct * A.nb + part * QW + q;
             if (A.state != nullptr && A.state[b].done) continue;
             const int e = A.xexp[((int64_t)T.m * A.batch + b) * 2 + T.part];
             const bool bad = e >= SPLIT_NAN;
@@ -681,7 +685,7 @@ __global__ void __launch_bounds__(SPLIT_THREADS, 1) k_split(const __grid_constan
   __syncthreads();
   // after a wait that gave up, the copies still in flight (at most the last
   // phase of each stage) land before the shared memory goes away
-  if (cta_bad && warp == SPLIT_DRAIN_WARPS && lane == 0)
+  if (cta_bad && warp == DRAIN && lane == 0)
     for (int c = max(0, issued - NS); c < issued; ++c) mbar_wait(&full[c % NS], (c / NS) & 1, A.err);
   fence_before_sync();
   __syncthreads();
@@ -1071,7 +1075,7 @@ static cudaError_t split_run(dm_plan *p, const SplitLaunches &C, const C2 *in, v
     auto go = [&](auto kern) {
       cudaError_t r = dyn_smem_allow(kern, smem);
       if (r) return r;
-      kern<<<grid, SPLIT_THREADS, smem, st>>>(map, A);
+      kern<<<grid, split_threads(nq), smem, st>>>(map, A);
       return cudaGetLastError();
     };
     switch (nq) {
