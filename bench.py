@@ -787,9 +787,9 @@ def main():
     stages = {
         "ring": hbm_line("k_ring<RING_ITER> (one launch per FFT-size class)", ring_bytes, stage["ms_ring"],
                          "k_ring_iter", ring_impl_bytes),
-        "synthesis": leg_line(("k_syn_b + k_syn_gen<0,1>" if gen_tiles else "k_syn_b + k_syn_tc<0,1>") if use_tc else ("k_leg_syn32" if mixed else "k_leg_syn64"),
+        "synthesis": leg_line(("k_syn_b + k_syn_gen<0,1>" if gen_tiles else "k_syn_b + k_syn_tc<0,1>") if use_tc else ("k_syn32 or k_split" if mixed else "k_split"),
                               stage["ms_synthesis"], "k_syn_tc" if use_tc else "k_leg_syn64"),
-        "analysis": leg_line(("k_ana_gen<0,1>" if gen_tiles else "k_ana_tc<0,1>") if use_tc else ("k_leg_ana32" if mixed else "k_leg_ana64"),
+        "analysis": leg_line(("k_ana_gen<0,1>" if gen_tiles else "k_ana_tc<0,1>") if use_tc else ("k_ana32 or k_split" if mixed else "k_split"),
                              stage["ms_analysis"], "k_ana_tc" if use_tc else "k_leg_ana64"),
         "reduce": hbm_line("k_ana_step_e32" if mixed else "k_ana_reduce", red_bytes, stage["ms_reduce"], "k_reduce"),
     }

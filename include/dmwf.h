@@ -63,15 +63,18 @@ typedef enum {
 } dm_status;
 
 /* Arithmetic of the Legendre contraction and of map storage.
- * DM_FP64: everything in FP64.
+ * DM_FP64: everything in FP64 precision.  The contractions (Legendre stages;
+ *   ring transforms and flat-patch columns of larger plans) run as products of
+ *   base-512 digits of the FP64 operands on the tensor cores, summed exactly
+ *   and rounded once; tables of digits are made on first use.  Where they
+ *   cannot be made (no memory, first use inside a stream capture) FP64 kernels
+ *   run instead.
  * DM_MIXED_FP32: FP64 recurrence (Legendre/Wigner values generated in FP64),
  *   FP32 contraction, FP32 ring FFTs and maps on the device; FP64 per-l 3x3
  *   filter, FP64 harmonic state and FP64 convergence norms.
- * DM_FLOAT_FLOAT: the FP64 path with the two Legendre stages computed in
- *   float-float arithmetic (pairs of FP32 numbers, about 48 significant bits)
- *   from FP64-generated tables on the FP32 pipe: FP64-class results (relative
- *   error near 1e-13 per transform) at a fraction of the FP64 cost on GPUs
- *   whose FP64 rate is low.  Not in the paper (an arithmetic choice). */
+ * DM_FLOAT_FLOAT: FP64-class results (relative error of 1e-13 or less per
+ *   transform); runs the same digit products as DM_FP64.  Not in the paper
+ *   (an arithmetic choice). */
 typedef enum { DM_FP64 = 0, DM_MIXED_FP32 = 1, DM_FLOAT_FLOAT = 2 } dm_precision;
 
 /* Cooling and stopping schedule of Algorithm 1 (Section 3.2).
@@ -99,8 +102,7 @@ typedef struct {
 /* Per-RHS statistics, valid after the call returns.
  * true_resid and chi2 are the paper's quality measures of the final iterate
  * (Section 3.2, Table 1; Appendix C), evaluated on the device in FP64-class
- * arithmetic (FP64, or float-float Legendre stages in DM_FLOAT_FLOAT and for
- * the mixed mode's float-float anchors):
+ * arithmetic:
  *  true_resid = ||A x - y|| / ||y||, A = 1 + S^1/2 Y^T N^-1 Y S^1/2,
  *               x = S^-1/2 a, y = S^1/2 Y^T N^-1 d  (with the analysis
  *               A = Omega Y^T standing in for Y^T, as in the iteration);
@@ -128,8 +130,7 @@ typedef struct {
  * CUDA device.  1 <= nside <= 2048 (a power of two is not required),
  * 2 <= lmax <= 4 nside, 1 <= batch <= 4096, and above nside 1024 at most
  * 2^31 - 1 pixel-components per plan (batch x 3 x 12 nside^2; nside 2048
- * allows 14 RHS).  The mixed and float-float modes also need their FP32
- * hi/lo tables (3 x nalm x 2 nside x 8 bytes) to fit.  Builds the ring geometry, the
+ * allows 14 RHS).  Builds the ring geometry, the
  * FFT chirps, the recurrence coefficient and seed tables, and allocates the
  * workspace (DM_ENOMEM if it does not fit). */
 dm_status dm_plan_create(int nside, int lmax, int batch, dm_plan **out);
@@ -239,7 +240,9 @@ dm_status dm_set_anchor_precision(dm_plan *plan, dm_precision prec);
 /* Tensor cores for the mixed-precision Legendre stages (default on): with a
  * batch of 8, 16, 32 or 64 RHS the contractions over l and over ring pairs
  * run as tcgen05 GEMMs with BF16 hi/lo split operands and FP32 accumulation
- * (three products per K step); other batches use the FP32 CUDA-core kernels.
+ * (three products per K step); other batches use FP32 kernels
+ * (small plans; the analysis of one or two RHS) or products of 27-bit operands'
+ * digits, exactly summed.
  * A pipeline wait that gives up (after 1 s) makes the solve calls return
  * DM_ETIMEOUT; the single-stage calls (dm_alm2map, dm_legendre_synthesis, ...)
  * return without synchronising and do not check it.  Each solve starts with
@@ -258,23 +261,22 @@ dm_status dm_set_tensor_cores(dm_plan *plan, int on);
  * 0: they stream tiles of stored BF16 hi/lo tables (16 GB at nside 512 /
  *    lmax 1024), built on first use.
  * Both give the same products to within the BF16 hi/lo rounding.  Without
- * stored tiles the plan keeps no full FP32 tables either: the float-float
- * anchors generate theirs per slab of orders (1 GiB).  DM_EINVAL for a null
+ * stored tiles the anchors' tables are made per slab of orders (1 GiB) where
+ * the whole ones do not fit.  DM_EINVAL for a null
  * plan, DM_EBUSY during a solve session. */
 dm_status dm_set_tc_tiles(dm_plan *plan, int generate);
 
-/* Memory for the float-float stages' per-slab Legendre tables, used when the
- * plan has no full FP32 tables (DM_FLOAT_FLOAT, and DM_MIXED_FP32's anchors
- * with generated tiles): each stage call generates the tables of one slab of
- * orders m (FP64 recurrence, hi and lo in FP32) and contracts it before the
- * next.  bytes: the largest slab (default 1 GiB; at least one order m is
- * always taken).  By default a plan keeps the full tables instead when they
- * fit in one slab, and in DM_FLOAT_FLOAT when they take at most 32 GiB;
- * after this call only the first rule applies.  Takes effect at the next stage call; DM_EINVAL for a null
+/* Memory for the per-slab Legendre digit tables of the FP64-class stages and
+ * the mixed mode's anchors: each stage call generates the tables of one slab
+ * of orders m (FP64 recurrence) and contracts it before the next.  bytes: the
+ * largest slab (default 1 GiB; at least one order m is always taken).  By
+ * default a plan keeps the full tables instead when they take at most 24 GiB;
+ * after this call it never does.  Takes effect at the next stage call; DM_EINVAL for a null
  * plan or bytes < 1, DM_EBUSY during a solve session. */
 dm_status dm_set_ff_slab_bytes(dm_plan *plan, int64_t bytes);
 
-/* Memory for the partial sums of the FP64 and float-float analysis: one
+/* Memory for the partial sums of the FP64 analysis that runs without digit
+ * tables: one
  * slot per RHS and chunk of 64 ring pairs (3 nalm FP64 complex values).  By
  * default a plan holds every chunk while that takes at most 24 GiB, else as
  * many slots as fit in it (at least 2); with fewer slots than chunks the
@@ -287,7 +289,9 @@ dm_status dm_set_analysis_slots(dm_plan *plan, int slots);
  * power of two in [512, 4096] run as fixed-size kernels of radix 2^lr with
  * M / 2^lr threads per ring and (RHS, field) lane; lr = 3 (radix 8, the
  * default) or 4 (radix 16); lr = 0 selects the generic radix-2^2 kernels for
- * every size.  The results agree to rounding.  DM_EINVAL for other lr. */
+ * every size.  In the FP64-class modes, whose larger plans run their ring and
+ * column transforms as digit products, a call selects the FFT kernels.  The
+ * results agree to rounding.  DM_EINVAL for other lr. */
 dm_status dm_set_ring_radix(dm_plan *plan, int lr);
 
 /* Constrained realisations, Section 2.2, Eq. 19:
