@@ -7,11 +7,22 @@
 // fixed-point number of S digits in base 512, every digit an integer in
 // [-256, 256] and so exact in BF16.  A product of two digits is at most 2^16,
 // and the FP32 accumulators of tcgen05.mma (kind::f16) add integers exactly up
-// to 2^24: sums of 128 products stay exact.  Digit products of equal weight
-// (i + j = k) share one accumulator; after every 128 terms the accumulators are
-// added to 64-bit integers, so no rounding happens between the splitting of
-// the inputs (2^-54 of the scale for S = 6, 2^-27 for S = 3) and the final
-// conversion, but for the dropped products i + j > S (i + j >= S for S = 3).
+// to 2^24.  Digit products of equal weight (i + j = k) share one accumulator;
+// after every 128 terms the accumulators are added to 64-bit integers, so no
+// rounding happens between the splitting of the inputs (2^-54 of the scale for
+// S = 6, 2^-27 for S = 3) and the final conversion, but for the dropped
+// products i + j > S (i + j >= S for S = 3).
+//
+// Is 128 terms short enough?  Weights 0 and 1 hold 1 and 2 products a term:
+// 2^24 at most.  From weight 4 on a unit is 2^-52 of the largest term, so a sum
+// beyond 2^24 would cost no more than FP64 does.  Weights 2 and 3 (3 and 4
+// products) could pass 2^24 only where three digits of both operands keep their
+// signs over a chunk; a digit that varies adds up as noise, near 2^20.  Harmonic
+// functions of few values on a ring (orders n / 4, n / 8, ... against a map of
+// that period) reach 0.82 of 2^24 over all amplitudes.  lambda_00 is the same
+// on every ring: against a constant map it reaches 1.17 (0.6 % of amplitudes pass
+// 1), but all terms are equal there, so every K step of 16 adds a multiple of 16,
+// which FP32 holds up to 2^28.
 // S = 6 serves DM_FP64, DM_FLOAT_FLOAT, the anchors and the diagnostics; S = 3
 // (27 bits against the 24 of FP32) the mixed mode's batches outside the BF16
 // kernels.
