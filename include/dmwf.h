@@ -271,7 +271,9 @@ dm_status dm_set_tc_tiles(dm_plan *plan, int generate);
  * of orders m (FP64 recurrence) and contracts it before the next.  bytes: the
  * largest slab (default 1 GiB; at least one order m is always taken).  By
  * default a plan keeps the full tables instead when they take at most 24 GiB;
- * after this call it never does.  Takes effect at the next stage call; DM_EINVAL for a null
+ * after this call it never does.  Takes effect at the next stage call and
+ * frees the tables made so far (a CUDA graph that recorded a stage call of the
+ * plan must not be replayed after it); DM_EINVAL for a null
  * plan or bytes < 1, DM_EBUSY during a solve session. */
 dm_status dm_set_ff_slab_bytes(dm_plan *plan, int64_t bytes);
 

@@ -82,10 +82,9 @@ struct DftCut {
   DftCol *cols = nullptr;              // device
   DftTile *tiles[2][5] = {};           // device, by direction and NQ
   int ntiles[2][5] = {};
-  int ncol = 0;
-  size_t xbytes = 0, vcount = 0;
 };
 struct DftTables {
+  int batch = 0;                       // the plan's right-hand sides (its views have one)
   std::vector<DftSet> sets;
   std::vector<int64_t> off;            // digit table offset of each set
   unsigned char *dig = nullptr;
@@ -93,12 +92,10 @@ struct DftTables {
   CUtensorMap *maps = nullptr;         // device: [set][inverse, forward]
   int *pair_of = nullptr, *set_of = nullptr;  // pair list and its sets
   int nlist = 0;
-  std::vector<DftCut> cuts;
-  unsigned char *x = nullptr;
-  size_t xbytes = 0;
-  double *v = nullptr;
-  size_t vcount = 0;
-  int *xexp = nullptr;                 // [2][columns]
+  std::vector<DftCut> cuts;            // by lanes: the groups of the plan and of its one-RHS views, three at most
+  unsigned char *x = nullptr;          // column digits of the largest group
+  double *v = nullptr;                 // orbit sums
+  int *xexp = nullptr;                 // [2][xexp_n] column exponents
   int xexp_n = 0;
   int64_t bytes = 0;
   bool failed = false;
@@ -910,62 +907,12 @@ void dft_release(dm_plan *p) {
   delete T;
   p->dft = nullptr;
 }
-void dft_new(dm_plan *p) { p->dft = new DftTables(); }
+void dft_new(dm_plan *p) {
+  p->dft = new DftTables();
+  p->dft->batch = p->batch;
+}
 void dft_disable(dm_plan *p) { p->dft->failed = true; }
 int64_t dft_bytes(const dm_plan *p) { return p->dft ? p->dft->bytes : 0; }
-
-static cudaError_t dft_setup(dm_plan *p, cudaStream_t st) {
-  DftTables *T = p->dft;
-  if (T->dig) return cudaSuccess;
-  if (!encode_fn()) return cudaErrorNotSupported;
-  std::vector<int> pairs, set_of;
-  T->sets = dft_sets(p, &pairs, &set_of);
-  T->nlist = (int)pairs.size();
-  const int ns = (int)T->sets.size();
-  int64_t total = 0;
-  T->off.clear();
-  for (const DftSet &s : T->sets) {
-    T->off.push_back(total);
-    total += (int64_t)set_bytes(s);
-  }
-  cudaError_t e;
-  unsigned char *dig = nullptr;
-  auto up = [&](auto **dst, const auto *src, size_t count) {
-    if (*dst == nullptr)
-      if (cudaError_t r = cudaMalloc((void **)dst, sizeof(*src) * count)) return r;
-    return cudaMemcpyAsync((void *)*dst, src, sizeof(*src) * count, cudaMemcpyHostToDevice, st);
-  };
-  if ((e = cudaMalloc(&dig, (size_t)total))) return e;
-  std::vector<CUtensorMap> maps(2 * ns);
-  for (int k = 0; k < ns && !e; ++k) {
-    const DftSet &s = T->sets[k];
-    for (int dir = 0; dir < 2; ++dir) {
-      const cuuint64_t dims[4] = {64, (cuuint64_t)s.nyo, (cuuint64_t)(4 * s.rq), SPLIT_S};
-      const cuuint64_t strides[3] = {128, (cuuint64_t)s.nyo * 128, (cuuint64_t)(4 * s.rq) * s.nyo * 128};
-      const cuuint32_t box[4] = {64, dir == 0 ? 16u : 2u, dir == 0 ? 2u : 16u, SPLIT_S};
-      const cuuint32_t one[4] = {1, 1, 1, 1};
-      if (encode_fn()(&maps[2 * k + dir], CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, dig + T->off[k], dims, strides, box,
-                      one, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
-                      CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
-        e = cudaErrorInvalidValue;
-    }
-    const int64_t items = (int64_t)4 * s.rq * 8 * s.nyo;
-    k_dft_gen<<<(unsigned)std::min<int64_t>((items + 127) / 128, 4096), 128, 0, st>>>(s, dig + T->off[k]);
-  }
-  if (!e) e = cudaGetLastError();
-  if (!e) e = up(&T->maps, maps.data(), maps.size());
-  if (!e) e = up(&T->sets_dev, T->sets.data(), T->sets.size());
-  if (!e) e = up(&T->pair_of, pairs.data(), pairs.size());
-  if (!e) e = up(&T->set_of, set_of.data(), set_of.size());
-  if (!e) e = cudaStreamSynchronize(st);
-  if (e) {
-    cudaFree(dig);
-    return e;
-  }
-  T->dig = dig;
-  T->bytes += total + (int64_t)(sizeof(CUtensorMap) * maps.size() + sizeof(DftSet) * ns + 2 * sizeof(int) * pairs.size());
-  return cudaSuccess;
-}
 
 // Column digits of nl lanes: bytes of the larger direction.
 static size_t cut_layout(const DftTables *T, int nl, std::vector<DftCol> *cols, int *ncol, size_t *vcount) {
@@ -998,12 +945,105 @@ static size_t cut_layout(const DftTables *T, int nl, std::vector<DftCol> *cols, 
   return std::max(xi, xf);
 }
 
+// Right-hand sides per group: as many as the column digits of DFT_SCRATCH bytes hold.
+static int dft_group(const DftTables *T, int batch) {
+  std::vector<DftCol> cols;
+  int nc;
+  size_t v;
+  int g = batch;
+  while (g > 1 && cut_layout(T, 3 * g, &cols, &nc, &v) > DFT_SCRATCH) g = (g + 1) / 2;
+  return g;
+}
+
+// Matrix sets, tensor maps and the scratch of the largest group: once per plan,
+// and kept until it goes, because a captured graph may name them.
+static cudaError_t dft_setup(dm_plan *p, cudaStream_t st) {
+  DftTables *T = p->dft;
+  if (T->dig) return cudaSuccess;
+  if (!encode_fn()) return cudaErrorNotSupported;
+  std::vector<int> pairs, set_of;
+  T->sets = dft_sets(p, &pairs, &set_of);
+  T->nlist = (int)pairs.size();
+  const int ns = (int)T->sets.size();
+  int64_t total = 0;
+  T->off.clear();
+  for (const DftSet &s : T->sets) {
+    T->off.push_back(total);
+    total += (int64_t)set_bytes(s);
+  }
+  cudaError_t e;
+  unsigned char *dig = nullptr;
+  auto up = [&](auto **dst, const auto *src, size_t count) {
+    if (*dst == nullptr)
+      if (cudaError_t r = cudaMalloc((void **)dst, sizeof(*src) * count)) return r;
+    return cudaMemcpyAsync((void *)*dst, src, sizeof(*src) * count, cudaMemcpyHostToDevice, st);
+  };
+  // the scratch of one right-hand side, of a whole group and of the last one
+  size_t xb = 0, vc = 0;
+  int nc = 0;
+  const int g = dft_group(T, T->batch);
+  for (int n : {1, g, T->batch % g}) {
+    if (n == 0) continue;
+    std::vector<DftCol> cols;
+    int c;
+    size_t v;
+    xb = std::max(xb, cut_layout(T, 3 * n, &cols, &c, &v));
+    vc = std::max(vc, v);
+    nc = std::max(nc, c);
+  }
+  if (!T->x) {
+    if ((e = cudaMalloc(&T->x, xb))) return T->x = nullptr, e;
+    T->bytes += (int64_t)xb;
+  }
+  if (!T->v) {
+    if ((e = cudaMalloc(&T->v, sizeof(double) * vc))) return T->v = nullptr, e;
+    T->bytes += (int64_t)(sizeof(double) * vc);
+  }
+  if (!T->xexp) {
+    if ((e = cudaMalloc(&T->xexp, sizeof(int) * 2 * nc))) return T->xexp = nullptr, e;
+    T->xexp_n = nc;
+    T->bytes += (int64_t)(sizeof(int) * 2 * nc);
+  }
+  if ((e = cudaMalloc(&dig, (size_t)total))) return e;
+  std::vector<CUtensorMap> maps(2 * ns);
+  for (int k = 0; k < ns && !e; ++k) {
+    const DftSet &s = T->sets[k];
+    for (int dir = 0; dir < 2; ++dir) {
+      const cuuint64_t dims[4] = {64, (cuuint64_t)s.nyo, (cuuint64_t)(4 * s.rq), SPLIT_S};
+      const cuuint64_t strides[3] = {128, (cuuint64_t)s.nyo * 128, (cuuint64_t)(4 * s.rq) * s.nyo * 128};
+      const cuuint32_t box[4] = {64, dir == 0 ? 16u : 2u, dir == 0 ? 2u : 16u, SPLIT_S};
+      const cuuint32_t one[4] = {1, 1, 1, 1};
+      if (encode_fn()(&maps[2 * k + dir], CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, dig + T->off[k], dims, strides, box,
+                      one, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
+                      CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
+        e = cudaErrorInvalidValue;
+    }
+    const int64_t items = (int64_t)4 * s.rq * 8 * s.nyo;
+    k_dft_gen<<<(unsigned)std::min<int64_t>((items + 127) / 128, 4096), 128, 0, st>>>(s, dig + T->off[k]);
+  }
+  if (!e) e = cudaGetLastError();
+  if (!e) e = up(&T->maps, maps.data(), maps.size());
+  if (!e) e = up(&T->sets_dev, T->sets.data(), T->sets.size());
+  if (!e) e = up(&T->pair_of, pairs.data(), pairs.size());
+  if (!e) e = up(&T->set_of, set_of.data(), set_of.size());
+  if (!e) e = cudaStreamSynchronize(st);
+  if (e) {
+    cudaFree(dig);
+    return e;
+  }
+  T->dig = dig;
+  T->bytes += total + (int64_t)(sizeof(CUtensorMap) * maps.size() + sizeof(DftSet) * ns + 2 * sizeof(int) * pairs.size());
+  return cudaSuccess;
+}
+
 static cudaError_t dft_cut(dm_plan *p, int nl, cudaStream_t st) {
   DftTables *T = p->dft;
   DftCut K;
   K.nl = nl;
   std::vector<DftCol> cols;
-  K.xbytes = cut_layout(T, nl, &cols, &K.ncol, &K.vcount);
+  int ncol;
+  size_t vcount;
+  cut_layout(T, nl, &cols, &ncol, &vcount);
   cudaError_t e = cudaMalloc(&K.cols, sizeof(DftCol) * cols.size());
   if (!e) e = cudaMemcpyAsync(K.cols, cols.data(), sizeof(DftCol) * cols.size(), cudaMemcpyHostToDevice, st);
   for (int dir = 0; dir < 2 && !e; ++dir) {
@@ -1044,46 +1084,12 @@ static cudaError_t dft_cut(dm_plan *p, int nl, cudaStream_t st) {
     }
   }
   if (!e) e = cudaStreamSynchronize(st);
-  if (!e && T->xbytes < K.xbytes) {
-    if (T->x) cudaFree(T->x);
-    T->bytes += (int64_t)K.xbytes - (int64_t)T->xbytes;
-    T->x = nullptr;
-    T->xbytes = 0;
-    if (!(e = cudaMalloc(&T->x, K.xbytes))) T->xbytes = K.xbytes;
-  }
-  if (!e && T->vcount < K.vcount) {
-    if (T->v) cudaFree(T->v);
-    T->bytes += (int64_t)(8 * (K.vcount - T->vcount));
-    T->v = nullptr;
-    T->vcount = 0;
-    if (!(e = cudaMalloc(&T->v, sizeof(double) * K.vcount))) T->vcount = K.vcount;
-  }
-  if (!e && T->xexp_n < K.ncol) {
-    if (T->xexp) cudaFree(T->xexp);
-    T->xexp = nullptr;
-    T->xexp_n = 0;
-    if (!(e = cudaMalloc(&T->xexp, sizeof(int) * 2 * K.ncol))) T->xexp_n = K.ncol;
-  }
   if (e) {
     drop_cut(K);
     return e;
   }
-  if (T->cuts.size() >= 6) {
-    for (DftCut &c : T->cuts) drop_cut(c);
-    T->cuts.clear();
-  }
   T->cuts.push_back(K);
   return cudaSuccess;
-}
-
-// Right-hand sides per group: as many as the column digits of DFT_SCRATCH bytes hold.
-static int dft_group(const dm_plan *p) {
-  std::vector<DftCol> cols;
-  int nc;
-  size_t v;
-  int g = p->batch;
-  while (g > 1 && cut_layout(p->dft, 3 * g, &cols, &nc, &v) > DFT_SCRATCH) g = (g + 1) / 2;
-  return g;
 }
 
 size_t dft_scratch_bytes(int nside, int batch) {  // bound of the column digits and orbit sums
@@ -1169,8 +1175,8 @@ static size_t pix_smem(const dm_plan *p) { return sizeof(double) * 8 * slots4((p
 static bool dft_use(dm_plan *p, cudaStream_t st) {
   if (!p->dft || p->dft->failed || p->ring_fft || p->tune_only_class >= 0) return false;
   if (p->npix * p->batch < DFT_MIN_PIXELS || std::max(xinv_smem(p), pix_smem(p)) > DFT_SMEM) return false;
-  if (!p->dft->dig && !dft_ready(p, 3, st)) return false;  // the tables, before the group is known
-  const int gb = dft_group(p);
+  if (!p->dft->dig && !dft_ready(p, 3, st)) return false;  // the sets, before the group is known
+  const int gb = dft_group(p->dft, p->batch);
   for (int b0 = 0; b0 < p->batch; b0 += gb)
     if (!dft_ready(p, 3 * std::min(gb, p->batch - b0), st)) return false;
   return true;
@@ -1181,7 +1187,7 @@ static bool dft_use(dm_plan *p, cudaStream_t st) {
 cudaError_t dft_ring_stage(dm_plan *p, int mode, const double *in_map, double *out_map, cudaStream_t st, bool *ran) {
   *ran = false;
   if (!dft_use(p, st)) return cudaSuccess;
-  const int gb = dft_group(p);
+  const int gb = dft_group(p->dft, p->batch);
   *ran = true;
   DftTables *T = p->dft;
   const int eq = p->flat ? -1 : p->npairs - 1;
@@ -1235,7 +1241,7 @@ cudaError_t dft_flat_columns(dm_plan *p, const double2 *alm, const SolveState *s
   if (!dft_use(p, st)) return cudaSuccess;
   *ran = true;
   DftTables *T = p->dft;
-  const int N = p->flatN, gb = dft_group(p);
+  const int N = p->flatN, gb = dft_group(p->dft, p->batch);
   const size_t sx = sizeof(double) * (8 * slots4(N / 4) + N), sf = sizeof(double) * 8 * slots4(N / 4 + 1);
   for (int b0 = 0; b0 < p->batch; b0 += gb) {
     const int nb = std::min(gb, p->batch - b0), nl = 3 * nb, lane0 = 3 * b0;

@@ -198,7 +198,8 @@ struct dm_plan {
   int tc_withhold = 0;          // test hook: one withheld arrival in the spin-0 analysis (dm_test_tc_withhold)
   // tiled BF16 hi/lo Legendre tables of the tensor-core stages ([0] = lambda, [1] = lam+/lam-)
   unsigned char *tc_synA[2] = {nullptr, nullptr}, *tc_anaA[2] = {nullptr, nullptr};
-  int *tc_ks = nullptr;         // first K step of every tile (visible_steps)
+  int *tc_ks = nullptr;         // first K step of every tile (visible_steps): stored tiles, FP32 tables
+  int *gen_ks = nullptr;        // the same of the generated tiles (gen_setup)
   int64_t *tc_soff = nullptr, *tc_aoff = nullptr;  // block offsets per m / per (m, parity)
   unsigned char *tc_synB[2] = {nullptr, nullptr};   // per-iteration synthesis B operand tiles
   // tensor-core Legendre tiles generated in the kernels (dm_legendre_otf.cu):

@@ -910,8 +910,7 @@ cudaError_t gen_setup(dm_plan *p) {
                                                               ck2, lf, p->lmax, p->npairs);
   if ((e = first_steps(lf, ks, p->mmax, p->npairs, npt, nlt)) || (e = cudaDeviceSynchronize())) return fail(e);
   cudaFree(lf);
-  cudaFree(p->tc_ks);
-  p->tc_ks = ks;
+  p->gen_ks = ks;
   p->ck0 = ck0;
   p->ck2 = ck2;
   p->rq0 = rq0;
@@ -968,7 +967,7 @@ cudaError_t syn_gen_launch(dm_plan *p, bool run0, bool run1, cudaStream_t st) {
     const size_t sm = tc_smem_n(stage, ns, nc);
     dyn_smem_allow(k_syn_gen<0>, sm);
     k_syn_gen<0><<<g, 160, sm, st>>>(p->ck0, p->ck2, p->cko, p->rq0, p->rq2, p->rq2d, p->pairs, p->tc_synB[0], p->tc_soff,
-                                     p->tc_ks, ks_stride, p->rc32, p->lmax, p->mmax, p->npairs, B, ns, nc, p->tc_err);
+                                     p->gen_ks, ks_stride, p->rc32, p->lmax, p->mmax, p->npairs, B, ns, nc, p->tc_err);
   }
   if (run1) {
     const int stage = 2 * 2 * TILE_A + 2 * 2 * (4 * B * 32);
@@ -978,7 +977,7 @@ cudaError_t syn_gen_launch(dm_plan *p, bool run0, bool run1, cudaStream_t st) {
     const size_t sm = tc_smem_n(stage, ns, nc);
     dyn_smem_allow(k_syn_gen<1>, sm);
     k_syn_gen<1><<<g, 160, sm, st>>>(p->ck0, p->ck2, p->cko, p->rq0, p->rq2, p->rq2d, p->pairs, p->tc_synB[1], p->tc_soff,
-                                     p->tc_ks, ks_stride, p->rc32, p->lmax, p->mmax, p->npairs, B, ns, nc, p->tc_err);
+                                     p->gen_ks, ks_stride, p->rc32, p->lmax, p->mmax, p->npairs, B, ns, nc, p->tc_err);
   }
   return cudaGetLastError();
 }
@@ -1017,12 +1016,12 @@ cudaError_t ana_gen_launch(dm_plan *p, cudaStream_t st) {
     dim3 g((ltiles + LT - 1) / LT, 2, p->mmax + 1);
     if (part == 0) {
       dyn_smem_allow(k_ana_gen<0>, sm);
-      k_ana_gen<0><<<g, AGEN_THREADS, sm, st>>>(p->ck0, p->ck2, p->cko, p->rq0, p->rq2, p->rq2d, p->pairs, p->tc_ks,
+      k_ana_gen<0><<<g, AGEN_THREADS, sm, st>>>(p->ck0, p->ck2, p->cko, p->rq0, p->rq2, p->rq2d, p->pairs, p->gen_ks,
                                                 npt, nlt, p->rc32, p->apart32, p->lmax, p->mmax, p->npairs, p->nalm, B, LT, nc, S,
                                                 p->tc_err, p->tc_withhold);
     } else {
       dyn_smem_allow(k_ana_gen<1>, sm);
-      k_ana_gen<1><<<g, AGEN_THREADS, sm, st>>>(p->ck0, p->ck2, p->cko, p->rq0, p->rq2, p->rq2d, p->pairs, p->tc_ks,
+      k_ana_gen<1><<<g, AGEN_THREADS, sm, st>>>(p->ck0, p->ck2, p->cko, p->rq0, p->rq2, p->rq2d, p->pairs, p->gen_ks,
                                                 npt, nlt, p->rc32, p->apart32, p->lmax, p->mmax, p->npairs, p->nalm, B, LT, nc, S,
                                                 p->tc_err, 0);
     }

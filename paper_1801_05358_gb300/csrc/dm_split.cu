@@ -114,11 +114,10 @@ struct SplitTables {
   CUtensorMap map_syn[2], map_ana[2];  // [0]: all six digits, [1]: the first three
   std::vector<int> roff;           // [mmax + 2] first table row of each order
   std::vector<int> ks_syn, ks_ana; // first K step per (part, m, row tile), from lfirst
-  unsigned char *x = nullptr;      // column digits of one launch
-  size_t xbytes = 0;
-  int *xexp = nullptr;             // [mmax + 1][batch][2] column exponents
-  int xexp_n = 0;
-  std::vector<SplitLaunches> cuts; // launches per kind of batch (a plan's own and its one-RHS views')
+  unsigned char *x = nullptr;      // column digits of one launch: six digits of every right-hand side, whatever runs
+  int *xexp = nullptr;             // [mmax + 1][batch][2] column exponents, behind x
+  int batch = 0;                   // the plan's right-hand sides (its views have one)
+  std::vector<SplitLaunches> cuts; // launches per kind of batch (a plan's own and its one-RHS views') and S: four at most
   int64_t bytes = 0;               // device memory held
   bool failed = false;             // the tables do not fit: the direct kernels run
 };
@@ -735,13 +734,16 @@ void split_release(dm_plan *p) {
   SplitTables *T = p->split;
   if (!T) return;
   drop_cuts(T);
-  for (void *q : {(void *)T->esc, (void *)T->dig, (void *)T->x, (void *)T->xexp})
+  for (void *q : {(void *)T->esc, (void *)T->dig, (void *)T->x})
     if (q) cudaFree(q);
   delete T;
   p->split = nullptr;
 }
 
-void split_new(dm_plan *p) { p->split = new SplitTables(); }
+void split_new(dm_plan *p) {
+  p->split = new SplitTables();
+  p->split->batch = p->batch;
+}
 
 void split_disable(dm_plan *p) { p->split->failed = true; }
 
@@ -802,9 +804,11 @@ cudaError_t visible_steps(dm_plan *p, int floor_exp, int **out) {
   return cudaSuccess;
 }
 
-// Row exponents, first visible multipoles, slabs and tensor maps: once per
-// plan.  The whole table is kept when it takes at most p->split_cap bytes,
-// else slabs of p->ffs_cap bytes are generated before their products.
+// Row exponents, first visible multipoles, column scratch, slabs and tensor
+// maps: once per plan, and kept until it goes, because a captured graph may
+// name them (the slabs until dm_set_ff_slab_bytes).  The whole table is kept
+// when it takes at most p->split_cap bytes, else slabs of p->ffs_cap bytes are
+// generated before their products.
 static cudaError_t split_setup(dm_plan *p, cudaStream_t st) {
   SplitTables *T = p->split;
   const int nm = p->mmax + 1, lmax = p->lmax, npairs = p->npairs;
@@ -852,6 +856,16 @@ static cudaError_t split_setup(dm_plan *p, cudaStream_t st) {
       std::copy_n(&h[(size_t)r * (npt + nlt)], npt, &T->ks_syn[(size_t)r * npt]);
       std::copy_n(&h[(size_t)r * (npt + nlt) + npt], nlt, &T->ks_ana[(size_t)r * nlt]);
     }
+  }
+  if (!T->x) {
+    const size_t xb = (split_scratch_bytes(lmax, npairs, T->batch) + 127) / 128 * 128;
+    const size_t all = xb + sizeof(int) * 2 * (size_t)nm * T->batch;
+    if ((e = cudaMalloc(&T->x, all))) {
+      T->x = nullptr;
+      return e;
+    }
+    T->xexp = reinterpret_cast<int *>(T->x + xb);
+    T->bytes += (int64_t)all;
   }
   if (!T->dig) {
     const size_t row_bytes = (size_t)3 * SPLIT_S * 128 * T->npoct;
@@ -914,7 +928,6 @@ static cudaError_t split_cut(dm_plan *p, int S, cudaStream_t st) {
   C.S = S;
   cudaError_t e = cudaSuccess;
   const size_t blk = (size_t)S * C.n0 * 32, cap = SPLIT_SCRATCH;
-  size_t need = 0;
   const int npt = (npairs + 127) / 128, nlt = (lmax + 128) / 128, nkp = (npairs + 15) / 16;
   for (int dir = 0; dir < 2 && !e; ++dir) {
     std::vector<SplitTile> tiles;
@@ -928,7 +941,6 @@ static cudaError_t split_cut(dm_plan *p, int S, cudaStream_t st) {
           if (m1 > m0 && bytes + add > cap) break;
           bytes += add;
         }
-        need = std::max(need, bytes);
         const size_t first = tiles.size();
         for (int m = m0; m < m1; ++m)
           for (int part = 0; part < 2; ++part)
@@ -957,29 +969,11 @@ static cudaError_t split_cut(dm_plan *p, int S, cudaStream_t st) {
       e = cudaMemcpyAsync(C.tiles[dir], tiles.data(), sizeof(SplitTile) * tiles.size(), cudaMemcpyHostToDevice, st);
     if (!e) e = cudaStreamSynchronize(st);
   }
-  const int nexp = 2 * nm * p->batch;
-  if (!e && T->xexp_n < nexp) {
-    if (T->xexp) cudaFree(T->xexp);
-    T->bytes += (int64_t)sizeof(int) * (nexp - T->xexp_n);
-    T->xexp = nullptr;
-    T->xexp_n = 0;
-    e = cudaMalloc(&T->xexp, sizeof(int) * nexp);
-    if (!e) T->xexp_n = nexp;
-  }
-  if (!e && T->xbytes < need) {
-    if (T->x) cudaFree(T->x);
-    T->bytes += (int64_t)need - (int64_t)T->xbytes;
-    T->x = nullptr;
-    T->xbytes = 0;
-    e = cudaMalloc(&T->x, need);
-    if (!e) T->xbytes = need;
-  }
   if (e) {
     for (SplitTile *t : C.tiles)
       if (t) cudaFree(t);
     return e;
   }
-  if (T->cuts.size() >= 6) drop_cuts(T);
   T->cuts.push_back(C);
   return cudaSuccess;
 }
@@ -988,7 +982,7 @@ static const SplitLaunches *split_find(const dm_plan *p, int S) {
   const SplitTables *T = p->split;
   int nct, nb, nq;
   split_cols(p->batch, &nct, &nb, &nq);
-  if (!T->dig || T->xexp_n < 2 * (p->mmax + 1) * p->batch) return nullptr;
+  if (!T->dig) return nullptr;
   for (const SplitLaunches &c : T->cuts)
     if (c.nct == nct && c.n0 == 8 * nq && c.S == S) return &c;
   return nullptr;
