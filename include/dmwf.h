@@ -68,7 +68,7 @@ typedef enum {
  *   base-512 digits of the FP64 operands on the tensor cores, summed exactly
  *   and rounded once; tables of digits are made on first use.  Where they
  *   cannot be made (no memory, first use inside a stream capture) FP64 kernels
- *   run instead.
+ *   run instead, and a later call makes them once there is more memory.
  * DM_MIXED_FP32: FP64 recurrence (Legendre/Wigner values generated in FP64),
  *   FP32 contraction, FP32 ring FFTs and maps on the device; FP64 per-l 3x3
  *   filter, FP64 harmonic state and FP64 convergence norms.
@@ -528,6 +528,13 @@ dm_status dm_set_noise_flat(dm_plan *plan, const double *sigma, const uint8_t *m
  * DM_ETIMEOUT.  The plan and the CUDA context stay usable: turn it off and
  * the next solve is normal.  Not for production use. */
 dm_status dm_test_tc_withhold(dm_plan *plan, int on);
+
+/* Failure test of the tables made on first use (Legendre digits, DFT
+ * matrices, FP32 Legendre values): from now on an allocation of more than
+ * `bytes` for them reports that the device has no memory (-1: the device
+ * decides).  The calls then run as they do where the tables do not fit, and
+ * make them once the limit is lifted.  Not for production use. */
+dm_status dm_test_table_memory(dm_plan *plan, int64_t bytes);
 
 /* --- serving: continuous batching of requests of different geometries ---- */
 

@@ -951,6 +951,12 @@ dm_status dm_set_analysis_slots(dm_plan *p, int slots) {
   return DM_OK;
 }
 
+dm_status dm_test_table_memory(dm_plan *p, int64_t bytes) {
+  if (!p) return DM_EINVAL;
+  p->table_limit = bytes;
+  return DM_OK;
+}
+
 dm_status dm_test_tc_withhold(dm_plan *p, int on) {
   if (!p) return DM_EINVAL;
   p->tc_withhold = on != 0;

@@ -98,7 +98,8 @@ struct DftTables {
   int *xexp = nullptr;                 // [2][xexp_n] column exponents
   int xexp_n = 0;
   int64_t bytes = 0;
-  bool failed = false;
+  bool disabled = false;               // the plan's owner chose the FFT kernels, or the matrices pass dft_cap
+  Shortage shortage;                   // they did not fit
 };
 
 namespace {
@@ -897,21 +898,33 @@ size_t dft_table_bytes(int nside, int mmax) {
   return (size_t)b;
 }
 
-void dft_release(dm_plan *p) {
-  DftTables *T = p->dft;
-  if (!T) return;
+// All that the device holds of the tables goes.
+static void drop_tables(DftTables *T) {
   for (DftCut &c : T->cuts) drop_cut(c);
+  T->cuts.clear();
   for (void *q : {(void *)T->dig, (void *)T->sets_dev, (void *)T->maps, (void *)T->pair_of, (void *)T->set_of,
                   (void *)T->x, (void *)T->v, (void *)T->xexp})
     if (q) cudaFree(q);
-  delete T;
+  T->dig = T->x = nullptr;
+  T->sets_dev = nullptr;
+  T->maps = nullptr;
+  T->pair_of = T->set_of = T->xexp = nullptr;
+  T->v = nullptr;
+  T->xexp_n = 0;
+  T->bytes = 0;
+}
+
+void dft_release(dm_plan *p) {
+  if (!p->dft) return;
+  drop_tables(p->dft);
+  delete p->dft;
   p->dft = nullptr;
 }
 void dft_new(dm_plan *p) {
   p->dft = new DftTables();
   p->dft->batch = p->batch;
 }
-void dft_disable(dm_plan *p) { p->dft->failed = true; }
+void dft_disable(dm_plan *p) { p->dft->disabled = true; }
 int64_t dft_bytes(const dm_plan *p) { return p->dft ? p->dft->bytes : 0; }
 
 // Column digits of nl lanes: bytes of the larger direction.
@@ -992,19 +1005,19 @@ static cudaError_t dft_setup(dm_plan *p, cudaStream_t st) {
     nc = std::max(nc, c);
   }
   if (!T->x) {
-    if ((e = cudaMalloc(&T->x, xb))) return T->x = nullptr, e;
+    if ((e = table_alloc(p, (void **)&T->x, xb))) return e;
     T->bytes += (int64_t)xb;
   }
   if (!T->v) {
-    if ((e = cudaMalloc(&T->v, sizeof(double) * vc))) return T->v = nullptr, e;
+    if ((e = table_alloc(p, (void **)&T->v, sizeof(double) * vc))) return e;
     T->bytes += (int64_t)(sizeof(double) * vc);
   }
   if (!T->xexp) {
-    if ((e = cudaMalloc(&T->xexp, sizeof(int) * 2 * nc))) return T->xexp = nullptr, e;
+    if ((e = table_alloc(p, (void **)&T->xexp, sizeof(int) * 2 * nc))) return e;
     T->xexp_n = nc;
     T->bytes += (int64_t)(sizeof(int) * 2 * nc);
   }
-  if ((e = cudaMalloc(&dig, (size_t)total))) return e;
+  if ((e = table_alloc(p, (void **)&dig, (size_t)total))) return e;
   std::vector<CUtensorMap> maps(2 * ns);
   for (int k = 0; k < ns && !e; ++k) {
     const DftSet &s = T->sets[k];
@@ -1098,25 +1111,10 @@ size_t dft_scratch_bytes(int nside, int batch) {  // bound of the column digits 
          ((size_t)32 << 20);
 }
 
-static const DftCut *dft_ready(dm_plan *p, int nl, cudaStream_t st) {
-  DftTables *T = p->dft;
-  if (!T || T->failed) return nullptr;
+static const DftCut *dft_find(const DftTables *T, int nl) {
   for (const DftCut &c : T->cuts)
     if (c.nl == nl) return &c;
-  cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
-  if (cudaStreamIsCapturing(st, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone) {
-    cudaGetLastError();
-    return nullptr;
-  }
-  cudaError_t e = !p->flat && (int64_t)dft_table_bytes(p->nside, p->mmax) > p->dft_cap ? cudaErrorMemoryAllocation
-                                                                            : dft_setup(p, st);
-  if (!e) e = dft_cut(p, nl, st);
-  if (e) {
-    cudaGetLastError();
-    T->failed = true;
-    return nullptr;
-  }
-  return &T->cuts.back();
+  return nullptr;
 }
 
 template <bool FWD>
@@ -1171,31 +1169,61 @@ static cudaError_t dft_products(dm_plan *p, const DftCut &K, int lane0, const So
 static size_t xinv_smem(const dm_plan *p) { return sizeof(double) * 8 * slots4(p->mmax / 2 + 1); }
 static size_t pix_smem(const dm_plan *p) { return sizeof(double) * 8 * slots4((p->flat ? p->flatN / 4 : p->nside) + 1); }
 
-// Whether the products run, their tables and the cuts of all groups made.
-static bool dft_use(dm_plan *p, cudaStream_t st) {
-  if (!p->dft || p->dft->failed || p->ring_fft || p->tune_only_class >= 0) return false;
-  if (p->npix * p->batch < DFT_MIN_PIXELS || std::max(xinv_smem(p), pix_smem(p)) > DFT_SMEM) return false;
-  if (!p->dft->dig && !dft_ready(p, 3, st)) return false;  // the sets, before the group is known
-  const int gb = dft_group(p->dft, p->batch);
-  for (int b0 = 0; b0 < p->batch; b0 += gb)
-    if (!dft_ready(p, 3 * std::min(gb, p->batch - b0), st)) return false;
-  return true;
+// Whether the products run; then their tables and the cuts of all groups exist.
+static cudaError_t dft_use(dm_plan *p, cudaStream_t st, bool *use) {
+  DftTables *T = p->dft;
+  *use = false;
+  if (!T || T->disabled || p->ring_fft || p->tune_only_class >= 0) return cudaSuccess;
+  if (p->npix * p->batch < DFT_MIN_PIXELS || std::max(xinv_smem(p), pix_smem(p)) > DFT_SMEM) return cudaSuccess;
+  const int B = p->batch;
+  auto found = [&](int gb) {
+    for (int b0 = 0; b0 < B; b0 += gb)
+      if (!dft_find(T, 3 * std::min(gb, B - b0))) return false;
+    return true;
+  };
+  if (T->dig && found(dft_group(T, B))) {
+    *use = true;
+    return cudaSuccess;
+  }
+  if (!T->dig && !p->flat && (int64_t)dft_table_bytes(p->nside, p->mmax) > p->dft_cap) {
+    T->disabled = true;
+    return cudaSuccess;
+  }
+  cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(st, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone) {
+    cudaGetLastError();
+    return cudaSuccess;
+  }
+  if (T->shortage.lasts(p)) return cudaSuccess;
+  const bool fresh = T->cuts.empty();
+  cudaError_t e = dft_setup(p, st);
+  const int gb = e ? B : dft_group(T, B);
+  for (int b0 = 0; !e && b0 < B; b0 += gb)
+    if (!dft_find(T, 3 * std::min(gb, B - b0))) e = dft_cut(p, 3 * std::min(gb, B - b0), st);
+  if (e) {
+    if (fresh) drop_tables(T);  // no launch has named them yet
+    cudaGetLastError();
+    if (e == cudaErrorNotSupported) T->disabled = true;
+    if (e == cudaErrorMemoryAllocation) T->shortage.note(p);
+    return e == cudaErrorMemoryAllocation || e == cudaErrorNotSupported ? cudaSuccess : e;
+  }
+  T->shortage = Shortage();
+  *use = true;
+  return cudaSuccess;
 }
 
 // The FP64 ring stage (modes of ring_stage) as split products; *ran = false
 // when the FFT kernels have to do it.
 cudaError_t dft_ring_stage(dm_plan *p, int mode, const double *in_map, double *out_map, cudaStream_t st, bool *ran) {
-  *ran = false;
-  if (!dft_use(p, st)) return cudaSuccess;
+  const cudaError_t eu = dft_use(p, st, ran);
+  if (eu || !*ran) return eu;
   const int gb = dft_group(p->dft, p->batch);
-  *ran = true;
   DftTables *T = p->dft;
   const int eq = p->flat ? -1 : p->npairs - 1;
   const SolveState *state = (mode == RING_ITER || mode == RING_INIT) ? p->state : nullptr;
   for (int b0 = 0; b0 < p->batch; b0 += gb) {
     const int nl = 3 * std::min(gb, p->batch - b0), lane0 = 3 * b0;
-    const DftCut *K = dft_ready(p, nl, st);
-    if (!K) return cudaErrorMemoryAllocation;
+    const DftCut *K = dft_find(T, nl);
     cudaError_t e;
     int *ei = T->xexp, *ef = T->xexp + T->xexp_n;
     if (mode == RING_ITER || mode == RING_INV_MAP) {
@@ -1237,16 +1265,14 @@ cudaError_t dft_ring_stage(dm_plan *p, int mode, const double *in_map, double *o
 // the FFT kernels have to do them.  Synthesis: modes to the ring coefficients;
 // analysis: in place, to F[lane][kx][ky] (without the Nyquist modes).
 cudaError_t dft_flat_columns(dm_plan *p, const double2 *alm, const SolveState *state, cudaStream_t st, bool *ran) {
-  *ran = false;
-  if (!dft_use(p, st)) return cudaSuccess;
-  *ran = true;
+  const cudaError_t eu = dft_use(p, st, ran);
+  if (eu || !*ran) return eu;
   DftTables *T = p->dft;
   const int N = p->flatN, gb = dft_group(p->dft, p->batch);
   const size_t sx = sizeof(double) * (8 * slots4(N / 4) + N), sf = sizeof(double) * 8 * slots4(N / 4 + 1);
   for (int b0 = 0; b0 < p->batch; b0 += gb) {
     const int nb = std::min(gb, p->batch - b0), nl = 3 * nb, lane0 = 3 * b0;
-    const DftCut *K = dft_ready(p, nl, st);
-    if (!K) return cudaErrorMemoryAllocation;
+    const DftCut *K = dft_find(T, nl);
     cudaError_t e;
     int *ei = T->xexp, *ef = T->xexp + T->xexp_n;
     if (alm) {

@@ -67,6 +67,14 @@ struct RingClass {
   int poff, pcount;  // pair_order[poff .. poff + pcount): the northern (or equatorial) rings of the class
 };
 
+// Device memory that did not suffice for a plan's tables: tried again once
+// there is more of it than there was then.
+struct Shortage {
+  size_t room = SIZE_MAX;
+  void note(const dm_plan *p);
+  bool lasts(const dm_plan *p) const;
+};
+
 struct SplitTables;  // dm_split.cu
 struct DftTables;    // dm_dft.cu
 
@@ -160,12 +168,13 @@ struct dm_plan {
   bool fp32_ready = false;      // the buffers of the FP32 modes exist (setup_fp32 succeeded)
   // FP32 Legendre tables of the mixed mode's small plans and batches (dm_legendre32.cu)
   float *tab32 = nullptr;       // [3][nalm][npairs up to a multiple of 4] lambda, lam+, lam-
-  bool tab32_failed = false;    // they did not fit: the split products run
+  dmwf::Shortage tab32_short;   // they did not fit: the split products run
   bool is_view = false;         // a one-RHS view of a serving pool (makes no tables of its own)
   // digit tables of the split products (dm_split.cu): shared with the views of the plan
   dmwf::SplitTables *split = nullptr;
   // ring DFT matrices of the FP64-class modes (dm_dft.cu), shared likewise
   dmwf::DftTables *dft = nullptr;
+  int64_t table_limit = -1;     // test hook (dm_test_table_memory): bytes that one table may take, -1: what the device has
   int64_t dft_cap = (int64_t)8 << 30;  // largest matrix table kept (else the FFT kernels)
   int64_t split_cap = (int64_t)24 << 30;  // largest whole table kept
   int64_t ffs_cap = (int64_t)1 << 30;  // bytes of the largest slab when the table is not kept whole
@@ -329,6 +338,10 @@ inline cudaError_t dyn_smem_allow(F *func, size_t bytes) {
 }
 // first alm index of order m (m = mmax + 1 = lmax + 1 gives nalm): idx(l, m) = start(m) + l - m
 inline int64_t alm_start_h(int lmax, int m) { return (int64_t)m * (2 * lmax + 3 - m) / 2; }
+// Tables made on first use, beyond the workspace of dm_plan_create (dm_setup.cu):
+// device memory free for them, and their allocation.
+size_t table_room(const dm_plan *p);
+cudaError_t table_alloc(const dm_plan *p, void **ptr, size_t bytes);
 // FP64-class ring transforms as split products (dm_dft.cu)
 void dft_new(dm_plan *p);
 void dft_release(dm_plan *p);

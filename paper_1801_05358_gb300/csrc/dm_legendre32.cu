@@ -222,7 +222,6 @@ int64_t order_entries(const dm_plan *p) { return (int64_t)p->npairs * (p->lmax +
 // plan that shares another's tables, or beyond 8 GiB.
 bool tables(dm_plan *p, cudaStream_t st) {
   if (p->tab32) return true;
-  if (p->tab32_failed) return false;
   const double bytes = 12.0 * (double)p->nalm * table_ld(p);
   cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
   if (bytes > 8.0 * (1u << 30) || p->is_view || cudaStreamIsCapturing(st, &cs) != cudaSuccess ||
@@ -230,16 +229,17 @@ bool tables(dm_plan *p, cudaStream_t st) {
     cudaGetLastError();
     return false;
   }
+  if (p->tab32_short.lasts(p)) return false;
   float *t = nullptr;
   int *ks = nullptr;
-  cudaError_t e = cudaMalloc(&t, (size_t)bytes);
+  cudaError_t e = table_alloc(p, (void **)&t, (size_t)bytes);
   if (!e && table_ld(p) != p->npairs) e = cudaMemsetAsync(t, 0, (size_t)bytes, st);
   if (!e) e = gen_tables32(p, t, table_ld(p), st);
   if (!e && !p->tc_ks) e = visible_steps(p, TC_FLOOR_EXP, &ks);
   if (e) {
     cudaGetLastError();
     cudaFree(t);
-    p->tab32_failed = true;
+    p->tab32_short.note(p);
     return false;
   }
   p->tab32 = t;

@@ -598,6 +598,27 @@ __global__ void k_d2f2(const double2 *in, float2 *out, int64_t n) {
     out[i] = make_float2((float)in[i].x, (float)in[i].y);
 }
 
+size_t table_room(const dm_plan *p) {
+  size_t fr = 0, all = 0;
+  if (cudaMemGetInfo(&fr, &all) != cudaSuccess) {
+    cudaGetLastError();
+    return 0;
+  }
+  return p->table_limit >= 0 ? std::min(fr, (size_t)p->table_limit) : fr;
+}
+cudaError_t table_alloc(const dm_plan *p, void **ptr, size_t bytes) {
+  *ptr = nullptr;
+  if (p->table_limit >= 0 && bytes > (size_t)p->table_limit) return cudaErrorMemoryAllocation;
+  const cudaError_t e = cudaMalloc(ptr, bytes);
+  if (e) {
+    *ptr = nullptr;
+    cudaGetLastError();
+  }
+  return e;
+}
+void Shortage::note(const dm_plan *p) { room = table_room(p); }
+bool Shortage::lasts(const dm_plan *p) const { return room != SIZE_MAX && table_room(p) <= room; }
+
 // Buffers of DM_MIXED_FP32 and DM_FLOAT_FLOAT: FP32 copies of the FFT tables,
 // FP32 ring coefficients and maps.  The Legendre tables are made on first use
 // (dm_split.cu, dm_legendre_tc.cu, dm_legendre_otf.cu).

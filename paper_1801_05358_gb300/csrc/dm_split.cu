@@ -119,7 +119,8 @@ struct SplitTables {
   int batch = 0;                   // the plan's right-hand sides (its views have one)
   std::vector<SplitLaunches> cuts; // launches per kind of batch (a plan's own and its one-RHS views') and S: four at most
   int64_t bytes = 0;               // device memory held
-  bool failed = false;             // the tables do not fit: the direct kernels run
+  bool disabled = false;           // the plan's owner chose the direct kernels
+  Shortage shortage;               // the tables did not fit: the direct kernels run
 };
 
 namespace {
@@ -730,13 +731,23 @@ static void drop_cuts(SplitTables *T) {
 
 int64_t split_bytes(const dm_plan *p) { return p->split ? p->split->bytes : 0; }
 
-void split_release(dm_plan *p) {
-  SplitTables *T = p->split;
-  if (!T) return;
+// All that the device holds of the tables goes.
+static void drop_tables(SplitTables *T) {
   drop_cuts(T);
   for (void *q : {(void *)T->esc, (void *)T->dig, (void *)T->x})
     if (q) cudaFree(q);
-  delete T;
+  T->esc = nullptr;
+  T->dig = T->x = nullptr;
+  T->xexp = nullptr;
+  T->full = false;
+  T->slab.clear();
+  T->bytes = 0;
+}
+
+void split_release(dm_plan *p) {
+  if (!p->split) return;
+  drop_tables(p->split);
+  delete p->split;
   p->split = nullptr;
 }
 
@@ -745,7 +756,7 @@ void split_new(dm_plan *p) {
   p->split->batch = p->batch;
 }
 
-void split_disable(dm_plan *p) { p->split->failed = true; }
+void split_disable(dm_plan *p) { p->split->disabled = true; }
 
 // Column digits of one launch: those of every order, at most SPLIT_SCRATCH
 // bytes unless one order alone takes more.
@@ -767,7 +778,6 @@ void split_forget(dm_plan *p) {
   }
   T->dig = nullptr;
   T->full = false;
-  T->failed = false;
   T->slab.clear();
   drop_cuts(T);
 }
@@ -824,8 +834,8 @@ static cudaError_t split_setup(dm_plan *p, cudaStream_t st) {
     const int npt = (npairs + 127) / 128, nlt = (lmax + 128) / 128;
     const size_t nks = 2 * (size_t)nm * (npt + nlt);
     unsigned char *esc = nullptr, *tmp = nullptr;  // tmp: first multipoles, then K steps
-    if ((e = cudaMalloc(&esc, eb + sizeof(int) * (nm + 1)))) return e;
-    if ((e = cudaMalloc(&tmp, (sizeof(uint16_t) * n + 15) / 16 * 16 + sizeof(int) * nks))) {
+    if ((e = table_alloc(p, (void **)&esc, eb + sizeof(int) * (nm + 1)))) return e;
+    if ((e = table_alloc(p, (void **)&tmp, (sizeof(uint16_t) * n + 15) / 16 * 16 + sizeof(int) * nks))) {
       cudaFree(esc);
       return e;
     }
@@ -860,10 +870,7 @@ static cudaError_t split_setup(dm_plan *p, cudaStream_t st) {
   if (!T->x) {
     const size_t xb = (split_scratch_bytes(lmax, npairs, T->batch) + 127) / 128 * 128;
     const size_t all = xb + sizeof(int) * 2 * (size_t)nm * T->batch;
-    if ((e = cudaMalloc(&T->x, all))) {
-      T->x = nullptr;
-      return e;
-    }
+    if ((e = table_alloc(p, (void **)&T->x, all))) return e;
     T->xexp = reinterpret_cast<int *>(T->x + xb);
     T->bytes += (int64_t)all;
   }
@@ -884,10 +891,8 @@ static cudaError_t split_setup(dm_plan *p, cudaStream_t st) {
       }
       T->slab.push_back(nm);
       T->rows_cap = most;
-      e = cudaMalloc(&T->dig, row_bytes * (size_t)most);
-      if (e == cudaErrorMemoryAllocation) cudaGetLastError();
-      if (!e) break;
-      T->dig = nullptr;
+      e = table_alloc(p, (void **)&T->dig, row_bytes * (size_t)most);
+      if (e != cudaErrorMemoryAllocation) break;
     }
     if (e) return e;
     T->bytes += (int64_t)(row_bytes * (size_t)T->rows_cap);
@@ -991,24 +996,30 @@ static const SplitLaunches *split_find(const dm_plan *p, int S) {
 // The launches of the plan's batch when the split products can run: the
 // tables exist or can be made now; else null (tables that do not fit, a
 // stream under capture, where nothing can be allocated).
-static const SplitLaunches *split_ready(dm_plan *p, int S, cudaStream_t st) {
+static cudaError_t split_ready(dm_plan *p, int S, cudaStream_t st, const SplitLaunches **out) {
   SplitTables *T = p->split;
-  if (!T || T->failed) return nullptr;
-  if (const SplitLaunches *c = split_find(p, S)) return c;
+  *out = nullptr;
+  if (!T || T->disabled) return cudaSuccess;
+  if ((*out = split_find(p, S))) return cudaSuccess;
   cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
   if (cudaStreamIsCapturing(st, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone) {
     cudaGetLastError();
-    return nullptr;
+    return cudaSuccess;
   }
+  if (T->shortage.lasts(p)) return cudaSuccess;
+  const bool fresh = T->cuts.empty();
   cudaError_t e = split_setup(p, st);
   if (!e) e = split_cut(p, S, st);
   if (e) {
+    if (fresh) drop_tables(T);  // no launch has named them yet
     cudaGetLastError();
-    split_forget(p);
-    T->failed = true;
-    return nullptr;
+    if (e == cudaErrorNotSupported) T->disabled = true;
+    if (e == cudaErrorMemoryAllocation) T->shortage.note(p);
+    return e == cudaErrorMemoryAllocation || e == cudaErrorNotSupported ? cudaSuccess : e;
   }
-  return split_find(p, S);
+  T->shortage = Shortage();
+  *out = split_find(p, S);
+  return cudaSuccess;
 }
 
 template <bool SYN, int S, typename C2>
@@ -1097,26 +1108,32 @@ static cudaError_t split_run(dm_plan *p, const SplitLaunches &C, const C2 *in, v
 // FP64-class synthesis of alm into p->rc; *ran = false when the direct
 // kernels have to do it.
 cudaError_t split_synthesis64(dm_plan *p, const double2 *alm, cudaStream_t st, bool *ran) {
-  const SplitLaunches *c = split_ready(p, 6, st);
+  const SplitLaunches *c = nullptr;
+  const cudaError_t e = split_ready(p, 6, st, &c);
   *ran = c != nullptr;
+  if (e) return e;
   return c ? split_run<true, 6>(p, *c, alm, p->rc, 0, st) : cudaSuccess;
 }
 // FP64-class analysis of p->rc into slot 0 of p->apart
 cudaError_t split_analysis64(dm_plan *p, cudaStream_t st, bool *ran) {
-  const SplitLaunches *c = split_ready(p, 6, st);
+  const SplitLaunches *c = nullptr;
+  const cudaError_t e = split_ready(p, 6, st, &c);
   *ran = c != nullptr;
+  if (e) return e;
   return c ? split_run<false, 6>(p, *c, p->rc, p->apart, (int64_t)p->nslot * 3 * p->nalm, st) : cudaSuccess;
 }
 
 // The mixed mode's stages for batches outside the BF16 kernels: of the FP32
 // state e32 (or of alm) into p->rc32, and of p->rc32 into p->apart32.
 cudaError_t split_synthesis32(dm_plan *p, const double2 *alm, const float2 *e32, cudaStream_t st) {
-  const SplitLaunches *c = split_ready(p, 3, st);
+  const SplitLaunches *c = nullptr;
+  if (const cudaError_t e = split_ready(p, 3, st, &c)) return e;
   if (!c) return cudaErrorMemoryAllocation;
   return e32 ? split_run<true, 3>(p, *c, e32, p->rc32, 0, st) : split_run<true, 3>(p, *c, alm, p->rc32, 0, st);
 }
 cudaError_t split_analysis32(dm_plan *p, cudaStream_t st) {
-  const SplitLaunches *c = split_ready(p, 3, st);
+  const SplitLaunches *c = nullptr;
+  if (const cudaError_t e = split_ready(p, 3, st, &c)) return e;
   if (!c) return cudaErrorMemoryAllocation;
   return split_run<false, 3>(p, *c, p->rc32, p->apart32, 3 * p->nalm, st);
 }
