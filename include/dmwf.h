@@ -241,8 +241,10 @@ dm_status dm_set_anchor_precision(dm_plan *plan, dm_precision prec);
  * batch of 8, 16, 32 or 64 RHS the contractions over l and over ring pairs
  * run as tcgen05 GEMMs with BF16 hi/lo split operands and FP32 accumulation
  * (three products per K step); other batches use FP32 kernels
- * (small plans; the analysis of one or two RHS) or products of 27-bit operands'
- * digits, exactly summed.
+ * (small plans; the analysis of one or two RHS; wherever the digit tables are
+ * not kept whole, see dm_set_ff_slab_bytes) or products of 27-bit operands'
+ * digits.  0: the FP32 kernels for every batch, where their tables (12 bytes
+ * per multipole, order and ring pair) fit; the FP64-class anchors run as ever.
  * A pipeline wait that gives up (after 1 s) makes the solve calls return
  * DM_ETIMEOUT; the single-stage calls (dm_alm2map, dm_legendre_synthesis, ...)
  * return without synchronising and do not check it.  Each solve starts with
@@ -270,8 +272,10 @@ dm_status dm_set_tc_tiles(dm_plan *plan, int generate);
  * the mixed mode's anchors: each stage call generates the tables of one slab
  * of orders m (FP64 recurrence) and contracts it before the next.  bytes: the
  * largest slab (default 1 GiB; at least one order m is always taken).  By
- * default a plan keeps the full tables instead when they take at most 24 GiB;
- * after this call it never does.  Takes effect at the next stage call and
+ * default a plan keeps the full tables instead when they take at most 48 GiB;
+ * after this call it never does.  Without the full tables one right-hand side
+ * alone runs the FP64 recurrence kernels, and the mixed mode's batches outside
+ * 8, 16, 32 and 64 FP32 kernels, where their tables fit.  Takes effect at the next stage call and
  * frees the tables made so far (a CUDA graph that recorded a stage call of the
  * plan must not be replayed after it); DM_EINVAL for a null
  * plan or bytes < 1, DM_EBUSY during a solve session. */

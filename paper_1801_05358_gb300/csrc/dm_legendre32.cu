@@ -1,7 +1,7 @@
 // dm_legendre32.cu -- the mixed mode's Legendre stages on the FP32 pipe, from
 // FP32 tables (12 bytes per multipole, order and ring pair for lambda, lam+
-// and lam-): the synthesis of small plans, and the analysis of small plans and
-// of one or two right-hand sides.
+// and lam-): the synthesis of small plans, the analysis of small plans and of
+// one or two right-hand sides, and both wherever no digit table is kept whole.
 //
 // With few columns the tables are the work, read once.  The split products
 // (dm_split.cu) read 18 bytes per triple for any number of columns up to 32,
@@ -113,8 +113,9 @@ constexpr int A32_LB = 128;    // multipoles per block
 // Analysis: each warp takes four multipoles and all ring pairs, 16 bytes per
 // lane, function and multipole (12 loads in flight); values below
 // 2^TC_FLOOR_EXP (the evanescent region) are not read.  At nside 256, one
-// right-hand side: 105 us, split products 203.  grid (blocks of A32_LB
-// multipoles, orders, batch / NB); dynamic shared memory [NB][12][ldp]:
+// right-hand side: 105 us, split products 203.  grid (batch / NB, blocks of
+// A32_LB multipoles, orders): blocks that read the same values run together and
+// find them in L2; dynamic shared memory [NB][12][ldp]:
 // (T, Q, U) x (even re, im, odd re, im) of every ring pair.
 template <int NB>
 __global__ void __launch_bounds__(32 * A32_WARPS) k_ana32(const float *__restrict__ tab, int ldt,
@@ -124,9 +125,9 @@ __global__ void __launch_bounds__(32 * A32_WARPS) k_ana32(const float *__restric
                                                           int64_t nalm, int ldp,
                                                           const SolveState *__restrict__ state) {
   extern __shared__ __align__(16) float G[];
-  const int m = blockIdx.y, lb = blockIdx.x * A32_LB;  // l - m of the block's first multipole
+  const int m = blockIdx.z, lb = blockIdx.y * A32_LB;  // l - m of the block's first multipole
   if (lb > lmax - m) return;
-  const int b0 = blockIdx.z * NB;
+  const int b0 = blockIdx.x * NB;
   rc += (int64_t)b0 * 3 * (mmax + 1) * npairs * 2;
   out += (int64_t)b0 * 3 * nalm;
   if (state != nullptr) state += b0;
@@ -218,18 +219,31 @@ __global__ void __launch_bounds__(32 * A32_WARPS) k_ana32(const float *__restric
 int table_ld(const dm_plan *p) { return (p->npairs + 3) & ~3; }  // 16-byte rows
 int64_t order_entries(const dm_plan *p) { return (int64_t)p->npairs * (p->lmax + 1); }
 
+// The FP32 kernels take every size and batch where the split products would
+// have to make their digits again in each stage call (no whole table), and when
+// the tensor cores are turned off.  An iteration at nside 1024 / lmax 2048, one
+// and three right-hand sides: 14.5 and 28.5 ms here, 425 and 426 with slabs of
+// digits; at nside 512 / lmax 1535 with seven, slabs 103, whole digits 8.6.
+bool instead(const dm_plan *p) { return !p->use_tc || !split_whole(p); }
+
 // The FP32 tables, made on first use: not while the stream is captured, on a
-// plan that shares another's tables, or beyond 8 GiB.
+// plan that shares another's tables, or where they leave no room for the
+// anchors' digits (a slab at least).
 bool tables(dm_plan *p, cudaStream_t st) {
   if (p->tab32) return true;
   const double bytes = 12.0 * (double)p->nalm * table_ld(p);
   cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
-  if (bytes > 8.0 * (1u << 30) || p->is_view || cudaStreamIsCapturing(st, &cs) != cudaSuccess ||
-      cs != cudaStreamCaptureStatusNone) {
+  if (p->is_view || cudaStreamIsCapturing(st, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone) {
     cudaGetLastError();
     return false;
   }
   if (p->tab32_short.lasts(p)) return false;
+  const double digits = std::min((double)p->ffs_cap, (double)split_table_bytes(p->lmax, p->mmax, p->npairs)) +
+                        (double)split_scratch_bytes(p->lmax, p->npairs, p->batch);
+  if (bytes + digits > (double)table_room(p)) {
+    p->tab32_short.note(p);
+    return false;
+  }
   float *t = nullptr;
   int *ks = nullptr;
   cudaError_t e = table_alloc(p, (void **)&t, (size_t)bytes);
@@ -248,17 +262,20 @@ bool tables(dm_plan *p, cudaStream_t st) {
   return true;
 }
 
+constexpr size_t ANA32_SMEM = 220u << 10;
 size_t ana32_smem(const dm_plan *p, int nb) {
   return sizeof(float) * 12 * (size_t)((p->npairs + 127) / 128 * 128) * nb;
 }
 
 }  // namespace
 
-bool syn32_ready(dm_plan *p, cudaStream_t st) { return order_entries(p) < SYN32_MAX && tables(p, st); }
+bool syn32_ready(dm_plan *p, cudaStream_t st) {
+  return (order_entries(p) < SYN32_MAX || instead(p)) && tables(p, st);
+}
 
 bool ana32_ready(dm_plan *p, cudaStream_t st) {
-  if (p->batch > 2 && order_entries(p) >= ANA32_MAX) return false;
-  return ana32_smem(p, 2) <= (220u << 10) && tables(p, st);
+  if (p->batch > 2 && order_entries(p) >= ANA32_MAX && !instead(p)) return false;
+  return ana32_smem(p, 1) <= ANA32_SMEM && tables(p, st);
 }
 
 cudaError_t syn32(dm_plan *p, const double2 *alm, const float2 *e32, cudaStream_t st) {
@@ -275,11 +292,12 @@ cudaError_t syn32(dm_plan *p, const double2 *alm, const float2 *e32, cudaStream_
 
 cudaError_t ana32(dm_plan *p, cudaStream_t st) {
   const SolveState *state = p->state_active ? p->state : nullptr;
-  const int npt = (p->npairs + 127) / 128, nlt = (p->lmax + 128) / 128, nb = p->batch % 2 ? 1 : 2;
+  const int npt = (p->npairs + 127) / 128, nlt = (p->lmax + 128) / 128;
+  const int nb = p->batch % 2 || ana32_smem(p, 2) > ANA32_SMEM ? 1 : 2;
   auto go = [&](auto kern) {
     const size_t sm = ana32_smem(p, nb);
     if (cudaError_t e = dyn_smem_allow(kern, sm)) return e;
-    kern<<<dim3((p->lmax + A32_LB) / A32_LB, p->mmax + 1, p->batch / nb), 32 * A32_WARPS, sm, st>>>(
+    kern<<<dim3(p->batch / nb, (p->lmax + A32_LB) / A32_LB, p->mmax + 1), 32 * A32_WARPS, sm, st>>>(
         p->tab32, table_ld(p), p->tc_ks, npt, nlt, p->rc32, p->apart32, p->lmax, p->mmax, p->npairs, p->nalm,
         npt * 128, state);
     return cudaGetLastError();

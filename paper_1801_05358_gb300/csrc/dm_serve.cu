@@ -306,6 +306,11 @@ Pool *make_pool(dm_server *S, const Request &r, dm_status *why) {
     *why = rs;
     return nullptr;
   }
+  // the views that set the slots up make no FP32 tables of their own
+  if (prec == DM_MIXED_FP32 && !tc_batch_ok(slots) && !split_whole(p)) {
+    syn32_ready(p, 0);
+    cudaDeviceSynchronize();
+  }
   p->anchor_every = S->cfg.anchor_every > 0 ? S->cfg.anchor_every : 256;
   // Pools run their rounds concurrently; the strict-precision pools, whose
   // requests are the long ones, take the higher stream priority so that the

@@ -211,9 +211,15 @@ __global__ void __launch_bounds__(128) k_split_gen(const PairDev *__restrict__ p
                                                    const int *__restrict__ seed_exp,
                                                    const int16_t *__restrict__ esc, unsigned char *__restrict__ dig,
                                                    int lmax, int mmax, int npairs, int npoct, int m0, int row0,
-                                                   const int *__restrict__ roff, int64_t rows_cap) {
+                                                   const int *__restrict__ roff, int64_t rows_cap,
+                                                   const SolveState *__restrict__ state, int batch) {
   extern __shared__ __align__(16) unsigned char stage[];
   __shared__ RecCoef sc[64];
+  if (state != nullptr) {  // a slab for right-hand sides of which none goes on
+    int live = 0;
+    for (int b = threadIdx.x; b < batch; b += 128) live |= !state[b].done;
+    if (!__syncthreads_or(live)) return;
+  }
   const int m = m0 + blockIdx.y, t = threadIdx.x, p = blockIdx.x * 128 + t;
   const bool act = p < npairs;
   const int pp = act ? p : npairs - 1;
@@ -722,6 +728,13 @@ size_t split_table_bytes(int lmax, int mmax, int npairs) {
   return (size_t)(rows * 3 * SPLIT_S * 128.0 * ((npairs + 7) / 8));
 }
 
+bool split_whole(const dm_plan *p) {
+  const SplitTables *T = p->split;
+  if (!T || T->disabled) return false;
+  if (T->dig) return T->full;
+  return !p->ffs_cap_set && split_table_bytes(p->lmax, p->mmax, p->npairs) <= (size_t)p->split_cap;
+}
+
 static void drop_cuts(SplitTables *T) {
   for (SplitLaunches &c : T->cuts)
     for (SplitTile *t : c.tiles)
@@ -913,7 +926,7 @@ static cudaError_t split_setup(dm_plan *p, cudaStream_t st) {
       if ((e = dyn_smem_allow(k_split_gen, GEN_STAGE))) return e;
       k_split_gen<<<dim3((npairs + 127) / 128, nm), 128, GEN_STAGE, st>>>(
           p->pairs, p->rec, p->seed, p->seed_exp, T->esc, T->dig, lmax, p->mmax, npairs, T->npoct, 0, 0,
-          T->roff_dev, T->rows_cap);
+          T->roff_dev, T->rows_cap, nullptr, 0);
       if ((e = cudaGetLastError())) return e;
       T->full = true;
     }
@@ -1044,7 +1057,7 @@ static cudaError_t split_run(dm_plan *p, const SplitLaunches &C, const C2 *in, v
         if ((e = dyn_smem_allow(k_split_gen, GEN_STAGE))) return e;
         k_split_gen<<<dim3((p->npairs + 127) / 128, T->slab[s + 1] - T->slab[s]), 128, GEN_STAGE, st>>>(
             p->pairs, p->rec, p->seed, p->seed_exp, T->esc, T->dig, p->lmax, p->mmax, p->npairs, T->npoct, T->slab[s],
-            T->roff[T->slab[s]], T->roff_dev, T->rows_cap);
+            T->roff[T->slab[s]], T->roff_dev, T->rows_cap, state, p->batch);
         slab_made = s;
       }
     }
@@ -1105,11 +1118,17 @@ static cudaError_t split_run(dm_plan *p, const SplitLaunches &C, const C2 *in, v
   return cudaSuccess;
 }
 
+// The digits of a slab are made in each stage call, for any number of
+// right-hand sides; the direct kernels run their recurrence once for each.  One
+// iteration, slabs and direct kernels: nside 512 / lmax 1535, one right-hand
+// side 109 and 100 ms, two 110 and 200; nside 1024 / lmax 2048, one 460 and 351.
+static bool direct64(const dm_plan *p) { return p->batch == 1 && !split_whole(p); }
+
 // FP64-class synthesis of alm into p->rc; *ran = false when the direct
 // kernels have to do it.
 cudaError_t split_synthesis64(dm_plan *p, const double2 *alm, cudaStream_t st, bool *ran) {
   const SplitLaunches *c = nullptr;
-  const cudaError_t e = split_ready(p, 6, st, &c);
+  const cudaError_t e = direct64(p) ? cudaSuccess : split_ready(p, 6, st, &c);
   *ran = c != nullptr;
   if (e) return e;
   return c ? split_run<true, 6>(p, *c, alm, p->rc, 0, st) : cudaSuccess;
@@ -1117,7 +1136,7 @@ cudaError_t split_synthesis64(dm_plan *p, const double2 *alm, cudaStream_t st, b
 // FP64-class analysis of p->rc into slot 0 of p->apart
 cudaError_t split_analysis64(dm_plan *p, cudaStream_t st, bool *ran) {
   const SplitLaunches *c = nullptr;
-  const cudaError_t e = split_ready(p, 6, st, &c);
+  const cudaError_t e = direct64(p) ? cudaSuccess : split_ready(p, 6, st, &c);
   *ran = c != nullptr;
   if (e) return e;
   return c ? split_run<false, 6>(p, *c, p->rc, p->apart, (int64_t)p->nslot * 3 * p->nalm, st) : cudaSuccess;
