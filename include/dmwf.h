@@ -75,6 +75,14 @@ typedef enum {
  * DM_FLOAT_FLOAT: FP64-class results (relative error of 1e-13 or less per
  *   transform); runs the same digit products as DM_FP64.  Not in the paper
  *   (an arithmetic choice). */
+/* The tensor-core kernels of every mode wait for their copies and products
+ * with a limit.  A wait that gives up (after 1 s) leaves results unwritten: the
+ * calls that synchronise (the solve calls, constrained realisations and
+ * refinements with their diagnostics, dm_draw_cr_inputs) then return
+ * DM_ETIMEOUT, and the server ends the requests of the pool with it.  The
+ * single-stage calls (dm_alm2map, dm_map2alm, dm_legendre_synthesis, ...)
+ * return without synchronising and do not check.  Each checking call starts
+ * with the flag cleared. */
 typedef enum { DM_FP64 = 0, DM_MIXED_FP32 = 1, DM_FLOAT_FLOAT = 2 } dm_precision;
 
 /* Cooling and stopping schedule of Algorithm 1 (Section 3.2).
@@ -245,10 +253,8 @@ dm_status dm_set_anchor_precision(dm_plan *plan, dm_precision prec);
  * not kept whole, see dm_set_ff_slab_bytes) or products of 27-bit operands'
  * digits.  0: the FP32 kernels for every batch, where their tables (12 bytes
  * per multipole, order and ring pair) fit; the FP64-class anchors run as ever.
- * A pipeline wait that gives up (after 1 s) makes the solve calls return
- * DM_ETIMEOUT; the single-stage calls (dm_alm2map, dm_legendre_synthesis, ...)
- * return without synchronising and do not check it.  Each solve starts with
- * the flag cleared. */
+ * A pipeline wait that gives up (after 1 s; see dm_precision) makes the solve
+ * calls return DM_ETIMEOUT. */
 dm_status dm_set_tensor_cores(dm_plan *plan, int on);
 
 /* Source of the tensor cores' Legendre operand (default -1: stored tiles when
@@ -533,6 +539,10 @@ dm_status dm_set_noise_flat(dm_plan *plan, const double *sigma, const uint8_t *m
  * the next solve is normal.  Not for production use. */
 dm_status dm_test_tc_withhold(dm_plan *plan, int on);
 
+/* Failure test of the reports of waits that gave up: the plan's flag is set,
+ * in stream order, as a kernel whose wait gave up would set it. */
+dm_status dm_test_wait_flag(dm_plan *plan, void *stream);
+
 /* Failure test of the tables made on first use (Legendre digits, DFT
  * matrices, FP32 Legendre values): from now on an allocation of more than
  * `bytes` for them reports that the device has no memory (-1: the device
@@ -582,7 +592,8 @@ typedef struct {
 } dm_request;
 
 typedef struct {
-  dm_status status;          /* DM_OK, DM_ENOTCONV, DM_ENOMEM (never fits), DM_EAGAIN (cancelled), ... */
+  dm_status status;          /* DM_OK, DM_ENOTCONV, DM_ENOMEM (never fits), DM_EAGAIN (cancelled), DM_ETIMEOUT (a kernel's
+                                wait gave up), ... */
   int iters;                 /* dual messenger iterations run */
   double cauchy_final;
   double latency_ms;         /* submit to completion (host wall clock) */
@@ -607,6 +618,9 @@ dm_status dm_serve_poll(dm_server *srv, uint64_t ticket, dm_result *out);
  * DM_EBUSY once admitted. */
 dm_status dm_serve_cancel(dm_server *srv, uint64_t ticket);
 dm_status dm_server_info(dm_server *srv, dm_server_info_t *out);
+/* Failure test: the next round (where = 1) or the next retirement of a request
+ * (2) finds its pool's wait flag set, as by a kernel whose wait gave up. */
+dm_status dm_test_server_wait_flag(dm_server *srv, int where);
 /* Completes every queued and running request, then frees the pools. */
 void dm_server_destroy(dm_server *srv);
 

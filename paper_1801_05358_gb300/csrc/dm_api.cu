@@ -241,9 +241,21 @@ dm_status anchor(dm_plan *p, cudaStream_t st, bool initial, const double *d, boo
   return DM_OK;
 }
 
+// The flag of the bounded tensor-core waits: cleared where a call that checks
+// it begins (a wait that gave up earlier does not count against that call),
+// read once the call's last kernel is enqueued.
+dm_status clear_waits(dm_plan *p, cudaStream_t st) {
+  DM_CU(cudaMemsetAsync(p->tc_err, 0, sizeof(int), st), "clear wait flag");
+  return DM_OK;
+}
+dm_status check_waits(dm_plan *p, cudaStream_t st) {
+  int gave_up = 0;
+  DM_CU(cudaMemcpyAsync(&gave_up, p->tc_err, sizeof(int), cudaMemcpyDeviceToHost, st), "wait flag");
+  DM_CU(cudaStreamSynchronize(st), "wait flag");
+  return gave_up ? fail(p, DM_ETIMEOUT, "a tensor-core pipeline wait gave up") : DM_OK;
+}
+
 dm_status solve_begin(dm_plan *p, const double *d, cudaStream_t st) {
-  // a tensor-core wait that gave up in an earlier solve does not count against this one
-  if (p->tc_err) DM_CU(cudaMemsetAsync(p->tc_err, 0, sizeof(int), st), "clear wait flag");
   DM_CU(cudaMemsetAsync(p->a, 0, sizeof(double2) * 3 * p->nalm * p->batch, st), "zero a");
   DM_CU(p->cov ? cov_prepare_wd(p, d, st) : prepare_wd(p, d, st), "w d");
   DM_CU(control_init(p, st), "control init");
@@ -289,7 +301,7 @@ dm_status solve_iterate(dm_plan *p, long max_iters, int *all_done, cudaStream_t 
     p->since_anchor += (int)window;
     cudaError_t e = cudaMemcpyAsync(hs.data(), p->state, sizeof(SolveState) * p->batch, cudaMemcpyDeviceToHost, st);
     int tcerr = 0;
-    if (!e && p->tc_err) e = cudaMemcpyAsync(&tcerr, p->tc_err, sizeof(int), cudaMemcpyDeviceToHost, st);
+    if (!e) e = cudaMemcpyAsync(&tcerr, p->tc_err, sizeof(int), cudaMemcpyDeviceToHost, st);
     if (!e) e = cudaStreamSynchronize(st);
     if (e) return cuda_fail(p, e, "poll state");
     if (tcerr) return fail(p, DM_ETIMEOUT, "a tensor-core pipeline wait gave up");
@@ -382,7 +394,8 @@ namespace {
 
 // Stats of every RHS after a solve (the stream is synchronised): counts,
 // Cauchy value, the FP64 diagnostics when enabled and ms_total from the
-// solve's begin and end events.
+// solve's begin and end events; *rs becomes DM_ETIMEOUT when a wait gave up in
+// the solve, its last synthesis or the diagnostics.
 void fill_stats(dm_plan *p, dm_stats *stats, dm_status *rs, cudaStream_t st) {
   std::vector<SolveState> hs(p->batch);
   cudaMemcpy(hs.data(), p->state, sizeof(SolveState) * p->batch, cudaMemcpyDeviceToHost);
@@ -419,6 +432,10 @@ void fill_stats(dm_plan *p, dm_stats *stats, dm_status *rs, cudaStream_t st) {
     }
   }
   if (notconv && *rs == DM_OK) *rs = fail(p, DM_ENOTCONV, "max_iter reached before the last level converged");
+  if (*rs == DM_OK || *rs == DM_ENOTCONV) {
+    const dm_status w = check_waits(p, st);
+    if (w != DM_OK) *rs = w;
+  }
 }
 
 }  // namespace
@@ -695,6 +712,7 @@ dm_status dm_wiener_filter(dm_plan *p, const double *d, double *s_out, double *a
   if (!d || !s_out) return fail(p, DM_EINVAL, "null buffer");
   cudaStream_t st = (cudaStream_t)stream;
   DM_CU(cudaEventRecord(p->ev_begin, st), "event");
+  if ((r = clear_waits(p, st)) != DM_OK) return r;
   r = run_dm(p, d, st);
   if (r != DM_OK && r != DM_ENOTCONV) return r;
   dm_status r2 = solve_end(p, s_out, alm_out, st, false);
@@ -713,6 +731,7 @@ dm_status dm_wiener_filter_host(dm_plan *p, const double *d_host, double *s_host
   cudaStream_t st = (cudaStream_t)stream;
   const size_t mb = sizeof(double) * 3 * p->npix * p->batch;
   DM_CU(cudaEventRecord(p->ev_begin, st), "event");
+  if ((r = clear_waits(p, st)) != DM_OK) return r;
   // tmpmap2 holds d
   DM_CU(cudaMemcpyAsync(p->tmpmap2, d_host, mb, cudaMemcpyHostToDevice, st), "h2d");
   r = run_dm(p, p->tmpmap2, st);
@@ -730,6 +749,8 @@ dm_status dm_draw_cr_inputs(dm_plan *p, const uint64_t *seeds, double *ahat, dou
   if (!p || !seeds) return DM_EINVAL;
   if (!p->have_cl || !p->have_noise) return fail(p, DM_EINVAL, "spectra and noise must be set");
   cudaStream_t st = (cudaStream_t)stream;
+  if (!p->session)  // (a solve in progress keeps what its own kernels reported)
+    if (const dm_status r = clear_waits(p, st)) return r;
   DM_CU(cudaMemcpyAsync(p->seeds_dev, seeds, sizeof(uint64_t) * p->batch, cudaMemcpyHostToDevice, st), "seeds");
   DM_CU(p->flat ? flat_draw_signal(p, p->seeds_dev, p->tmpalm, st) : draw_signal(p, p->seeds_dev, p->tmpalm, st),
         "draw signal");
@@ -741,8 +762,7 @@ dm_status dm_draw_cr_inputs(dm_plan *p, const uint64_t *seeds, double *ahat, dou
   if (ahat)
     DM_CU(cudaMemcpyAsync(ahat, p->tmpalm, sizeof(double2) * 3 * p->nalm * p->batch, cudaMemcpyDeviceToDevice, st),
           "copy ahat");
-  DM_CU(cudaStreamSynchronize(st), "sync");
-  return DM_OK;
+  return check_waits(p, st);
 }
 
 dm_status dm_constrained_realization(dm_plan *p, const double *d, const uint64_t *seeds, double *s_cr_out,
@@ -754,6 +774,7 @@ dm_status dm_constrained_realization(dm_plan *p, const double *d, const uint64_t
   const int64_t n = 3 * p->npix * p->batch;
   // shat -> tmpmap, ahat -> tmpalm, dhat -> tmpmap2, then tmpmap2 = d - dhat
   DM_CU(cudaEventRecord(p->ev_begin, st), "event");
+  if ((r = clear_waits(p, st)) != DM_OK) return r;
   DM_CU(cudaMemcpyAsync(p->seeds_dev, seeds, sizeof(uint64_t) * p->batch, cudaMemcpyHostToDevice, st), "seeds");
   DM_CU(p->flat ? flat_draw_signal(p, p->seeds_dev, p->tmpalm, st) : draw_signal(p, p->seeds_dev, p->tmpalm, st),
         "draw signal");
@@ -839,6 +860,7 @@ dm_status dm_solve_begin(dm_plan *p, const double *d, void *stream) {
   if (!d) return fail(p, DM_EINVAL, "null buffer");
   if (p->session) return fail(p, DM_EBUSY, "a solve is already in progress on this plan");
   DM_CU(cudaEventRecord(p->ev_begin, (cudaStream_t)stream), "event");
+  if ((r = clear_waits(p, (cudaStream_t)stream)) != DM_OK) return r;
   r = solve_begin(p, d, (cudaStream_t)stream);
   if (r != DM_OK) end_session(p);
   return r;
@@ -870,6 +892,7 @@ dm_status dm_jacobi_refine(dm_plan *p, const double *d, int n_refine, double *s_
   if (p->session) return fail(p, DM_EBUSY, "a solve is in progress on this plan");
   cudaStream_t st = (cudaStream_t)stream;
   DM_CU(cudaEventRecord(p->ev_begin, st), "event");
+  if ((r = clear_waits(p, st)) != DM_OK) return r;
   // the usual solve, whose per-level counts W~ then repeats
   r = run_dm(p, d, st);
   if (r != DM_OK && r != DM_ENOTCONV) return r;
@@ -954,6 +977,12 @@ dm_status dm_set_analysis_slots(dm_plan *p, int slots) {
 dm_status dm_test_table_memory(dm_plan *p, int64_t bytes) {
   if (!p) return DM_EINVAL;
   p->table_limit = bytes;
+  return DM_OK;
+}
+
+dm_status dm_test_wait_flag(dm_plan *p, void *stream) {
+  if (!p) return DM_EINVAL;
+  DM_CU(cudaMemsetAsync(p->tc_err, 1, sizeof(int), (cudaStream_t)stream), "wait flag");
   return DM_OK;
 }
 

@@ -417,6 +417,8 @@ inline cudaError_t chunk_waves(dm_plan *p, int m0, int m1, cudaStream_t st, F la
 
 // driver (dm_api.cu), shared with the server (dm_serve.cu)
 dm_status upload_levels(dm_plan *p);
+dm_status clear_waits(dm_plan *p, cudaStream_t st);
+dm_status check_waits(dm_plan *p, cudaStream_t st);
 cudaError_t enqueue_iteration(dm_plan *p, cudaStream_t st, cudaEvent_t *E);
 dm_status anchor(dm_plan *p, cudaStream_t st, bool initial, const double *d, bool need_g);
 dm_status solve_begin(dm_plan *p, const double *d, cudaStream_t st);

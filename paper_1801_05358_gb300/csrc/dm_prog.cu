@@ -125,7 +125,6 @@ __global__ void k_change_band(const double2 *__restrict__ in, double2 *__restric
 // The usual level loop from the iterate the plan holds in p->a (instead of
 // a = 0, t_0 = d): the first step is a <- F [a + A(w (d - Y a))].
 dm_status solve_begin_warm(dm_plan *p, const double *d, cudaStream_t st) {
-  if (p->tc_err && cudaMemsetAsync(p->tc_err, 0, sizeof(int), st)) return DM_ECUDA;
   if (prepare_wd(p, d, st) || control_init(p, st)) return DM_ECUDA;
   p->launches += 2;
   if (p->prec == DM_FP64) {
@@ -306,6 +305,7 @@ dm_status run_progressive(dm_plan *p, const double *d, cudaStream_t st) {
     // data at this resolution
     const double *dq = d;
     if (q != p) {
+      if ((r = clear_waits(q, st)) != DM_OK) break;
       const int64_t npk = q->npix;
       k_degrade<<<2048, 256, 0, st>>>(d, lp->child, lp->v, q->tmpmap2, p->npix, npk, lp->per, p->batch);
       if (cudaGetLastError()) {
@@ -324,6 +324,7 @@ dm_status run_progressive(dm_plan *p, const double *d, cudaStream_t st) {
     int all = 0;
     if (r == DM_OK) r = solve_iterate(q, s1.max_iter + 4, &all, st);
     if (r == DM_OK) r = solve_end(q, nullptr, nullptr, st, false);
+    if (r == DM_OK && q != p) r = check_waits(q, st);  // (the call that began the solve checks p)
     if (r != DM_OK) {
       q->session = q->state_active = q->anchor_active = false;
       break;

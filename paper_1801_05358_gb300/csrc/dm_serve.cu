@@ -63,6 +63,7 @@ struct Slot {
   bool busy = false;
   std::unique_ptr<Request> req;
   int since_anchor = 0;
+  bool begun = false;  // set up: kernels of its request have run
 };
 
 struct Pool {
@@ -73,9 +74,12 @@ struct Pool {
   size_t reserved = 0;          // bytes of the memory budget it holds
   cudaStream_t stream = nullptr;
   std::vector<Slot> slots;
-  // a round in flight: its iterations and the copy of the solver states into
-  // hs (pinned) are enqueued, done_ev is recorded after them
+  // a round in flight: its iterations and the copies of the solver states into
+  // hs and of the plan's wait flag into gave_up (pinned) are enqueued, done_ev
+  // is recorded after them
   bool inflight = false;
+  dm_status round_status = DM_OK;  // of enqueuing it
+  int *gave_up = nullptr;
   cudaEvent_t done_ev = nullptr;
   SolveState *hs = nullptr;
   int busy() const {
@@ -205,6 +209,7 @@ struct dm_server {
   std::thread worker;
   std::string err;
   std::atomic<int64_t> rounds{0}, admitted{0}, retired{0};  // written by the worker, read by dm_server_info
+  std::atomic<int> test_wait{0};  // test hook: where the next wait is to have given up (1: a round, 2: a retirement)
 };
 
 namespace {
@@ -229,6 +234,7 @@ dm_precision request_prec(const dm_server *S, const Request &r) {
 void release_pool(Pool *q) {
   if (q->done_ev) cudaEventDestroy(q->done_ev);
   if (q->hs) cudaFreeHost(q->hs);
+  if (q->gave_up) cudaFreeHost(q->gave_up);
   cudaStreamDestroy(q->stream);
   dm_plan_destroy(q->plan);
 }
@@ -324,8 +330,10 @@ Pool *make_pool(dm_server *S, const Request &r, dm_status *why) {
     return nullptr;
   }
   if (cudaEventCreateWithFlags(&pool->done_ev, cudaEventDisableTiming) != cudaSuccess ||
-      cudaMallocHost(&pool->hs, sizeof(SolveState) * slots) != cudaSuccess) {
+      cudaMallocHost(&pool->hs, sizeof(SolveState) * slots) != cudaSuccess ||
+      cudaMallocHost(&pool->gave_up, sizeof(int)) != cudaSuccess) {
     if (pool->done_ev) cudaEventDestroy(pool->done_ev);
+    if (pool->hs) cudaFreeHost(pool->hs);
     cudaStreamDestroy(pool->stream);
     dm_plan_destroy(p);
     *why = DM_ECUDA;
@@ -355,6 +363,21 @@ Pool *find_pool(dm_server *S, const Request &r, bool *full) {
       *full = true;
     }
   return nullptr;
+}
+
+// Test hook (dm_test_server_wait_flag): as if a wait of the pool's kernels had given up here.
+void test_wait(dm_server *S, Pool *pool) {
+  S->test_wait = 0;
+  cudaMemsetAsync(pool->plan->tc_err, 1, sizeof(int), pool->stream);
+}
+
+// The pool's wait flag after everything enqueued so far (synchronises): it is
+// the slots' common one, so that once set it fails every slot that has begun
+// (fail_slots), and only that clears it.
+dm_status pool_waits(Pool *pool) {
+  cudaMemcpyAsync(pool->gave_up, pool->plan->tc_err, sizeof(int), cudaMemcpyDeviceToHost, pool->stream);
+  if (cudaStreamSynchronize(pool->stream) != cudaSuccess) return DM_ECUDA;
+  return *pool->gave_up ? DM_ETIMEOUT : DM_OK;
 }
 
 // Set slot b up alone and run its first iteration (t_0 = d), then anchor.
@@ -399,6 +422,7 @@ dm_status slot_begin(Pool *pool, int b, Request &r) {
     cudaMemcpyAsync(v.tmpmap2, v.rhi, sizeof(double) * n3, cudaMemcpyDeviceToDevice, st);
     v.prec = pr;
   }
+  pool->slots[b].begun = true;
   dm_status rs = solve_begin(&v, v.tmpmap2, st);
   if (rs != DM_OK) return rs;
   if (enqueue_iteration(&v, st, nullptr) != cudaSuccess) return DM_ECUDA;
@@ -407,10 +431,29 @@ dm_status slot_begin(Pool *pool, int b, Request &r) {
     if (rs != DM_OK) return rs;
   }
   pool->slots[b].since_anchor = 0;
-  return cudaStreamSynchronize(st) == cudaSuccess ? DM_OK : DM_ECUDA;
+  return pool_waits(pool);
 }
 
-void slot_end(dm_server *S, Pool *pool, int b, const SolveState &ss) {
+void free_slot(dm_server *S, Pool *pool, int b) {
+  std::lock_guard<std::mutex> lk(S->mu);
+  pool->slots[b].busy = pool->slots[b].begun = false;
+  pool->slots[b].req.reset();
+}
+
+// Every slot that has begun ends with status rs; the plan's wait flag is cleared.
+void fail_slots(dm_server *S, Pool *pool, dm_status rs) {
+  for (int b = 0; b < (int)pool->slots.size(); ++b) {
+    if (!pool->slots[b].busy || !pool->slots[b].begun) continue;
+    finish(S, *pool->slots[b].req, rs, 0, 0.0);
+    k_mark_done<<<1, 1, 0, pool->stream>>>(pool->plan->state + b, 1);
+    free_slot(S, pool, b);
+  }
+  cudaMemsetAsync(pool->plan->tc_err, 0, sizeof(int), pool->stream);
+  *pool->gave_up = 0;
+  cudaStreamSynchronize(pool->stream);
+}
+
+dm_status slot_end(dm_server *S, Pool *pool, int b, const SolveState &ss) {
   dm_plan *p = pool->plan;
   cudaStream_t st = pool->stream;
   Request &r = *pool->slots[b].req;
@@ -419,13 +462,14 @@ void slot_end(dm_server *S, Pool *pool, int b, const SolveState &ss) {
   if (v.prec != DM_FP64) rs = anchor(&v, st, false, nullptr, false);  // s = Y a in FP64
   const int64_t n3 = 3 * p->npix;
   if (rs == DM_OK && r.kind == DM_REQ_CR) axpy_maps(n3, v.tmpmap, 1.0, v.s64, st);
+  if (S->test_wait == 2) test_wait(S, pool);
   if (rs == DM_OK) cudaMemcpyAsync(r.s_out, v.s64, sizeof(double) * n3, cudaMemcpyDeviceToHost, st);
-  if (cudaStreamSynchronize(st) != cudaSuccess) rs = DM_ECUDA;
+  const dm_status w = pool_waits(pool);
+  if (rs == DM_OK) rs = w;
   finish(S, r, rs != DM_OK ? rs : (ss.notconv ? DM_ENOTCONV : DM_OK), ss.iters_total, ss.cauchy);
-  std::lock_guard<std::mutex> lk(S->mu);
-  pool->slots[b].busy = false;
-  pool->slots[b].req.reset();
+  free_slot(S, pool, b);
   S->retired++;
+  return w;
 }
 
 void worker_main(dm_server *S) {
@@ -502,12 +546,12 @@ void worker_main(dm_server *S) {
       const int b = pb.second;
       dm_status rs = slot_begin(pool, b, *pool->slots[b].req);
       S->admitted++;
-      if (rs != DM_OK) {
+      if (rs == DM_ETIMEOUT) {
+        fail_slots(S, pool, rs);
+      } else if (rs != DM_OK) {
         finish(S, *pool->slots[b].req, rs, 0, 0.0);
         k_mark_done<<<1, 1, 0, pool->stream>>>(pool->plan->state + b, 1);
-        std::lock_guard<std::mutex> lk(S->mu);
-        pool->slots[b].busy = false;
-        pool->slots[b].req.reset();
+        free_slot(S, pool, b);
       }
     }
     // ---- rounds: every pool with busy slots and no round in flight starts
@@ -517,9 +561,15 @@ void worker_main(dm_server *S) {
     for (auto &qq : S->pools) {
       Pool *q = qq.get();
       if (q->inflight || q->busy() == 0) continue;
-      for (int k = 0; k < N; ++k) enqueue_iteration(q->plan, q->stream, nullptr);
+      q->round_status = DM_OK;
+      for (int k = 0; k < N && q->round_status == DM_OK; ++k) {
+        const cudaError_t e = enqueue_iteration(q->plan, q->stream, nullptr);
+        if (e) q->round_status = e == cudaErrorMemoryAllocation ? DM_ENOMEM : DM_ECUDA;
+      }
+      if (S->test_wait == 1) test_wait(S, q);
       cudaMemcpyAsync(q->hs, q->plan->state, sizeof(SolveState) * q->slots.size(), cudaMemcpyDeviceToHost,
                       q->stream);
+      cudaMemcpyAsync(q->gave_up, q->plan->tc_err, sizeof(int), cudaMemcpyDeviceToHost, q->stream);
       cudaEventRecord(q->done_ev, q->stream);
       q->inflight = true;
     }
@@ -530,17 +580,29 @@ void worker_main(dm_server *S) {
       q->inflight = false;
       progressed = true;
       S->rounds++;
+      if (q->round_status != DM_OK || *q->gave_up) {
+        fail_slots(S, q, q->round_status != DM_OK ? q->round_status : DM_ETIMEOUT);
+        continue;
+      }
       for (int b = 0; b < (int)q->slots.size(); ++b) {
         Slot &sl = q->slots[b];
         if (!sl.busy) continue;
         if (q->hs[b].done) {
-          slot_end(S, q, b, q->hs[b]);
+          const dm_status w = slot_end(S, q, b, q->hs[b]);
+          if (w != DM_OK) {
+            fail_slots(S, q, w);
+            break;
+          }
           continue;
         }
         sl.since_anchor += N;
         if (q->plan->prec != DM_FP64 && sl.since_anchor >= q->plan->anchor_every) {
           dm_plan v = make_view(q->plan, b);
-          anchor(&v, q->stream, false, nullptr, true);
+          const dm_status w = anchor(&v, q->stream, false, nullptr, true);
+          if (w != DM_OK) {
+            fail_slots(S, q, w);
+            break;
+          }
           sl.since_anchor = 0;
         }
       }
@@ -648,6 +710,12 @@ dm_status dm_server_info(dm_server *S, dm_server_info_t *out) {
   out->rounds = S->rounds.load();
   out->admitted = S->admitted.load();
   out->retired = S->retired.load();
+  return DM_OK;
+}
+
+dm_status dm_test_server_wait_flag(dm_server *S, int where) {
+  if (!S || where < 0 || where > 2) return DM_EINVAL;
+  S->test_wait = where;
   return DM_OK;
 }
 

@@ -29,7 +29,7 @@ EXPORTS = [
     "dm_serve_poll", "dm_serve_cancel", "dm_server_info", "dm_server_destroy", "dm_set_tensor_cores", "dm_set_tc_tiles", "dm_set_ff_slab_bytes", "dm_set_analysis_slots", "dm_set_ring_radix",
     "dm_set_anchor_precision", "dm_set_noise_cov",
     "dm_legendre_analysis_noalloc", "dm_set_diagnostics", "dm_autotune", "dm_get_tuning", "dm_set_tuning",
-    "dm_jacobi_refine", "dm_test_tc_withhold", "dm_test_table_memory", "dm_plan_create_flat", "dm_set_spectra_flat", "dm_set_noise_flat",
+    "dm_jacobi_refine", "dm_test_tc_withhold", "dm_test_table_memory", "dm_test_wait_flag", "dm_test_server_wait_flag", "dm_plan_create_flat", "dm_set_spectra_flat", "dm_set_noise_flat",
     "dm_set_progressive", "dm_get_progressive_levels",
 ]
 DM_REQ_WF, DM_REQ_CR = 0, 1
@@ -144,6 +144,8 @@ def lib():
         L.dm_autotune.argtypes = [vp, ctypes.c_int, vp]
         L.dm_jacobi_refine.argtypes = [vp, vp, ctypes.c_int, vp, vp, vp, vp]
         L.dm_test_tc_withhold.argtypes = [vp, ctypes.c_int]
+        L.dm_test_wait_flag.argtypes = [vp, vp]
+        L.dm_test_server_wait_flag.argtypes = [vp, ctypes.c_int]
         L.dm_test_table_memory.argtypes = [vp, ctypes.c_int64]
         L.dm_set_progressive.argtypes = [vp, ctypes.c_double, ctypes.c_int]
         L.dm_get_progressive_levels.argtypes = [vp, vp, vp]
@@ -304,6 +306,10 @@ class Plan:
     def test_tc_withhold(self, on=True):
         """Failure-test hook: one withheld mbarrier arrival in the tensor-core analysis."""
         self._check(lib().dm_test_tc_withhold(self.h, 1 if on else 0))
+
+    def test_wait_flag(self, stream=None):
+        """Failure-test hook: as if a kernel of the plan had given up a wait."""
+        self._check(lib().dm_test_wait_flag(self.h, _stream(stream)))
 
     def test_table_memory(self, limit=-1):
         """Failure-test hook: tables of more than `limit` bytes find no memory (-1: the device decides)."""
@@ -491,6 +497,10 @@ class Server:
         out = self._live.pop(ticket)
         return dict(status=r.status, iters=r.iters, cauchy_final=r.cauchy_final, latency_ms=r.latency_ms,
                     queue_ms=r.queue_ms), out
+
+    def test_wait_flag(self, where):
+        """Failure-test hook: the next round (1) or retirement (2) finds that a wait gave up."""
+        return lib().dm_test_server_wait_flag(self.h, where)
 
     def cancel(self, ticket):
         return lib().dm_serve_cancel(self.h, ctypes.c_uint64(ticket))
