@@ -1037,6 +1037,7 @@ dm_status dm_set_tc_tiles(dm_plan *p, int generate) {
 
 dm_status dm_set_ring_radix(dm_plan *p, int lr) {
   if (!p || (lr != 0 && lr != 3 && lr != 4)) return DM_EINVAL;
+  prog_release(p);
   p->ring_lr = lr;
   p->ring_fft = true;
   for (int i = 0; i < DM_TUNE_MAX_CLASSES; ++i) p->tune_ring_lr[i] = -1;  // an explicit radix overrides a tuned one

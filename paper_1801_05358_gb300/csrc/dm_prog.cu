@@ -211,6 +211,7 @@ dm_status make_level_plan(dm_plan *p, int nk, int L, ProgLevelPlan &lp, std::str
   q->anchor_every = p->anchor_every;
   q->anchor_ff = p->anchor_ff;
   q->ring_lr = p->ring_lr;
+  q->ring_fft = p->ring_fft;
   if (cudaMalloc(&lp.child, sizeof(int) * ch.size()) || cudaMalloc(&lp.v, sizeof(double) * v.size()) ||
       cudaMemcpy(lp.child, ch.data(), sizeof(int) * ch.size(), cudaMemcpyHostToDevice) ||
       cudaMemcpy(lp.v, v.data(), sizeof(double) * v.size(), cudaMemcpyHostToDevice)) {
