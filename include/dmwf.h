@@ -423,7 +423,10 @@ dm_status dm_legendre_analysis_noalloc(dm_plan *plan, const double *rc, double *
  * pipeline stages of the two analysis kernels.  A value of 0 (-1 for a
  * radix) means the built-in heuristic.  The ms_ fields report the stage time
  * per iteration of the pick and of the heuristic, as measured by
- * dm_autotune (0 when not measured). */
+ * dm_autotune (0 when not measured).  Where the rings run as digit products
+ * (larger plans of the FP64-class modes, see dm_set_ring_radix) there is
+ * nothing to pick: both ring times are theirs, and the ring fields hold the
+ * FFT kernels' defaults. */
 typedef struct {
   int n_ring_classes;
   int ring_radix_lr[DM_TUNE_MAX_CLASSES];

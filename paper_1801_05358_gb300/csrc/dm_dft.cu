@@ -1170,7 +1170,7 @@ static size_t xinv_smem(const dm_plan *p) { return sizeof(double) * 8 * slots4(p
 static size_t pix_smem(const dm_plan *p) { return sizeof(double) * 8 * slots4((p->flat ? p->flatN / 4 : p->nside) + 1); }
 
 // Whether the products run; then their tables and the cuts of all groups exist.
-static cudaError_t dft_use(dm_plan *p, cudaStream_t st, bool *use) {
+cudaError_t dft_use(dm_plan *p, cudaStream_t st, bool *use) {
   DftTables *T = p->dft;
   *use = false;
   if (!T || T->disabled || p->ring_fft || p->tune_only_class >= 0) return cudaSuccess;

@@ -350,6 +350,7 @@ void dft_disable(dm_plan *p);
 int64_t dft_bytes(const dm_plan *p);
 size_t dft_table_bytes(int nside, int mmax);
 size_t dft_scratch_bytes(int nside, int batch);
+cudaError_t dft_use(dm_plan *p, cudaStream_t st, bool *use);  // whether the products run
 cudaError_t dft_flat_columns(dm_plan *p, const double2 *alm, const SolveState *state, cudaStream_t st, bool *ran);
 cudaError_t dft_ring_stage(dm_plan *p, int mode, const double *in_map, double *out_map, cudaStream_t st, bool *ran);
 // split products of the Legendre stages (dm_split.cu)

@@ -31,7 +31,8 @@ std::string tune_key(const dm_plan *p) {
     dev = std::string(prop.name) + "/" + std::to_string(prop.multiProcessorCount);
   return dev + "|" + std::to_string(p->nside) + "|" + std::to_string(p->lmax) + "|" + std::to_string(p->batch) +
          "|" + std::to_string((int)p->prec) + "|" + std::to_string((int)p->ff_legendre) + "|" +
-         std::to_string((int)(p->use_tc && tc_batch_ok(p->batch))) + "|" + std::to_string(p->tc_gen);
+         std::to_string((int)(p->use_tc && tc_batch_ok(p->batch))) + "|" + std::to_string(p->tc_gen) + "|" +
+         std::to_string((int)p->ring_fft);
 }
 
 void apply(dm_plan *p, const dm_tuning &t) {
@@ -89,9 +90,22 @@ dm_status autotune(dm_plan *p, cudaStream_t st, std::string &err) {
   const bool sa = p->state_active, aa = p->anchor_active;
   p->state_active = false;
   p->anchor_active = false;
+  // no right-hand side counts as finished (an earlier solve's state, or none yet)
+  if (cudaMemsetAsync(p->state, 0, sizeof(SolveState) * p->batch, st) != cudaSuccess) {
+    err = "state";
+    return DM_ECUDA;
+  }
   dm_tuning t{};
   t.n_ring_classes = ncls;
   dm_status rs = DM_OK;
+  // The FP64-class rings of larger plans run as digit products, which have
+  // nothing to pick: the reported time is theirs, the FFT launches (what runs
+  // where the products cannot) keep their defaults.
+  bool products = false;
+  if (p->prec == DM_FP64 && dft_use(p, st, &products) != cudaSuccess) {
+    err = "tables of the ring transforms";
+    rs = DM_ECUDA;
+  }
   // ---- ring stage: per class, every (radix, lanes per block) the launch allows
   for (int ci = 0; ci < ncls && rs == DM_OK; ++ci) {
     p->tune_only_class = ci;
@@ -116,7 +130,7 @@ dm_status autotune(dm_plan *p, cudaStream_t st, std::string &err) {
     std::array<int, 3> bestc = used_now();
     std::vector<std::array<int, 3>> seen{bestc};
     const int lrs[3] = {3, 4, 0};
-    for (int li = 0; li < 3; ++li)
+    for (int li = 0; li < (products ? 0 : 3); ++li)
       for (int fu : {1, 0, 2}) {
         if (lrs[li] == 0 && fu != 1) continue;
         if (fu == 2 && (lrs[li] != 4 || p->prec == DM_FP64)) continue;
@@ -147,6 +161,14 @@ dm_status autotune(dm_plan *p, cudaStream_t st, std::string &err) {
     t.ms_ring_default += t_def;
   }
   p->tune_only_class = -1;
+  if (products && rs == DM_OK) {
+    t.ms_ring = t.ms_ring_default =
+        time_it(p, st, [&]() { return ring_stage(p, RING_ITER, nullptr, p->s64, st); }, reps, e0, e1);
+    if (t.ms_ring < 0.f) {
+      err = "ring stage failed";
+      rs = DM_ECUDA;
+    }
+  }
   // ---- tensor-core Legendre stages
   if (tc && rs == DM_OK) {
     for (int part = 0; part < 2 && rs == DM_OK; ++part) {
