@@ -76,6 +76,7 @@ struct DftTile {
   int z, zfun;          // table row octet of the tile; distance to the sine matrix
   int n0;
   int64_t x, xfun;      // column digits of K step 0; distance to the sine columns
+  int b0, b1;           // first and last right-hand side (of the group) with a column here
 };
 struct DftCut {
   int nl = 0;
@@ -152,7 +153,11 @@ __global__ void k_dft_gen(const DftSet s, unsigned char *__restrict__ dig) {
   }
 }
 
-// column of (pair of the set, lane, side): its tile and place there
+// Columns of a set run over the pairs' two sides, then over the lanes, so that a
+// tile holds as few right-hand sides as it can: it is left out once they are
+// finished.
+__device__ __forceinline__ int col_of(const DftSet &s, int pair, int lane) { return (lane * s.npr + pair) * 2; }
+// a column's tile and place there
 __device__ __forceinline__ void col_place(const DftCol &c, int col, int &ct, int &cit) {
   ct = col / c.w;
   cit = col - ct * c.w;
@@ -190,7 +195,7 @@ __device__ __forceinline__ void digit_items(unsigned char *x, const DftCol &C, i
 __global__ void __launch_bounds__(128) k_dft_xinv(const double2 *__restrict__ rc, unsigned char *__restrict__ x,
                                                   int *__restrict__ xexp, const DftSet *__restrict__ sets,
                                                   const DftCol *__restrict__ cols, const int *__restrict__ pair_of,
-                                                  const int *__restrict__ set_of, int nl, int lane0, int mmax,
+                                                  const int *__restrict__ set_of, int lane0, int mmax,
                                                   int npairs, int eq, const SolveState *__restrict__ state) {
   extern __shared__ __align__(16) double vals[];  // [side][CE, CO, SE, SO][slots of an order's half]
   __shared__ double2 part[256];                   // partial alias sums of the short rings
@@ -250,7 +255,7 @@ __global__ void __launch_bounds__(128) k_dft_xinv(const double2 *__restrict__ rc
       }
   }
   int e[2];
-  const int col = ((g - S.pair0) * nl + lane) * 2, nsides = equator ? 1 : 2;
+  const int col = col_of(S, g - S.pair0, lane), nsides = equator ? 1 : 2;
   for (int side = 0; side < 2; ++side) {
     e[side] = max(-1000, block_max(ex[side], red));  // (its barriers cover the staged values too)
     if (e[side] >= SPLIT_NAN) e[side] = SPLIT_NAN;
@@ -276,7 +281,7 @@ __global__ void __launch_bounds__(256) k_dft_pix(const RingDev *__restrict__ rin
                                                  unsigned char *__restrict__ x, const int *__restrict__ xexp_in,
                                                  int *__restrict__ xexp_out, const DftSet *__restrict__ sets,
                                                  const DftCol *__restrict__ cols, const int *__restrict__ pair_of,
-                                                 const int *__restrict__ set_of, int nl, int lane0, int eq,
+                                                 const int *__restrict__ set_of, int lane0, int eq,
                                                  int nrings, int64_t npix, const double *__restrict__ in_map,
                                                  double *__restrict__ out_map, const double *__restrict__ w,
                                                  const double *__restrict__ wd, double *__restrict__ norms,
@@ -292,7 +297,7 @@ __global__ void __launch_bounds__(256) k_dft_pix(const RingDev *__restrict__ rin
   const int nsides = pair == eq ? 1 : 2;
   const bool on = side < nsides;
   const int ring = side ? nrings - 1 - pair : pair;
-  const int col = ((g - S.pair0) * nl + lane) * 2;
+  const int col = col_of(S, g - S.pair0, lane);
   const int n = S.n, nj = S.nj, ld = slots4(nj);
   double dd = 0.0, ss = 0.0;
   int ex = -100000;
@@ -490,7 +495,7 @@ __global__ void __launch_bounds__(256) k_flat_xsyn(const double2 *__restrict__ a
       keep(1, cs.y, -sn.x);
     }
     int e[2];
-    const int col = (kx * nl + 3 * b + f) * 2;
+    const int col = col_of(S, kx, 3 * b + f);
     for (int ri = 0; ri < 2; ++ri) {
       e[ri] = max(-1000, block_max(ex[ri], red));  // (its barriers cover the staged values too)
       if (e[ri] >= SPLIT_NAN) e[ri] = SPLIT_NAN;
@@ -517,12 +522,12 @@ __device__ __forceinline__ void flat_orbit(int j, int N, int at[4]) {
 // Orbit sums of a column into its rows.  grid (columns, lanes)
 __global__ void __launch_bounds__(256) k_flat_unfold(const double *__restrict__ v, const int *__restrict__ xexp,
                                                      double2 *__restrict__ rc, const DftSet *__restrict__ sets,
-                                                     const DftCol *__restrict__ cols, int nl, int lane0, int mmax,
+                                                     const DftCol *__restrict__ cols, int lane0, int mmax,
                                                      const SolveState *__restrict__ state) {
   const int kx = blockIdx.x, lane = blockIdx.y, al = lane0 + lane;
   if (state != nullptr && state[al / 3].done) return;
   const DftCol C = cols[0];
-  const int N = sets[0].n, col = (kx * nl + lane) * 2;
+  const int N = sets[0].n, col = col_of(sets[0], kx, lane);
   const double *vc = v + C.v + (int64_t)col * 4 * C.njp;
   double2 *o = rc + ((int64_t)al * (mmax + 1) + kx) * N;
   for (int j = threadIdx.x; j < N / 4; j += 256) {
@@ -556,7 +561,7 @@ __global__ void __launch_bounds__(256) k_flat_unfold(const double *__restrict__ 
 // The rows of a column folded over their orbits, as digits.  grid (columns, lanes)
 __global__ void __launch_bounds__(256) k_flat_xana(const double2 *__restrict__ rc, unsigned char *__restrict__ x,
                                                    int *__restrict__ xexp, const DftSet *__restrict__ sets,
-                                                   const DftCol *__restrict__ cols, int nl, int lane0, int mmax,
+                                                   const DftCol *__restrict__ cols, int lane0, int mmax,
                                                    const SolveState *__restrict__ state) {
   extern __shared__ __align__(16) double vals[];  // [re, im][CE, CO, SE, SO][slots of nj]
   __shared__ int red[8];
@@ -564,7 +569,7 @@ __global__ void __launch_bounds__(256) k_flat_xana(const double2 *__restrict__ r
   if (state != nullptr && state[al / 3].done) return;
   const DftSet S = sets[0];
   const DftCol C = cols[0];
-  const int N = S.n, ld = slots4(S.nj), col = (kx * nl + lane) * 2;
+  const int N = S.n, ld = slots4(S.nj), col = col_of(S, kx, lane);
   const double2 *src = rc + ((int64_t)al * (mmax + 1) + kx) * N;
   int ex[2] = {-100000, -100000};
   for (int j = threadIdx.x; j < N / 4; j += 256) {
@@ -645,6 +650,7 @@ __global__ void __launch_bounds__(dft_threads(NQ), 1) k_dft(const DftArgs A) {
   __shared__ uint64_t bars[2 * DFT_MAX_STAGES + 5];
   __shared__ uint32_t tslot;
   __shared__ int cta_bad;
+  __shared__ uint32_t live[128];  // unfinished right-hand sides of the group (4096 at most)
   uint64_t *full = bars, *empty = bars + DFT_MAX_STAGES, *tfull = bars + 2 * DFT_MAX_STAGES, *tempty = tfull + 2,
            *fin = tempty + 2;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -667,9 +673,20 @@ __global__ void __launch_bounds__(dft_threads(NQ), 1) k_dft(const DftArgs A) {
         make_uint4(0, 0, 0, 0);
   fence_proxy_async();
   if (warp == 0) tmem_alloc(&tslot, COLS);
+  if (A.state != nullptr)
+    for (int b = tid; (b & ~31) < A.nl / 3; b += THREADS) {
+      const uint32_t word = __ballot_sync(0xffffffffu, b < A.nl / 3 && !A.state[A.lane0 / 3 + b].done);
+      if (lane == 0) live[b >> 5] = word;
+    }
   fence_before_sync();
   __syncthreads();
   fence_after_sync();
+  auto finished = [&](const DftTile &T) {  // the same for every role: the states do not change under the kernel
+    if (A.state == nullptr) return false;
+    for (int b = T.b0; b <= T.b1; ++b)
+      if ((live[b >> 5] >> (b & 31)) & 1u) return false;
+    return true;
+  };
   const uint32_t tbase = tslot;
   int issued = 0;
   const uint32_t sm_a = smem_u32(sm), full_a = smem_u32(full), empty_a = smem_u32(empty);
@@ -680,6 +697,7 @@ __global__ void __launch_bounds__(dft_threads(NQ), 1) k_dft(const DftArgs A) {
       StageAt at;
       for (int t = blockIdx.x; ok && t < A.ntiles; t += gridDim.x) {
         const DftTile T = A.tiles[t];
+        if (finished(T)) continue;
         const CUtensorMap *map = A.maps + 2 * T.set + (FWD ? 1 : 0);
         map_acquire(map);
         for (int k0 = 0; ok && k0 < T.ks; k0 += DFT_CHUNK)
@@ -711,6 +729,7 @@ __global__ void __launch_bounds__(dft_threads(NQ), 1) k_dft(const DftArgs A) {
       const uint64_t ad0 = FWD ? split_desc(sm_a, 128, 256) : split_desc(sm_a, 2048, 128);
       const uint64_t bd0 = split_desc(sm_a + ABYTES, 128, 256);
       for (int t = blockIdx.x; ok && t < A.ntiles; t += gridDim.x) {
+        if (finished(A.tiles[t])) continue;
         const int ks = A.tiles[t].ks, nch = NF * ((ks + DFT_CHUNK - 1) / DFT_CHUNK);
         for (int c = 0; ok && c < nch; ++c, ++cc) {
           const int set = cc & 1;
@@ -748,6 +767,7 @@ __global__ void __launch_bounds__(dft_threads(NQ), 1) k_dft(const DftArgs A) {
     int cc = 0;
     for (int t = blockIdx.x; ok && t < A.ntiles; t += gridDim.x) {
       const DftTile T = A.tiles[t];
+      if (finished(T)) continue;
       const DftSet D = A.sets[T.set];
       const DftCol C = A.cols[T.set];
       const int ncol = D.npr * A.nl * 2, c0 = T.ct * C.w + part * QW * 4;
@@ -807,7 +827,7 @@ __global__ void __launch_bounds__(dft_threads(NQ), 1) k_dft(const DftArgs A) {
             for (int e = 0; e < 4; e += 2) {  // the two sides of one pair and lane
               const int col = c0 + 4 * q + e;
               if (col >= cend) break;
-              const int pc = col >> 1, pl = pc / A.nl, ln = pc - pl * A.nl, al = A.lane0 + ln;
+              const int pc = col >> 1, ln = pc / D.npr, pl = pc - ln * D.npr, al = A.lane0 + ln;
               if (A.state != nullptr && A.state[al / 3].done) continue;
               const int pair = A.pair_of[D.pair0 + pl];
               const bool equator = pair == A.eq;
@@ -1079,6 +1099,8 @@ static cudaError_t dft_cut(dm_plan *p, int nl, cudaStream_t st) {
             t.z = fun * s.rq + (dir == 0 ? 0 : 16 * r);
             t.zfun = 2 * s.rq;
             t.n0 = c.n0;
+            t.b0 = ct * c.w / (6 * s.npr);
+            t.b1 = (std::min(2 * s.npr * nl, (ct + 1) * c.w) - 1) / (6 * s.npr);
             t.x = (dir == 0 ? c.xi : c.xf) + ((int64_t)fun * c.nct + ct) * ks * blk;
             t.xfun = (int64_t)2 * c.nct * ks * blk;
             tiles[c.n0 / 8].push_back(t);
@@ -1229,7 +1251,7 @@ cudaError_t dft_ring_stage(dm_plan *p, int mode, const double *in_map, double *o
     if (mode == RING_ITER || mode == RING_INV_MAP) {
       const size_t sm = xinv_smem(p);
       if ((e = dyn_smem_allow(k_dft_xinv, sm))) return e;
-      k_dft_xinv<<<dim3(T->nlist, nl), 128, sm, st>>>(p->rc, T->x, ei, T->sets_dev, K->cols, T->pair_of, T->set_of, nl,
+      k_dft_xinv<<<dim3(T->nlist, nl), 128, sm, st>>>(p->rc, T->x, ei, T->sets_dev, K->cols, T->pair_of, T->set_of,
                                                       lane0, p->mmax, p->npairs, eq, state);
       if ((e = dft_products<false>(p, *K, lane0, state, st))) return e;
     }
@@ -1237,7 +1259,7 @@ cudaError_t dft_ring_stage(dm_plan *p, int mode, const double *in_map, double *o
     auto pix = [&](auto kern) {
       if (cudaError_t r = dyn_smem_allow(kern, sp)) return r;
       kern<<<dim3(T->nlist, nl), 256, sp, st>>>(p->rings, T->v, T->x, ei, ef, T->sets_dev, K->cols, T->pair_of,
-                                                T->set_of, nl, lane0, eq, p->nrings, p->npix, in_map, out_map, p->w,
+                                                T->set_of, lane0, eq, p->nrings, p->npix, in_map, out_map, p->w,
                                                 p->wd, p->norms, state);
       return cudaGetLastError();
     };
@@ -1280,12 +1302,12 @@ cudaError_t dft_flat_columns(dm_plan *p, const double2 *alm, const SolveState *s
       k_flat_xsyn<<<dim3(N / 2, 3 * ((nb + FLAT_NB - 1) / FLAT_NB)), 256, sx, st>>>(
           alm, T->x, ei, T->sets_dev, K->cols, nl, b0, 1.0 / (p->flatL * p->flatL), p->nmodes, state);
       if ((e = dft_products<false>(p, *K, lane0, state, st))) return e;
-      k_flat_unfold<<<dim3(N / 2, nl), 256, 0, st>>>(T->v, ei, p->rc, T->sets_dev, K->cols, nl, lane0, p->mmax,
+      k_flat_unfold<<<dim3(N / 2, nl), 256, 0, st>>>(T->v, ei, p->rc, T->sets_dev, K->cols, lane0, p->mmax,
                                                      state);
       if ((e = cudaGetLastError())) return e;
     } else {
       if ((e = dyn_smem_allow(k_flat_xana, sf))) return e;
-      k_flat_xana<<<dim3(N / 2, nl), 256, sf, st>>>(p->rc, T->x, ef, T->sets_dev, K->cols, nl, lane0, p->mmax,
+      k_flat_xana<<<dim3(N / 2, nl), 256, sf, st>>>(p->rc, T->x, ef, T->sets_dev, K->cols, lane0, p->mmax,
                                                     state);
       if ((e = dft_products<true>(p, *K, lane0, state, st, true))) return e;
     }
