@@ -21,8 +21,9 @@
 // functions of few values on a ring (orders n / 4, n / 8, ... against a map of
 // that period) reach 0.82 of 2^24 over all amplitudes.  lambda_00 is the same
 // on every ring: against a constant map it reaches 1.17 (0.6 % of amplitudes pass
-// 1), but all terms are equal there, so every K step of 16 adds a multiple of 16,
-// which FP32 holds up to 2^28.
+// 1).  Its tile of the analysis therefore drains every 64 terms, where weights 2
+// and 3 cannot pass; every other function changes over 128 rings by far more
+// than a unit of its third digit (relative 2^-26).
 // S = 6 serves DM_FP64, DM_FLOAT_FLOAT, the anchors and the diagnostics; S = 3
 // (27 bits against the 24 of FP32) the mixed mode's batches outside the BF16
 // kernels.
@@ -74,7 +75,7 @@ namespace dmwf {
 using namespace tc;
 
 constexpr int SPLIT_ROWS = 128;        // rows of a tile (ring pairs or multipoles)
-constexpr int SPLIT_CHUNK = 8;         // K steps of 16 per drain
+constexpr int SPLIT_CHUNK = 8;         // K steps of 16 per drain (half of it in the analysis tile of l = 0)
 constexpr int SPLIT_MIN_EXP = -600;    // smallest row scale
 // Drain warps: 16 where the columns divide (the drain is latency bound).  Both
 // stages and the rings' products alike, a solve at nside 128 with 8 right-hand
@@ -92,6 +93,7 @@ struct SplitTile {
   int trow;        // table row (octet of multipoles) of the tile's first row octet (analysis) or K step 0 (synthesis)
   int xstep;       // K step 0 of the tile in the column scratch, in steps (of one column tile)
   int xlen;        // K steps of the whole order (scratch stride between column tiles)
+  int chunk;       // K steps per drain
 };
 
 // Launches of both directions for one kind of batch: device tile lists, and
@@ -512,9 +514,9 @@ __global__ void __launch_bounds__(split_threads(NQ), 1) k_split(const __grid_con
         const unsigned char *x0 = A.x + (int64_t)T.part * A.xpart +
                                   (T.xstep * (int64_t)A.nct + (int64_t)ct * T.xlen + T.k0) * BBYTES;
         // chunks alternate p and q over the same K steps
-        for (int k0 = 0; ok && k0 < T.nk; k0 += SPLIT_CHUNK)
+        for (int k0 = 0; ok && k0 < T.nk; k0 += T.chunk)
           for (int fun = 0; ok && fun < nfun; ++fun)
-            for (int k = k0; k < min(k0 + SPLIT_CHUNK, T.nk); k += KS) {
+            for (int k = k0; k < min(k0 + T.chunk, T.nk); k += KS) {
               if (issued >= NS && !mbar_wait_at(empty_a + 8 * at.s, at.phase ^ 1, A.err)) {
                 ok = false;
                 break;
@@ -547,8 +549,8 @@ __global__ void __launch_bounds__(split_threads(NQ), 1) k_split(const __grid_con
         const int ct = t % A.nct;
         if (!((live_mask[ct >> 5] >> (ct & 31)) & 1u)) continue;
         const SplitTile *T = A.tiles + t / A.nct;
-        const int nk = T->nk, nfun = T->part == 0 ? 1 : 2;
-        const int nch = nfun * ((nk + SPLIT_CHUNK - 1) / SPLIT_CHUNK);
+        const int nk = T->nk, nfun = T->part == 0 ? 1 : 2, chunk = T->chunk;
+        const int nch = nfun * ((nk + chunk - 1) / chunk);
         for (int c = 0; ok && c < nch; ++c, ++cc) {
           const int set = cc & 1;
           if (cc >= 2 && !mbar_wait(&tempty[set], ((cc >> 1) - 1) & 1, A.err)) {
@@ -556,7 +558,7 @@ __global__ void __launch_bounds__(split_threads(NQ), 1) k_split(const __grid_con
             break;
           }
           fence_after_sync();
-          const int nstep = min(SPLIT_CHUNK, nk - (nfun == 2 ? c >> 1 : c) * SPLIT_CHUNK);
+          const int nstep = min(chunk, nk - (nfun == 2 ? c >> 1 : c) * chunk);
           const uint32_t d = tbase + set * SET;
           for (int k = 0; k < nstep; k += KS) {
             if (!mbar_wait_at(full_a + 8 * at.s, at.phase, A.err)) {
@@ -593,7 +595,7 @@ __global__ void __launch_bounds__(split_threads(NQ), 1) k_split(const __grid_con
       if (!((live_mask[ct >> 5] >> (ct & 31)) & 1u)) continue;
       const SplitTile T = A.tiles[t / A.nct];
       const int nfun = T.part == 0 ? 1 : 2;
-      const int nch = nfun * ((T.nk + SPLIT_CHUNK - 1) / SPLIT_CHUNK);
+      const int nch = nfun * ((T.nk + T.chunk - 1) / T.chunk);
       const int nrhs = min(QW, min(A.nb, A.batch - ct * A.nb) - part * QW);  // of this warp group (may be <= 0)
       constexpr int NF = SYN ? 2 : 1;
       Acc<S> acc[NF][QW][4];
@@ -971,6 +973,7 @@ static cudaError_t split_cut(dm_plan *p, int S, cudaStream_t st) {
               t.k0 = std::min(t.xlen, dir == 0 ? T->ks_syn[((size_t)part * nm + m) * npt + r]
                                                : T->ks_ana[((size_t)part * nm + m) * nlt + r]);
               t.nk = t.xlen - t.k0;
+              t.chunk = dir == 1 && m == 0 && part == 0 && r == 0 ? SPLIT_CHUNK / 2 : SPLIT_CHUNK;
               t.trow = T->roff[m] - T->roff[T->slab[k]] + (dir == 0 ? 0 : 16 * r);
               t.xstep = dir == 0 ? (T->roff[m] - T->roff[m0]) / 2 : (m - m0) * nkp;
               tiles.push_back(t);

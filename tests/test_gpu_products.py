@@ -130,6 +130,26 @@ def test_products_not_finite(bad):
         assert np.array_equal(bm[b], gm[b]) and np.array_equal(ba[b], ga[b])
 
 
+# Constant maps: lambda_00 is one value on every ring, so the digits of both
+# operands keep their signs and the digit sums are the largest there are: for
+# the first four amplitudes (over all of them), and a sweep of one power of two.
+# The monopole of c is c sqrt(4 pi); operands and values are rounded at 2^-52 of
+# theirs at most, four times: bar 4e-15, a lost unit of a sum is 1e-12.
+def test_products_constant_maps():
+    nside, lmax, B = 256, 96, 64
+    amp = np.concatenate([[0.9628561361180136, 0.8613087756796693, 0.9354665353746234, 0.6738011761632003, 2.7255],
+                          0.5 * 2.0 ** np.random.default_rng(8).random(B - 5)])
+    maps = np.zeros((B, 3, 12 * nside * nside))
+    maps[:, 0] = amp[:, None]
+    p = dmwf.Plan(nside, lmax, B)
+    out = torch.zeros((B, 3, (lmax + 1) * (lmax + 2) // 2, 2), dtype=torch.float64, device="cuda")
+    p.map2alm(dev(maps), out)
+    torch.cuda.synchronize()
+    p.close()
+    mono = out[:, 0, 0, 0].cpu().numpy()
+    assert np.abs(mono / (amp * np.sqrt(4.0 * np.pi)) - 1.0).max() < 4e-15
+
+
 # Mixed mode outside the tensor-core batches: FP32 kernels below the size rules
 # (23: ring pairs not a multiple of 4; 64, 190: the largest analysis, 100, 244:
 # the largest synthesis; batch 4: four right-hand sides a thread; batch 2 above
