@@ -65,8 +65,14 @@ typedef enum {
 /* Arithmetic of the Legendre contraction and of map storage.
  * DM_FP64: everything in FP64 precision.  The contractions (Legendre stages;
  *   ring transforms and flat-patch columns of larger plans) run as products of
- *   base-512 digits of the FP64 operands on the tensor cores, summed exactly
- *   and rounded once; tables of digits are made on first use.  Where they
+ *   base-512 digits of the FP64 operands on the tensor cores, whose sums stay
+ *   within what FP32 accumulators hold exactly and are rounded to FP64 once.
+ *   The operands are fixed-point, 54 bits below the largest value of their row
+ *   (an order and ring pair of the Legendre functions) or column (an order of
+ *   one RHS): errors are FP64's relative to those, not to each value of its
+ *   own; the calls that return the coefficients themselves
+ *   (dm_legendre_synthesis, dm_legendre_analysis) run FP64 kernels, which keep
+ *   every value's bits.  Tables of digits are made on first use.  Where they
  *   cannot be made (no memory, first use inside a stream capture) FP64 kernels
  *   run instead, and a later call makes them once there is more memory.
  * DM_MIXED_FP32: FP64 recurrence (Legendre/Wigner values generated in FP64),

@@ -830,7 +830,10 @@ dm_status dm_ring_fft_inverse(dm_plan *p, const double *rc, double *map, void *s
 dm_status dm_legendre_synthesis(dm_plan *p, const double *alm, double *rc, void *stream) {
   if (!p || !alm || !rc) return DM_EINVAL;
   cudaStream_t st = (cudaStream_t)stream;
-  DM_CU(legendre_synthesis(p, (const double2 *)alm, st), "synthesis");
+  p->each_value = true;
+  const cudaError_t e = legendre_synthesis(p, (const double2 *)alm, st);
+  p->each_value = false;
+  DM_CU(e, "synthesis");
   DM_CU(rc_to_public(p, (double2 *)rc, st), "layout");
   return DM_OK;
 }
@@ -839,7 +842,10 @@ dm_status dm_legendre_analysis(dm_plan *p, const double *rc, double *alm, void *
   if (!p || !alm || !rc) return DM_EINVAL;
   cudaStream_t st = (cudaStream_t)stream;
   DM_CU(rc_from_public(p, (const double2 *)rc, st), "layout");
-  DM_CU(legendre_analysis(p, ANA_PLAIN, (double2 *)alm, st), "analysis");
+  p->each_value = true;
+  const cudaError_t e = legendre_analysis(p, ANA_PLAIN, (double2 *)alm, st);
+  p->each_value = false;
+  DM_CU(e, "analysis");
   return DM_OK;
 }
 

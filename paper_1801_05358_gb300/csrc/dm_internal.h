@@ -169,6 +169,7 @@ struct dm_plan {
   // FP32 Legendre tables of the mixed mode's small plans and batches (dm_legendre32.cu)
   float *tab32 = nullptr;       // [3][nalm][npairs up to a multiple of 4] lambda, lam+, lam-
   dmwf::Shortage tab32_short;   // they did not fit: the split products run
+  bool each_value = false;      // inside a stage call that returns coefficients: kernels that keep every value's own precision
   bool is_view = false;         // a one-RHS view of a serving pool (makes no tables of its own)
   // digit tables of the split products (dm_split.cu): shared with the views of the plan
   dmwf::SplitTables *split = nullptr;

@@ -220,11 +220,11 @@ int table_ld(const dm_plan *p) { return (p->npairs + 3) & ~3; }  // 16-byte rows
 int64_t order_entries(const dm_plan *p) { return (int64_t)p->npairs * (p->lmax + 1); }
 
 // The FP32 kernels take every size and batch where the split products would
-// have to make their digits again in each stage call (no whole table), and when
-// the tensor cores are turned off.  An iteration at nside 1024 / lmax 2048, one
+// have to make their digits again in each stage call (no whole table), when the
+// tensor cores are turned off and where every value's precision counts.  An iteration at nside 1024 / lmax 2048, one
 // and three right-hand sides: 14.5 and 28.5 ms here, 425 and 426 with slabs of
 // digits; at nside 512 / lmax 1535 with seven, slabs 103, whole digits 8.6.
-bool instead(const dm_plan *p) { return !p->use_tc || !split_whole(p); }
+bool instead(const dm_plan *p) { return !p->use_tc || p->each_value || !split_whole(p); }
 
 // The FP32 tables, made on first use: not while the stream is captured, on a
 // plan that shares another's tables, or where they leave no room for the

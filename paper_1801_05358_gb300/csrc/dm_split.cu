@@ -1125,7 +1125,11 @@ static cudaError_t split_run(dm_plan *p, const SplitLaunches &C, const C2 *in, v
 // right-hand sides; the direct kernels run their recurrence once for each.  One
 // iteration, slabs and direct kernels: nside 512 / lmax 1535, one right-hand
 // side 109 and 100 ms, two 110 and 200; nside 1024 / lmax 2048, one 460 and 351.
-static bool direct64(const dm_plan *p) { return p->batch == 1 && !split_whole(p); }
+// Digits are fixed-point: a value far below the largest of its row or column
+// keeps few bits or none.  No pixel and no sum notices, but the coefficients of
+// a red spectrum near the poles (lambda of low multipoles beside that of the
+// highest) are such values: the calls that return them take the direct kernels.
+static bool direct64(const dm_plan *p) { return p->each_value || (p->batch == 1 && !split_whole(p)); }
 
 // FP64-class synthesis of alm into p->rc; *ran = false when the direct
 // kernels have to do it.
