@@ -179,6 +179,7 @@ struct dm_plan {
   int64_t dft_cap = (int64_t)8 << 30;  // largest matrix table kept (else the FFT kernels)
   int64_t split_cap = (int64_t)48 << 30;  // largest whole table kept (41 GiB at nside 512 / lmax 1535: an
                                           // FP64-class iteration of two RHS takes 110 ms in slabs, 14.4 whole)
+  int64_t scratch_cap = (int64_t)1 << 30;  // column digits of one launch of the split products
   int64_t ffs_cap = (int64_t)1 << 30;  // bytes of the largest slab when the table is not kept whole
   bool ffs_cap_set = false;     // dm_set_ff_slab_bytes was called: slabs of that size, no whole table
   bool ff_legendre = false;     // DM_FLOAT_FLOAT: Legendre stages in float-float
@@ -362,7 +363,8 @@ void split_release(dm_plan *p);
 void split_forget(dm_plan *p);
 int64_t split_bytes(const dm_plan *p);
 size_t split_table_bytes(int lmax, int mmax, int npairs);
-size_t split_scratch_bytes(int lmax, int npairs, int batch);  // upper bound of the column digits
+size_t split_order_bytes(int lmax, int npairs);  // of the largest order
+size_t split_scratch_bytes(int lmax, int npairs, int batch, int64_t cap);  // upper bound of the column digits
 bool split_whole(const dm_plan *p);                            // the digit table is (to be) kept whole
 void split_disable(dm_plan *p);                                // the direct kernels only
 cudaError_t split_synthesis64(dm_plan *p, const double2 *alm, cudaStream_t st, bool *ran);

@@ -180,7 +180,7 @@ size_t estimate_bytes(int nside, int lmax, int S, dm_precision prec, double *tab
       *tables = (double)(1u << 30);
     }
     b += S * 3 * (lmax + 1.0) * npairs * 2 * 8;  // rc32
-    b += S * nchunk * 3 * nalm * 8;              // apart32
+    b += S * 3 * nalm * 8;                       // apart32
     b += S * 3 * npix * 4 * 4;                   // s32, w32, wd32, shi32
     b += S * 3 * nalm * 16 * 2;                  // a_hi, g_hi
     b += S * 3 * nalm * 8 * 2;                   // e32, c32
@@ -279,7 +279,7 @@ Pool *make_pool(dm_server *S, const Request &r, dm_status *why) {
     // slabs, else none (the direct FP64 kernels), so that no request the
     // budget held without them is turned away for them.
     const double room = tables + (double)(S->cfg.hbm_budget_bytes - S->used - need);
-    const double scratch = (double)split_scratch_bytes(r.lmax, p->npairs, slots);
+    const double scratch = (double)split_scratch_bytes(r.lmax, p->npairs, slots, p->scratch_cap);
     const double whole = (double)split_table_bytes(r.lmax, p->mmax, p->npairs);
     double take = 0;
     if (whole <= (double)p->split_cap && whole + scratch <= room) {
@@ -289,10 +289,11 @@ Pool *make_pool(dm_server *S, const Request &r, dm_status *why) {
       take = std::min(whole, (double)p->ffs_cap) + scratch;
     } else if (prec == DM_FP64) {
       split_disable(p);
-    } else {  // the other modes have no kernels without tables: slabs within what the estimate left
+    } else {  // the other modes' estimate leaves room for tables: slabs in one half of it, their column digits in the other
       p->split_cap = 0;
-      p->ffs_cap = (int64_t)std::max((double)(1 << 20), std::min(whole, tables));
-      take = tables;
+      p->ffs_cap = p->scratch_cap = (int64_t)std::max((double)(1 << 20), tables / 2);
+      const double slab = std::max((double)p->ffs_cap, (double)split_order_bytes(r.lmax, p->npairs));
+      take = std::min(whole, slab) + (double)split_scratch_bytes(r.lmax, p->npairs, slots, p->scratch_cap);
     }
     // the ring DFT matrices with what is left, else the FFT kernels
     const double rings = (double)dft_table_bytes(r.nside, p->mmax) + (double)dft_scratch_bytes(r.nside, slots);

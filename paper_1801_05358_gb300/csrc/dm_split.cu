@@ -83,7 +83,6 @@ constexpr int SPLIT_MIN_EXP = -600;    // smallest row scale
 __host__ __device__ constexpr int split_drain_warps(int nq) { return nq % 2 == 0 ? 16 : 8; }
 __host__ __device__ constexpr int split_threads(int nq) { return 32 * (split_drain_warps(nq) + 2); }
 constexpr int SPLIT_MAX_STAGES = 12;
-constexpr size_t SPLIT_SCRATCH = (size_t)1 << 30;  // column digits of one launch
 
 // One tile of work: 128 rows of one order and part, K steps [k0, k0 + nk) of each function.
 struct SplitTile {
@@ -737,6 +736,10 @@ bool split_whole(const dm_plan *p) {
   return !p->ffs_cap_set && split_table_bytes(p->lmax, p->mmax, p->npairs) <= (size_t)p->split_cap;
 }
 
+size_t split_order_bytes(int lmax, int npairs) {
+  return (size_t)table_rows(lmax, 0) * 3 * SPLIT_S * 128 * ((npairs + 7) / 8);
+}
+
 static void drop_cuts(SplitTables *T) {
   for (SplitLaunches &c : T->cuts)
     for (SplitTile *t : c.tiles)
@@ -773,14 +776,14 @@ void split_new(dm_plan *p) {
 
 void split_disable(dm_plan *p) { p->split->disabled = true; }
 
-// Column digits of one launch: those of every order, at most SPLIT_SCRATCH
-// bytes unless one order alone takes more.
-size_t split_scratch_bytes(int lmax, int npairs, int batch) {
+// Column digits of one launch: those of every order, at most cap bytes unless
+// one order alone takes more.
+size_t split_scratch_bytes(int lmax, int npairs, int batch, int64_t cap) {
   int nct, nb, nq;
   split_cols(batch, &nct, &nb, &nq);
   const double blk = (double)SPLIT_S * 8 * nq * 32 * nct, nkp = (npairs + 15) / 16;
   const double one = blk * std::max(3.0 * nkp, (double)table_rows(lmax, 0)), all = one * (lmax + 1);
-  return (size_t)std::max(one, std::min(all, (double)SPLIT_SCRATCH));
+  return (size_t)std::max(one, std::min(all, (double)cap));
 }
 
 // Forget the digit slabs (a new slab size); the row exponents stay.
@@ -883,7 +886,7 @@ static cudaError_t split_setup(dm_plan *p, cudaStream_t st) {
     }
   }
   if (!T->x) {
-    const size_t xb = (split_scratch_bytes(lmax, npairs, T->batch) + 127) / 128 * 128;
+    const size_t xb = (split_scratch_bytes(lmax, npairs, T->batch, p->scratch_cap) + 127) / 128 * 128;
     const size_t all = xb + sizeof(int) * 2 * (size_t)nm * T->batch;
     if ((e = table_alloc(p, (void **)&T->x, all))) return e;
     T->xexp = reinterpret_cast<int *>(T->x + xb);
@@ -947,7 +950,7 @@ static cudaError_t split_cut(dm_plan *p, int S, cudaStream_t st) {
   C.n0 = 8 * nq;
   C.S = S;
   cudaError_t e = cudaSuccess;
-  const size_t blk = (size_t)S * C.n0 * 32, cap = SPLIT_SCRATCH;
+  const size_t blk = (size_t)S * C.n0 * 32, cap = (size_t)p->scratch_cap;
   const int npt = (npairs + 127) / 128, nlt = (lmax + 128) / 128, nkp = (npairs + 15) / 16;
   for (int dir = 0; dir < 2 && !e; ++dir) {
     std::vector<SplitTile> tiles;
