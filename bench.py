@@ -643,7 +643,7 @@ def main():
         fms = timed_single_steps(plan, d, nf, torch)
         fp64_line = {"value": B / (fms * 1e-3), "unit": "DM iterations/s", "steps": nf,
                      "ms_per_step": fms, "note": f"median of {nf} single timed iterations"}
-    # ---- the float-float Legendre path (FP64-class results on the FP32 pipe) ----
+    # ---- DM_FLOAT_FLOAT (the FP64-class path under its other name) ----
     ff_line = None
     if args.fp64_steps > 0 and prec != dmwf.DM_FP64:
         nf = args.fp64_steps

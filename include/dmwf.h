@@ -247,8 +247,9 @@ dm_status dm_set_diagnostics(dm_plan *plan, int on);
  * precision iterative refinement; no counterpart in the paper). */
 dm_status dm_set_refinement(dm_plan *plan, int anchor_every);
 
-/* Arithmetic of those anchors: DM_FLOAT_FLOAT (default; FP64-class accuracy
- * on the FP32 pipe) or DM_FP64 (FP64 pipe); DM_EINVAL for other values. */
+/* Arithmetic of those anchors: DM_FLOAT_FLOAT or DM_FP64, which are one
+ * FP64-class path (see dm_precision), so that the call changes nothing;
+ * DM_EINVAL for other values. */
 dm_status dm_set_anchor_precision(dm_plan *plan, dm_precision prec);
 
 /* Tensor cores for the mixed-precision Legendre stages (default on): with a

@@ -158,9 +158,10 @@ dm_status check_ready(dm_plan *p) {
 namespace dmwf {
 
 // The iteration driver.  Device stages per iteration:
-//   analysis + harmonic step  a <- F_k [a + A (t - s)]      (k_leg_ana + k_ana_reduce)
-//   synthesis                 F_m(theta) from a             (k_leg_syn)
-//   ring stage                s, Cauchy partials, t - s, G_m (k_ring<RING_ITER>)
+//   analysis + harmonic step  a <- F_k [a + A (t - s)]      (k_split, k_ana_tc, k_ana_gen, k_ana32 or k_leg_ana64;
+//                                                            k_ana_reduce, k_ana_reduce32 or k_ana_step_e32)
+//   synthesis                 F_m(theta) from a             (k_split, k_syn_tc, k_syn_gen, k_syn32 or k_leg_syn64)
+//   ring stage                s, Cauchy partials, t - s, G_m (k_dft and k_dft_pix, or k_ring<RING_ITER>)
 //   control                   Cauchy ratio, level, stop     (k_control_step)
 // Mixed precision adds FP64 anchors (iterative refinement): a = a_hi + e, the
 // FP32 stages transform e only, and g_hi = A W (d - Y a_hi) is recomputed in
@@ -191,7 +192,6 @@ dm_status anchor(dm_plan *p, cudaStream_t st, bool initial, const double *d, boo
   const size_t mn = sizeof(double) * 3 * p->npix * p->batch;
   p->state_active = false;
   p->prec = DM_FP64;
-  p->ff_now = p->anchor_ff;
   cudaError_t e = cudaSuccess;
   cudaEvent_t ta = nullptr, tb = nullptr;
   if (p->prof_on) {
@@ -221,7 +221,6 @@ dm_status anchor(dm_plan *p, cudaStream_t st, bool initial, const double *d, boo
     p->launches += 4;
   }
   p->prec = DM_MIXED_FP32;
-  p->ff_now = false;
   if (!e) e = cudaMemsetAsync(p->s32, 0, sizeof(float) * 3 * p->npix * p->batch, st);
   if (!e)
     e = cudaMemsetAsync(p->rc32, 0, sizeof(float2) * (size_t)p->batch * 3 * (p->mmax + 1) * p->npairs * 2, st);
@@ -560,18 +559,15 @@ dm_status dm_set_precision(dm_plan *p, dm_precision prec) {
   if (p->flat && prec != DM_FP64) return fail(p, DM_EINVAL, "flat-sky plans run in DM_FP64");
   if (p->session) return fail(p, DM_EBUSY, "a solve is in progress");
   prog_release(p);
-  if (prec != DM_FP64) DM_CU(setup_fp32(p), "float tables");
-  // DM_FLOAT_FLOAT runs the FP64 path with float-float Legendre stages
-  p->prec = prec == DM_MIXED_FP32 ? DM_MIXED_FP32 : DM_FP64;
-  p->ff_legendre = prec == DM_FLOAT_FLOAT;
+  if (prec == DM_MIXED_FP32) DM_CU(setup_fp32(p), "float tables");
+  p->prec = prec == DM_MIXED_FP32 ? DM_MIXED_FP32 : DM_FP64;  // DM_FLOAT_FLOAT runs the FP64 path
   return DM_OK;
 }
 
 dm_status dm_set_anchor_precision(dm_plan *p, dm_precision prec) {
   if (!p) return DM_EINVAL;
   if (prec != DM_FP64 && prec != DM_FLOAT_FLOAT) return fail(p, DM_EINVAL, "anchors run in DM_FP64 or DM_FLOAT_FLOAT");
-  p->anchor_ff = prec == DM_FLOAT_FLOAT;
-  return DM_OK;
+  return DM_OK;  // one FP64-class path serves both
 }
 
 dm_status dm_set_spectra(dm_plan *p, const double *cl) {

@@ -11,7 +11,7 @@
 //  chi^2          (d - s)^T N^-1 (d - s) + a^T S^-1 a (Eq. 3), the data term over
 //                 observed pixel-components, the prior with C^+ (m > 0 twice).
 //
-// Both reuse the FP64 (or float-float) stages of the plan: one ring analysis
+// Both reuse the FP64-class stages of the plan: one ring analysis
 // of w d and one of the residual map w (d - Y a), where s = Y a is the final
 // map the solve already holds.  Under correlated noise (Appendix B) w is the
 // 3 x 3 block W = alpha N^-1 of each pixel, and the data term of chi^2 is
@@ -261,8 +261,7 @@ cudaError_t diag_tables_flat(dm_plan *p, const std::vector<double> &cl) {
 }
 
 // The diagnostics of every RHS of the plan's final iterate (p->a, with
-// s64 = Y a).  Runs the FP64-class stages (FP64 or float-float, as the
-// plan's anchors do in the mixed mode); synchronises the stream.
+// s64 = Y a).  Runs the FP64-class stages; synchronises the stream.
 cudaError_t diagnostics(dm_plan *p, cudaStream_t st, std::vector<double> &resid, std::vector<double> &chi2) {
   const int B = p->batch;
   resid.assign(B, NAN);
@@ -293,12 +292,8 @@ cudaError_t diagnostics(dm_plan *p, cudaStream_t st, std::vector<double> &resid,
   // the FP64-class stages, on every RHS
   const bool sa = p->state_active;
   const dm_precision prec = p->prec;
-  const bool ffn = p->ff_now;
   p->state_active = false;
-  if (prec != DM_FP64) {
-    p->prec = DM_FP64;
-    p->ff_now = p->anchor_ff;
-  }
+  p->prec = DM_FP64;
   const int64_t n3 = 3 * p->npix;
   // r = w (d - Y a) (W (d - Y a) under correlated noise) into tmpmap2, and
   // the data term of chi^2
@@ -325,7 +320,6 @@ cudaError_t diagnostics(dm_plan *p, cudaStream_t st, std::vector<double> &resid,
     e = cudaGetLastError();
   }
   p->prec = prec;
-  p->ff_now = ffn;
   p->state_active = sa;
   p->launches += 7;
   if (e) return e;

@@ -182,9 +182,6 @@ struct dm_plan {
   int64_t scratch_cap = (int64_t)1 << 30;  // column digits of one launch of the split products
   int64_t ffs_cap = (int64_t)1 << 30;  // bytes of the largest slab when the table is not kept whole
   bool ffs_cap_set = false;     // dm_set_ff_slab_bytes was called: slabs of that size, no whole table
-  bool ff_legendre = false;     // DM_FLOAT_FLOAT: Legendre stages in float-float
-  bool anchor_ff = true;        // mixed-mode anchors in float-float (else FP64)
-  bool ff_now = false;          // inside a float-float anchor
   float2 *rc32 = nullptr;       // [B][3][mmax+1][npairs][2]
   float2 *apart32 = nullptr;    // [B][3][nalm] analysis sums
   float *s32 = nullptr;         // [B][3][npix] iteration map

@@ -61,21 +61,15 @@ __global__ void k_jacobi_source(double2 *__restrict__ g, const double2 *__restri
   }
 }
 
-// run f with the plan's FP64-class stages (FP64, or float-float where the
-// plan's anchors are), on every RHS
+// run f with the plan's FP64-class stages, on every RHS
 template <typename F>
 cudaError_t fp64_class(dm_plan *p, F f) {
   const bool sa = p->state_active;
   const dm_precision prec = p->prec;
-  const bool ffn = p->ff_now;
   p->state_active = false;
-  if (prec != DM_FP64) {
-    p->prec = DM_FP64;
-    p->ff_now = p->anchor_ff;
-  }
+  p->prec = DM_FP64;
   cudaError_t e = f();
   p->prec = prec;
-  p->ff_now = ffn;
   p->state_active = sa;
   return e;
 }

@@ -202,14 +202,12 @@ dm_status make_level_plan(dm_plan *p, int nk, int L, ProgLevelPlan &lp, std::str
     err = q->err;
     return r;
   }
-  const dm_precision prec = p->ff_legendre ? DM_FLOAT_FLOAT : p->prec;
-  if ((r = dm_set_precision(q, prec)) != DM_OK) {
+  if ((r = dm_set_precision(q, p->prec)) != DM_OK) {
     err = q->err;
     return r;
   }
   q->use_tc = p->use_tc;
   q->anchor_every = p->anchor_every;
-  q->anchor_ff = p->anchor_ff;
   q->ring_lr = p->ring_lr;
   q->ring_fft = p->ring_fft;
   if (cudaMalloc(&lp.child, sizeof(int) * ch.size()) || cudaMalloc(&lp.v, sizeof(double) * v.size()) ||

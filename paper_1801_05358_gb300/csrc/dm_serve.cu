@@ -169,8 +169,8 @@ size_t estimate_bytes(int nside, int lmax, int S, dm_precision prec, double *tab
   b += nalm * 48 + (lmax + 1.0) * npairs * 28;   // coefficients, seeds
   const bool tc = prec == DM_MIXED_FP32 && dmwf::tc_batch_ok(S);
   const bool stored = tc && dmwf::tc_tables_fit(lmax, lmax, (int)npairs, S);
-  if (prec != DM_FP64) {                         // DM_MIXED_FP32 and DM_FLOAT_FLOAT
-    const double full = 3 * nalm * npairs * 4 * 2;  // FP32 tables, hi and lo
+  if (prec != DM_FP64) {  // DM_MIXED_FP32 and DM_FLOAT_FLOAT: tables, 24 bytes per multipole, order and ring pair
+    const double full = 3 * nalm * npairs * 4 * 2;
     const bool fp32_tab = stored || (prec == DM_MIXED_FP32 && !tc);
     if (fp32_tab || (prec == DM_FLOAT_FLOAT && full <= 32.0 * (1u << 30)) || full <= (double)(1u << 30)) {
       b += full;
@@ -179,6 +179,8 @@ size_t estimate_bytes(int nside, int lmax, int S, dm_precision prec, double *tab
       b += (double)(1u << 30);
       *tables = (double)(1u << 30);
     }
+  }
+  if (prec == DM_MIXED_FP32) {
     b += S * 3 * (lmax + 1.0) * npairs * 2 * 8;  // rc32
     b += S * 3 * nalm * 8;                       // apart32
     b += S * 3 * npix * 4 * 4;                   // s32, w32, wd32, shi32

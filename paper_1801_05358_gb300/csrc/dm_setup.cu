@@ -619,7 +619,7 @@ cudaError_t table_alloc(const dm_plan *p, void **ptr, size_t bytes) {
 void Shortage::note(const dm_plan *p) { room = table_room(p); }
 bool Shortage::lasts(const dm_plan *p) const { return room != SIZE_MAX && table_room(p) <= room; }
 
-// Buffers of DM_MIXED_FP32 and DM_FLOAT_FLOAT: FP32 copies of the FFT tables,
+// Buffers of DM_MIXED_FP32: FP32 copies of the FFT tables,
 // FP32 ring coefficients and maps.  The Legendre tables are made on first use
 // (dm_split.cu, dm_legendre_tc.cu, dm_legendre_otf.cu).
 cudaError_t setup_fp32(dm_plan *p) {

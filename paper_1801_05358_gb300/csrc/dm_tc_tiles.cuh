@@ -16,7 +16,9 @@ constexpr int TILE_A = 4096;  // 128 x 16 BF16
 
 // K steps before the first Legendre value of a tile that reaches 2^-60 are
 // left out: the evanescent region (m well above l sin theta), where a value
-// this small changes no bit of an FP32 sum with those of the other rings.  It
+// this small changes no bit of an FP32 sum with those of the other rings.  (The
+// stored tiles and FP32 tables, whose list visible_steps makes, leave out what
+// lies 2^-55 below the largest value of its ring too.)  It
 // holds 10 % of the K steps at nside 256 / lmax 512, 20 % at nside 512 / 1024.
 constexpr int TC_FLOOR_EXP = -60;
 

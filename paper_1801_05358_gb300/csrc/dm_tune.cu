@@ -30,7 +30,7 @@ std::string tune_key(const dm_plan *p) {
   if (cudaGetDeviceProperties(&prop, p->device) == cudaSuccess)
     dev = std::string(prop.name) + "/" + std::to_string(prop.multiProcessorCount);
   return dev + "|" + std::to_string(p->nside) + "|" + std::to_string(p->lmax) + "|" + std::to_string(p->batch) +
-         "|" + std::to_string((int)p->prec) + "|" + std::to_string((int)p->ff_legendre) + "|" +
+         "|" + std::to_string((int)p->prec) + "|" +
          std::to_string((int)(p->use_tc && tc_batch_ok(p->batch))) + "|" + std::to_string(p->tc_gen) + "|" +
          std::to_string((int)p->ring_fft);
 }

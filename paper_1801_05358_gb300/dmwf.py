@@ -373,7 +373,7 @@ class Plan:
         self._check(lib().dm_set_analysis_slots(self.h, int(slots)))
 
     def set_ff_slab_bytes(self, nbytes):
-        """Largest per-slab table of the float-float stages when the plan keeps no full FP32 tables."""
+        """Largest slab of Legendre digits; the plan then keeps no whole table."""
         self._check(lib().dm_set_ff_slab_bytes(self.h, int(nbytes)))
 
     def set_ring_radix(self, lr):
