@@ -20,7 +20,11 @@ namespace {
 // (below the line), B 3 92 and 102, B 9 199 and 186; nside 128 (above), B 1 124
 // and 91, B 9 271 and 235.
 constexpr int64_t SYN32_MAX = 48 * 1024;
-// The analysis of more than two right-hand sides runs here below this many.
+// The analysis of more than two right-hand sides runs here below this many, and
+// of more than 16 where four of them share a block.  map2alm, k_ana32 and split
+// products: nside 64 / lmax 128, B 12 79.9 and 89.1 us, B 40 231 and 246, B 50
+// (two share) 340 and 304, B 25 (each alone) 174 and 167; nside 64 / lmax 190
+// (the line), B 12 101 and 115.
 constexpr int64_t ANA32_MAX = 24 * 1024;
 
 constexpr int SYN_THREADS = 128;
@@ -107,10 +111,40 @@ __global__ void __launch_bounds__(SYN_THREADS) k_syn32(const float *__restrict__
 }
 
 constexpr int A32_WARPS = 8;
-constexpr int A32_ROWS = 4;    // multipoles per warp and pass
+// multipoles per warp and pass: with four right-hand sides two, so that two blocks share an SM
+__host__ __device__ constexpr int a32_rows(int nb) { return nb == 4 ? 2 : 4; }
 constexpr int A32_LB = 128;    // multipoles per block
 
-// Analysis: each warp takes four multipoles and all ring pairs, 16 bytes per
+// The sums over a warp of N values a lane, each left in the lanes that the
+// folding assigns it to: every step halves the values that a lane still holds
+// (N = 48: 48 shuffles instead of 240 for a tree each, more than the products
+// of 64 ring pairs); what is added to what is as in the trees.
+template <int N, int O>
+__device__ __forceinline__ void fold_sums(float *a, int lane, int &first) {
+  if constexpr (O > 0) {
+    if constexpr (N % 2 == 0) {
+      const bool up = lane & O;
+#pragma unroll
+      for (int i = 0; i < N / 2; ++i) {
+        const float keep = up ? a[N / 2 + i] : a[i], give = up ? a[i] : a[N / 2 + i];
+        a[i] = keep + __shfl_xor_sync(0xffffffffu, give, O);
+      }
+      if (up) first += N / 2;
+      fold_sums<N / 2, O / 2>(a, lane, first);
+    } else {
+#pragma unroll
+      for (int i = 0; i < N; ++i) a[i] += __shfl_xor_sync(0xffffffffu, a[i], O);
+      fold_sums<N, O / 2>(a, lane, first);
+    }
+  }
+}
+// values that a lane is left with, and the lane bits of those that share them
+__host__ __device__ constexpr int folded(int n, int o) { return o == 0 ? n : folded(n % 2 ? n : n / 2, o / 2); }
+__host__ __device__ constexpr int sharers(int n, int o) {
+  return o == 0 ? 0 : (n % 2 ? o : 0) | sharers(n % 2 ? n : n / 2, o / 2);
+}
+
+// Analysis: each warp takes a32_rows multipoles and all ring pairs, 16 bytes per
 // lane, function and multipole (12 loads in flight); values below
 // 2^TC_FLOOR_EXP (the evanescent region) are not read.  At nside 256, one
 // right-hand side: 105 us, split products 203.  grid (batch / NB, blocks of
@@ -118,12 +152,13 @@ constexpr int A32_LB = 128;    // multipoles per block
 // find them in L2; dynamic shared memory [NB][12][ldp]:
 // (T, Q, U) x (even re, im, odd re, im) of every ring pair.
 template <int NB>
-__global__ void __launch_bounds__(32 * A32_WARPS) k_ana32(const float *__restrict__ tab, int ldt,
+__global__ void __launch_bounds__(32 * A32_WARPS, NB == 4 ? 2 : 0) k_ana32(const float *__restrict__ tab, int ldt,
                                                           const int *__restrict__ ks,
                                                           int npt, int nlt, const float2 *__restrict__ rc,
                                                           float2 *__restrict__ out, int lmax, int mmax, int npairs,
                                                           int64_t nalm, int ldp,
                                                           const SolveState *__restrict__ state) {
+  constexpr int A32_ROWS = a32_rows(NB);
   extern __shared__ __align__(16) float G[];
   const int m = blockIdx.z, lb = blockIdx.y * A32_LB;  // l - m of the block's first multipole
   if (lb > lmax - m) return;
@@ -135,7 +170,6 @@ __global__ void __launch_bounds__(32 * A32_WARPS) k_ana32(const float *__restric
   for (int k = 0; k < NB && !any; ++k) any = !state[k].done;
   if (!any) return;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int64_t fs = (int64_t)(mmax + 1) * npairs * 2;
   // first ring pair visible at the block's last multipole, down to a multiple of 128
   const int64_t kr = (int64_t)m * (npt + nlt) + npt + min(nlt - 1, lb / 128), ks2 = (int64_t)(mmax + 1) * (npt + nlt);
   const int p0 = min(16 * min(ks[kr], ks[kr + ks2]), npairs - 1) & ~127;
@@ -198,21 +232,35 @@ __global__ void __launch_bounds__(32 * A32_WARPS) k_ana32(const float *__restric
         }
       }
     }
+    if constexpr (NB > 1) {
+      constexpr int V = A32_ROWS * NB * 6;
+      float *v = &acc[0][0][0];
+      int first = 0;
+      fold_sums<V, 16>(v, lane, first);
+      if ((lane & sharers(V, 16)) == 0)
 #pragma unroll
-    for (int r = 0; r < A32_ROWS; ++r)
-#pragma unroll
-      for (int k = 0; k < NB; ++k) {
-#pragma unroll
-        for (int c = 0; c < 6; ++c)
-#pragma unroll
-          for (int o = 16; o > 0; o >>= 1) acc[r][k][c] += __shfl_xor_sync(0xffffffffu, acc[r][k][c], o);
-        if (lane == 0 && r0 + r <= lmax - m && (state == nullptr || !state[k].done)) {
-          float2 *o = out + (int64_t)k * 3 * nalm + base + m + r0 + r;
-          o[0] = make_float2(acc[r][k][0], acc[r][k][1]);
-          o[nalm] = make_float2(acc[r][k][2], acc[r][k][3]);
-          o[2 * nalm] = make_float2(acc[r][k][4], acc[r][k][5]);
+        for (int i = 0; i < folded(V, 16); ++i) {
+          const int r = (first + i) / (6 * NB), k = (first + i) / 6 % NB, c = (first + i) % 6;
+          if (r0 + r <= lmax - m && (state == nullptr || !state[k].done))
+            reinterpret_cast<float *>(out)[2 * ((int64_t)(3 * k + c / 2) * nalm + base + m + r0 + r) + c % 2] = v[i];
         }
-      }
+    } else {
+#pragma unroll
+      for (int r = 0; r < A32_ROWS; ++r)
+#pragma unroll
+        for (int k = 0; k < NB; ++k) {
+#pragma unroll
+          for (int c = 0; c < 6; ++c)
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) acc[r][k][c] += __shfl_xor_sync(0xffffffffu, acc[r][k][c], o);
+          if (lane == 0 && r0 + r <= lmax - m && (state == nullptr || !state[k].done)) {
+            float2 *o = out + (int64_t)k * 3 * nalm + base + m + r0 + r;
+            o[0] = make_float2(acc[r][k][0], acc[r][k][1]);
+            o[nalm] = make_float2(acc[r][k][2], acc[r][k][3]);
+            o[2 * nalm] = make_float2(acc[r][k][4], acc[r][k][5]);
+          }
+        }
+    }
   }
 }
 
@@ -274,7 +322,8 @@ bool syn32_ready(dm_plan *p, cudaStream_t st) {
 }
 
 bool ana32_ready(dm_plan *p, cudaStream_t st) {
-  if (p->batch > 2 && order_entries(p) >= ANA32_MAX && !instead(p)) return false;
+  const bool few = p->batch <= 16 || p->batch % 4 == 0;
+  if (p->batch > 2 && (order_entries(p) >= ANA32_MAX || !few) && !instead(p)) return false;
   return ana32_smem(p, 1) <= ANA32_SMEM && tables(p, st);
 }
 
@@ -293,7 +342,8 @@ cudaError_t syn32(dm_plan *p, const double2 *alm, const float2 *e32, cudaStream_
 cudaError_t ana32(dm_plan *p, cudaStream_t st) {
   const SolveState *state = p->state_active ? p->state : nullptr;
   const int npt = (p->npairs + 127) / 128, nlt = (p->lmax + 128) / 128;
-  const int nb = p->batch % 2 || ana32_smem(p, 2) > ANA32_SMEM ? 1 : 2;
+  int nb = p->batch % 4 == 0 && p->batch >= 8 ? 4 : p->batch % 2 == 0 ? 2 : 1;
+  while (ana32_smem(p, nb) > ANA32_SMEM) nb /= 2;
   auto go = [&](auto kern) {
     const size_t sm = ana32_smem(p, nb);
     if (cudaError_t e = dyn_smem_allow(kern, sm)) return e;
@@ -302,7 +352,7 @@ cudaError_t ana32(dm_plan *p, cudaStream_t st) {
         npt * 128, state);
     return cudaGetLastError();
   };
-  return nb == 1 ? go(k_ana32<1>) : go(k_ana32<2>);
+  return nb == 1 ? go(k_ana32<1>) : nb == 2 ? go(k_ana32<2>) : go(k_ana32<4>);
 }
 
 }  // namespace dmwf
