@@ -47,9 +47,19 @@ constexpr size_t DFT_SMEM = 224u << 10;  // dynamic shared memory that a block m
 // faster: a stage here is five dependent launches of few tiles, there one to
 // three.  64 iterations of a solve, products against FFTs: nside 16, B 1 22.1
 // and 11.5 ms; nside 64, B 1 23.8 and 19.7; nside 64, B 2 (the line) 26.7 and
-// 30.0; nside 32, B 8 (the line) 28.9 and 29.8; nside 128, B 2 58 and 101;
-// flat N = 256, B 1 15.6 and 13.3, B 2 20.9 and 24.1; N = 1024, B 4 387 and 510.
+// 30.0; nside 32, B 8 (the line) 28.9 and 29.8; nside 128, B 2 58 and 101.
 constexpr int64_t DFT_MIN_PIXELS = 12 * 64 * 64 * 2;
+// The rows and columns of a flat patch have no Bluestein rings, and on a small
+// grid nothing makes up for the passes around the products: from 2^18 pixels
+// on, of grids below 256 from 2^18 (256 / N)^2, below 128 never.  20 iterations
+// of a solve, products against FFTs: N = 64, B 24 5.5 and 3.7 ms, B 400 54 and
+// 48; N = 128, B 24 8.4 and 8.1, B 100 28.6 and 30.5 (the line: 64); N = 256, B 2
+// 3.5 and 3.2, B 4 (the line) 4.9 and 5.0, B 8 7.4 and 8.4; N = 512, B 1 4.6 and
+// 5.0; N = 1024, B 1 12.7 and 18.2.
+static bool flat_products(int N, int batch) {
+  const int64_t px = (int64_t)N * N * batch, line = (int64_t)1 << 18;
+  return N >= 256 ? px >= line : N >= 128 && px * N * N >= line * 256 * 256;
+}
 constexpr size_t DFT_SCRATCH = (size_t)1 << 30;  // column digits of one direction and group of right-hand sides
 
 // A matrix set: the rings of one length and shift.
@@ -1196,7 +1206,8 @@ cudaError_t dft_use(dm_plan *p, cudaStream_t st, bool *use) {
   DftTables *T = p->dft;
   *use = false;
   if (!T || T->disabled || p->ring_fft || p->tune_only_class >= 0) return cudaSuccess;
-  if (p->npix * p->batch < DFT_MIN_PIXELS || std::max(xinv_smem(p), pix_smem(p)) > DFT_SMEM) return cudaSuccess;
+  if (p->flat ? !flat_products(p->flatN, p->batch) : p->npix * p->batch < DFT_MIN_PIXELS) return cudaSuccess;
+  if (std::max(xinv_smem(p), pix_smem(p)) > DFT_SMEM) return cudaSuccess;
   const int B = p->batch;
   auto found = [&](int gb) {
     for (int b0 = 0; b0 < B; b0 += gb)

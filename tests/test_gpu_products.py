@@ -165,3 +165,29 @@ def test_mixed_small_batches(orc, nside, lmax, B):
     for b in (0, B - 1):
         assert rel(gm[b], orc.alm2map(nside, lmax, alm[b])) < 2e-6
         assert rel(ga[b], orc.map2alm(nside, lmax, maps[b])) < 2e-6
+
+
+# Flat patches on both sides of the size rule of their products: at the line and
+# one right-hand side below it, and a grid that never takes them.  The matrices
+# show in the plan's bytes; either way the transforms agree with the FFT kernels.
+@pytest.mark.parametrize("N,B,products", [(64, 70, False), (128, 63, False), (128, 64, True), (256, 3, False),
+                                          (256, 4, True), (512, 1, True)])
+def test_flat_size_rule(N, B, products):
+    rng = np.random.default_rng(N + B)
+    d = dev(rng.standard_normal((B, 3, N * N)))
+    out = []
+    for fft in (False, True):
+        p = dmwf.FlatPlan(N, W.FLAT_L, B)
+        if fft:
+            p.set_ring_radix(0)
+        held = p.info()["workspace_bytes"]
+        a, m = torch.zeros((B, 3, N * N // 2, 2), dtype=torch.float64, device="cuda"), torch.zeros_like(d)
+        p.map2alm(d, a)
+        p.alm2map(a, m)
+        torch.cuda.synchronize()
+        assert (p.info()["workspace_bytes"] > held) == (products and not fft)
+        out.append((a.cpu().numpy(), m.cpu().numpy()))
+        p.close()
+    for x, y in zip(*out):
+        for b in (0, B - 1):
+            assert rel(x[b], y[b]) < 1e-12
