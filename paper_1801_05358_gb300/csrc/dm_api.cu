@@ -47,7 +47,7 @@ void free_all(dm_plan *p) {
                   p->filt, p->w, p->mask, p->sigma, p->rc, p->a, p->apart, p->wd, p->norms, p->state,
                   p->lev, p->tmpmap, p->tmpmap2, p->tmpalm, p->seeds_dev, p->coef_tmp,
                   p->rc32, p->apart32, p->s32, p->w32, p->wd32, p->phase32, p->bhat32, p->twid32,
-                  p->a_hi, p->g_hi, p->shi32, p->s64, p->rhi, p->tc_err, p->ring_order, p->pair_order,
+                  p->a_hi, p->g_hi, p->shi32, p->s64, p->rhi, p->ring_order, p->pair_order,
                   p->tc_synA[0], p->tc_synA[1], p->tc_anaA[0], p->tc_anaA[1], p->tc_soff, p->tc_aoff, p->tc_ks, p->gen_ks, p->tab32,
                   p->tc_synB[0], p->tc_synB[1], p->e32, p->c32, p->clev, p->filt32,
                   p->twr, p->twr32, p->chirp, p->chirp32, p->wcov, p->diag_tab, p->diag_alm, p->diag_part,
@@ -248,10 +248,16 @@ dm_status clear_waits(dm_plan *p, cudaStream_t st) {
   return DM_OK;
 }
 dm_status check_waits(dm_plan *p, cudaStream_t st) {
-  int gave_up = 0;
-  DM_CU(cudaMemcpyAsync(&gave_up, p->tc_err, sizeof(int), cudaMemcpyDeviceToHost, st), "wait flag");
+  int flag = 0;
+  DM_CU(cudaMemcpyAsync(&flag, p->tc_err, sizeof(int), cudaMemcpyDeviceToHost, st), "wait flag");
   DM_CU(cudaStreamSynchronize(st), "wait flag");
-  return gave_up ? fail(p, DM_ETIMEOUT, "a tensor-core pipeline wait gave up") : DM_OK;
+  return flag ? fail(p, DM_ETIMEOUT, "a tensor-core pipeline wait gave up") : DM_OK;
+}
+
+static bool gave_up(const std::vector<SolveState> &hs) {  // the flag behind a copy of the states
+  int flag;
+  memcpy(&flag, &hs.back(), sizeof(int));
+  return flag != 0;
 }
 
 dm_status solve_begin(dm_plan *p, const double *d, cudaStream_t st) {
@@ -284,7 +290,7 @@ dm_status solve_iterate(dm_plan *p, long max_iters, int *all_done, cudaStream_t 
     p->ev.resize(6 * every);
     for (int i = have; i < 6 * every; ++i) cudaEventCreate(&p->ev[i]);
   }
-  std::vector<SolveState> hs(p->batch);
+  std::vector<SolveState> hs(p->batch + 1);  // and the wait flag
   const bool mixed = p->prec != DM_FP64;
   long done_iters = 0;
   *all_done = 0;
@@ -298,12 +304,11 @@ dm_status solve_iterate(dm_plan *p, long max_iters, int *all_done, cudaStream_t 
     done_iters += window;
     p->iters_launched += window;
     p->since_anchor += (int)window;
-    cudaError_t e = cudaMemcpyAsync(hs.data(), p->state, sizeof(SolveState) * p->batch, cudaMemcpyDeviceToHost, st);
-    int tcerr = 0;
-    if (!e) e = cudaMemcpyAsync(&tcerr, p->tc_err, sizeof(int), cudaMemcpyDeviceToHost, st);
+    cudaError_t e = cudaMemcpyAsync(hs.data(), p->state, sizeof(SolveState) * p->batch + sizeof(int),
+                                    cudaMemcpyDeviceToHost, st);
     if (!e) e = cudaStreamSynchronize(st);
     if (e) return cuda_fail(p, e, "poll state");
-    if (tcerr) return fail(p, DM_ETIMEOUT, "a tensor-core pipeline wait gave up");
+    if (gave_up(hs)) return fail(p, DM_ETIMEOUT, "a tensor-core pipeline wait gave up");
     if (p->prof_on) {
       for (long k = 0; k < window; ++k) {
         float t[5];
@@ -317,7 +322,7 @@ dm_status solve_iterate(dm_plan *p, long max_iters, int *all_done, cudaStream_t 
       }
     }
     bool all = true;
-    for (auto &s : hs) all = all && s.done;
+    for (int b = 0; b < p->batch; ++b) all = all && hs[b].done;
     if (all) {
       *all_done = 1;
       break;
@@ -396,8 +401,8 @@ namespace {
 // solve's begin and end events; *rs becomes DM_ETIMEOUT when a wait gave up in
 // the solve, its last synthesis or the diagnostics.
 void fill_stats(dm_plan *p, dm_stats *stats, dm_status *rs, cudaStream_t st) {
-  std::vector<SolveState> hs(p->batch);
-  cudaMemcpy(hs.data(), p->state, sizeof(SolveState) * p->batch, cudaMemcpyDeviceToHost);
+  std::vector<SolveState> hs(p->batch + 1);  // and the wait flag
+  cudaMemcpy(hs.data(), p->state, sizeof(SolveState) * p->batch + sizeof(int), cudaMemcpyDeviceToHost);
   std::vector<double> resid(p->batch, NAN), chi2(p->batch, NAN);
   float ms = NAN;
   if (stats) {
@@ -475,7 +480,10 @@ dm_status plan_workspace(dm_plan *p, dm_plan **out) {
   if (!p->flat && (e = dalloc(p, &p->apart, (size_t)B * p->nslot * 3 * p->nalm))) return bad(e, "alloc apart");
   if ((e = dalloc(p, &p->wd, (size_t)B * n3))) return bad(e, "alloc wd");
   if ((e = dalloc(p, &p->norms, (size_t)B * 3 * p->nrings * 2))) return bad(e, "alloc norms");
-  if ((e = dalloc(p, &p->state, (size_t)B))) return bad(e, "alloc state");
+  // one more: the wait flag, so that one copy brings the states and it
+  if ((e = dalloc(p, &p->state, (size_t)B + 1))) return bad(e, "alloc state");
+  p->tc_err = reinterpret_cast<int *>(p->state + B);
+  cudaMemset(p->state, 0, sizeof(SolveState) * ((size_t)B + 1));
   if ((e = dalloc(p, &p->lev, (size_t)B))) return bad(e, "alloc lev");
   if ((e = dalloc(p, &p->tmpmap, (size_t)B * n3))) return bad(e, "alloc tmp");
   if ((e = dalloc(p, &p->tmpmap2, (size_t)B * n3))) return bad(e, "alloc tmp");
@@ -484,8 +492,6 @@ dm_status plan_workspace(dm_plan *p, dm_plan **out) {
   if ((e = dalloc(p, &p->coef_tmp, 4 * (size_t)L))) return bad(e, "alloc coef");
   if ((e = dalloc(p, &p->s64, (size_t)B * n3))) return bad(e, "alloc s");
   if ((e = dalloc(p, &p->rhi, (size_t)B * n3))) return bad(e, "alloc rhi");
-  if ((e = dalloc(p, &p->tc_err, 1))) return bad(e, "alloc");
-  cudaMemset(p->tc_err, 0, sizeof(int));
   if (!p->flat) split_new(p);
   dft_new(p);
   if ((e = cudaEventCreate(&p->ev_begin)) || (e = cudaEventCreate(&p->ev_end))) return bad(e, "events");

@@ -154,7 +154,7 @@ struct dm_plan {
   int nslot = 0;                // chunk slots of apart per RHS (nslot < nchunk: the analysis runs in waves)
   double *wd = nullptr;         // [B][3][npix] w * d
   double *norms = nullptr;      // [B][3][nrings][2] Cauchy partial sums
-  dmwf::SolveState *state = nullptr;   // [B]
+  dmwf::SolveState *state = nullptr;   // [B], then tc_err
   dmwf::LevelDev *lev = nullptr;         // [B] per-RHS stopping schedule
   std::vector<double> eps_final_rhs;     // per RHS (serving sets it per request)
   double *tmpmap = nullptr;     // [B][3][npix] scratch map (CR, host-buffer entry)
@@ -203,7 +203,7 @@ struct dm_plan {
   bool anchor_active = false;
   int anchor_every = 256;
   bool use_tc = true;           // tcgen05 Legendre stages when the batch allows
-  int *tc_err = nullptr;        // device flag: a bounded tensor-core wait gave up
+  int *tc_err = nullptr;        // device flag behind the states: a bounded tensor-core wait gave up
   int tc_withhold = 0;          // test hook: one withheld arrival in the spin-0 analysis (dm_test_tc_withhold)
   // tiled BF16 hi/lo Legendre tables of the tensor-core stages ([0] = lambda, [1] = lam+/lam-)
   unsigned char *tc_synA[2] = {nullptr, nullptr}, *tc_anaA[2] = {nullptr, nullptr};

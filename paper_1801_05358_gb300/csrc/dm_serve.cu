@@ -74,9 +74,9 @@ struct Pool {
   size_t reserved = 0;          // bytes of the memory budget it holds
   cudaStream_t stream = nullptr;
   std::vector<Slot> slots;
-  // a round in flight: its iterations and the copies of the solver states into
-  // hs and of the plan's wait flag into gave_up (pinned) are enqueued, done_ev
-  // is recorded after them
+  // a round in flight: its iterations and the copy of the solver states and of
+  // the plan's wait flag behind them into hs and gave_up (pinned, one block) are
+  // enqueued, done_ev is recorded after them
   bool inflight = false;
   dm_status round_status = DM_OK;  // of enqueuing it
   int *gave_up = nullptr;
@@ -236,7 +236,6 @@ dm_precision request_prec(const dm_server *S, const Request &r) {
 void release_pool(Pool *q) {
   if (q->done_ev) cudaEventDestroy(q->done_ev);
   if (q->hs) cudaFreeHost(q->hs);
-  if (q->gave_up) cudaFreeHost(q->gave_up);
   cudaStreamDestroy(q->stream);
   dm_plan_destroy(q->plan);
 }
@@ -333,15 +332,15 @@ Pool *make_pool(dm_server *S, const Request &r, dm_status *why) {
     return nullptr;
   }
   if (cudaEventCreateWithFlags(&pool->done_ev, cudaEventDisableTiming) != cudaSuccess ||
-      cudaMallocHost(&pool->hs, sizeof(SolveState) * slots) != cudaSuccess ||
-      cudaMallocHost(&pool->gave_up, sizeof(int)) != cudaSuccess) {
+      cudaMallocHost(&pool->hs, sizeof(SolveState) * (slots + 1)) != cudaSuccess) {
     if (pool->done_ev) cudaEventDestroy(pool->done_ev);
-    if (pool->hs) cudaFreeHost(pool->hs);
     cudaStreamDestroy(pool->stream);
     dm_plan_destroy(p);
     *why = DM_ECUDA;
     return nullptr;
   }
+  pool->gave_up = reinterpret_cast<int *>(pool->hs + slots);
+  *pool->gave_up = 0;
   pool->slots.resize(slots);
   k_mark_done<<<(slots + 127) / 128, 128, 0, pool->stream>>>(p->state, slots);
   p->session = true;
@@ -570,9 +569,8 @@ void worker_main(dm_server *S) {
         if (e) q->round_status = e == cudaErrorMemoryAllocation ? DM_ENOMEM : DM_ECUDA;
       }
       if (S->test_wait == 1) test_wait(S, q);
-      cudaMemcpyAsync(q->hs, q->plan->state, sizeof(SolveState) * q->slots.size(), cudaMemcpyDeviceToHost,
-                      q->stream);
-      cudaMemcpyAsync(q->gave_up, q->plan->tc_err, sizeof(int), cudaMemcpyDeviceToHost, q->stream);
+      cudaMemcpyAsync(q->hs, q->plan->state, sizeof(SolveState) * q->slots.size() + sizeof(int),
+                      cudaMemcpyDeviceToHost, q->stream);
       cudaEventRecord(q->done_ev, q->stream);
       q->inflight = true;
     }
