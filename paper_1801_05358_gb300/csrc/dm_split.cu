@@ -733,7 +733,8 @@ bool split_whole(const dm_plan *p) {
   const SplitTables *T = p->split;
   if (!T || T->disabled) return false;
   if (T->dig) return T->full;
-  return !p->ffs_cap_set && split_table_bytes(p->lmax, p->mmax, p->npairs) <= (size_t)p->split_cap;
+  const int64_t bytes = (int64_t)split_table_bytes(p->lmax, p->mmax, p->npairs);
+  return bytes <= p->ffs_cap || (!p->ffs_cap_set && bytes <= p->split_cap);  // (one slab may hold all of it)
 }
 
 size_t split_order_bytes(int lmax, int npairs) {
