@@ -286,8 +286,10 @@ bool tables(dm_plan *p, cudaStream_t st) {
     return false;
   }
   if (p->tab32_short.lasts(p)) return false;
-  const double digits = std::min((double)p->ffs_cap, (double)split_table_bytes(p->lmax, p->mmax, p->npairs)) +
-                        (double)split_scratch_bytes(p->lmax, p->npairs, p->batch, p->scratch_cap);
+  const double digits =
+      split_bytes(p) > 0 ? 0.0  // made already
+                         : std::min((double)p->ffs_cap, (double)split_table_bytes(p->lmax, p->mmax, p->npairs)) +
+                               (double)split_scratch_bytes(p->lmax, p->npairs, p->batch, p->scratch_cap);
   if (bytes + digits > (double)table_room(p)) {
     p->tab32_short.note(p);
     return false;

@@ -106,3 +106,25 @@ def test_mixed_batches(orc, nside, lmax, B):
     p.set_precision(dmwf.DM_MIXED_FP32)
     _check(orc, p, nside, lmax, B, 2e-6)
     p.close()
+
+
+# The anchors' digits are made first in a solve: room for them is not asked for again.
+def test_tables_beside_the_anchors_digits():
+    nside, lmax, B = 128, 256, 3
+    npix = 12 * nside * nside
+    p = dmwf.Plan(nside, lmax, B)
+    p.set_precision(dmwf.DM_MIXED_FP32)
+    p.set_ring_radix(3)
+    p.set_diagnostics(False)
+    p.set_ff_slab_bytes(2_000_000)
+    p.set_noise_mask(np.full((3, npix), 0.5), np.ones(npix, np.uint8))
+    cl = np.zeros((4, lmax + 1))
+    cl[:3, 2:] = 1.0 / np.arange(2, lmax + 1) ** 2.0
+    p.set_spectra(cl)
+    p.set_schedule(lambda0=10.0, n_levels=1, iters_per_level=2, check_every=2)
+    p.test_table_memory(_table_bytes(nside, lmax))
+    held = p.info()["workspace_bytes"]
+    d = dev(W.random_maps(nside, B, 90))
+    p.wiener_filter(d, torch.zeros_like(d))
+    assert p.info()["workspace_bytes"] - held > _table_bytes(nside, lmax)
+    p.close()
