@@ -20,11 +20,10 @@ namespace {
 // (below the line), B 3 92 and 102, B 9 199 and 186; nside 128 (above), B 1 124
 // and 91, B 9 271 and 235.
 constexpr int64_t SYN32_MAX = 48 * 1024;
-// The analysis of more than two right-hand sides runs here below this many, and
-// of more than 16 where four of them share a block.  map2alm, k_ana32 and split
-// products: nside 64 / lmax 128, B 12 79.9 and 89.1 us, B 40 231 and 246, B 50
-// (two share) 340 and 304, B 25 (each alone) 174 and 167; nside 64 / lmax 190
-// (the line), B 12 101 and 115.
+// The analysis of more than two right-hand sides runs here below this many.
+// map2alm, k_ana32 and split products: nside 64 / lmax 128, B 12 79.9 and 89.1 us,
+// B 25 149 and 167, B 50 291 and 304; nside 64 / lmax 190 (the line), B 12 102 and
+// 115, B 17 152 and 155, B 50 402 and 393.
 constexpr int64_t ANA32_MAX = 24 * 1024;
 
 constexpr int SYN_THREADS = 128;
@@ -156,18 +155,18 @@ __global__ void __launch_bounds__(32 * A32_WARPS, NB == 4 ? 2 : 0) k_ana32(const
                                                           const int *__restrict__ ks,
                                                           int npt, int nlt, const float2 *__restrict__ rc,
                                                           float2 *__restrict__ out, int lmax, int mmax, int npairs,
-                                                          int64_t nalm, int ldp,
+                                                          int64_t nalm, int ldp, int batch,
                                                           const SolveState *__restrict__ state) {
   constexpr int A32_ROWS = a32_rows(NB);
   extern __shared__ __align__(16) float G[];
   const int m = blockIdx.z, lb = blockIdx.y * A32_LB;  // l - m of the block's first multipole
   if (lb > lmax - m) return;
-  const int b0 = blockIdx.x * NB;
+  const int b0 = blockIdx.x * NB, nb = NB == 4 ? min(NB, batch - b0) : NB;  // (of four the last block may hold fewer)
   rc += (int64_t)b0 * 3 * (mmax + 1) * npairs * 2;
   out += (int64_t)b0 * 3 * nalm;
   if (state != nullptr) state += b0;
   bool any = state == nullptr;
-  for (int k = 0; k < NB && !any; ++k) any = !state[k].done;
+  for (int k = 0; k < nb && !any; ++k) any = !state[k].done;
   if (!any) return;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   // first ring pair visible at the block's last multipole, down to a multiple of 128
@@ -176,7 +175,7 @@ __global__ void __launch_bounds__(32 * A32_WARPS, NB == 4 ? 2 : 0) k_ana32(const
   for (int i = tid; i < (ldp - p0) * 3 * NB; i += 32 * A32_WARPS) {
     const int p = p0 + i % (ldp - p0), kf = i / (ldp - p0);
     float2 n = make_float2(0.f, 0.f), s = n;
-    if (p < npairs) {
+    if (p < npairs && kf < 3 * nb) {
       const float2 *g = rc + ((int64_t)kf * (mmax + 1) + m) * npairs * 2 + 2 * p;
       n = g[0];
       if (p != npairs - 1) s = g[1];
@@ -241,7 +240,7 @@ __global__ void __launch_bounds__(32 * A32_WARPS, NB == 4 ? 2 : 0) k_ana32(const
 #pragma unroll
         for (int i = 0; i < folded(V, 16); ++i) {
           const int r = (first + i) / (6 * NB), k = (first + i) / 6 % NB, c = (first + i) % 6;
-          if (r0 + r <= lmax - m && (state == nullptr || !state[k].done))
+          if (r0 + r <= lmax - m && k < nb && (state == nullptr || !state[k].done))
             reinterpret_cast<float *>(out)[2 * ((int64_t)(3 * k + c / 2) * nalm + base + m + r0 + r) + c % 2] = v[i];
         }
     } else {
@@ -324,8 +323,7 @@ bool syn32_ready(dm_plan *p, cudaStream_t st) {
 }
 
 bool ana32_ready(dm_plan *p, cudaStream_t st) {
-  const bool few = p->batch <= 16 || p->batch % 4 == 0;
-  if (p->batch > 2 && (order_entries(p) >= ANA32_MAX || !few) && !instead(p)) return false;
+  if (p->batch > 2 && order_entries(p) >= ANA32_MAX && !instead(p)) return false;
   return ana32_smem(p, 1) <= ANA32_SMEM && tables(p, st);
 }
 
@@ -344,14 +342,17 @@ cudaError_t syn32(dm_plan *p, const double2 *alm, const float2 *e32, cudaStream_
 cudaError_t ana32(dm_plan *p, cudaStream_t st) {
   const SolveState *state = p->state_active ? p->state : nullptr;
   const int npt = (p->npairs + 127) / 128, nlt = (p->lmax + 128) / 128;
-  int nb = p->batch % 4 == 0 && p->batch >= 8 ? 4 : p->batch % 2 == 0 ? 2 : 1;
+  // four where that still makes 200 blocks for the 152 SMs (map2alm, four a block and one or two: nside 32, B 9, 195
+  // blocks, 34.9 and 31.3 us; nside 21, B 25, 301, 45.1 and 48.4; nside 8, B 50, 221, 30.7 and 34.8)
+  const int64_t blocks4 = (int64_t)((p->batch + 3) / 4) * (p->mmax + 1) * ((p->lmax + A32_LB) / A32_LB);
+  int nb = p->batch >= 8 && blocks4 >= 200 ? 4 : p->batch % 2 == 0 ? 2 : 1;
   while (ana32_smem(p, nb) > ANA32_SMEM) nb /= 2;
   auto go = [&](auto kern) {
     const size_t sm = ana32_smem(p, nb);
     if (cudaError_t e = dyn_smem_allow(kern, sm)) return e;
-    kern<<<dim3(p->batch / nb, (p->lmax + A32_LB) / A32_LB, p->mmax + 1), 32 * A32_WARPS, sm, st>>>(
+    kern<<<dim3((p->batch + nb - 1) / nb, (p->lmax + A32_LB) / A32_LB, p->mmax + 1), 32 * A32_WARPS, sm, st>>>(
         p->tab32, table_ld(p), p->tc_ks, npt, nlt, p->rc32, p->apart32, p->lmax, p->mmax, p->npairs, p->nalm,
-        npt * 128, state);
+        npt * 128, p->batch, state);
     return cudaGetLastError();
   };
   return nb == 1 ? go(k_ana32<1>) : nb == 2 ? go(k_ana32<2>) : go(k_ana32<4>);

@@ -96,11 +96,11 @@ def test_mixed_solve_in_slabs(orc):
         assert rel(s[b].cpu().numpy(), ref["s"]) < 1e-5
 
 
-# The default choice of the analysis: four right-hand sides a block from eight
-# on, two or one of other batches, digit products from 17 on that four do not
-# divide; ring pairs within one warp's pass and in several, odd rows at the end.
+# The default choice of the analysis: four right-hand sides a block from eight on
+# where that fills the chip (the last block with one to four), two or one else;
+# ring pairs within one warp's pass and in several, odd rows at the end.
 @pytest.mark.parametrize("nside,lmax,B", [(2, 4, 12), (23, 60, 12), (64, 190, 12), (33, 67, 20), (64, 128, 14),
-                                          (64, 128, 18), (33, 70, 17), (16, 33, 4)])
+                                          (64, 128, 19), (33, 70, 17), (16, 33, 4), (16, 33, 17), (16, 33, 50)])
 def test_mixed_batches(orc, nside, lmax, B):
     p = dmwf.Plan(nside, lmax, B)
     p.set_precision(dmwf.DM_MIXED_FP32)
